@@ -12,9 +12,12 @@
 // P passes costs P - 1 shared-memory round trips and no global traffic.
 //
 // Twiddles: per-pass tables built on the host in long double, laid out
-// [pass][r][j] (r = 0..R-1, j = 0..NS-1; entries r = 0 are 1), so the lanes
-// of a warp, which hold consecutive j, read consecutive entries.  Kernels
-// copy the tables to shared memory first.  No device trigonometry is used.
+// [pass][r][j] (j = 0..NS-1), so the lanes of a warp, which hold consecutive
+// j, read consecutive entries.  FP32: r = 0..R-1, entry r the twiddle of
+// input r (r = 0 is 1), multiplied in before a constant-root butterfly.
+// FP64: R / 2 entries per j, the roots of the pass's radix-2 stages with the
+// twiddle folded in (fused_dft).  Kernels copy the tables to shared memory
+// first.  No device trigonometry is used.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -150,6 +153,19 @@ __device__ __forceinline__ C twiddle_small(C a, int k, int len) {
   return cmul(a, mk<C>(cr, DIR * sr));
 }
 
+// Radix-2 butterfly with the root folded in: u' = u + w v, v' = u - w v with
+// w = (wx, DIR < 0 ? wy : -wy), as u' by four fused multiply-adds and
+// v' = 2 u - u' by two more: 6 instructions against 8 for the product
+// followed by two complex additions.
+template <int DIR, typename C>
+__device__ __forceinline__ void fused_bfly(C& u, C& v, decltype(C::x) wx, decltype(C::x) wy0) {
+  using T = decltype(C::x);
+  const T wy = DIR < 0 ? wy0 : -wy0;
+  const C x = mk<C>(fma(wx, v.x, fma(-wy, v.y, u.x)), fma(wx, v.y, fma(wy, v.x, u.y)));
+  v = mk<C>(fma(T(2), u.x, -x.x), fma(T(2), u.y, -x.y));
+  u = x;
+}
+
 // In-register DFT of length R (R <= 32) on a[0], a[S], ..., a[(R-1) S],
 // natural order in and out, X[k] = sum_n x[n] exp(DIR 2 pi i n k / R).
 template <int R, int DIR, int S, typename C>
@@ -187,6 +203,15 @@ __device__ __forceinline__ void reg_dft(C* a) {
       for (int i = 0; i < R; i += len) {
 #pragma unroll
         for (int k = 0; k < len / 2; ++k) {
+          if constexpr (sizeof(C) == 16) {
+            // FP64: roots other than 1 and -+i in the fused butterfly
+            if (k != 0 && 4 * k != len) {
+              const int j = k * 32 / len;  // angle -2 pi j / 32, 0 < j < 16
+              const double wx = j < 8 ? cos32(j) : -cos32(16 - j), wy = j < 8 ? -sin32(j) : -sin32(16 - j);
+              fused_bfly<DIR>(t[i + k], t[i + k + len / 2], wx, wy);
+              continue;
+            }
+          }
           C u = t[i + k];
           C v = twiddle_small<DIR>(t[i + k + len / 2], k, len);
           t[i + k] = cadd(u, v);
@@ -199,28 +224,79 @@ __device__ __forceinline__ void reg_dft(C* a) {
   }
 }
 
+// DFT of length R on a[0], a[S], ... whose input r carries the twiddle
+// exp(DIR 2 pi i r j / (NS R)) (decimation in time): in stage `len` butterfly
+// k takes the root exp(DIR 2 pi i (j + k NS) / (NS len)), so the twiddles cost
+// nothing beyond the stages' own fused butterflies: 3 instructions per value
+// and stage, against 3.5 to 3.6 for a separate twiddle product at radix 8 or
+// 16.  The FP64 passes are bound by the FP64 pipe, so fewer instructions are
+// less time: 1024^2, p = 2, a step 596 us against 652 us; 64^3, p = 4, 290 us
+// against 305 us.  Roots with k >= len / 4 are -+i times those of k - len / 4.  tw: the
+// R / 2 roots of this j, NS entries apart, stage 2 first (stages of length
+// len = 2, 4, 8, 16 hold 1, 1, 2, 4).
+template <int R, int DIR, int S, int NS, typename C>
+__device__ __forceinline__ void fused_dft(C* a, const C* __restrict__ tw) {
+  constexpr int B = ilog2(R);
+  C t[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) t[i] = a[bitrev(i, B) * S];
+#pragma unroll
+  for (int len = 2; len <= R; len <<= 1) {
+    const int nk = len >= 4 ? len / 4 : 1, base = len == 2 ? 0 : len / 4;
+#pragma unroll
+    for (int k = 0; k < nk; ++k) {
+      const C w = tw[(base + k) * NS];
+#pragma unroll
+      for (int i = 0; i < R; i += len) {
+        fused_bfly<DIR>(t[i + k], t[i + k + len / 2], w.x, w.y);
+        if (len >= 4) {
+          C v = mul_i<DIR>(t[i + k + len / 4 + len / 2]);
+          fused_bfly<DIR>(t[i + k + len / 4], v, w.x, w.y);
+          t[i + k + len / 4 + len / 2] = v;
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i) a[i * S] = t[i];
+}
+
 // ---- pass structure (identical on host and device) -------------------------
+// Table entries of a pass of radix r after sub-length ns.
+__host__ __device__ constexpr int pass_entries(int ns, int r, bool f64) { return f64 ? ns * (r / 2) : ns * r; }
 template <int L, int E, int NS>
 struct PassRadix {
   static constexpr int R = imin(E, L / NS);
 };
+// FP64 table entry q of a pass at j (see fused_dft): q = 0 is stage 2, then
+// stage 4, two of stage 8, four of stage 16; the angle is -2 pi num / den.
+__host__ inline void stage_root(int q, int j, int ns, long long* num, long long* den) {
+  int len = 2, k = q;
+  if (q > 0) {
+    len = 4;
+    while (q >= len / 2) len <<= 1;  // stage len holds q in [len / 4, len / 2)
+    k = q - len / 4;
+  }
+  *num = j + (long long)k * ns;
+  *den = (long long)ns * len;
+}
 // offset (in complex entries) of the table of the pass starting at NS
 template <int L, int E, int NS>
-constexpr int pass_table_offset() {
+constexpr int pass_table_offset(bool f64) {
   int off = 0;
   for (int ns = 1; ns < NS;) {
     int r = imin(E, L / ns);
-    if (ns > 1) off += ns * r;
+    if (ns > 1) off += pass_entries(ns, r, f64);
     ns *= r;
   }
   return off;
 }
 // total table size of a line FFT of length L with E per thread
-__host__ __device__ constexpr int pass_table_size(int L, int E) {
+__host__ __device__ constexpr int pass_table_size(int L, int E, bool f64 = false) {
   int off = 0;
   for (int ns = 1; ns < L;) {
     int r = E < L / ns ? E : L / ns;
-    if (ns > 1) off += ns * r;
+    if (ns > 1) off += pass_entries(ns, r, f64);
     ns *= r;
   }
   return off;
@@ -241,10 +317,16 @@ __device__ __forceinline__ void stockham(C (&v)[E], int t, const C* __restrict__
   for (int q = 0; q < Q; ++q) {
     const int b = t + TPL * q;
     if constexpr (NS > 1) {
+      constexpr bool F64 = sizeof(C) == 16;
       const int j = b & (NS - 1);
-      const C* w = twp + pass_table_offset<L, E, NS>() + j;
+      const C* w = twp + pass_table_offset<L, E, NS>(F64) + j;
+      if constexpr (F64) {
+        fused_dft<R, DIR, Q, NS>(&v[q], w);
+        continue;
+      } else {
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[q + Q * r] = mul_tw<DIR>(v[q + Q * r], w[r * NS]);
+        for (int r = 1; r < R; ++r) v[q + Q * r] = mul_tw<DIR>(v[q + Q * r], w[r * NS]);
+      }
     }
     reg_dft<R, DIR, Q>(&v[q]);
   }

@@ -666,13 +666,13 @@ TableLayout table_layout(const fs_params& prm, bool f64) {
   t.k2z = o;
   o = align16(o + rs * nz);
   t.tw_row = o;
-  o = align16(o + cs * fs::pass_table_size(t.Lrow, t.Erow));
+  o = align16(o + cs * fs::pass_table_size(t.Lrow, t.Erow, f64));
   t.tw_row_w = o;  // wide x-pass variant (32 values per thread): FP32 rows of 1024
   o = align16(o + (wide_rows(prm, f64) ? cs * fs::pass_table_size(t.Lrow, 32) : 0));
   t.tw_col = o;
-  o = align16(o + cs * fs::pass_table_size(t.Lcol, t.Ecol));
+  o = align16(o + cs * fs::pass_table_size(t.Lcol, t.Ecol, f64));
   t.tw_z = o;
-  o = align16(o + cs * (nz > 1 ? fs::pass_table_size(t.Lz, t.Ez) : 0));
+  o = align16(o + cs * (nz > 1 ? fs::pass_table_size(t.Lz, t.Ez, f64) : 0));
   t.tw_half = o;
   o = align16(o + cs * (nx / 2));
   t.tc_b = o;
@@ -693,16 +693,18 @@ size_t member_table_bytes(const fs_params& prm, bool f64) { return table_layout(
 
 // Stockham pass tables of a line FFT of length L with E values per thread:
 // for every pass after the first (sub-length NS, radix R = min(E, L/NS)),
-// entries [r][j] = exp(-2 pi i r j / (NS R)), r < R, j < NS.
-void pass_table(int L, int E, std::vector<long double>& re, std::vector<long double>& im) {
+// FP32 entries [r][j] = exp(-2 pi i r j / (NS R)), r < R, j < NS; FP64 entries
+// [q][j], q < R / 2, the roots of the pass's radix-2 stages (fs::stage_root).
+void pass_table(int L, int E, bool f64, std::vector<long double>& re, std::vector<long double>& im) {
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int ns = 1; ns < L;) {
     int r = E < L / ns ? E : L / ns;
     if (ns > 1)
-      for (int q = 0; q < r; ++q)
+      for (int q = 0; q < (f64 ? r / 2 : r); ++q)
         for (int j = 0; j < ns; ++j) {
-          long long e = (long long)q * j % ((long long)ns * r);
-          long double ang = 2.0L * pi * (long double)e / (long double)(ns * r);
+          long long num = (long long)q * j, den = (long long)ns * r;
+          if (f64) fs::stage_root(q, j, ns, &num, &den);
+          long double ang = 2.0L * pi * (long double)(num % den) / (long double)den;
           re.push_back(cosl(ang));
           im.push_back(-sinl(ang));
         }
@@ -735,14 +737,14 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   for (int k = 0; k < ny; ++k) ky[k] = axis_k2(prm.lap, k, ny, prm.dx[1]);
   for (int k = 0; k < nz && prm.ndim > 2; ++k) kz[k] = axis_k2(prm.lap, k, nz, prm.dx[2]);
   std::vector<long double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i;
-  if (row2_form(prm, f64)) pass_table(nx, nx / 32, r2r, r2i);
-  if (col2_form(prm, f64) && ny <= 1024) pass_table(ny, ny / 32, c2r, c2i);
-  if (row2_form(prm, f64) && nx >= 128) pass_table(nx, nx / 64, r3r, r3i);
-  if (col2_form(prm, f64) && ny >= 128) pass_table(ny, ny / 64, c3r, c3i);
-  pass_table(t.Lrow, t.Erow, rr, ii);
-  if (wide_rows(prm, f64)) pass_table(t.Lrow, 32, wr, wi);
-  pass_table(t.Lcol, t.Ecol, cr, ci);
-  if (nz > 1) pass_table(t.Lz, t.Ez, zr, zi);
+  if (row2_form(prm, f64)) pass_table(nx, nx / 32, f64, r2r, r2i);
+  if (col2_form(prm, f64) && ny <= 1024) pass_table(ny, ny / 32, f64, c2r, c2i);
+  if (row2_form(prm, f64) && nx >= 128) pass_table(nx, nx / 64, f64, r3r, r3i);
+  if (col2_form(prm, f64) && ny >= 128) pass_table(ny, ny / 64, f64, c3r, c3i);
+  pass_table(t.Lrow, t.Erow, f64, rr, ii);
+  if (wide_rows(prm, f64)) pass_table(t.Lrow, 32, f64, wr, wi);
+  pass_table(t.Lcol, t.Ecol, f64, cr, ci);
+  if (nz > 1) pass_table(t.Lz, t.Ez, f64, zr, zi);
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int k = 0; k < nx / 2; ++k) {
     long double ang = 2.0L * pi * (long double)k / (long double)nx;
