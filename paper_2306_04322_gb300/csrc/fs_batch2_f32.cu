@@ -11,7 +11,7 @@ namespace fs {
 
 #define FS_V2_SIZES(X) X(64) X(128) X(256) X(512) X(1024)
 
-__global__ void __launch_bounds__(Row2Cfg<1024>::MAX_THREADS, 3)
+__global__ void __launch_bounds__(Row2Cfg<float, 1024>::MAX_THREADS, 3)
     fs_row2_batch_kernel(const KArgs* __restrict__ mem, const long long* __restrict__ begin, int nm,
                          long long total) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(Row2Cfg<1024>::MAX_THREADS, 3)
     bool ok = true;
     switch (a.nx) {
 #define FS_CASE(n) \
-  case n: ok = row2_body<n>(a, rp, smem_raw, bar, parity); break;
+  case n: ok = row2_body<float, n>(a, rp, smem_raw, bar, parity); break;
       FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
       default: break;
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(128, 4)
     bool ok = true;
     switch (a.ny) {
 #define FS_CASE(n) \
-  case n: ok = col2_body<n>(a, &maps[m], cp, group, smem_raw, bar, parity); break;
+  case n: ok = col2_body<float, n>(a, &maps[m], cp, group, smem_raw, bar, parity); break;
       FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
       default: break;
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(128, 4)
 size_t row2_smem_f32(int nx, int nf) {
   switch (nx) {
 #define FS_CASE(n) \
-  case n: return row2_smem_bytes<n>(nf);
+  case n: return row2_smem_bytes<float, n>(nf);
     FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
     default: return 0;
@@ -83,7 +83,7 @@ size_t row2_smem_f32(int nx, int nf) {
 size_t col2_smem_f32(int ny) {
   switch (ny) {
 #define FS_CASE(n) \
-  case n: return col2_smem_bytes<n>();
+  case n: return col2_smem_bytes<float, n>();
     FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
     default: return 0;

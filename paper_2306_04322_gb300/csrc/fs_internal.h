@@ -90,6 +90,12 @@ cudaError_t col_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t s
 // cudaErrorNotSupported for other requests.
 cudaError_t row2_launch_f32(const KArgs& a, cudaStream_t s);
 cudaError_t col2_launch_f32(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
+// The same in FP64: rows of 64 to 2048 points, columns of 64 to 512; warps
+// per line (0: no such kernel).
+cudaError_t row2_launch_f64(const KArgs& a, cudaStream_t s);
+cudaError_t col2_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
+int row2_g64(int nx);
+int col2_g64(int ny);
 bool row2_supported(int nx, int nf);
 bool col2_supported(int ny, int nf);
 // Fused step (pass form 4, fs_step2_f32.cu): `nsteps` steady-state steps

@@ -1,9 +1,10 @@
-// Warp-per-line forms of the row and column passes (FP32, lines of 256, 512
-// or 1024 points).  Every line transform is held by one warp, E = L / 32
-// values per thread (radix 32 x 32 at L = 1024: one exchange), so the FFT
-// exchanges synchronise the warp only; CTA-wide barriers remain only where
-// fields meet (the pointwise stage of the row pass) and named 64-thread
-// barriers where the column pass hands df/dc^ to the c update.
+// Warp-per-line forms of the row and column passes.  FP32: every line
+// transform is held by one warp, E = L / 32 values per thread (radix 32 x 32
+// at L = 1024: one exchange), so the FFT exchanges synchronise the warp only;
+// CTA-wide barriers remain only where fields meet (the pointwise stage of the
+// row pass) and named 64-thread barriers where the column pass hands df/dc^
+// to the c update.  FP64: G warps per line with 2 to 8 values per thread
+// (see row2_g64).
 //
 // Row pass, pair form.  Grid rows a and b of one field are transformed as
 // the single complex line z = a + i b of length nx:
@@ -40,23 +41,39 @@ __device__ __forceinline__ void warp_line_fft(C (&v)[E], int t, const C* __restr
   else line_fft<L, E, DIR>(v, t, twp, st, ld, sync);
 }
 
-// G warps per line (1, or 2 to double the warps in flight when lines are
-// few); a line's TPL = 32 G threads hold E = NX / TPL values each.
-template <int NX, int G = 1>
+// Padded exchange layout of a line: FP32 one spare slot every 32 elements;
+// FP64 (16-byte elements, 8 lanes per shared-memory wavefront) every 8, so
+// that the writes of E consecutive elements per thread fall on different
+// banks (every 16 at 2048 points, where six padded areas must fit an SM).
+template <typename T, int L>
+__device__ __forceinline__ int line_pad(int i) {
+  if constexpr (sizeof(T) == 4) return pad32(i);
+  else return i + (i >> (L >= 2048 ? 4 : 3));
+}
+template <typename T>
+constexpr int line_pad_len(int L) {
+  return sizeof(T) == 4 ? (padded_len(L) + 1) & ~1 : L + (L >> (L >= 2048 ? 4 : 3)) + 1;
+}
+
+// G warps per line (FP32: 1, or 2 to double the warps in flight when lines
+// are few); a line's TPL = 32 G threads hold E = NX / TPL values each.
+template <typename T, int NX, int G = 1>
 struct Row2Cfg {
+  static constexpr bool F64 = sizeof(T) == 8;
   static constexpr int TPL = 32 * G;                          // threads per line
   static constexpr int E = NX / TPL;                          // values per thread
   static constexpr int H = NX / 2;                            // packed bins per row
-  static constexpr int PL = (padded_len(NX) + 1) & ~1;        // complex per field area (16-byte multiple)
-  static constexpr int TWS = pass_table_size(NX, E);
-  static constexpr int TW_BYTES = ((TWS * 8) + 127) & ~127;
+  static constexpr int PL = line_pad_len<T>(NX);           // complex per field area (16-byte multiple)
+  static constexpr int TWS = pass_table_size(NX, E, F64);
+  static constexpr int TW_BYTES = ((TWS * (int)sizeof(cplx<T>)) + 127) & ~127;
   static constexpr int BAR_BYTES = 128;
   static constexpr int MAX_THREADS = TPL * 5;                 // one line per field, nf <= 5
 };
 
-template <int NX, int G = 1>
+template <typename T, int NX, int G = 1>
 constexpr size_t row2_smem_bytes(int nf) {
-  return Row2Cfg<NX, G>::BAR_BYTES + Row2Cfg<NX, G>::TW_BYTES + (size_t)(nf + 1) * Row2Cfg<NX, G>::PL * 8;
+  using Cfg = Row2Cfg<T, NX, G>;
+  return Cfg::BAR_BYTES + Cfg::TW_BYTES + (size_t)(nf + 1) * Cfg::PL * sizeof(cplx<T>);
 }
 
 // Synchronisation of the threads of one line: the warp itself, or the two
@@ -71,16 +88,16 @@ struct LineSync {
 };
 
 // Pointwise stage of the pair-form row pass (Section 2.1 derivatives, lane-
-// wise on the two rows of a pair) with p = P known at compile time: four
-// independent points per iteration -- all loads, then the arithmetic, then
+// wise on the two rows of a pair) with p = P known at compile time: U (FP32:
+// four) independent points per iteration -- all loads, then the arithmetic, then
 // the stores (points past the row repeat point n).  areas: [nf + 1][PL],
 // c, eta_i (replaced by g_i), df/dc in area nf.  df/dc is non-finite
 // whenever c or any eta_i is (see the row pass of fs_kernels.cuh): one test
 // of the sum of its lanes covers all inputs.
-template <int P, int NX, int PL>
-__device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<float>& pw, float2* areas, bool& bad) {
-  using C = float2;
-  constexpr int PE = P > 0 ? P : 1, U = 4;
+template <typename T, int P, int NX, int PL>
+__device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cplx<T>* areas, bool& bad) {
+  using C = cplx<T>;
+  constexpr int PE = P > 0 ? P : 1, U = sizeof(T) == 4 ? 4 : 1;  // FP64: bound by its pipe, not by latency
   for (int n = threadIdx.x; n < NX; n += U * blockDim.x) {
     int k[U];
     C c[U], e[U][PE], fc[U], g[U][PE];
@@ -91,10 +108,10 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<float>& pw,
 #pragma unroll
       for (int i = 0; i < P; ++i) e[u][i] = areas[(1 + i) * PL + k[u]];
     }
-    float chk = 0.f;
+    T chk = T(0);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      C h = vsplat<C>(0.f), S2 = vsplat<C>(0.f);
+      C h = vsplat<C>(T(0)), S2 = vsplat<C>(T(0));
 #pragma unroll
       for (int i = 0; i < P; ++i) {
         h = cadd(h, pw.hpoly2(e[u][i]));
@@ -124,11 +141,11 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<float>& pw,
 // wait gave up.  PC >= 0: the caller guarantees nf = PC + 1, and the
 // pointwise stage is compiled for that p alone (the 96-thread kernel, whose
 // nf is 3: a kernel holding the code for every p measured slower there).
-template <int NX, int G = 1, int PC = -1>
+template <typename T, int NX, int G = 1, int PC = -1>
 __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsigned char* smem_raw, uint64_t* bar,
                                           uint32_t parity) {
-  using C = float2;
-  using Cfg = Row2Cfg<NX, G>;
+  using C = cplx<T>;
+  using Cfg = Row2Cfg<T, NX, G>;
   constexpr int E = Cfg::E, H = Cfg::H, PL = Cfg::PL, TPL = Cfg::TPL;
   C* tw = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
   C* areas = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES + Cfg::TW_BYTES);
@@ -148,10 +165,10 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
     const uint32_t tbytes = (uint32_t)(Cfg::TWS * sizeof(C));
     mbar_arrive_expect_tx(bar, tbytes + bytes * nf);
     // the constant pass table first, overlapping the previous grid's tail
-    bulk_g2s(tw, G == 1 ? a.tw_row2 : a.tw_row2w, tbytes, bar);
+    bulk_g2s(tw, G == 1 || Cfg::F64 ? a.tw_row2 : a.tw_row2w, tbytes, bar);
     griddep_wait();  // the spectra are the previous pass's output
     const C* spec = reinterpret_cast<const C*>(a.spec);
-    const float* real = reinterpret_cast<const float*>(a.real);
+    const T* real = reinterpret_cast<const T*>(a.real);
     for (int f = 0; f < nf; ++f) {
       // 3D carry: c's x spectrum sits in slot nf
       const int sl = (f == 0 && a.carry3) ? nf : f;
@@ -168,7 +185,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
   }
 
   C* spec = reinterpret_cast<C*>(a.spec);
-  float* real = reinterpret_cast<float*>(a.real);
+  T* real = reinterpret_cast<T*>(a.real);
   bool bad = false;
   // Both transform phases share one FFT call site (the inverse is computed as
   // conj(FFT(conj(.)))): ph 0 inverse of the nf fields (modes 0, 2; mode 1
@@ -181,14 +198,14 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
     for (int i = line; i < items; i += nw) {
       const int f = f0 + i;
       C* s = areas + f * PL;
-      auto st = [s](int q, C x) { s[pad32(q)] = x; };
-      auto ld = [s](int q) { return s[pad32(q)]; };
+      auto st = [s](int q, C x) { s[line_pad<T, NX>(q)] = x; };
+      auto ld = [s](int q) { return s[line_pad<T, NX>(q)]; };
       C v[E];
       if (inv) {
         if (from_real) {
           // rows a and b (NX reals each) -> pairs (a[n], b[n]) in natural order
-          const float* r = reinterpret_cast<const float*>(s);
-          float xa[E], xb[E];
+          const T* r = reinterpret_cast<const T*>(s);
+          T xa[E], xb[E];
 #pragma unroll
           for (int m = 0; m < E; ++m) {
             xa[m] = r[t + TPL * m];
@@ -196,7 +213,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
           }
           lsync();
 #pragma unroll
-          for (int m = 0; m < E; ++m) s[t + TPL * m] = make_float2(xa[m], xb[m]);
+          for (int m = 0; m < E; ++m) s[t + TPL * m] = mk<C>(xa[m], xb[m]);
           continue;
         }
         // conj(Z), Z[k] = X_a[k] + i X_b[k]; staging: row a bins [0, H), row b [H, 2H);
@@ -207,12 +224,12 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
           C z;
           if (k < H) {
             const C xa = s[k], xb = s[H + k];
-            z = (k == 0) ? make_float2(xa.x, xb.x) : make_float2(xa.x - xb.y, xa.y + xb.x);
+            z = (k == 0) ? mk<C>(xa.x, xb.x) : mk<C>(xa.x - xb.y, xa.y + xb.x);
           } else if (k == H) {
-            z = make_float2(s[0].y, s[H].y);
+            z = mk<C>(s[0].y, s[H].y);
           } else {
             const C xa = s[NX - k], xb = s[H + NX - k];
-            z = make_float2(xa.x + xb.y, xb.x - xa.y);
+            z = mk<C>(xa.x + xb.y, xb.x - xa.y);
           }
           v[m] = cconj(z);
         }
@@ -225,12 +242,12 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
       if (inv) {
         // a + i b = conj(v)
         if (a.mode == 2) {
-          float* ra = real + f * a.npts + row0 * NX;
+          T* ra = real + f * a.npts + row0 * NX;
 #pragma unroll
           for (int m = 0; m < E; ++m) {
             const int n = t + TPL * m;
-            if (real_ok(a, &ra[n], 4)) ra[n] = v[m].x;
-            if (real_ok(a, &ra[NX + n], 4)) ra[NX + n] = -v[m].y;
+            if (real_ok(a, &ra[n], sizeof(T))) ra[n] = v[m].x;
+            if (real_ok(a, &ra[NX + n], sizeof(T))) ra[NX + n] = -v[m].y;
           }
         } else {
           lsync();
@@ -244,7 +261,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
         for (int m = 0; m < E; ++m) s[t + TPL * m] = v[m];
         lsync();
         const bool c_carried = (f == 0);  // mode 1: c stored as x spectrum / nx
-        const float cs = c_carried ? 0.5f / (float)NX : 1.0f;
+        const T cs = c_carried ? T(0.5) / T(NX) : T(1);
         C* Pa = spec + f * a.slot_stride + row0 * H;
         C* Pb = Pa + H;
 #pragma unroll
@@ -254,12 +271,12 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
           C pa, pb;
           if (k == 0) {
             const C zh = s[H];
-            pa = make_float2(2.f * zk.x, 2.f * zh.x);
-            pb = make_float2(2.f * zk.y, 2.f * zh.y);
+            pa = mk<C>(T(2) * zk.x, T(2) * zh.x);
+            pb = mk<C>(T(2) * zk.y, T(2) * zh.y);
           } else {
             const C zm = s[NX - k];
-            pa = make_float2(zk.x + zm.x, zk.y - zm.y);
-            pb = make_float2(zk.y + zm.y, zm.x - zk.x);
+            pa = mk<C>(zk.x + zm.x, zk.y - zm.y);
+            pb = mk<C>(zk.y + zm.y, zm.x - zk.x);
           }
           if (c_carried) {
             pa = cscale(pa, cs);
@@ -275,16 +292,16 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
     __syncthreads();
 
     // pointwise stage: pairs (row a, row b) of every field, lane-wise
-    const Pointwise<float> pw(a);
+    const Pointwise<T> pw(a);
     if constexpr (PC >= 0) {
-      row2_pointwise_fixed<PC, NX, PL>(pw, areas, bad);
+      row2_pointwise_fixed<T, PC, NX, PL>(pw, areas, bad);
     } else {
       switch (nf) {  // p known at compile time for every supported field count
-        case 1: row2_pointwise_fixed<0, NX, PL>(pw, areas, bad); break;
-        case 2: row2_pointwise_fixed<1, NX, PL>(pw, areas, bad); break;
-        case 3: row2_pointwise_fixed<2, NX, PL>(pw, areas, bad); break;
-        case 4: row2_pointwise_fixed<3, NX, PL>(pw, areas, bad); break;
-        case 5: row2_pointwise_fixed<4, NX, PL>(pw, areas, bad); break;
+        case 1: row2_pointwise_fixed<T, 0, NX, PL>(pw, areas, bad); break;
+        case 2: row2_pointwise_fixed<T, 1, NX, PL>(pw, areas, bad); break;
+        case 3: row2_pointwise_fixed<T, 2, NX, PL>(pw, areas, bad); break;
+        case 4: row2_pointwise_fixed<T, 3, NX, PL>(pw, areas, bad); break;
+        case 5: row2_pointwise_fixed<T, 4, NX, PL>(pw, areas, bad); break;
         default: break;
       }
     }
@@ -301,8 +318,14 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
 // thread; otherwise three 160-thread CTAs (136).  Measured (L2 flushed
 // before each step, p = 2): 512^2 step 17.1 us against 19.1 us, 1024^2
 // unchanged; with nf = 2 the 1024^2 step lost 4 %, so only nf = 3 takes it.
-template <int NX, int G, int NW>
-__global__ void __launch_bounds__(32 * G * NW, (G == 1 && NW <= 3) ? 4 : (G == 1 ? 3 : 2))
+// FP64: as many CTAs as leave the registers of E values per thread.
+template <typename T, int G, int NW>
+constexpr int row2_min_blocks() {
+  if (sizeof(T) == 8) return 32 * G * NW > 400 ? 1 : (32 * G * NW > 250 ? 2 : 4);
+  return (G == 1 && NW <= 3) ? 4 : (G == 1 ? 3 : 2);
+}
+template <typename T, int NX, int G, int NW>
+__global__ void __launch_bounds__(32 * G * NW, row2_min_blocks<T, G, NW>())
     fs_row2_kernel(KArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
@@ -311,32 +334,36 @@ __global__ void __launch_bounds__(32 * G * NW, (G == 1 && NW <= 3) ? 4 : (G == 1
     fence_mbar_init();
   }
   __syncthreads();
-  row2_body<NX, G, (G == 1 && NW == 3) ? 2 : -1>(a, blockIdx.x, smem_raw, bar, 0);
+  row2_body<T, NX, G, (sizeof(T) == 4 && G == 1 && NW == 3) ? 2 : -1>(a, blockIdx.x, smem_raw, bar, 0);
 }
 
-template <int NY, int G = 1>
+template <typename T, int NY, int G = 1>
 struct Col2Cfg {
+  static constexpr bool F64 = sizeof(T) == 8;
+  static constexpr int CS = 2 * (int)sizeof(T);               // bytes of a complex value
   static constexpr int TPL = 32 * G;                          // threads per line
   static constexpr int E = NY / TPL;
   static constexpr int TK = 2;                                // kx columns per CTA
   static constexpr int BH = NY < 256 ? NY : 256;              // TMA box height (rows)
-  static constexpr int PL = (padded_len(NY) + 1) & ~1;        // complex per compact column area
+  static constexpr int PL = line_pad_len<T>(NY);           // complex per compact column area
   // slot region: the [NY][TK] tile as loaded, then TK compact areas, then the
   // [NY][TK] tile again for the TMA store; a multiple of 16 complex so every
   // region starts on 128 bytes (TMA)
   static constexpr int SLOT = (((NY * TK > TK * PL) ? NY * TK : TK * PL) + 15) & ~15;
-  static constexpr int TWS = pass_table_size(NY, E);
-  static constexpr int TW_BYTES = ((TWS * 8) + 127) & ~127;
-  static constexpr int K2_BYTES = ((NY * 4) + 127) & ~127;
+  static constexpr int TWS = pass_table_size(NY, E, F64);
+  static constexpr int TW_BYTES = ((TWS * CS) + 127) & ~127;
+  static constexpr int K2_BYTES = ((NY * (int)sizeof(T)) + 127) & ~127;
   static constexpr int HEAD = 128 + TW_BYTES + K2_BYTES;
-  // CTAs per SM the registers are budgeted for: 128 per thread at 32 values
-  static constexpr int MIN_BLOCKS = E >= 32 ? 4 / G : (G == 1 ? 4 : 3);
+  // CTAs per SM the registers are budgeted for: FP32 128 per thread at 32
+  // values, FP64 at least 64
+  static constexpr int MIN_BLOCKS = F64 ? (G == 1 ? 6 : 8 / G) : (E >= 32 ? 4 / G : (G == 1 ? 4 : 3));
 };
 
 // Shared memory of one CTA: the head and two slot regions.
-template <int NY, int G = 1>
+template <typename T, int NY, int G = 1>
 constexpr size_t col2_smem_bytes() {
-  return Col2Cfg<NY, G>::HEAD + (size_t)2 * Col2Cfg<NY, G>::SLOT * 8;
+  using Cfg = Col2Cfg<T, NY, G>;
+  return Cfg::HEAD + (size_t)2 * Cfg::SLOT * Cfg::CS;
 }
 
 // The packed kx = 0 / Nyquist column of the first CTA: y holds this warp's
@@ -348,27 +375,27 @@ constexpr size_t col2_smem_bytes() {
 // B, and the update is real-linear with the same K2 at ky and ny - ky), so a
 // thread owns both entries of its pairs and no other thread touches them.  A
 // few warps of the grid run this, so it stays out of line and rolled.
-template <int NY, int TPL>
-__device__ __noinline__ void col2_packed_update(float2* __restrict__ y, const float2* __restrict__ fz, int t,
-                                                bool isC, KUpdate<float> up, float kx2, float kxn2,
-                                                const float* __restrict__ k2yt, const double* csum,
+template <typename T, int NY, int TPL>
+__device__ __noinline__ void col2_packed_update(cplx<T>* __restrict__ y, const cplx<T>* __restrict__ fz, int t,
+                                                bool isC, KUpdate<T> up, T kx2, T kxn2,
+                                                const T* __restrict__ k2yt, const double* csum,
                                                 double inv_npts) {
-  using C = float2;
+  using C = cplx<T>;
 #pragma unroll 1
   for (int m = 0; m <= NY / (2 * TPL); ++m) {
     const int ky = t + TPL * m;  // pairs ky = 0 .. ny/2
     if (ky > NY / 2) break;
     const int kq = (NY - ky) & (NY - 1);
-    const float ky2 = k2yt[ky];
+    const T ky2 = k2yt[ky];
     const C z = y[ky], pz = cconj(y[kq]);
-    const C A = cscale(cadd(z, pz), 0.5f), B = cscale(mul_i<-1>(csub(z, pz)), 0.5f);
+    const C A = cscale(cadd(z, pz), T(0.5)), B = cscale(mul_i<-1>(csub(z, pz)), T(0.5));
     C An, Bn;
     if (isC) {
       const C zf = fz[ky], pf = cconj(fz[kq]);
-      const C Af = cscale(cadd(zf, pf), 0.5f), Bf = cscale(mul_i<-1>(csub(zf, pf)), 0.5f);
+      const C Af = cscale(cadd(zf, pf), T(0.5)), Bf = cscale(mul_i<-1>(csub(zf, pf)), T(0.5));
       An = up.c(A, Af, kx2 + ky2);
       Bn = up.c(B, Bf, kxn2 + ky2);
-      if (ky == 0 && csum) An = make_float2((float)(*csum * inv_npts), 0.f);
+      if (ky == 0 && csum) An = mk<C>((T)(*csum * inv_npts), T(0));
     } else {
       An = up.eta(A, kx2 + ky2);
       Bn = up.eta(B, kxn2 + ky2);
@@ -389,15 +416,15 @@ __device__ __noinline__ void col2_packed_update(float2* __restrict__ y, const fl
 // TMA, so the global writes are whole 16-byte rows instead of one 8-byte
 // value per lane and row.
 // Column pair `cpair`, field group `group` of the simulation `a` (blockDim =
-// 128); `bar` as for row2_body.  Returns false if a bounded wait gave up.
-template <int NY, int G = 1>
+// 128 G); `bar` as for row2_body.  Returns false if a bounded wait gave up.
+template <typename T, int NY, int G = 1>
 __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tmap, int cpair, int group,
                                           unsigned char* smem_raw, uint64_t* bar, uint32_t parity) {
-  using C = float2;
-  using Cfg = Col2Cfg<NY, G>;
+  using C = cplx<T>;
+  using Cfg = Col2Cfg<T, NY, G>;
   constexpr int E = Cfg::E, BH = Cfg::BH, PL = Cfg::PL, SLOT = Cfg::SLOT, TPL = Cfg::TPL;
   C* tw = reinterpret_cast<C*>(smem_raw + 128);
-  float* k2yt = reinterpret_cast<float*>(smem_raw + 128 + Cfg::TW_BYTES);
+  T* k2yt = reinterpret_cast<T*>(smem_raw + 128 + Cfg::TW_BYTES);
   C* regions = reinterpret_cast<C*>(smem_raw + Cfg::HEAD);
   const int nf = a.nf, p = nf - 1;
   const int line = (threadIdx.x >> 5) / G, t = threadIdx.x % TPL;  // line (region, column), thread in it
@@ -414,19 +441,19 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
     // the ensemble kernel reuses the regions: order the previous item's
     // generic accesses (ended by the caller's CTA barrier) before the TMA writes
     fence_proxy_async_smem();
-    const uint32_t tbytes = (uint32_t)(Cfg::TWS * sizeof(C)), kbytes = (uint32_t)(NY * sizeof(float));
+    const uint32_t tbytes = (uint32_t)(Cfg::TWS * sizeof(C)), kbytes = (uint32_t)(NY * sizeof(T));
     mbar_arrive_expect_tx(bar, tbytes + kbytes + (uint32_t)(nreg * NY * Cfg::TK * sizeof(C)));
     // the constant tables first, overlapping the previous grid's tail
-    bulk_g2s(tw, G == 1 ? a.tw_col2 : a.tw_col2w, tbytes, bar);
+    bulk_g2s(tw, G == 1 || Cfg::F64 ? a.tw_col2 : a.tw_col2w, tbytes, bar);
     bulk_g2s(k2yt, a.k2y, kbytes, bar);
     griddep_wait();  // the tiles are the previous pass's output
     for (int q = 0; q < nreg; ++q)
-      // innermost coordinate kx0 (8-byte units) is even: 16-byte aligned
+      // innermost coordinate kx0 in 8-byte units is even: 16-byte aligned
       for (int y0 = 0; y0 < NY; y0 += BH)
-        tma_load_3d(regions + q * SLOT + y0 * Cfg::TK, tmap, kx0, y0, slot_of(q), bar);
+        tma_load_3d(regions + q * SLOT + y0 * Cfg::TK, tmap, kx0 * (Cfg::CS / 8), y0, slot_of(q), bar);
   }
-  const float* __restrict__ k2xt = reinterpret_cast<const float*>(a.k2x);
-  const float kx2 = k2xt[kx];
+  const T* __restrict__ k2xt = reinterpret_cast<const T*>(a.k2x);
+  const T kx2 = k2xt[kx];
   griddep_launch_dependents();
   if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
@@ -446,9 +473,9 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   // both columns of this region have left the tile: it becomes two compact areas
   region_sync();
   C* xa = reg + j * PL;
-  auto st = [xa](int q, C x) { xa[pad32(q)] = x; };
-  auto ld = [xa](int q) { return xa[pad32(q)]; };
-  const KUpdate<float> up(a);
+  auto st = [xa](int q, C x) { xa[line_pad<T, NY>(q)] = x; };
+  auto ld = [xa](int q) { return xa[line_pad<T, NY>(q)]; };
+  const KUpdate<T> up(a);
   const bool special = (a.kx_base + kx0 == 0 && j == 0);  // the packed kx = 0 / Nyquist column
   const C* fz = regions + j * PL;             // df/dc^ of this column (region 0 of group 0)
 
@@ -473,10 +500,22 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
 #pragma unroll
       for (int m = 0; m < E; ++m) xa[t + TPL * m] = v[m];
       lsync();
-      col2_packed_update<NY, TPL>(xa, fz, t, isC, up, kx2, k2xt[H], k2yt, a.csum, a.inv_npts);
+      col2_packed_update<T, NY, TPL>(xa, fz, t, isC, up, kx2, k2xt[H], k2yt, a.csum, a.inv_npts);
       lsync();
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = cconj(xa[t + TPL * m]);
+    } else if constexpr (Cfg::F64) {
+      // bound by the FP64 pipe: c and eta each with their own operations only
+      if (isC) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+          const int ky = t + TPL * m;
+          v[m] = cconj(up.c(v[m], fz[ky], kx2 + k2yt[ky]));
+        }
+      } else {
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = cconj(up.eta(v[m], kx2 + k2yt[t + TPL * m]));
+      }
     } else {
       // c^' = (c^ - M dt K2 f^) / (1 + M dt kappa_c K2^2), eta^' = g^ / (1 + L dt kappa_eta K2)
       // (scales folded as in KUpdate); one code path for both, the quotient by
@@ -502,15 +541,15 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   fence_proxy_async_smem();
   region_sync();
   if (j == 0 && t == 0) {  // one thread of the region's column-0 line
-    for (int y0 = 0; y0 < NY; y0 += BH) tma_store_3d(tmap, kx0, y0, slot_of(r), reg + y0 * Cfg::TK);
+    for (int y0 = 0; y0 < NY; y0 += BH) tma_store_3d(tmap, kx0 * (Cfg::CS / 8), y0, slot_of(r), reg + y0 * Cfg::TK);
     bulk_commit();
     bulk_wait_all();  // the tile is read (and written out) before the region is reused or the CTA exits
   }
   return true;
 }
 
-template <int NY, int G>
-__global__ void __launch_bounds__(128 * G, Col2Cfg<NY, G>::MIN_BLOCKS)
+template <typename T, int NY, int G>
+__global__ void __launch_bounds__(128 * G, Col2Cfg<T, NY, G>::MIN_BLOCKS)
     fs_col2_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
@@ -519,33 +558,29 @@ __global__ void __launch_bounds__(128 * G, Col2Cfg<NY, G>::MIN_BLOCKS)
     fence_mbar_init();
   }
   __syncthreads();
-  col2_body<NY, G>(a, &tmap, blockIdx.x, blockIdx.y, smem_raw, bar, 0);
+  col2_body<T, NY, G>(a, &tmap, blockIdx.x, blockIdx.y, smem_raw, bar, 0);
 }
 
 // Launchers: cudaErrorNotSupported when this form does not cover the
 // request (the caller falls back to the half-length / tile kernels).
-template <int NX, int G, int NW>
+template <typename T, int NX, int G, int NW>
 cudaError_t row2_launch_nw(const KArgs& a, cudaStream_t s) {
   static unsigned done = 0;
-  cudaError_t e = allow_big_smem(fs_row2_kernel<NX, G, NW>, &done);
+  cudaError_t e = allow_big_smem(fs_row2_kernel<T, NX, G, NW>, &done);
   if (e != cudaSuccess) return e;
-  return launch_pdl(fs_row2_kernel<NX, G, NW>, dim3((unsigned)(a.lines / 2)), dim3((unsigned)(32 * G * a.nf)),
-                    row2_smem_bytes<NX, G>(a.nf), s, a);
-}
-template <int NX, int G>
-cudaError_t row2_launch_n(const KArgs& a, cudaStream_t s) {
-  if (G == 1 && a.nf == 3) return row2_launch_nw<NX, G, 3>(a, s);
-  return row2_launch_nw<NX, G, 5>(a, s);
+  const int lines = a.nf < NW ? a.nf : NW;  // lines in flight; more fields take a second round
+  return launch_pdl(fs_row2_kernel<T, NX, G, NW>, dim3((unsigned)(a.lines / 2)), dim3((unsigned)(32 * G * lines)),
+                    row2_smem_bytes<T, NX, G>(a.nf), s, a);
 }
 
-template <int NY, int G>
+template <typename T, int NY, int G>
 cudaError_t col2_launch_n(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
   static unsigned done = 0;
-  cudaError_t e = allow_big_smem(fs_col2_kernel<NY, G>, &done);
+  cudaError_t e = allow_big_smem(fs_col2_kernel<T, NY, G>, &done);
   if (e != cudaSuccess) return e;
   const unsigned groups = (unsigned)(1 + (a.nf - 1 + 1) / 2);  // {df/dc, c} and the eta pairs
-  return launch_pdl(fs_col2_kernel<NY, G>, dim3((unsigned)(a.nx / 2 / Col2Cfg<NY, G>::TK), groups),
-                    dim3((unsigned)(128 * G)), col2_smem_bytes<NY, G>(), s, a, tm);
+  return launch_pdl(fs_col2_kernel<T, NY, G>, dim3((unsigned)(a.nx / 2 / Col2Cfg<T, NY, G>::TK), groups),
+                    dim3((unsigned)(128 * G)), col2_smem_bytes<T, NY, G>(), s, a, tm);
 }
 
 }  // namespace fs

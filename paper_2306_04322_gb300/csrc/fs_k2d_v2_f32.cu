@@ -9,6 +9,11 @@ static bool v2_size(int n) { return n == 64 || n == 128 || n == 256 || n == 512 
 bool row2_supported(int nx, int nf) { return v2_size(nx) && nf >= 1 && nf <= 5; }
 bool col2_supported(int ny, int nf) { return (v2_size(ny) || ny == 2048) && nf >= 1 && nf <= 5; }
 
+template <int NX, int G>
+static cudaError_t row2_launch_n(const KArgs& a, cudaStream_t s) {
+  if (G == 1 && a.nf == 3) return row2_launch_nw<float, NX, G, 3>(a, s);
+  return row2_launch_nw<float, NX, G, 5>(a, s);
+}
 template <int G>
 cudaError_t row2_launch_g(const KArgs& a, cudaStream_t s) {
   switch (a.nx) {
@@ -23,12 +28,12 @@ cudaError_t row2_launch_g(const KArgs& a, cudaStream_t s) {
 template <int G>
 cudaError_t col2_launch_g(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
   switch (a.ny) {
-    case 64: if constexpr (G == 1) return col2_launch_n<64, G>(a, tm, s); else return cudaErrorNotSupported;
-    case 128: return col2_launch_n<128, G>(a, tm, s);
-    case 256: return col2_launch_n<256, G>(a, tm, s);
-    case 512: return col2_launch_n<512, G>(a, tm, s);
-    case 1024: return col2_launch_n<1024, G>(a, tm, s);
-    case 2048: if constexpr (G == 2) return col2_launch_n<2048, G>(a, tm, s); else return cudaErrorNotSupported;
+    case 64: if constexpr (G == 1) return col2_launch_n<float, 64, G>(a, tm, s); else return cudaErrorNotSupported;
+    case 128: return col2_launch_n<float, 128, G>(a, tm, s);
+    case 256: return col2_launch_n<float, 256, G>(a, tm, s);
+    case 512: return col2_launch_n<float, 512, G>(a, tm, s);
+    case 1024: return col2_launch_n<float, 1024, G>(a, tm, s);
+    case 2048: if constexpr (G == 2) return col2_launch_n<float, 2048, G>(a, tm, s); else return cudaErrorNotSupported;
     default: return cudaErrorNotSupported;
   }
 }

@@ -266,9 +266,12 @@ fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {
   // several-row CTAs of the half-length kernel there -- always with form 2,
   // never with form 1; ensemble members keep both tables (the autotuner
   // picks the form per pass)
+  // (FP64: the pair form saves a third of the row transforms' instructions
+  // on every grid, so form 0 takes it wherever it exists)
   const bool r2 = p->batch || p->row_form == 2 || p->row_form == 4 ||
-                  (p->row_form == 0 && m.prm.n[0] >= 256 && m.prm.ndim == 2);
-  const bool c2 = p->batch || p->col_form == 2 || p->col_form == 4 || (p->col_form == 0 && m.prm.n[1] >= 256);
+                  (p->row_form == 0 && (p->f64 || (m.prm.n[0] >= 256 && m.prm.ndim == 2)));
+  const bool c2 = p->batch || p->col_form == 2 || p->col_form == 4 ||
+                  (p->col_form == 0 && (p->f64 || m.prm.n[1] >= 256));
   a.tw_row2 = r2 ? m.tw_row2 : nullptr;
   a.tw_col2 = c2 ? m.tw_col2 : nullptr;
   a.tw_row2w = (!p->batch && p->row_form == 3) ? m.tw_row2w : nullptr;
@@ -316,18 +319,18 @@ fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {
   return a;
 }
 
-// FP32 plans take the warp-per-line forms where they apply (KArgs::tw_row2 /
+// Plans take the warp-per-line forms where they apply (KArgs::tw_row2 /
 // tw_col2 set), else the half-length row / tile column kernels.
 cudaError_t launch_row(const fs_plan* p, const fs::KArgs& a, cudaStream_t s) {
-  if (!p->f64 && (a.tw_row2 || a.tw_row2w)) {
-    cudaError_t e = fs::row2_launch_f32(a, s);
+  if (a.tw_row2 || a.tw_row2w) {
+    cudaError_t e = p->f64 ? fs::row2_launch_f64(a, s) : fs::row2_launch_f32(a, s);
     if (e != cudaErrorNotSupported) return e;
   }
   return p->f64 ? fs::row_launch_f64(a, s) : fs::row_launch_f32(a, s);
 }
 cudaError_t launch_col(const fs_plan* p, const Member& m, const fs::KArgs& a, cudaStream_t s) {
-  if (!p->f64 && (a.tw_col2 || a.tw_col2w)) {
-    cudaError_t e = fs::col2_launch_f32(a, m.tmap_col2, s);
+  if (a.tw_col2 || a.tw_col2w) {
+    cudaError_t e = p->f64 ? fs::col2_launch_f64(a, m.tmap_col2, s) : fs::col2_launch_f32(a, m.tmap_col2, s);
     if (e != cudaErrorNotSupported) return e;
   }
   return p->f64 ? fs::col_launch_f64(a, m.tmap_col, s) : fs::col_launch_f32(a, m.tmap_col, s);
@@ -356,12 +359,15 @@ EncodeTiledFn encode_tiled() {
 // for the tensor-core precisions, whose stage is in the column transforms),
 // semi-implicit FS; rows of 256, 512 or 1024 points (2D rows and 3D x
 // lines); 2D columns of 256, 512 or 1024 points with no tensor-core stage.
+// FP64: any x line of 64 to 2048 points, 2D columns of 64 to 512 points.
 bool row2_form(const fs_params& prm, bool f64) {
-  return !f64 && prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && fs::row2_supported(prm.n[0], 1 + prm.p);
+  if (f64) return prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && fs::row2_g64(prm.n[0]) != 0;
+  return prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && fs::row2_supported(prm.n[0], 1 + prm.p);
 }
 // (columns of 2048 points: two warps per line only)
 bool col2_form(const fs_params& prm, bool f64) {
-  return !f64 && prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && prm.ndim == 2 && prm.precision == FS_F32 &&
+  if (f64) return prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && prm.ndim == 2 && fs::col2_g64(prm.n[1]) != 0;
+  return prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && prm.ndim == 2 && prm.precision == FS_F32 &&
          fs::col2_supported(prm.n[1], 1 + prm.p);
 }
 
@@ -388,10 +394,10 @@ bool encode_col_map(Member& m, int nslots, bool f64) {
     if (r != CUDA_SUCCESS) return false;
   }
   if (col2_form(m.prm, f64)) {
-    // [slot][y][kx]: two-column tiles (16-byte rows) of the warp-per-column pass
+    // [slot][y][kx]: two-column tiles of the warp-per-column pass
     cuuint64_t dims[3] = {W, (cuuint64_t)ny, (cuuint64_t)nslots};
     cuuint64_t strides[2] = {W * 8, W * 8 * ny};
-    cuuint32_t box[3] = {2, (cuuint32_t)(ny < 256 ? ny : 256), 1};
+    cuuint32_t box[3] = {(cuuint32_t)(2 * units), (cuuint32_t)(ny < 256 ? ny : 256), 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(&m.tmap_col2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, m.spec, dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -645,6 +651,20 @@ void tc_table(int mode, uint32_t* out) {
       }
 }
 
+// Values per thread of the warp-per-line forms (one warp per line in FP32;
+// 0: no table).
+int row2_e(const fs_params& prm, bool f64) {
+  if (!row2_form(prm, f64)) return 0;
+  return prm.n[0] / (32 * (f64 ? fs::row2_g64(prm.n[0]) : 1));
+}
+int col2_e(const fs_params& prm, bool f64) {
+  if (!col2_form(prm, f64) || (!f64 && prm.n[1] > 1024)) return 0;
+  return prm.n[1] / (32 * (f64 ? fs::col2_g64(prm.n[1]) : 1));
+}
+// FP32 only: the same with two warps per line.
+bool row2w_form(const fs_params& prm, bool f64) { return !f64 && row2_form(prm, f64) && prm.n[0] >= 128; }
+bool col2w_form(const fs_params& prm, bool f64) { return !f64 && col2_form(prm, f64) && prm.n[1] >= 128; }
+
 // Rows of 1024 in FP32 run the x-pass variant with 32 values per thread.
 bool wide_rows(const fs_params& prm, bool f64) { return !f64 && prm.n[0] == 1024; }
 
@@ -677,14 +697,15 @@ TableLayout table_layout(const fs_params& prm, bool f64) {
   o = align16(o + cs * (nx / 2));
   t.tc_b = o;
   o = align16(o + (tc_split(prm.precision) ? 2048 * sizeof(float) : 0));
-  t.tw_row2 = o;  // pair-form row pass: L = nx, E = nx / 32
-  o = align16(o + (row2_form(prm, f64) ? cs * fs::pass_table_size(nx, nx / 32) : 0));
-  t.tw_col2 = o;  // warp-per-column pass: L = ny, E = ny / 32 (up to 1024 points)
-  o = align16(o + (col2_form(prm, f64) && ny <= 1024 ? cs * fs::pass_table_size(ny, ny / 32) : 0));
+  const int er = row2_e(prm, f64), ec = col2_e(prm, f64);
+  t.tw_row2 = o;  // pair-form row pass: L = nx (FP32 E = nx / 32)
+  o = align16(o + (er ? cs * fs::pass_table_size(nx, er, f64) : 0));
+  t.tw_col2 = o;  // warp-per-column pass: L = ny (FP32 E = ny / 32, up to 1024 points)
+  o = align16(o + (ec ? cs * fs::pass_table_size(ny, ec, f64) : 0));
   t.tw_row2w = o;  // two warps per line: E = nx / 64, ny / 64
-  o = align16(o + (row2_form(prm, f64) && nx >= 128 ? cs * fs::pass_table_size(nx, nx / 64) : 0));
+  o = align16(o + (row2w_form(prm, f64) ? cs * fs::pass_table_size(nx, nx / 64) : 0));
   t.tw_col2w = o;
-  o = align16(o + (col2_form(prm, f64) && ny >= 128 ? cs * fs::pass_table_size(ny, ny / 64) : 0));
+  o = align16(o + (col2w_form(prm, f64) ? cs * fs::pass_table_size(ny, ny / 64) : 0));
   t.total = o;
   return t;
 }
@@ -737,10 +758,11 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   for (int k = 0; k < ny; ++k) ky[k] = axis_k2(prm.lap, k, ny, prm.dx[1]);
   for (int k = 0; k < nz && prm.ndim > 2; ++k) kz[k] = axis_k2(prm.lap, k, nz, prm.dx[2]);
   std::vector<long double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i;
-  if (row2_form(prm, f64)) pass_table(nx, nx / 32, f64, r2r, r2i);
-  if (col2_form(prm, f64) && ny <= 1024) pass_table(ny, ny / 32, f64, c2r, c2i);
-  if (row2_form(prm, f64) && nx >= 128) pass_table(nx, nx / 64, f64, r3r, r3i);
-  if (col2_form(prm, f64) && ny >= 128) pass_table(ny, ny / 64, f64, c3r, c3i);
+  const int er = row2_e(prm, f64), ec = col2_e(prm, f64);
+  if (er) pass_table(nx, er, f64, r2r, r2i);
+  if (ec) pass_table(ny, ec, f64, c2r, c2i);
+  if (row2w_form(prm, f64)) pass_table(nx, nx / 64, f64, r3r, r3i);
+  if (col2w_form(prm, f64)) pass_table(ny, ny / 64, f64, c3r, c3i);
   pass_table(t.Lrow, t.Erow, f64, rr, ii);
   if (wide_rows(prm, f64)) pass_table(t.Lrow, 32, f64, wr, wi);
   pass_table(t.Lcol, t.Ecol, f64, cr, ci);
@@ -759,6 +781,8 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
     put_cplx<double>(buf, t.tw_col, cr, ci);
     put_cplx<double>(buf, t.tw_z, zr, zi);
     put_cplx<double>(buf, t.tw_half, hr, hi);
+    put_cplx<double>(buf, t.tw_row2, r2r, r2i);
+    put_cplx<double>(buf, t.tw_col2, c2r, c2i);
   } else {
     put_real<float>(buf, t.k2x, kx);
     put_real<float>(buf, t.k2y, ky);
@@ -781,10 +805,10 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   m.tw_col = dev + t.tw_col;
   m.tw_z = dev + t.tw_z;
   m.tw_half = dev + t.tw_half;
-  m.tw_row2 = row2_form(prm, f64) ? dev + t.tw_row2 : nullptr;
-  m.tw_col2 = col2_form(prm, f64) && ny <= 1024 ? dev + t.tw_col2 : nullptr;
-  m.tw_row2w = row2_form(prm, f64) && nx >= 128 ? dev + t.tw_row2w : nullptr;
-  m.tw_col2w = col2_form(prm, f64) && ny >= 128 ? dev + t.tw_col2w : nullptr;
+  m.tw_row2 = er ? dev + t.tw_row2 : nullptr;
+  m.tw_col2 = ec ? dev + t.tw_col2 : nullptr;
+  m.tw_row2w = row2w_form(prm, f64) ? dev + t.tw_row2w : nullptr;
+  m.tw_col2w = col2w_form(prm, f64) ? dev + t.tw_col2w : nullptr;
   if (const int mode = tc_split(prm.precision)) {
     tc_table(mode, reinterpret_cast<uint32_t*>(buf.data() + t.tc_b));
     m.tc_b = dev + t.tc_b;
@@ -1469,8 +1493,8 @@ fs_status fs_set_pass_forms(fs_plan_t p, int row_form, int col_form) {
   if (row_form == 4 && (p->batch || p->f64 || m.prm.ndim != 2 || !m.tw_row2 || !m.tw_col2 ||
                         !fs::step2_supported(m.prm.n[0], m.prm.n[1], p->nf)))
     return fail(p, FS_ERR_UNSUPPORTED, "the fused step covers single 2D FP32 plans of 256^2, 512^2 or 1024^2, p <= 3");
-  const bool r2ok = p->batch ? p->bargs.maps2 != nullptr : m.tw_row2 != nullptr;
-  const bool c2ok = p->batch ? p->bargs.maps2 != nullptr : m.tw_col2 != nullptr;
+  const bool r2ok = p->batch ? p->bargs.maps2 != nullptr : !p->f64 && m.tw_row2 != nullptr;
+  const bool c2ok = p->batch ? p->bargs.maps2 != nullptr : !p->f64 && m.tw_col2 != nullptr;
   const bool r3ok = !p->batch && m.tw_row2w != nullptr, c3ok = !p->batch && m.tw_col2w != nullptr;
   if ((row_form == 2 && !r2ok) || (col_form == 2 && !c2ok) || (row_form == 3 && !r3ok) || (col_form == 3 && !c3ok))
     return fail(p, FS_ERR_UNSUPPORTED, "the warp-per-line form does not cover this plan's grid or precision");
