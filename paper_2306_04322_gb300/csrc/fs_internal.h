@@ -24,7 +24,26 @@ struct Coef {
   T Mdt, Mdtkc, Ldtke, scale;                               // k-space update
   T idx2, idy2, idz2, kc, ke, dtM, dtL;                     // explicit FD scheme
   T dt;                                                     // adjoint
+  // pointwise stage with the constants multiplied out (Pointwise::fc2, g2)
+  T fc_c, fc_0, fc_h, g_c, g_0, g_dw, g_pair;
 };
+
+// The multiplied-out constants, formed in FP64:
+//   df/dc = fc_c c + fc_0 + fc_h h,
+//   eta - L dt df/deta = eta + q ((g_c c + g_0) q + g_dw (1 - 2 eta)) + g_pair eta (S2 - eta^2),
+//   q = eta (1 - eta).
+template <typename T>
+inline void fill_pointwise(Coef<T>& k, double rho2, double c_alpha, double c_beta, double w, double alpha,
+                           double Ldt) {
+  const double d = c_beta - c_alpha;
+  k.fc_c = (T)(2.0 * rho2);
+  k.fc_0 = (T)(-2.0 * rho2 * c_alpha);
+  k.fc_h = (T)(-2.0 * rho2 * d);
+  k.g_c = (T)(60.0 * Ldt * rho2 * d);
+  k.g_0 = (T)(-30.0 * Ldt * rho2 * d * (c_beta + c_alpha));
+  k.g_dw = (T)(-2.0 * Ldt * w);
+  k.g_pair = (T)(-4.0 * alpha * Ldt * w);
+}
 
 // Arguments of one pass over one simulation (passed by value).  Array
 // pointers are in the plan's precision T (float or double) unless noted.

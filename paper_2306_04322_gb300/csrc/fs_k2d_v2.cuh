@@ -114,7 +114,7 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
       C h = vsplat<C>(T(0)), S2 = vsplat<C>(T(0));
 #pragma unroll
       for (int i = 0; i < P; ++i) {
-        h = cadd(h, pw.hpoly2(e[u][i]));
+        h = pw.add_h2(e[u][i], h);
         S2 = vfma(e[u][i], e[u][i], S2);
       }
       fc[u] = pw.fc2(c[u], h);

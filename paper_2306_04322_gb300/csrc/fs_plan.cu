@@ -248,6 +248,7 @@ void fill_coef(fs::Coef<T>& k, const fs_params& q, double scale) {
   k.Mdtkc = (T)(q.M * q.dt * q.kappa_c);
   k.Ldtke = (T)(q.L * q.dt * q.kappa_eta);
   k.scale = (T)scale;
+  fs::fill_pointwise(k, q.rho2, q.c_alpha, q.c_beta, q.w, q.alpha, q.L * q.dt);
 }
 
 fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {

@@ -103,6 +103,7 @@ void fill_coef_static(fs::Coef<T>& k, const fs_params& q, double scale) {
   k.dtM = (T)(q.dt * q.M);
   k.dtL = (T)(q.dt * q.L);
   k.dt = (T)q.dt;
+  fs::fill_pointwise(k, q.rho2, q.c_alpha, q.c_beta, q.w, q.alpha, q.L * q.dt);
 }
 
 // Byte size of the tables build_tables writes for grid (nx, ny).
