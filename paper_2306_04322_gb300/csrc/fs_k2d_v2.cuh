@@ -76,14 +76,25 @@ constexpr size_t row2_smem_bytes(int nf) {
   return Cfg::BAR_BYTES + Cfg::TW_BYTES + (size_t)(nf + 1) * Cfg::PL * sizeof(cplx<T>);
 }
 
-// Synchronisation of the threads of one line: the warp itself, or the two
-// warps of a line through named barrier 1 + line (64 threads).
-template <int G>
+// Synchronisation of the threads of one line: the warp itself, or the G
+// warps of a line through named barrier BASE + line (32 G threads).  The ids
+// are compile-time constants of a warp-uniform switch: with an id in a
+// register a kernel reserves all 16 barriers, which limits an SM to four CTAs.
+template <int G, int BASE>
 struct LineSync {
-  int id;
+  int line;
   __device__ __forceinline__ void operator()() const {
-    if constexpr (G == 1) __syncwarp();
-    else bar_sync(id, 32 * G);
+    if constexpr (G == 1) {
+      __syncwarp();
+    } else {
+      switch (line) {
+        case 0: bar_sync(BASE, 32 * G); break;
+        case 1: bar_sync(BASE + 1, 32 * G); break;
+        case 2: bar_sync(BASE + 2, 32 * G); break;
+        case 3: bar_sync(BASE + 3, 32 * G); break;
+        default: bar_sync(BASE + 4, 32 * G); break;
+      }
+    }
   }
 };
 
@@ -153,7 +164,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
   const int line = (threadIdx.x >> 5) / G, t = threadIdx.x % TPL;  // line of this thread, thread within it
   const int nw = blockDim.x / TPL;  // lines per CTA = nf
   const long long row0 = 2LL * pair;  // row a; row b = row0 + 1
-  const LineSync<G> lsync{1 + line};
+  const LineSync<G, 1> lsync{line};
   const bool from_real = (a.mode == 1);
 
   if (threadIdx.x == 0) {
@@ -343,7 +354,8 @@ struct Col2Cfg {
   static constexpr int CS = 2 * (int)sizeof(T);               // bytes of a complex value
   static constexpr int TPL = 32 * G;                          // threads per line
   static constexpr int E = NY / TPL;
-  static constexpr int TK = 2;                                // kx columns per CTA
+  static constexpr int TK = F64 ? 1 : 2;                      // kx columns per CTA (16-byte TMA rows)
+  static constexpr int NE = F64 ? 1 : 2;                      // eta_i per field group
   static constexpr int BH = NY < 256 ? NY : 256;              // TMA box height (rows)
   static constexpr int PL = line_pad_len<T>(NY);           // complex per compact column area
   // slot region: the [NY][TK] tile as loaded, then TK compact areas, then the
@@ -356,7 +368,7 @@ struct Col2Cfg {
   static constexpr int HEAD = 128 + TW_BYTES + K2_BYTES;
   // CTAs per SM the registers are budgeted for: FP32 128 per thread at 32
   // values, FP64 at least 64
-  static constexpr int MIN_BLOCKS = F64 ? (G == 1 ? 6 : 8 / G) : (E >= 32 ? 4 / G : (G == 1 ? 4 : 3));
+  static constexpr int MIN_BLOCKS = F64 ? (G <= 2 ? 8 / G : (G == 4 ? 3 : 1)) : (E >= 32 ? 4 / G : (G == 1 ? 4 : 3));
 };
 
 // Shared memory of one CTA: the head and two slot regions.
@@ -405,9 +417,13 @@ __device__ __noinline__ void col2_packed_update(cplx<T>* __restrict__ y, const c
   }
 }
 
-// CTA: two adjacent kx columns (kx0 = 2 blockIdx.x, kx0 + 1) of one field
+// FP32 CTA: two adjacent kx columns (kx0 = 2 blockIdx.x, kx0 + 1) of one field
 // group (blockIdx.y): group 0 holds df/dc and c, group g >= 1 eta_{2g-1} and
-// eta_{2g}; warp (region r, column j), r = 0, 1.  Four warps per CTA and
+// eta_{2g}; warp (region r, column j), r = 0, 1.  FP64 CTA: one column of
+// {df/dc, c} or of one eta_i, the smallest unit there is: the pass is bound by
+// the FP64 pipe, so its time is the busiest SM's share of the transforms
+// (256^2, p = 4: 9.3 transforms per SM on average; 16 on the busiest with the
+// FP32 units, 11 with these).  Four warps per CTA and
 // 1 + ceil(p / 2) groups, so every CTA carries about two transforms per warp
 // and several CTAs share an SM.  The tiles come in by TMA, every warp copies
 // its column to registers, then its region becomes two compact per-column
@@ -415,8 +431,8 @@ __device__ __noinline__ void col2_packed_update(cplx<T>* __restrict__ y, const c
 // transform the results go back to the interleaved tile layout and out by
 // TMA, so the global writes are whole 16-byte rows instead of one 8-byte
 // value per lane and row.
-// Column pair `cpair`, field group `group` of the simulation `a` (blockDim =
-// 128 G); `bar` as for row2_body.  Returns false if a bounded wait gave up.
+// Column pair (FP64: column) `cpair`, field group `group` of the simulation
+// `a` (blockDim = 64 TK G); `bar` as for row2_body.  Returns false if a bounded wait gave up.
 template <typename T, int NY, int G = 1>
 __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tmap, int cpair, int group,
                                           unsigned char* smem_raw, uint64_t* bar, uint32_t parity) {
@@ -428,10 +444,11 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   C* regions = reinterpret_cast<C*>(smem_raw + Cfg::HEAD);
   const int nf = a.nf, p = nf - 1;
   const int line = (threadIdx.x >> 5) / G, t = threadIdx.x % TPL;  // line (region, column), thread in it
-  const int j = line & 1, r = line >> 1;
-  const int nreg = group == 0 ? 2 : (p - 2 * (group - 1) >= 2 ? 2 : 1);
-  // slot of region q of this group: group 0: df/dc (nf), c (0); else eta_{2g-1+q}
-  auto slot_of = [nf, group](int q) { return group == 0 ? (q == 0 ? nf : 0) : 2 * group - 1 + q; };
+  constexpr int TK = Cfg::TK, NE = Cfg::NE;
+  const int j = line % TK, r = line / TK;
+  const int nreg = group == 0 ? 2 : (p - NE * (group - 1) >= NE ? NE : 1);
+  // slot of region q of this group: group 0: df/dc (nf), c (0); else eta_{NE (g - 1) + 1 + q}
+  auto slot_of = [nf, group](int q) { return group == 0 ? (q == 0 ? nf : 0) : NE * (group - 1) + 1 + q; };
   const bool isF = (group == 0 && r == 0), isC = (group == 0 && r == 1);
   const int kx0 = cpair * Cfg::TK, kx = kx0 + j;
   const int H = a.nx / 2;
@@ -468,8 +485,8 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   // named barriers with compile-time ids: 1, 2 per region (its two column
   // lines), 3, 4 per column (df/dc^ handed to the c line), 5.. per line (its
   // G warps, G = 2)
-  auto region_sync = [r]() { if (r == 0) bar_sync(1, 64 * G); else bar_sync(2, 64 * G); };
-  const LineSync<G> lsync{5 + line};
+  auto region_sync = [r]() { if (r == 0) bar_sync(1, 32 * TK * G); else bar_sync(2, 32 * TK * G); };
+  const LineSync<G, 5> lsync{line};
   // both columns of this region have left the tile: it becomes two compact areas
   region_sync();
   C* xa = reg + j * PL;
@@ -549,7 +566,7 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
 }
 
 template <typename T, int NY, int G>
-__global__ void __launch_bounds__(128 * G, Col2Cfg<T, NY, G>::MIN_BLOCKS)
+__global__ void __launch_bounds__(64 * Col2Cfg<T, NY, G>::TK * G, Col2Cfg<T, NY, G>::MIN_BLOCKS)
     fs_col2_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
@@ -578,9 +595,10 @@ cudaError_t col2_launch_n(const KArgs& a, const CUtensorMap& tm, cudaStream_t s)
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_col2_kernel<T, NY, G>, &done);
   if (e != cudaSuccess) return e;
-  const unsigned groups = (unsigned)(1 + (a.nf - 1 + 1) / 2);  // {df/dc, c} and the eta pairs
-  return launch_pdl(fs_col2_kernel<T, NY, G>, dim3((unsigned)(a.nx / 2 / Col2Cfg<T, NY, G>::TK), groups),
-                    dim3((unsigned)(128 * G)), col2_smem_bytes<T, NY, G>(), s, a, tm);
+  using Cfg = Col2Cfg<T, NY, G>;
+  const unsigned groups = (unsigned)(1 + (a.nf - 1 + Cfg::NE - 1) / Cfg::NE);  // {df/dc, c}; NE eta_i each
+  return launch_pdl(fs_col2_kernel<T, NY, G>, dim3((unsigned)(a.nx / 2 / Cfg::TK), groups),
+                    dim3((unsigned)(64 * Cfg::TK * G)), col2_smem_bytes<T, NY, G>(), s, a, tm);
 }
 
 }  // namespace fs

@@ -9,8 +9,8 @@ namespace fs {
 // and that a warp's own chain is short: few values per thread (2 at 64 points,
 // 4 at 128 and 256, 8 above), which costs the fused butterflies almost no
 // instructions (3 per value and radix-2 stage whatever the radix).
-#define FS_ROW64_SIZES(X) X(64, 1) X(128, 1) X(256, 2) X(512, 2) X(1024, 4) X(2048, 8)
-#define FS_COL64_SIZES(X) X(64, 1) X(128, 1) X(256, 2) X(512, 4)
+#define FS_ROW64_SIZES(X) X(64, 1) X(128, 1) X(256, 4) X(512, 4) X(1024, 4) X(2048, 8)
+#define FS_COL64_SIZES(X) X(64, 1) X(128, 1) X(256, 2) X(512, 2) X(1024, 4) X(2048, 8)
 
 int row2_g64(int nx) {
   switch (nx) {

@@ -32,7 +32,9 @@ struct LineCfg {
   static constexpr bool F64 = sizeof(T) == 8;
   static constexpr int E = col_E(NL, F64);
   static constexpr int TPL = NL / E;
-  static constexpr int TK = col_tk(NL, F64, 128);  // 3D line passes: about 128 threads per CTA
+  // about 128 threads per CTA; FP64 64, so that the tiles of a small grid
+  // spread evenly over the SMs (the passes are bound by the FP64 pipe)
+  static constexpr int TK = col_tk(NL, F64, F64 ? 64 : 128);
   static constexpr int THREADS = TPL * TK;
   static constexpr int BH = NL < 256 ? NL : 256;  // TMA box extent along the line
   static constexpr int BAR_BYTES = 128;

@@ -395,10 +395,10 @@ bool encode_col_map(Member& m, int nslots, bool f64) {
     if (r != CUDA_SUCCESS) return false;
   }
   if (col2_form(m.prm, f64)) {
-    // [slot][y][kx]: two-column tiles of the warp-per-column pass
+    // [slot][y][kx]: tiles of the warp-per-column pass with 16-byte rows (FP32 two columns, FP64 one)
     cuuint64_t dims[3] = {W, (cuuint64_t)ny, (cuuint64_t)nslots};
     cuuint64_t strides[2] = {W * 8, W * 8 * ny};
-    cuuint32_t box[3] = {(cuuint32_t)(2 * units), (cuuint32_t)(ny < 256 ? ny : 256), 1};
+    cuuint32_t box[3] = {2, (cuuint32_t)(ny < 256 ? ny : 256), 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(&m.tmap_col2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, m.spec, dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
