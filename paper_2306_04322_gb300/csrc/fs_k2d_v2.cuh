@@ -103,8 +103,8 @@ struct LineSync {
 // four) independent points per iteration -- all loads, then the arithmetic, then
 // the stores (points past the row repeat point n).  areas: [nf + 1][PL],
 // c, eta_i (replaced by g_i), df/dc in area nf.  df/dc is non-finite
-// whenever c or any eta_i is (see the row pass of fs_kernels.cuh): one test
-// of the sum of its lanes covers all inputs.
+// whenever c or any eta_i is (see the row pass of fs_kernels.cuh), so testing
+// it covers all inputs.
 template <typename T, int P, int NX, int PL>
 __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cplx<T>* areas, bool& bad) {
   using C = cplx<T>;
@@ -119,7 +119,7 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
 #pragma unroll
       for (int i = 0; i < P; ++i) e[u][i] = areas[(1 + i) * PL + k[u]];
     }
-    T chk = T(0);
+    FiniteCheck<T> chk;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       C h = vsplat<C>(T(0)), S2 = vsplat<C>(T(0));
@@ -129,11 +129,11 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
         S2 = vfma(e[u][i], e[u][i], S2);
       }
       fc[u] = pw.fc2(c[u], h);
-      chk += fc[u].x + fc[u].y;
+      chk.add(fc[u]);
 #pragma unroll
       for (int i = 0; i < P; ++i) g[u][i] = pw.g2(c[u], e[u][i], S2);
     }
-    bad |= !finite_val(chk);
+    bad |= chk.bad();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       areas[(P + 1) * PL + k[u]] = fc[u];

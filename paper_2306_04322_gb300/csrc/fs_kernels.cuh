@@ -133,6 +133,23 @@ __device__ __forceinline__ bool finite_val(T x) {
   return isfinite(x);
 }
 
+// Finds a NaN or infinity among the pairs shown to it.  FP32: 0 v is NaN for
+// either, one packed instruction per pair; FP64: the exponent bits, off the
+// FP64 pipe.
+template <typename T> struct FiniteCheck;
+template <> struct FiniteCheck<float> {
+  float2 acc = make_float2(0.f, 0.f);
+  __device__ __forceinline__ void add(float2 v) { acc = vfma(v, make_float2(0.f, 0.f), acc); }
+  __device__ __forceinline__ bool bad() const { return !(acc.x == 0.f && acc.y == 0.f); }
+};
+template <> struct FiniteCheck<double> {
+  unsigned acc = 0;
+  __device__ __forceinline__ void add(double2 v) {
+    acc = max(acc, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+  }
+  __device__ __forceinline__ bool bad() const { return acc >= 0x7ff00000u; }
+};
+
 // ---------------------------------------------------------------------------
 // Row pass.  Lines along x.  A CTA holds R rows and four warps; warp w
 // works on fields w, w + 4, ... of all R rows (TPL = L / E threads per line,

@@ -228,13 +228,8 @@ void plan_free_all(fs_plan* p) {
 
 template <typename T>
 void fill_coef(fs::Coef<T>& k, const fs_params& q, double scale) {
-  k.idx2 = (T)(1.0 / (q.dx[0] * q.dx[0]));
-  k.idy2 = (T)(1.0 / (q.dx[1] * q.dx[1]));
-  k.idz2 = (T)(q.ndim > 2 ? 1.0 / (q.dx[2] * q.dx[2]) : 0.0);
   k.kc = (T)q.kappa_c;
   k.ke = (T)q.kappa_eta;
-  k.dtM = (T)(q.dt * q.M);
-  k.dtL = (T)(q.dt * q.L);
   k.dt = (T)q.dt;
   k.two_rho2 = (T)(2.0 * q.rho2);
   k.ca = (T)q.c_alpha;
@@ -249,6 +244,9 @@ void fill_coef(fs::Coef<T>& k, const fs_params& q, double scale) {
   k.Ldtke = (T)(q.L * q.dt * q.kappa_eta);
   k.scale = (T)scale;
   fs::fill_pointwise(k, q.rho2, q.c_alpha, q.c_beta, q.w, q.alpha, q.L * q.dt);
+  const double i2[3] = {1.0 / (q.dx[0] * q.dx[0]), 1.0 / (q.dx[1] * q.dx[1]),
+                        q.ndim > 2 ? 1.0 / (q.dx[2] * q.dx[2]) : 0.0};
+  fs::fill_fd(k, q.rho2, q.kappa_c, q.kappa_eta, q.dt * q.M, q.dt * q.L, i2);
 }
 
 fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {

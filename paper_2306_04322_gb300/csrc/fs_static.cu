@@ -95,13 +95,8 @@ void fill_coef_static(fs::Coef<T>& k, const fs_params& q, double scale) {
   k.Mdtkc = (T)(q.M * q.dt * q.kappa_c);
   k.Ldtke = (T)(q.L * q.dt * q.kappa_eta);
   k.scale = (T)scale;
-  k.idx2 = (T)(1.0 / (q.dx[0] * q.dx[0]));
-  k.idy2 = (T)(1.0 / (q.dx[1] * q.dx[1]));
-  k.idz2 = (T)0;
   k.kc = (T)q.kappa_c;
   k.ke = (T)q.kappa_eta;
-  k.dtM = (T)(q.dt * q.M);
-  k.dtL = (T)(q.dt * q.L);
   k.dt = (T)q.dt;
   fs::fill_pointwise(k, q.rho2, q.c_alpha, q.c_beta, q.w, q.alpha, q.L * q.dt);
 }
