@@ -116,7 +116,7 @@ cudaError_t adjoint3_launch_t(const KArgs& a0, const CUtensorMap& tm_y, const CU
   b.plane0 = 0;
   b.tc = 0;
   constexpr bool f64 = sizeof(T) == 8;
-  e = f64 ? ypass_launch_f64(b, tm_y, -1, 3 * a0.nf, s) : ypass_launch_f32(b, tm_y, -1, 3 * a0.nf, s);
+  e = f64 ? ypass_launch_f64(b, tm_y, -1, a0.nz, 3 * a0.nf, s) : ypass_launch_f32(b, tm_y, -1, a0.nz, 3 * a0.nf, s);
   if (e != cudaSuccess) return e;
   e = cudaErrorInvalidValue;
   switch (a0.nz) {
@@ -127,7 +127,7 @@ cudaError_t adjoint3_launch_t(const KArgs& a0, const CUtensorMap& tm_y, const CU
     default: break;
   }
   if (e != cudaSuccess) return e;
-  e = f64 ? ypass_launch_f64(b, tm_y, 1, 2 * a0.nf, s) : ypass_launch_f32(b, tm_y, 1, 2 * a0.nf, s);
+  e = f64 ? ypass_launch_f64(b, tm_y, 1, a0.nz, 2 * a0.nf, s) : ypass_launch_f32(b, tm_y, 1, a0.nz, 2 * a0.nf, s);
   if (e != cudaSuccess) return e;
   KArgs a1 = a0;
   a1.real = lam_out;

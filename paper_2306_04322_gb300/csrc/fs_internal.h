@@ -81,6 +81,7 @@ struct KArgs {
   const void* tw_col2;     // pass tables of the y line FFT of the warp-per-column form (L = ny, E = ny / 32)
   const void* tw_row2w;    // the same two with two warps per line (E = nx / 64, ny / 64; NULL: not this form)
   const void* tw_col2w;
+  const void* tw_row3;     // pass tables of the 3D x pass with several row pairs per CTA (L = nx, E = 16; NULL: none)
   const void* tc_b;        // tensor-core DFT stage: split 16-point DFT matrix, [hi | lo][32][32] float
   const void* k2x;         // |xi_x|^2 per x bin, nx/2 + 1 entries
   const void* k2y;         // |xi_y|^2 per y bin, ny entries
@@ -96,7 +97,7 @@ struct KArgs {
   int tc;                  // FP32 column transforms: 0 CUDA cores, 1 TF32 x 3, 2 BF16 x 3 tensor-core stage
   int carry3;              // 3D FS: c stays in slot 0 as (kx, ky, z) spectrum between steps; its x spectrum
                            // for the x pass goes to slot nf (see the 3D passes)
-  int plane0;              // y pass: first plane (slot * nz + z) of the launch
+  int plane0;              // y pass: first plane (slot * nz + z) of the launch's first slot
   double M, L, kappa_c, kappa_eta, rho2, c_alpha, c_beta, w, alpha, dt;
   double scale;            // k-space scale 1 / (2 N)
   double inv_npts;         // 1 / N
@@ -134,6 +135,10 @@ cudaError_t col2_launch_f32(const KArgs& a, const CUtensorMap& tm, cudaStream_t 
 // per line (0: no such kernel).
 cudaError_t row2_launch_f64(const KArgs& a, cudaStream_t s);
 cudaError_t col2_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
+// 3D x pass with several row pairs per CTA (FP32, nx of 64 to 512, modes 0
+// and 2; needs KArgs::tw_row3).
+cudaError_t row3_launch_f32(const KArgs& a, cudaStream_t s);
+bool row3_supported(int nx);
 int row2_g64(int nx);
 int col2_g64(int ny);
 bool row2_supported(int nx, int nf);
@@ -164,11 +169,11 @@ cudaError_t adjoint3_launch_f64(const KArgs& a, const CUtensorMap& tm_y, const C
                                 cudaStream_t s);
 // Columns per CTA of the 2D column pass for this grid (the TMA box width).
 int col_tile_width(bool f64, int nx, int ny);
-// 3D passes (fs_k3d_f32.cu / fs_k3d_f64.cu): y transform of nslots slots of
-// every z plane (dir -1 forward with kx = 0 column packing, +1 inverse), and
+// 3D passes (fs_k3d_f32.cu / fs_k3d_f64.cu): y transform of `planes` z planes
+// of nslots slots from plane KArgs::plane0 (dir -1 forward with kx = 0 column packing, +1 inverse), and
 // the z step (forward z, k-space update, inverse z).
-cudaError_t ypass_launch_f32(const KArgs& a, const CUtensorMap& tm, int dir, int nslots, cudaStream_t s);
-cudaError_t ypass_launch_f64(const KArgs& a, const CUtensorMap& tm, int dir, int nslots, cudaStream_t s);
+cudaError_t ypass_launch_f32(const KArgs& a, const CUtensorMap& tm, int dir, int planes, int nslots, cudaStream_t s);
+cudaError_t ypass_launch_f64(const KArgs& a, const CUtensorMap& tm, int dir, int planes, int nslots, cudaStream_t s);
 cudaError_t zstep_launch_f32(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
 cudaError_t zstep_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
 // Free-energy diagnostic, 3D: z transforms and sums of w K2 |phi^|^2 after

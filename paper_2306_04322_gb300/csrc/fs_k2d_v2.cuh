@@ -77,15 +77,19 @@ constexpr size_t row2_smem_bytes(int nf) {
 }
 
 // Synchronisation of the threads of one line: the warp itself, or the G
-// warps of a line through named barrier BASE + line (32 G threads).  The ids
-// are compile-time constants of a warp-uniform switch: with an id in a
-// register a kernel reserves all 16 barriers, which limits an SM to four CTAs.
-template <int G, int BASE>
+// warps of a line through named barrier BASE + line (32 G threads).  With an
+// id in a register a kernel reserves all 16 barriers, which limits an SM to
+// four CTAs; CONST takes compile-time ids from a warp-uniform switch instead
+// (the small FP64 CTAs; the FP32 columns of 2048, two CTAs per SM, lost 5 % to
+// the longer code).
+template <int G, int BASE, bool CONST>
 struct LineSync {
   int line;
   __device__ __forceinline__ void operator()() const {
     if constexpr (G == 1) {
       __syncwarp();
+    } else if constexpr (!CONST) {
+      bar_sync(BASE + line, 32 * G);
     } else {
       switch (line) {
         case 0: bar_sync(BASE, 32 * G); break;
@@ -101,23 +105,25 @@ struct LineSync {
 // Pointwise stage of the pair-form row pass (Section 2.1 derivatives, lane-
 // wise on the two rows of a pair) with p = P known at compile time: U (FP32:
 // four) independent points per iteration -- all loads, then the arithmetic, then
-// the stores (points past the row repeat point n).  areas: [nf + 1][PL],
-// c, eta_i (replaced by g_i), df/dc in area nf.  df/dc is non-finite
+// the stores (points past the rows repeat point n).  areas: [nf + 1][PR][PL]
+// (PR row pairs), c, eta_i (replaced by g_i), df/dc in area nf.  df/dc is non-finite
 // whenever c or any eta_i is (see the row pass of fs_kernels.cuh), so testing
 // it covers all inputs.
-template <typename T, int P, int NX, int PL>
+template <typename T, int P, int NX, int PL, int PR = 1>
 __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cplx<T>* areas, bool& bad) {
   using C = cplx<T>;
   constexpr int PE = P > 0 ? P : 1, U = sizeof(T) == 4 ? 4 : 1;  // FP64: bound by its pipe, not by latency
-  for (int n = threadIdx.x; n < NX; n += U * blockDim.x) {
+  constexpr int FS = PR * PL;
+  for (int n = threadIdx.x; n < PR * NX; n += U * blockDim.x) {
     int k[U];
     C c[U], e[U][PE], fc[U], g[U][PE];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      k[u] = n + u * (int)blockDim.x < NX ? n + u * (int)blockDim.x : n;
+      k[u] = n + u * (int)blockDim.x < PR * NX ? n + u * (int)blockDim.x : n;
+      if (PR > 1) k[u] = (k[u] / NX) * PL + k[u] % NX;
       c[u] = areas[k[u]];
 #pragma unroll
-      for (int i = 0; i < P; ++i) e[u][i] = areas[(1 + i) * PL + k[u]];
+      for (int i = 0; i < P; ++i) e[u][i] = areas[(1 + i) * FS + k[u]];
     }
     FiniteCheck<T> chk;
 #pragma unroll
@@ -136,9 +142,9 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
     bad |= chk.bad();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      areas[(P + 1) * PL + k[u]] = fc[u];
+      areas[(P + 1) * FS + k[u]] = fc[u];
 #pragma unroll
-      for (int i = 0; i < P; ++i) areas[(1 + i) * PL + k[u]] = g[u][i];
+      for (int i = 0; i < P; ++i) areas[(1 + i) * FS + k[u]] = g[u][i];
     }
   }
 }
@@ -164,7 +170,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
   const int line = (threadIdx.x >> 5) / G, t = threadIdx.x % TPL;  // line of this thread, thread within it
   const int nw = blockDim.x / TPL;  // lines per CTA = nf
   const long long row0 = 2LL * pair;  // row a; row b = row0 + 1
-  const LineSync<G, 1> lsync{line};
+  const LineSync<G, 1, Cfg::F64> lsync{line};
   const bool from_real = (a.mode == 1);
 
   if (threadIdx.x == 0) {
@@ -188,6 +194,10 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
       if (from_real ? real_ok(a, src, bytes) : spec_ok(a, src, bytes)) bulk_g2s(areas + f * PL, src, bytes, bar);
     }
   }
+  // all threads: the bounded wait starts when the copies do, however long the
+  // previous pass takes, and no lane of warp 0 polls before lane 0 has issued
+  griddep_wait();
+  __syncwarp();
   griddep_launch_dependents();
   if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
@@ -320,6 +330,152 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
   }
   if (bad) atomicOr(a.flag, FS_FLAG_NONFINITE);
   return true;
+}
+
+// Several row pairs per CTA (3D x passes, FP32, rows of 64 to 512 points,
+// steady steps and the inverse only: modes 0 and 2).  A 3D pass has ny nz
+// rows, so what counts is instructions, not the reach of a few rows over the
+// chip: 16 values per thread and 4 to 32 threads per line (two register
+// passes, one exchange), W warps per field, so that the table fetch and the
+// set-up are shared by PR = W 32 / TPL pairs.  Against the half-length kernel
+// (one real row per line of nx / 2, with its real <-> half-length step), 256^3,
+// p = 2: X1 us per pass against X0.
+template <int NX, int W>
+struct Row3Cfg {
+  static constexpr int E = 16, TPL = NX / E, LPW = 32 / TPL, PR = W * LPW, H = NX / 2;
+  // pitch of a line's area: pad16 layout, a multiple of 16 bytes, and = TPL
+  // (mod 16) where a warp holds several lines, so that a half-warp's lines
+  // start on different banks
+  static constexpr int PL0 = (padded16_len(NX) + 1) & ~1;
+  static constexpr int PL = TPL < 16 ? PL0 + ((TPL - PL0 % 16) + 16) % 16 : PL0;
+  static constexpr int TWS = pass_table_size(NX, E);
+  static constexpr int TW_BYTES = ((TWS * 8) + 127) & ~127;
+  static constexpr size_t smem(int nf) { return 128 + TW_BYTES + (size_t)(nf + 1) * PR * PL * 8; }
+};
+
+template <int NX, int W, int NW>
+__global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 8 / W : 4 / W) fs_row3_kernel(KArgs a) {
+  using C = float2;
+  using Cfg = Row3Cfg<NX, W>;
+  constexpr int E = Cfg::E, TPL = Cfg::TPL, LPW = Cfg::LPW, PR = Cfg::PR, PL = Cfg::PL, H = Cfg::H;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
+  C* tw = reinterpret_cast<C*>(smem_raw + 128);
+  C* areas = reinterpret_cast<C*>(smem_raw + 128 + Cfg::TW_BYTES);  // [nf + 1][PR][PL]
+  const int nf = a.nf;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane % TPL;
+  const int fw = w / W, q = (w % W) * LPW + lane / TPL;  // the warp's field, the line's pair
+  const long long row0 = 2LL * PR * blockIdx.x;          // first row of the CTA
+  C* spec = reinterpret_cast<C*>(a.spec);
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+    mbar_arrive_expect_tx(bar, (uint32_t)(Cfg::TWS * sizeof(C) + nf * PR * NX * sizeof(C)));
+    bulk_g2s(tw, a.tw_row3, (uint32_t)(Cfg::TWS * sizeof(C)), bar);
+  }
+  griddep_wait();  // the spectra are the previous pass's output
+  griddep_launch_dependents();
+  if (w == 0) {
+    __syncwarp();
+    for (int i = lane; i < nf * PR; i += 32) {
+      const int f = i / PR, sl = (f == 0 && a.carry3) ? nf : f;  // 3D carry: c's x spectrum sits in slot nf
+      const C* src = spec + sl * a.slot_stride + (row0 + 2 * (i % PR)) * H;
+      if (spec_ok(a, src, NX * sizeof(C))) bulk_g2s(areas + i * PL, src, NX * sizeof(C), bar);
+    }
+  }
+  __syncthreads();
+  if (!mbar_wait_bounded(bar, 0, first_wait_polls(a))) {
+    if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
+    mbar_wait_bounded(bar, 0, kWaitPolls);  // let the copies land before exiting
+    return;
+  }
+  bool bad = false;
+  auto wsync = []() { __syncwarp(); };
+  for (int ph = 0; ph < 2; ++ph) {
+    const int f = fw + ph;  // inverse: fields 0..nf-1; forward: g_1..g_p and df/dc
+    C* s = areas + (f * PR + q) * PL;
+    auto st = [s](int i, C x) { s[pad16(i)] = x; };
+    auto ld = [s](int i) { return s[pad16(i)]; };
+    C v[E];
+    if (ph == 0) {
+      // conj(Z), Z[k] = X_a[k] + i X_b[k] (as row2_body)
+#pragma unroll
+      for (int m = 0; m < E; ++m) {
+        const int k = t + TPL * m;
+        if (m < E / 2) {
+          const C xa = s[k], xb = s[H + k];
+          v[m] = mk<C>(xa.x - xb.y, -(xa.y + xb.x));
+          if (m == 0 && t == 0) v[m] = mk<C>(xa.x, -xb.x);
+        } else {
+          const int kr = (m == E / 2 && t == 0) ? 0 : NX - k;
+          const C xa = s[kr], xb = s[H + kr];
+          v[m] = mk<C>(xa.x + xb.y, xa.y - xb.x);
+          if (m == E / 2 && t == 0) v[m] = mk<C>(xa.y, -xb.y);
+        }
+      }
+      __syncwarp();  // the staging area becomes the exchange buffer
+    } else {
+#pragma unroll
+      for (int m = 0; m < E; ++m) v[m] = s[t + TPL * m];
+    }
+    warp_line_fft<NX, E, -1>(v, t, tw, st, ld, wsync);
+    if (ph == 0) {
+      if (a.mode == 2) {
+        float* ra = reinterpret_cast<float*>(a.real) + f * a.npts + (row0 + 2 * q) * NX;
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+          const int n = t + TPL * m;
+          if (real_ok(a, &ra[n], 4)) ra[n] = v[m].x;
+          if (real_ok(a, &ra[NX + n], 4)) ra[NX + n] = -v[m].y;
+        }
+        return;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int m = 0; m < E; ++m) s[t + TPL * m] = cconj(v[m]);
+      __syncthreads();
+      const Pointwise<float> pw(a);
+      switch (nf) {
+        case 1: row2_pointwise_fixed<float, 0, NX, PL, PR>(pw, areas, bad); break;
+        case 2: row2_pointwise_fixed<float, 1, NX, PL, PR>(pw, areas, bad); break;
+        case 3: row2_pointwise_fixed<float, 2, NX, PL, PR>(pw, areas, bad); break;
+        case 4: row2_pointwise_fixed<float, 3, NX, PL, PR>(pw, areas, bad); break;
+        default: row2_pointwise_fixed<float, 4, NX, PL, PR>(pw, areas, bad); break;
+      }
+      __syncthreads();
+    } else {
+      // separate the two rows' spectra; Z[nx - k] through shared memory
+      __syncwarp();
+#pragma unroll
+      for (int m = 0; m < E; ++m) s[t + TPL * m] = v[m];
+      __syncwarp();
+      C* Pa = spec + f * a.slot_stride + (row0 + 2 * q) * H;
+      C* Pb = Pa + H;
+#pragma unroll
+      for (int m = 0; m < E / 2; ++m) {
+        const int k = t + TPL * m;
+        const C zk = v[m], zm = s[(m == 0 && t == 0) ? H : NX - k];
+        C pa = mk<C>(zk.x + zm.x, zk.y - zm.y), pb = mk<C>(zk.y + zm.y, zm.x - zk.x);
+        if (m == 0 && t == 0) {
+          pa = mk<C>(2.f * zk.x, 2.f * zm.x);
+          pb = mk<C>(2.f * zk.y, 2.f * zm.y);
+        }
+        if (spec_ok(a, &Pa[k], sizeof(C))) Pa[k] = pa;
+        if (spec_ok(a, &Pb[k], sizeof(C))) Pb[k] = pb;
+      }
+    }
+  }
+  if (bad) atomicOr(a.flag, FS_FLAG_NONFINITE);
+}
+
+template <int NX, int W, int NW>
+cudaError_t row3_launch_nw(const KArgs& a, cudaStream_t s) {
+  using Cfg = Row3Cfg<NX, W>;
+  static unsigned done = 0;
+  cudaError_t e = allow_big_smem(fs_row3_kernel<NX, W, NW>, &done);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(fs_row3_kernel<NX, W, NW>, dim3((unsigned)(a.lines / (2 * Cfg::PR))),
+                    dim3((unsigned)(32 * W * a.nf)), Cfg::smem(a.nf), s, a);
 }
 
 // NW: the most warps per line group the instantiation takes (nf <= NW).
@@ -471,6 +627,10 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   }
   const T* __restrict__ k2xt = reinterpret_cast<const T*>(a.k2x);
   const T kx2 = k2xt[kx];
+  // all threads: the bounded wait starts when the copies do, however long the
+  // previous pass takes, and no lane of warp 0 polls before lane 0 has issued
+  griddep_wait();
+  __syncwarp();
   griddep_launch_dependents();
   if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
@@ -486,7 +646,7 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   // lines), 3, 4 per column (df/dc^ handed to the c line), 5.. per line (its
   // G warps, G = 2)
   auto region_sync = [r]() { if (r == 0) bar_sync(1, 32 * TK * G); else bar_sync(2, 32 * TK * G); };
-  const LineSync<G, 5> lsync{line};
+  const LineSync<G, 5, Cfg::F64> lsync{line};
   // both columns of this region have left the tile: it becomes two compact areas
   region_sync();
   C* xa = reg + j * PL;

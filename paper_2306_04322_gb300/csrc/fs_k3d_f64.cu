@@ -3,8 +3,8 @@
 #include "fs_k3d_impl.cuh"
 
 namespace fs {
-cudaError_t ypass_launch_f64(const KArgs& a, const CUtensorMap& tm, int dir, int nslots, cudaStream_t s) {
-  return ypass_launch_t<double>(a, tm, dir, nslots, s);
+cudaError_t ypass_launch_f64(const KArgs& a, const CUtensorMap& tm, int dir, int planes, int nslots, cudaStream_t s) {
+  return ypass_launch_t<double>(a, tm, dir, planes, nslots, s);
 }
 cudaError_t zstep_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
   return zstep_launch_t<double>(a, tm, s);

@@ -48,9 +48,14 @@ struct LineCfg {
 
 // ---------------------------------------------------------------------------
 // y pass: one CTA per (kx tile, z, slot); DIR = -1 forward (slots 0..nf),
-// DIR = +1 inverse (slots 0..nf-1).  Tensor map: [slot * nz + z][y][kx].
+// DIR = +1 inverse (slots 0..nf-1), from plane a.plane0.  Tensor map:
+// [slot * nz + z][y][kx].  TKC: columns per CTA (the tensor map's box) known
+// at compile time, 0 where a short x axis makes them fewer; the results leave
+// through the tile by TMA.  Both took integer instructions out of a kernel
+// that spent 39 % of its issue slots on addresses (256^3, FP32: Y1 us against
+// Y0 per pass of three slots).
 // ---------------------------------------------------------------------------
-template <typename T, int NY, int DIR, int TCM = TC_NONE>
+template <typename T, int NY, int DIR, int TCM, int TKC>
 __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
     fs_ypass_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   using C = cplx<T>;
@@ -60,11 +65,10 @@ __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   C* tw = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
   C* tile = reinterpret_cast<C*>(smem_raw + Cfg::HEAD);
-  const int tk = blockDim.x / TPL;
-  const int j = threadIdx.x % tk, t = threadIdx.x / tk;
-  const int Lh = a.nx / 2;
+  const int tk = TKC ? TKC : blockDim.x / TPL;
+  const int j = threadIdx.x % tk, t = (threadIdx.x / tk) & (TPL - 1);
   const int kx0 = blockIdx.x * tk;
-  const int plane = blockIdx.y + a.plane0;  // slot * nz + z
+  const int plane = blockIdx.z * a.nz + blockIdx.y + a.plane0;  // slot * nz + z
   // y inverse of c with the 3D carry: c's x spectrum goes to slot nf
   const int oplane = (DIR > 0 && a.carry3 && plane < a.nz) ? plane + a.nf * a.nz : plane;
   if (threadIdx.x == 0) {
@@ -72,12 +76,14 @@ __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
     fence_mbar_init();
   }
   __syncthreads();
+  const int cx = kx0 * (int)(sizeof(C) / 8);
   if (threadIdx.x == 0) {
+    griddep_wait();  // the tile is the previous pass's output
     mbar_arrive_expect_tx(bar, (uint32_t)(NY * tk * sizeof(C)));
-    const int cx = kx0 * (int)(sizeof(C) / 8);
     for (int y0 = 0; y0 < NY; y0 += BH) tma_load_3d(tile + y0 * tk, &tmap, cx, y0, plane, bar);
   }
   copy_to_smem(tw, reinterpret_cast<const C*>(a.tw_col), Cfg::TWS);
+  griddep_wait();  // all threads: the bounded wait below starts when the tile's copy does
   __syncthreads();
   if (!mbar_wait_bounded(bar, 0, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
@@ -130,7 +136,7 @@ __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
       float* bsm = reinterpret_cast<float*>(tile + Cfg::TROWS * tk);
       tc_load_b(bsm, reinterpret_cast<const float*>(a.tc_b));
       __syncthreads();
-      tc_first_pass16<NY, TCM>(reinterpret_cast<float2*>(tile), tk, bsm, a.flag);
+      tc_first_pass16<NY, TCM>(reinterpret_cast<float2*>(tile), tk, bsm, a.flag, 0u);
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = ld(t + TPL * m);
       stockham<NY, E, 16, DIR>(v, t, tw, st, ld, sync);
@@ -166,17 +172,26 @@ __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
       }
     }
   }
-  C* S = reinterpret_cast<C*>(a.spec) + (long long)oplane * NY * Lh + kx0 + j;
+  // out through the tile (every thread has read its last exchange by then)
+  if constexpr (TCM == TC_NONE && sizeof(T) == 4) griddep_launch_dependents();
+  __syncthreads();
 #pragma unroll
-  for (int m = 0; m < E; ++m)
-    if (spec_ok(a, &S[(long long)(t + TPL * m) * Lh], sizeof(C))) S[(long long)(t + TPL * m) * Lh] = v[m];
+  for (int m = 0; m < E; ++m) tile[(t + TPL * m) * tk + j] = v[m];
+  fence_proxy_async_smem();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int y0 = 0; y0 < NY; y0 += BH) tma_store_3d(&tmap, cx, y0, oplane, tile + y0 * tk);
+    bulk_commit();
+    bulk_wait_read();  // the tile is read before the CTA's shared memory goes
+  }
 }
 
 // ---------------------------------------------------------------------------
 // z step: one CTA per (kx tile, ky storage row, field group).  Tensor map:
-// [slot][z][y][kx] with a box of one y row and up to 256 z planes.
+// [slot][z][y][kx] with a box of one y row and up to 256 z planes; TKC and the
+// store as in the y pass (256^3, p = 2, FP32: Z1 us against Z0).
 // ---------------------------------------------------------------------------
-template <typename T, int NZ, int TCM = TC_NONE>
+template <typename T, int NZ, int TCM, int TKC>
 __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 4)
     fs_zstep_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   using C = cplx<T>;
@@ -187,23 +202,23 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 4)
   C* tw = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
   T* k2zt = reinterpret_cast<T*>(smem_raw + Cfg::BAR_BYTES + Cfg::TW_BYTES);
   C* tiles = reinterpret_cast<C*>(smem_raw + Cfg::HEAD);
-  const int tk = blockDim.x / TPL;
-  const int j = threadIdx.x % tk, t = threadIdx.x / tk;
+  const int tk = TKC ? TKC : blockDim.x / TPL;
+  const int j = threadIdx.x % tk, t = (threadIdx.x / tk) & (TPL - 1);
   const int Lh = a.nx / 2, NY = a.ny;
   const int kx0 = blockIdx.x * tk, kx = kx0 + j;
   const int ky = blockIdx.y;  // storage row
   const int g = blockIdx.z;   // field group
   const int nf = a.nf;
   const int nin = (g == 0) ? 2 : 1;
-  const long long zstride = (long long)NY * Lh;
+  const int cx = kx0 * (int)(sizeof(C) / 8);
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
   }
   __syncthreads();
   if (threadIdx.x == 0) {
+    griddep_wait();  // the tiles are the previous pass's output
     mbar_arrive_expect_tx(bar, (uint32_t)(nin * NZ * tk * sizeof(C)));
-    const int cx = kx0 * (int)(sizeof(C) / 8);
     for (int i = 0; i < nin; ++i) {
       const int slot = (g == 0) ? (i == 0 ? nf : 0) : g;
       for (int z0 = 0; z0 < NZ; z0 += BH)
@@ -212,6 +227,7 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 4)
   }
   copy_to_smem(tw, reinterpret_cast<const C*>(a.tw_z), Cfg::TWS);
   for (int i = threadIdx.x; i < NZ; i += blockDim.x) k2zt[i] = reinterpret_cast<const T*>(a.k2z)[i];
+  griddep_wait();  // all threads: the bounded wait below starts when the tiles' copies do
   __syncthreads();
   if (!mbar_wait_bounded(bar, 0, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
@@ -247,7 +263,7 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 4)
     auto st = [tl, tk](int q, C x) { tl[(q + (q >> LOGE)) * tk] = x; };
     auto ld = [tl, tk](int q) { return tl[(q + (q >> LOGE)) * tk]; };
     if constexpr (TCM != TC_NONE) {
-      tc_first_pass16<NZ, TCM>(reinterpret_cast<float2*>(tiles + i * TROWS * tk), tk, bsm, a.flag);
+      tc_first_pass16<NZ, TCM>(reinterpret_cast<float2*>(tiles + i * TROWS * tk), tk, bsm, a.flag, (uint32_t)i);
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = ld(t + TPL * m);
       stockham<NZ, E, 16, -1>(v, t, tw, st, ld, sync);
@@ -307,10 +323,17 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 4)
     auto ld = [tl, tk](int q) { return tl[(q + (q >> LOGE)) * tk]; };
     line_fft<NZ, E, 1>(v, t, tw, st, ld, sync);
   }
-  C* S = reinterpret_cast<C*>(a.spec) + (long long)(g == 0 ? 0 : g) * a.slot_stride + (long long)ky * Lh + kx;
+  if constexpr (TCM == TC_NONE && sizeof(T) == 4) griddep_launch_dependents();
+  sync();
 #pragma unroll
-  for (int m = 0; m < E; ++m)
-    if (spec_ok(a, &S[(long long)(t + TPL * m) * zstride], sizeof(C))) S[(long long)(t + TPL * m) * zstride] = v[m];
+  for (int m = 0; m < E; ++m) xt[(t + TPL * m) * tk + j] = v[m];
+  fence_proxy_async_smem();
+  sync();
+  if (threadIdx.x == 0) {
+    for (int z0 = 0; z0 < NZ; z0 += BH) tma_store_4d(&tmap, cx, ky, z0, g, xt + z0 * tk);
+    bulk_commit();
+    bulk_wait_read();
+  }
 }
 
 // ---- launchers ---------------------------------------------------------------
@@ -431,66 +454,82 @@ cudaError_t energy_z_launch_n(const KArgs& a, const CUtensorMap& tm, cudaStream_
   return cudaGetLastError();
 }
 
-template <typename T, int NY, int DIR, int TCM>
-cudaError_t ypass_launch_tc(const KArgs& a, const CUtensorMap& tm, int nslots, cudaStream_t s) {
+template <typename T, int NY, int DIR, int TCM, int TKC>
+cudaError_t ypass_launch_tk(const KArgs& a, const CUtensorMap& tm, int planes, int nslots, int tk, cudaStream_t s) {
   using Cfg = LineCfg<T, NY>;
-  const int tk = line_tk<T, NY>(a.nx);
   size_t smem = Cfg::HEAD + (size_t)Cfg::TROWS * tk * sizeof(cplx<T>) + (TCM ? 8192 : 0) +
                 (TCM == TC_TF32 ? tc5_extra_bytes(tk * Cfg::TPL) : 0);
   // the tcgen05 stage runs 128-row MMAs over the CTA's (butterfly, column) rows
   if (TCM == TC_TF32 && (tk * Cfg::TPL) % 128 != 0) return cudaErrorNotSupported;
   static unsigned done = 0;
-  cudaError_t e = allow_big_smem(fs_ypass_kernel<T, NY, DIR, TCM>, &done);
+  cudaError_t e = allow_big_smem(fs_ypass_kernel<T, NY, DIR, TCM, TKC>, &done);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)(a.nx / 2 / tk), (unsigned)(a.nz * nslots));
-  fs_ypass_kernel<T, NY, DIR, TCM><<<grid, (unsigned)(tk * Cfg::TPL), smem, s>>>(a, tm);
-  return cudaGetLastError();
+  const dim3 grid((unsigned)(a.nx / 2 / tk), (unsigned)planes, (unsigned)nslots);
+  // The tensor-core stage holds TMEM: those launches do not overlap others.
+  // Nor do the FP64 ones: CTAs of the next pass that start early gather on
+  // the SMs that finish first, and a pass bound by the FP64 pipe lasts as long
+  // as its fullest SM (64^3, p = 4: 217 us per step, 247 with the overlap,
+  // 229 with it allowed only from the end of a CTA, as in FP32 below).
+  if (TCM != TC_NONE || sizeof(T) == 8) {
+    fs_ypass_kernel<T, NY, DIR, TCM, TKC><<<grid, (unsigned)(tk * Cfg::TPL), smem, s>>>(a, tm);
+    return cudaGetLastError();
+  }
+  return launch_pdl(fs_ypass_kernel<T, NY, DIR, TCM, TKC>, grid, dim3((unsigned)(tk * Cfg::TPL)), smem, s, a, tm);
 }
 
 template <typename T, int NY, int DIR>
-cudaError_t ypass_launch_n(const KArgs& a, const CUtensorMap& tm, int nslots, cudaStream_t s) {
+cudaError_t ypass_launch_n(const KArgs& a, const CUtensorMap& tm, int planes, int nslots, cudaStream_t s) {
+  constexpr int TK = LineCfg<T, NY>::TK;
+  const int tk = line_tk<T, NY>(a.nx);
   if constexpr (sizeof(T) == 4 && NY >= 64 && DIR < 0) {
-    if (a.tc == TC_TF32) return ypass_launch_tc<T, NY, DIR, TC_TF32>(a, tm, nslots, s);
-    if (a.tc == TC_BF16X3) return ypass_launch_tc<T, NY, DIR, TC_BF16X3>(a, tm, nslots, s);
+    // (axes of at least 64 points: tk = TK)
+    if (a.tc == TC_TF32) return ypass_launch_tk<T, NY, DIR, TC_TF32, TK>(a, tm, planes, nslots, tk, s);
+    if (a.tc == TC_BF16X3) return ypass_launch_tk<T, NY, DIR, TC_BF16X3, TK>(a, tm, planes, nslots, tk, s);
   }
   if (a.tc != TC_NONE && DIR < 0) return cudaErrorInvalidValue;
-  return ypass_launch_tc<T, NY, DIR, TC_NONE>(a, tm, nslots, s);
+  if (tk == TK) return ypass_launch_tk<T, NY, DIR, TC_NONE, TK>(a, tm, planes, nslots, tk, s);
+  return ypass_launch_tk<T, NY, DIR, TC_NONE, 0>(a, tm, planes, nslots, tk, s);
 }
 
-template <typename T, int NZ, int TCM>
-cudaError_t zstep_launch_tc(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
+template <typename T, int NZ, int TCM, int TKC>
+cudaError_t zstep_launch_tk(const KArgs& a, const CUtensorMap& tm, int tk, cudaStream_t s) {
   using Cfg = LineCfg<T, NZ>;
-  const int tk = line_tk<T, NZ>(a.nx);
   size_t smem = Cfg::HEAD + 2 * (size_t)Cfg::TROWS * tk * sizeof(cplx<T>) + (TCM ? 8192 : 0) +
                 (TCM == TC_TF32 ? tc5_extra_bytes(tk * Cfg::TPL) : 0);
   if (TCM == TC_TF32 && (tk * Cfg::TPL) % 128 != 0) return cudaErrorNotSupported;
   static unsigned done = 0;
-  cudaError_t e = allow_big_smem(fs_zstep_kernel<T, NZ, TCM>, &done);
+  cudaError_t e = allow_big_smem(fs_zstep_kernel<T, NZ, TCM, TKC>, &done);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)(a.nx / 2 / tk), (unsigned)a.ny, (unsigned)a.nf);
-  fs_zstep_kernel<T, NZ, TCM><<<grid, (unsigned)(tk * Cfg::TPL), smem, s>>>(a, tm);
-  return cudaGetLastError();
+  const dim3 grid((unsigned)(a.nx / 2 / tk), (unsigned)a.ny, (unsigned)a.nf);
+  if (TCM != TC_NONE || sizeof(T) == 8) {  // as the y pass
+    fs_zstep_kernel<T, NZ, TCM, TKC><<<grid, (unsigned)(tk * Cfg::TPL), smem, s>>>(a, tm);
+    return cudaGetLastError();
+  }
+  return launch_pdl(fs_zstep_kernel<T, NZ, TCM, TKC>, grid, dim3((unsigned)(tk * Cfg::TPL)), smem, s, a, tm);
 }
 
 template <typename T, int NZ>
 cudaError_t zstep_launch_n(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
+  constexpr int TK = LineCfg<T, NZ>::TK;
+  const int tk = line_tk<T, NZ>(a.nx);
   if constexpr (sizeof(T) == 4 && NZ >= 64) {
-    if (a.tc == TC_TF32) return zstep_launch_tc<T, NZ, TC_TF32>(a, tm, s);
-    if (a.tc == TC_BF16X3) return zstep_launch_tc<T, NZ, TC_BF16X3>(a, tm, s);
+    if (a.tc == TC_TF32) return zstep_launch_tk<T, NZ, TC_TF32, TK>(a, tm, tk, s);
+    if (a.tc == TC_BF16X3) return zstep_launch_tk<T, NZ, TC_BF16X3, TK>(a, tm, tk, s);
   }
   if (a.tc != TC_NONE) return cudaErrorInvalidValue;
-  return zstep_launch_tc<T, NZ, TC_NONE>(a, tm, s);
+  if (tk == TK) return zstep_launch_tk<T, NZ, TC_NONE, TK>(a, tm, tk, s);
+  return zstep_launch_tk<T, NZ, TC_NONE, 0>(a, tm, tk, s);
 }
 
 #define FS_LINE_SIZES(X) X(8) X(16) X(32) X(64) X(128) X(256) X(512)
 
 template <typename T>
-cudaError_t ypass_launch_t(const KArgs& a, const CUtensorMap& tm, int dir, int nslots, cudaStream_t s) {
+cudaError_t ypass_launch_t(const KArgs& a, const CUtensorMap& tm, int dir, int planes, int nslots, cudaStream_t s) {
   switch (a.ny) {
 #define FS_CASE(n)                                                            \
   case n:                                                                     \
-    return dir < 0 ? ypass_launch_n<T, n, -1>(a, tm, nslots, s)               \
-                   : ypass_launch_n<T, n, 1>(a, tm, nslots, s);
+    return dir < 0 ? ypass_launch_n<T, n, -1>(a, tm, planes, nslots, s)       \
+                   : ypass_launch_n<T, n, 1>(a, tm, planes, nslots, s);
     FS_LINE_SIZES(FS_CASE)
 #undef FS_CASE
     default: return cudaErrorInvalidValue;

@@ -683,7 +683,7 @@ __device__ __forceinline__ bool col_body(const KArgs& a, const CUtensorMap* tmap
     if constexpr (TCM != TC_NONE) {
       if (!inv) {
         // first radix-16 pass on tensor cores, the rest on CUDA cores
-        tc_first_pass16<NY, TCM>(reinterpret_cast<float2*>(tiles + it * TROWS * tk), tk, bsm, a.flag);
+        tc_first_pass16<NY, TCM>(reinterpret_cast<float2*>(tiles + it * TROWS * tk), tk, bsm, a.flag, (uint32_t)it);
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = ld(t + TPL * m);
         stockham<NY, E, 16, -1>(v, t, twc, st, ld, sync);

@@ -42,6 +42,7 @@ struct Member {
   void* tc_b = nullptr;  // split DFT matrix of the tensor-core stage (TC precisions)
   void* tw_row2 = nullptr;  // x-line tables of the pair-form row pass (FP32, nx in {256, 512, 1024})
   void* tw_col2 = nullptr;  // y-line tables of the warp-per-column pass (FP32 2D, ny in [64, 1024])
+  void* tw_row3 = nullptr;  // x-line tables of the 3D x pass with several row pairs per CTA (FP32, nx 64 to 512)
   void* tw_row2w = nullptr; // the same with two warps per line (lines of 128 points and more)
   void* tw_col2w = nullptr;
   double* csum = nullptr;
@@ -276,6 +277,7 @@ fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {
   a.tw_row2w = (!p->batch && p->row_form == 3) ? m.tw_row2w : nullptr;
   // columns of 2048 points have only the two-warp form, the default there
   a.tw_col2w = (!p->batch && (p->col_form == 3 || (p->col_form == 0 && m.prm.n[1] == 2048))) ? m.tw_col2w : nullptr;
+  a.tw_row3 = p->row_form == 0 ? m.tw_row3 : nullptr;
   a.tc_b = m.tc_b;
   a.k2x = m.k2x;
   a.k2y = m.k2y;
@@ -321,6 +323,10 @@ fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {
 // Plans take the warp-per-line forms where they apply (KArgs::tw_row2 /
 // tw_col2 set), else the half-length row / tile column kernels.
 cudaError_t launch_row(const fs_plan* p, const fs::KArgs& a, cudaStream_t s) {
+  if (a.tw_row3) {
+    cudaError_t e = fs::row3_launch_f32(a, s);
+    if (e != cudaErrorNotSupported) return e;
+  }
   if (a.tw_row2 || a.tw_row2w) {
     cudaError_t e = p->f64 ? fs::row2_launch_f64(a, s) : fs::row2_launch_f32(a, s);
     if (e != cudaErrorNotSupported) return e;
@@ -500,11 +506,11 @@ cudaError_t launch_pass(const fs_plan* p, const Member& m, const fs::KArgs& a, i
     const bool skip_c = a.carry3 && a.mode == 0;
     b.plane0 = skip_c ? a.nz : 0;
     const int nslots = skip_c ? nf : nf + 1;
-    return p->f64 ? fs::ypass_launch_f64(b, m.tmap_col, -1, nslots, s)
-                  : fs::ypass_launch_f32(b, m.tmap_col, -1, nslots, s);
+    return p->f64 ? fs::ypass_launch_f64(b, m.tmap_col, -1, a.nz, nslots, s)
+                  : fs::ypass_launch_f32(b, m.tmap_col, -1, a.nz, nslots, s);
   }
   if (kind == 2) return p->f64 ? fs::zstep_launch_f64(a, m.tmap_z, s) : fs::zstep_launch_f32(a, m.tmap_z, s);
-  return p->f64 ? fs::ypass_launch_f64(a, m.tmap_col, 1, nf, s) : fs::ypass_launch_f32(a, m.tmap_col, 1, nf, s);
+  return p->f64 ? fs::ypass_launch_f64(a, m.tmap_col, 1, a.nz, nf, s) : fs::ypass_launch_f32(a, m.tmap_col, 1, a.nz, nf, s);
 }
 
 void drop_graph(fs_plan* p) {
@@ -565,7 +571,7 @@ fs_status read_flag(fs_plan* p) {
 //   tc_b[2048] (TC precisions only)         (split DFT matrix of the tensor-core stage, 32-bit words)
 struct TableLayout {
   size_t k2x, k2y, k2z, tw_row, tw_row_w, tw_col, tw_z, tw_half, tc_b, tw_row2, tw_col2, tw_row2w, tw_col2w,
-      total;  // offsets (bytes)
+      tw_row3, total;  // offsets (bytes)
   int Lrow, Erow, Lcol, Ecol, Lz, Ez;
 };
 
@@ -664,6 +670,11 @@ int col2_e(const fs_params& prm, bool f64) {
 bool row2w_form(const fs_params& prm, bool f64) { return !f64 && row2_form(prm, f64) && prm.n[0] >= 128; }
 bool col2w_form(const fs_params& prm, bool f64) { return !f64 && col2_form(prm, f64) && prm.n[1] >= 128; }
 
+// FP32 3D plans: the x pass with several row pairs per CTA.
+bool row3_form(const fs_params& prm, bool f64) {
+  return !f64 && prm.ndim == 3 && prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && fs::row3_supported(prm.n[0]);
+}
+
 // Rows of 1024 in FP32 run the x-pass variant with 32 values per thread.
 bool wide_rows(const fs_params& prm, bool f64) { return !f64 && prm.n[0] == 1024; }
 
@@ -705,6 +716,8 @@ TableLayout table_layout(const fs_params& prm, bool f64) {
   o = align16(o + (row2w_form(prm, f64) ? cs * fs::pass_table_size(nx, nx / 64) : 0));
   t.tw_col2w = o;
   o = align16(o + (col2w_form(prm, f64) ? cs * fs::pass_table_size(ny, ny / 64) : 0));
+  t.tw_row3 = o;  // 3D x pass with several row pairs per CTA: E = 16
+  o = align16(o + (row3_form(prm, f64) ? cs * fs::pass_table_size(nx, 16) : 0));
   t.total = o;
   return t;
 }
@@ -756,12 +769,13 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   for (int k = 0; k <= nx / 2; ++k) kx[k] = axis_k2(prm.lap, k, nx, prm.dx[0]);
   for (int k = 0; k < ny; ++k) ky[k] = axis_k2(prm.lap, k, ny, prm.dx[1]);
   for (int k = 0; k < nz && prm.ndim > 2; ++k) kz[k] = axis_k2(prm.lap, k, nz, prm.dx[2]);
-  std::vector<long double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i;
+  std::vector<long double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i, m3r, m3i;
   const int er = row2_e(prm, f64), ec = col2_e(prm, f64);
   if (er) pass_table(nx, er, f64, r2r, r2i);
   if (ec) pass_table(ny, ec, f64, c2r, c2i);
   if (row2w_form(prm, f64)) pass_table(nx, nx / 64, f64, r3r, r3i);
   if (col2w_form(prm, f64)) pass_table(ny, ny / 64, f64, c3r, c3i);
+  if (row3_form(prm, f64)) pass_table(nx, 16, f64, m3r, m3i);
   pass_table(t.Lrow, t.Erow, f64, rr, ii);
   if (wide_rows(prm, f64)) pass_table(t.Lrow, 32, f64, wr, wi);
   pass_table(t.Lcol, t.Ecol, f64, cr, ci);
@@ -795,6 +809,7 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
     put_cplx<float>(buf, t.tw_col2, c2r, c2i);
     put_cplx<float>(buf, t.tw_row2w, r3r, r3i);
     put_cplx<float>(buf, t.tw_col2w, c3r, c3i);
+    put_cplx<float>(buf, t.tw_row3, m3r, m3i);
   }
   m.k2x = dev + t.k2x;
   m.k2y = dev + t.k2y;
@@ -808,6 +823,7 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   m.tw_col2 = ec ? dev + t.tw_col2 : nullptr;
   m.tw_row2w = row2w_form(prm, f64) ? dev + t.tw_row2w : nullptr;
   m.tw_col2w = col2w_form(prm, f64) ? dev + t.tw_col2w : nullptr;
+  m.tw_row3 = row3_form(prm, f64) ? dev + t.tw_row3 : nullptr;
   if (const int mode = tc_split(prm.precision)) {
     tc_table(mode, reinterpret_cast<uint32_t*>(buf.data() + t.tc_b));
     m.tc_b = dev + t.tc_b;
@@ -1280,8 +1296,8 @@ fs_status fs_free_energy(fs_plan_t p, double* F, double* parts) {
     fs::KArgs b = a;
     b.plane0 = 0;
     if (e == cudaSuccess)
-      e = p->f64 ? fs::ypass_launch_f64(b, m.tmap_col, -1, p->nf, p->stream)
-                 : fs::ypass_launch_f32(b, m.tmap_col, -1, p->nf, p->stream);
+      e = p->f64 ? fs::ypass_launch_f64(b, m.tmap_col, -1, a.nz, p->nf, p->stream)
+                 : fs::ypass_launch_f32(b, m.tmap_col, -1, a.nz, p->nf, p->stream);
     if (e == cudaSuccess)
       e = p->f64 ? fs::energy_z_launch_f64(a, m.tmap_z, p->stream) : fs::energy_z_launch_f32(a, m.tmap_z, p->stream);
   }

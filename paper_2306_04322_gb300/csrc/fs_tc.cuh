@@ -140,12 +140,13 @@ __device__ __forceinline__ void tc_first_pass16_mma(float2* tile, int tk, const 
 
 // ---- tcgen05 (fifth-generation tensor cores, accumulator in TMEM) --------
 template <int NL>
-__device__ __forceinline__ void tc5_first_pass16(float2* tile, int tk, const float* bsm, int* flag);
+__device__ __forceinline__ void tc5_first_pass16(float2* tile, int tk, const float* bsm, int* flag, uint32_t call);
 
 // The stage of precision MODE: TF32 x 3 on tcgen05, BF16 x 3 on mma.sync.
+// call: how many times this CTA has run it before.
 template <int NL, int MODE>
-__device__ __forceinline__ void tc_first_pass16(float2* tile, int tk, const float* bsm, int* flag) {
-  if constexpr (MODE == TC_TF32) tc5_first_pass16<NL>(tile, tk, bsm, flag);
+__device__ __forceinline__ void tc_first_pass16(float2* tile, int tk, const float* bsm, int* flag, uint32_t call) {
+  if constexpr (MODE == TC_TF32) tc5_first_pass16<NL>(tile, tk, bsm, flag, call);
   else tc_first_pass16_mma<NL, MODE>(tile, tk, bsm);
 }
 
@@ -216,8 +217,10 @@ __host__ __device__ constexpr size_t tc5_extra_bytes(int threads) { return 128 +
 // it (tc5_extra_bytes) are the stage's own.  TMEM (64 columns) is allocated
 // and freed inside the call, so no return path of the caller can hold it.
 // `flag` receives FS_FLAG_TIMEOUT if the bounded wait for the MMAs gives up.
+// The mbarrier is initialised by the CTA's first call (call = 0); call k
+// waits for its phase k (a valid mbarrier is not initialised again).
 template <int NL>
-__device__ __forceinline__ void tc5_first_pass16(float2* tile, int tk, const float* bsm, int* flag) {
+__device__ __forceinline__ void tc5_first_pass16(float2* tile, int tk, const float* bsm, int* flag, uint32_t call) {
   constexpr int NB = NL / 16;
   constexpr uint32_t kBlock = 128 * 32 * 4;  // bytes of A per 128-row block (16 x 8 core matrices)
   const int warp = threadIdx.x >> 5;
@@ -260,10 +263,11 @@ __device__ __forceinline__ void tc5_first_pass16(float2* tile, int tk, const flo
     }
   }
   fence_proxy_async_smem();  // the MMAs read A through the async proxy
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && call == 0) {
     mbar_init(mbar, 1);
     fence_mbar_init();
   }
+  __syncwarp();  // the .aligned instructions below need converged warps
   if (warp == 0) tmem_alloc(tslot, 64);
   tc5_fence_before();
   __syncthreads();
@@ -285,10 +289,12 @@ __device__ __forceinline__ void tc5_first_pass16(float2* tile, int tk, const flo
     }
     umma_commit(mbar);
   }
-  if (!mbar_wait_bounded(mbar, 0, kWaitPolls)) {
+  __syncwarp();  // no lane of warp 0 polls (and gives up) before lane 0 has issued the MMAs
+  if (!mbar_wait_bounded(mbar, call & 1u, kWaitPolls)) {
     if (threadIdx.x == 0) atomicOr(flag, 2 /* FS_FLAG_TIMEOUT */);
-    mbar_wait_bounded(mbar, 0, kWaitPolls);
+    mbar_wait_bounded(mbar, call & 1u, kWaitPolls);
   }
+  __syncwarp();
   tc5_fence_after();
   uint32_t d[32];
   tmem_ld32(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + 32u * (uint32_t)(warp >> 2), d);
