@@ -354,7 +354,7 @@ struct Row3Cfg {
 };
 
 template <int NX, int W, int NW>
-__global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 8 / W : 4 / W) fs_row3_kernel(KArgs a) {
+__global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3_kernel(KArgs a) {
   using C = float2;
   using Cfg = Row3Cfg<NX, W>;
   constexpr int E = Cfg::E, TPL = Cfg::TPL, LPW = Cfg::LPW, PR = Cfg::PR, PL = Cfg::PL, H = Cfg::H;

@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
 // store as in the y pass (256^3, p = 2, FP32: Z1 us against Z0).
 // ---------------------------------------------------------------------------
 template <typename T, int NZ, int TCM, int TKC>
-__global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 4)
+__global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, sizeof(T) == 4 ? 5 : 4)
     fs_zstep_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   using C = cplx<T>;
   using Cfg = LineCfg<T, NZ>;
