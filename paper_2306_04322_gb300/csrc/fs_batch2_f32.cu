@@ -95,18 +95,16 @@ cudaError_t row2_batch_launch_f32(const BatchArgs& b, cudaStream_t s) {
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_row2_batch_kernel, &done);
   if (e != cudaSuccess) return e;
-  fs_row2_batch_kernel<<<(unsigned)b.row2_grid, (unsigned)(32 * (b.nf1 - 1)), b.row2_smem, s>>>(
-      b.mem, b.row2_begin, b.nm, b.row2_total);
-  return cudaGetLastError();
+  return launch_pdl(fs_row2_batch_kernel, dim3((unsigned)b.row2_grid), dim3((unsigned)(32 * (b.nf1 - 1))), b.row2_smem,
+                    s, b.mem, b.row2_begin, b.nm, b.row2_total);
 }
 
 cudaError_t col2_batch_launch_f32(const BatchArgs& b, cudaStream_t s) {
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_col2_batch_kernel, &done);
   if (e != cudaSuccess) return e;
-  fs_col2_batch_kernel<<<(unsigned)b.col2_grid, 128, b.col2_smem, s>>>(b.mem_col, b.maps2, b.col2_begin,
-                                                                      b.col2_pairs, b.nm, b.col2_total);
-  return cudaGetLastError();
+  return launch_pdl(fs_col2_batch_kernel, dim3((unsigned)b.col2_grid), dim3(128), b.col2_smem, s, b.mem_col, b.maps2,
+                    b.col2_begin, b.col2_pairs, b.nm, b.col2_total);
 }
 
 }  // namespace fs

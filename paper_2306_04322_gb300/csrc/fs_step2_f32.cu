@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(128, 4)
       if (__syncthreads_or(!ok)) return;
       parity ^= 1u;
     }
+    bulk_wait_all();  // the column pass waits only until its stores have left shared memory
     if (step + 1 < nsteps && !grid_barrier(gsync, gridDim.x, limit, a.flag)) return;
   }
 }
