@@ -12,12 +12,10 @@
 // P passes costs P - 1 shared-memory round trips and no global traffic.
 //
 // Twiddles: per-pass tables built on the host in long double, laid out
-// [pass][r][j] (j = 0..NS-1), so the lanes of a warp, which hold consecutive
-// j, read consecutive entries.  FP32: r = 0..R-1, entry r the twiddle of
-// input r (r = 0 is 1), multiplied in before a constant-root butterfly.
-// FP64: R / 2 entries per j, the roots of the pass's radix-2 stages with the
-// twiddle folded in (fused_dft).  Kernels copy the tables to shared memory
-// first.  No device trigonometry is used.
+// [pass][q][j] (q = 0..R/2-1, j = 0..NS-1): the roots of the pass's radix-2
+// stages with the pass twiddle folded in (fused_dft), so that the lanes of a
+// warp, which hold consecutive j, read consecutive entries.  Kernels copy the
+// tables to shared memory first.  No device trigonometry is used.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -94,6 +92,15 @@ template <> __device__ __forceinline__ float2 vfma<float2>(float2 a, float2 b, f
   return upk2(d);
 }
 
+// FP32 complex products as two packed instructions: the swapped, broadcast and
+// sign-changed operands are operand modifiers of the packed instructions.
+template <> __device__ __forceinline__ float2 cmul<float2>(float2 a, float2 b) {
+  return vfma(a, make_float2(b.x, b.x), vmul(make_float2(a.y, a.x), make_float2(-b.y, b.y)));
+}
+template <> __device__ __forceinline__ float2 cmulc<float2>(float2 a, float2 b) {
+  return vfma(a, make_float2(b.x, b.x), vmul(make_float2(a.y, a.x), make_float2(b.y, -b.y)));
+}
+
 // multiply by +i (DIR = +1) or -i (DIR = -1)
 template <int DIR, typename C> __device__ __forceinline__ C mul_i(C a) {
   return DIR > 0 ? mk<C>(-a.y, a.x) : mk<C>(a.y, -a.x);
@@ -154,16 +161,27 @@ __device__ __forceinline__ C twiddle_small(C a, int k, int len) {
 }
 
 // Radix-2 butterfly with the root folded in: u' = u + w v, v' = u - w v with
-// w = (wx, DIR < 0 ? wy : -wy), as u' by four fused multiply-adds and
-// v' = 2 u - u' by two more: 6 instructions against 8 for the product
-// followed by two complex additions.
+// w = (wx, DIR < 0 ? wy : -wy).  FP64: u' = (u + swap(v) (-wy, wy)) + v (wx, wx)
+// by fused multiply-adds and v' = 2 u - u' by two more, 6 instructions against
+// 8 for the product followed by two additions.  FP32: four packed instructions
+// -- the swap, the broadcasts and the sign changes are operand modifiers --
+// against four scalar and two packed ones.  (FP32 keeps the product apart: in
+// fields that are a mean plus a little, u is large and v small, and the FP64
+// form rounds twice at the size of u; it cost a packed instruction less but
+// doubled the error against 64 bits at 1024^2, 1.1e-6 against 5e-7.)
 template <int DIR, typename C>
 __device__ __forceinline__ void fused_bfly(C& u, C& v, decltype(C::x) wx, decltype(C::x) wy0) {
   using T = decltype(C::x);
   const T wy = DIR < 0 ? wy0 : -wy0;
-  const C x = mk<C>(fma(wx, v.x, fma(-wy, v.y, u.x)), fma(wx, v.y, fma(wy, v.x, u.y)));
-  v = mk<C>(fma(T(2), u.x, -x.x), fma(T(2), u.y, -x.y));
-  u = x;
+  if constexpr (sizeof(T) == 8) {
+    const C x = vfma(v, vsplat<C>(wx), vfma(mk<C>(v.y, v.x), mk<C>(-wy, wy), u));
+    v = vfma(u, vsplat<C>(T(2)), mk<C>(-x.x, -x.y));
+    u = x;
+  } else {
+    const C t = vfma(v, vsplat<C>(wx), vmul(mk<C>(v.y, v.x), mk<C>(-wy, wy)));
+    v = csub(u, t);
+    u = cadd(u, t);
+  }
 }
 
 // In-register DFT of length R (R <= 32) on a[0], a[S], ..., a[(R-1) S],
@@ -203,17 +221,15 @@ __device__ __forceinline__ void reg_dft(C* a) {
       for (int i = 0; i < R; i += len) {
 #pragma unroll
         for (int k = 0; k < len / 2; ++k) {
-          if constexpr (sizeof(C) == 16) {
-            // FP64: roots other than 1 and -+i in the fused butterfly
-            if (k != 0 && 4 * k != len) {
-              const int j = k * 32 / len;  // angle -2 pi j / 32, 0 < j < 16
-              const double wx = j < 8 ? cos32(j) : -cos32(16 - j), wy = j < 8 ? -sin32(j) : -sin32(16 - j);
-              fused_bfly<DIR>(t[i + k], t[i + k + len / 2], wx, wy);
-              continue;
-            }
+          if (k != 0 && 4 * k != len) {  // roots other than 1 and -+i
+            using T = decltype(C::x);
+            const int j = k * 32 / len;  // angle -2 pi j / 32, 0 < j < 16
+            fused_bfly<DIR>(t[i + k], t[i + k + len / 2], (T)(j < 8 ? cos32(j) : -cos32(16 - j)),
+                            (T)(j < 8 ? -sin32(j) : -sin32(16 - j)));
+            continue;
           }
-          C u = t[i + k];
-          C v = twiddle_small<DIR>(t[i + k + len / 2], k, len);
+          C u = t[i + k], v = t[i + k + len / 2];
+          if (k != 0) v = mul_i<DIR>(v);
           t[i + k] = cadd(u, v);
           t[i + k + len / 2] = csub(u, v);
         }
@@ -228,10 +244,10 @@ __device__ __forceinline__ void reg_dft(C* a) {
 // exp(DIR 2 pi i r j / (NS R)) (decimation in time): in stage `len` butterfly
 // k takes the root exp(DIR 2 pi i (j + k NS) / (NS len)), so the twiddles cost
 // nothing beyond the stages' own fused butterflies: 3 instructions per value
-// and stage, against 3.5 to 3.6 for a separate twiddle product at radix 8 or
-// 16.  The FP64 passes are bound by the FP64 pipe, so fewer instructions are
-// less time: 1024^2, p = 2, a step 596 us against 652 us; 64^3, p = 4, 290 us
-// against 305 us.  Roots with k >= len / 4 are -+i times those of k - len / 4.  tw: the
+// and stage (FP32 1.5), against 3.5 to 3.6 for a separate twiddle product at
+// radix 8 or 16.  The FP64 passes are bound by the FP64 pipe, so fewer
+// instructions are less time: 1024^2, p = 2, a step 596 us against 652 us;
+// 64^3, p = 4, 290 us against 305 us.  FP32 (folded twiddles, packed products): 1024^2, p = 2, 25.4 us against 27.4; 2048^2, p = 4, 139 us against 143.  Roots with k >= len / 4 are -+i times those of k - len / 4.  tw: the
 // R / 2 roots of this j, NS entries apart, stage 2 first (stages of length
 // len = 2, 4, 8, 16 hold 1, 1, 2, 4).
 template <int R, int DIR, int S, int NS, typename C>
@@ -263,12 +279,12 @@ __device__ __forceinline__ void fused_dft(C* a, const C* __restrict__ tw) {
 
 // ---- pass structure (identical on host and device) -------------------------
 // Table entries of a pass of radix r after sub-length ns.
-__host__ __device__ constexpr int pass_entries(int ns, int r, bool f64) { return f64 ? ns * (r / 2) : ns * r; }
+__host__ __device__ constexpr int pass_entries(int ns, int r) { return ns * (r / 2); }
 template <int L, int E, int NS>
 struct PassRadix {
   static constexpr int R = imin(E, L / NS);
 };
-// FP64 table entry q of a pass at j (see fused_dft): q = 0 is stage 2, then
+// Table entry q of a pass at j (see fused_dft): q = 0 is stage 2, then
 // stage 4, two of stage 8, four of stage 16; the angle is -2 pi num / den.
 __host__ inline void stage_root(int q, int j, int ns, long long* num, long long* den) {
   int len = 2, k = q;
@@ -282,21 +298,21 @@ __host__ inline void stage_root(int q, int j, int ns, long long* num, long long*
 }
 // offset (in complex entries) of the table of the pass starting at NS
 template <int L, int E, int NS>
-constexpr int pass_table_offset(bool f64) {
+constexpr int pass_table_offset() {
   int off = 0;
   for (int ns = 1; ns < NS;) {
     int r = imin(E, L / ns);
-    if (ns > 1) off += pass_entries(ns, r, f64);
+    if (ns > 1) off += pass_entries(ns, r);
     ns *= r;
   }
   return off;
 }
 // total table size of a line FFT of length L with E per thread
-__host__ __device__ constexpr int pass_table_size(int L, int E, bool f64 = false) {
+__host__ __device__ constexpr int pass_table_size(int L, int E) {
   int off = 0;
   for (int ns = 1; ns < L;) {
     int r = E < L / ns ? E : L / ns;
-    if (ns > 1) off += pass_entries(ns, r, f64);
+    if (ns > 1) off += pass_entries(ns, r);
     ns *= r;
   }
   return off;
@@ -316,19 +332,8 @@ __device__ __forceinline__ void stockham(C (&v)[E], int t, const C* __restrict__
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int b = t + TPL * q;
-    if constexpr (NS > 1) {
-      constexpr bool F64 = sizeof(C) == 16;
-      const int j = b & (NS - 1);
-      const C* w = twp + pass_table_offset<L, E, NS>(F64) + j;
-      if constexpr (F64) {
-        fused_dft<R, DIR, Q, NS>(&v[q], w);
-        continue;
-      } else {
-#pragma unroll
-        for (int r = 1; r < R; ++r) v[q + Q * r] = mul_tw<DIR>(v[q + Q * r], w[r * NS]);
-      }
-    }
-    reg_dft<R, DIR, Q>(&v[q]);
+    if constexpr (NS > 1) fused_dft<R, DIR, Q, NS>(&v[q], twp + pass_table_offset<L, E, NS>() + (b & (NS - 1)));
+    else reg_dft<R, DIR, Q>(&v[q]);
   }
   if constexpr (NS * R < L) {
     sync();
@@ -355,34 +360,6 @@ __device__ __forceinline__ void line_fft(C (&v)[E], int t, const C* __restrict__
                                          Sync sync) {
   static_assert(L % E == 0, "E must divide L");
   stockham<L, E, 1, DIR>(v, t, twp, st, ld, sync);
-}
-
-// Line FFT of length L = E * E held by one warp-sized group of E threads
-// with E values each (E = 32: 1024 points, one warp): two radix-E passes and
-// one exchange, as line_fft, but both passes run the same loop body, so the
-// radix-E butterfly code is emitted once (half the instruction footprint of
-// the unrolled pass sequence; the instruction cache is what the warp-per-line
-// kernels run short of).  twp: the pass table of (L, E), entries [r][j] of
-// the second pass (sub-length E).
-template <int E, int DIR, typename C, class Store, class Load, class Sync>
-__device__ __forceinline__ void line_fft_sq(C (&v)[E], int t, const C* __restrict__ twp, Store st, Load ld,
-                                            Sync sync) {
-#pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    if (pass == 1) {
-#pragma unroll
-      for (int r = 1; r < E; ++r) v[r] = mul_tw<DIR>(v[r], twp[r * E + t]);
-    }
-    reg_dft<E, DIR, 1>(v);
-    if (pass == 0) {
-      sync();
-#pragma unroll
-      for (int r = 0; r < E; ++r) st(t * E + r, v[r]);
-      sync();
-#pragma unroll
-      for (int m = 0; m < E; ++m) v[m] = ld(t + E * m);
-    }
-  }
 }
 
 // Padded shared-memory indices: one spare slot every 32 (pad32) or 16

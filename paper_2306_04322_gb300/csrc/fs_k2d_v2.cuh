@@ -32,15 +32,6 @@
 
 namespace fs {
 
-// Line FFT of the warp-per-line kernels: the looped two-pass form at 1024
-// points (E = 32), the pass sequence of line_fft otherwise.
-template <int L, int E, int DIR, typename C, class Store, class Load, class Sync>
-__device__ __forceinline__ void warp_line_fft(C (&v)[E], int t, const C* __restrict__ twp, Store st, Load ld,
-                                              Sync sync) {
-  if constexpr (L == E * E) line_fft_sq<E, DIR>(v, t, twp, st, ld, sync);
-  else line_fft<L, E, DIR>(v, t, twp, st, ld, sync);
-}
-
 // Padded exchange layout of a line: FP32 one spare slot every 32 elements;
 // FP64 (16-byte elements, 8 lanes per shared-memory wavefront) every 8, so
 // that the writes of E consecutive elements per thread fall on different
@@ -64,7 +55,7 @@ struct Row2Cfg {
   static constexpr int E = NX / TPL;                          // values per thread
   static constexpr int H = NX / 2;                            // packed bins per row
   static constexpr int PL = line_pad_len<T>(NX);           // complex per field area (16-byte multiple)
-  static constexpr int TWS = pass_table_size(NX, E, F64);
+  static constexpr int TWS = pass_table_size(NX, E);
   static constexpr int TW_BYTES = ((TWS * (int)sizeof(cplx<T>)) + 127) & ~127;
   static constexpr int BAR_BYTES = 128;
   static constexpr int MAX_THREADS = TPL * 5;                 // one line per field, nf <= 5
@@ -245,12 +236,12 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
           C z;
           if (k < H) {
             const C xa = s[k], xb = s[H + k];
-            z = (k == 0) ? mk<C>(xa.x, xb.x) : mk<C>(xa.x - xb.y, xa.y + xb.x);
+            z = (k == 0) ? mk<C>(xa.x, xb.x) : cadd(xa, mul_i<1>(xb));
           } else if (k == H) {
             z = mk<C>(s[0].y, s[H].y);
           } else {
             const C xa = s[NX - k], xb = s[H + NX - k];
-            z = mk<C>(xa.x + xb.y, xb.x - xa.y);
+            z = cadd(cconj(xa), mul_i<1>(cconj(xb)));
           }
           v[m] = cconj(z);
         }
@@ -259,7 +250,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = s[t + TPL * m];  // z = g_a + i g_b, natural order
       }
-      warp_line_fft<NX, E, -1>(v, t, tw, st, ld, lsync);
+      line_fft<NX, E, -1>(v, t, tw, st, ld, lsync);
       if (inv) {
         // a + i b = conj(v)
         if (a.mode == 2) {
@@ -296,8 +287,8 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
             pb = mk<C>(T(2) * zk.y, T(2) * zh.y);
           } else {
             const C zm = s[NX - k];
-            pa = mk<C>(zk.x + zm.x, zk.y - zm.y);
-            pb = mk<C>(zk.y + zm.y, zm.x - zk.x);
+            pa = cadd(zk, cconj(zm));
+            pb = cadd(mul_i<-1>(zk), mul_i<1>(cconj(zm)));
           }
           if (c_carried) {
             pa = cscale(pa, cs);
@@ -404,12 +395,12 @@ __global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3
         const int k = t + TPL * m;
         if (m < E / 2) {
           const C xa = s[k], xb = s[H + k];
-          v[m] = mk<C>(xa.x - xb.y, -(xa.y + xb.x));
+          v[m] = cadd(cconj(xa), mul_i<-1>(cconj(xb)));
           if (m == 0 && t == 0) v[m] = mk<C>(xa.x, -xb.x);
         } else {
           const int kr = (m == E / 2 && t == 0) ? 0 : NX - k;
           const C xa = s[kr], xb = s[H + kr];
-          v[m] = mk<C>(xa.x + xb.y, xa.y - xb.x);
+          v[m] = cadd(xa, mul_i<-1>(xb));
           if (m == E / 2 && t == 0) v[m] = mk<C>(xa.y, -xb.y);
         }
       }
@@ -418,7 +409,7 @@ __global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3
 #pragma unroll
       for (int m = 0; m < E; ++m) v[m] = s[t + TPL * m];
     }
-    warp_line_fft<NX, E, -1>(v, t, tw, st, ld, wsync);
+    line_fft<NX, E, -1>(v, t, tw, st, ld, wsync);
     if (ph == 0) {
       if (a.mode == 2) {
         float* ra = reinterpret_cast<float*>(a.real) + f * a.npts + (row0 + 2 * q) * NX;
@@ -455,7 +446,7 @@ __global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3
       for (int m = 0; m < E / 2; ++m) {
         const int k = t + TPL * m;
         const C zk = v[m], zm = s[(m == 0 && t == 0) ? H : NX - k];
-        C pa = mk<C>(zk.x + zm.x, zk.y - zm.y), pb = mk<C>(zk.y + zm.y, zm.x - zk.x);
+        C pa = cadd(zk, cconj(zm)), pb = cadd(mul_i<-1>(zk), mul_i<1>(cconj(zm)));
         if (m == 0 && t == 0) {
           pa = mk<C>(2.f * zk.x, 2.f * zm.x);
           pb = mk<C>(2.f * zk.y, 2.f * zm.y);
@@ -518,7 +509,7 @@ struct Col2Cfg {
   // [NY][TK] tile again for the TMA store; a multiple of 16 complex so every
   // region starts on 128 bytes (TMA)
   static constexpr int SLOT = (((NY * TK > TK * PL) ? NY * TK : TK * PL) + 15) & ~15;
-  static constexpr int TWS = pass_table_size(NY, E, F64);
+  static constexpr int TWS = pass_table_size(NY, E);
   static constexpr int TW_BYTES = ((TWS * CS) + 127) & ~127;
   static constexpr int K2_BYTES = ((NY * (int)sizeof(T)) + 127) & ~127;
   static constexpr int HEAD = 128 + TW_BYTES + K2_BYTES;
@@ -659,7 +650,7 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   // One FFT call site: it 0 forward (all warps), it 1 inverse (c, eta) as
   // conj(FFT(conj(.))).
   for (int it = 0; it < 2; ++it) {
-    warp_line_fft<NY, E, -1>(v, t, tw, st, ld, lsync);
+    line_fft<NY, E, -1>(v, t, tw, st, ld, lsync);
     if (it == 1) break;
     if (isF) {
       // df/dc^: natural layout for the c warp of this column

@@ -38,7 +38,7 @@ struct LineCfg {
   static constexpr int THREADS = TPL * TK;
   static constexpr int BH = NL < 256 ? NL : 256;  // TMA box extent along the line
   static constexpr int BAR_BYTES = 128;
-  static constexpr int TWS = pass_table_size(NL, E, F64);
+  static constexpr int TWS = pass_table_size(NL, E);
   static constexpr int TW_BYTES = ((TWS * (int)sizeof(cplx<T>)) + 127) & ~127;
   static constexpr int K2_BYTES = ((NL * (int)sizeof(T)) + 127) & ~127;
   static constexpr int LOGE = ilog2(E);

@@ -199,7 +199,7 @@ struct RowCfg {
   // registers of 16
   static constexpr int MIN_BLOCKS = F64 ? (E >= 32 ? 2 : 3) : (E >= 32 ? 4 : 7);
   static constexpr int BAR_BYTES = 128;
-  static constexpr int TWS = pass_table_size(L, E, F64);  // twiddle entries (complex)
+  static constexpr int TWS = pass_table_size(L, E);  // twiddle entries (complex)
   static constexpr int TW_BYTES = ((TWS * (int)sizeof(cplx<T>)) + 127) & ~127;
 };
 
@@ -544,7 +544,7 @@ struct ColCfg {
   static constexpr int THREADS = TPL * TK;
   static constexpr int BH = NY < 256 ? NY : 256;  // TMA box height (rows)
   static constexpr int BAR_BYTES = 128;
-  static constexpr int TWS = pass_table_size(NY, E, F64);  // twiddle entries (complex)
+  static constexpr int TWS = pass_table_size(NY, E);  // twiddle entries (complex)
   static constexpr int TW_BYTES = ((TWS * (int)sizeof(cplx<T>)) + 127) & ~127;
   static constexpr int K2_BYTES = ((NY * (int)sizeof(T)) + 127) & ~127;
   static constexpr int LOGE = ilog2(E);

@@ -696,22 +696,22 @@ TableLayout table_layout(const fs_params& prm, bool f64) {
   t.k2z = o;
   o = align16(o + rs * nz);
   t.tw_row = o;
-  o = align16(o + cs * fs::pass_table_size(t.Lrow, t.Erow, f64));
+  o = align16(o + cs * fs::pass_table_size(t.Lrow, t.Erow));
   t.tw_row_w = o;  // wide x-pass variant (32 values per thread): FP32 rows of 1024
   o = align16(o + (wide_rows(prm, f64) ? cs * fs::pass_table_size(t.Lrow, 32) : 0));
   t.tw_col = o;
-  o = align16(o + cs * fs::pass_table_size(t.Lcol, t.Ecol, f64));
+  o = align16(o + cs * fs::pass_table_size(t.Lcol, t.Ecol));
   t.tw_z = o;
-  o = align16(o + cs * (nz > 1 ? fs::pass_table_size(t.Lz, t.Ez, f64) : 0));
+  o = align16(o + cs * (nz > 1 ? fs::pass_table_size(t.Lz, t.Ez) : 0));
   t.tw_half = o;
   o = align16(o + cs * (nx / 2));
   t.tc_b = o;
   o = align16(o + (tc_split(prm.precision) ? 2048 * sizeof(float) : 0));
   const int er = row2_e(prm, f64), ec = col2_e(prm, f64);
   t.tw_row2 = o;  // pair-form row pass: L = nx (FP32 E = nx / 32)
-  o = align16(o + (er ? cs * fs::pass_table_size(nx, er, f64) : 0));
+  o = align16(o + (er ? cs * fs::pass_table_size(nx, er) : 0));
   t.tw_col2 = o;  // warp-per-column pass: L = ny (FP32 E = ny / 32, up to 1024 points)
-  o = align16(o + (ec ? cs * fs::pass_table_size(ny, ec, f64) : 0));
+  o = align16(o + (ec ? cs * fs::pass_table_size(ny, ec) : 0));
   t.tw_row2w = o;  // two warps per line: E = nx / 64, ny / 64
   o = align16(o + (row2w_form(prm, f64) ? cs * fs::pass_table_size(nx, nx / 64) : 0));
   t.tw_col2w = o;
@@ -726,17 +726,17 @@ size_t member_table_bytes(const fs_params& prm, bool f64) { return table_layout(
 
 // Stockham pass tables of a line FFT of length L with E values per thread:
 // for every pass after the first (sub-length NS, radix R = min(E, L/NS)),
-// FP32 entries [r][j] = exp(-2 pi i r j / (NS R)), r < R, j < NS; FP64 entries
-// [q][j], q < R / 2, the roots of the pass's radix-2 stages (fs::stage_root).
-void pass_table(int L, int E, bool f64, std::vector<long double>& re, std::vector<long double>& im) {
+// entries [q][j], q < R / 2, j < NS: the roots of the pass's radix-2 stages
+// (fs::stage_root).
+void pass_table(int L, int E, std::vector<long double>& re, std::vector<long double>& im) {
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int ns = 1; ns < L;) {
     int r = E < L / ns ? E : L / ns;
     if (ns > 1)
-      for (int q = 0; q < (f64 ? r / 2 : r); ++q)
+      for (int q = 0; q < r / 2; ++q)
         for (int j = 0; j < ns; ++j) {
-          long long num = (long long)q * j, den = (long long)ns * r;
-          if (f64) fs::stage_root(q, j, ns, &num, &den);
+          long long num, den;
+          fs::stage_root(q, j, ns, &num, &den);
           long double ang = 2.0L * pi * (long double)(num % den) / (long double)den;
           re.push_back(cosl(ang));
           im.push_back(-sinl(ang));
@@ -771,15 +771,15 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   for (int k = 0; k < nz && prm.ndim > 2; ++k) kz[k] = axis_k2(prm.lap, k, nz, prm.dx[2]);
   std::vector<long double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i, m3r, m3i;
   const int er = row2_e(prm, f64), ec = col2_e(prm, f64);
-  if (er) pass_table(nx, er, f64, r2r, r2i);
-  if (ec) pass_table(ny, ec, f64, c2r, c2i);
-  if (row2w_form(prm, f64)) pass_table(nx, nx / 64, f64, r3r, r3i);
-  if (col2w_form(prm, f64)) pass_table(ny, ny / 64, f64, c3r, c3i);
-  if (row3_form(prm, f64)) pass_table(nx, 16, f64, m3r, m3i);
-  pass_table(t.Lrow, t.Erow, f64, rr, ii);
-  if (wide_rows(prm, f64)) pass_table(t.Lrow, 32, f64, wr, wi);
-  pass_table(t.Lcol, t.Ecol, f64, cr, ci);
-  if (nz > 1) pass_table(t.Lz, t.Ez, f64, zr, zi);
+  if (er) pass_table(nx, er, r2r, r2i);
+  if (ec) pass_table(ny, ec, c2r, c2i);
+  if (row2w_form(prm, f64)) pass_table(nx, nx / 64, r3r, r3i);
+  if (col2w_form(prm, f64)) pass_table(ny, ny / 64, c3r, c3i);
+  if (row3_form(prm, f64)) pass_table(nx, 16, m3r, m3i);
+  pass_table(t.Lrow, t.Erow, rr, ii);
+  if (wide_rows(prm, f64)) pass_table(t.Lrow, 32, wr, wi);
+  pass_table(t.Lcol, t.Ecol, cr, ci);
+  if (nz > 1) pass_table(t.Lz, t.Ez, zr, zi);
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int k = 0; k < nx / 2; ++k) {
     long double ang = 2.0L * pi * (long double)k / (long double)nx;

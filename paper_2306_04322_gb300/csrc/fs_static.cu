@@ -57,20 +57,19 @@ double axis_k2_static(int lap, int k, int n, double dx) {
 size_t up16(size_t v) { return (v + 15) & ~(size_t)15; }
 
 // Writes the Stockham pass tables of (L, E) as complex T at dst, for every
-// pass after the first: FP32 entries [r][j] = exp(-2 pi i r j / (NS R)), FP64
-// the roots of the pass's radix-2 stages (fs::stage_root).
+// pass after the first: the roots of the pass's radix-2 stages
+// (fs::stage_root).
 template <typename T>
 size_t put_pass_table(T* dst, int L, int E) {
   const long double pi = 3.141592653589793238462643383279502884L;
-  const bool f64 = sizeof(T) == 8;
   size_t n = 0;
   for (int ns = 1; ns < L;) {
     int r = E < L / ns ? E : L / ns;
     if (ns > 1)
-      for (int q = 0; q < (f64 ? r / 2 : r); ++q)
+      for (int q = 0; q < r / 2; ++q)
         for (int j = 0; j < ns; ++j) {
-          long long num = (long long)q * j, den = (long long)ns * r;
-          if (f64) fs::stage_root(q, j, ns, &num, &den);
+          long long num, den;
+          fs::stage_root(q, j, ns, &num, &den);
           long double ang = 2.0L * pi * (long double)(num % den) / (long double)den;
           dst[2 * n] = (T)cosl(ang);
           dst[2 * n + 1] = (T)(-sinl(ang));
@@ -107,8 +106,8 @@ size_t tables_bytes(int nx, int ny) {
   const bool f64 = sizeof(T) == 8;
   size_t o = up16(sizeof(T) * (nx / 2 + 1));
   o = up16(o + sizeof(T) * ny);
-  o = up16(o + 2 * sizeof(T) * (size_t)fs::pass_table_size(nx / 2, fs::row_E(nx / 2, f64), f64));
-  o = up16(o + 2 * sizeof(T) * (size_t)fs::pass_table_size(ny, fs::col_E(ny, f64), f64));
+  o = up16(o + 2 * sizeof(T) * (size_t)fs::pass_table_size(nx / 2, fs::row_E(nx / 2, f64)));
+  o = up16(o + 2 * sizeof(T) * (size_t)fs::pass_table_size(ny, fs::col_E(ny, f64)));
   return up16(o + 2 * sizeof(T) * (nx / 2));
 }
 
