@@ -11,7 +11,7 @@ namespace fs {
 
 #define FS_V2_SIZES(X) X(64) X(128) X(256) X(512) X(1024)
 
-__global__ void __launch_bounds__(Row2Cfg<float, 1024>::MAX_THREADS, 3)
+__global__ void __launch_bounds__(Row2Cfg<float, 1024>::MAX_THREADS, 4)
     fs_row2_batch_kernel(const KArgs* __restrict__ mem, const long long* __restrict__ begin, int nm,
                          long long total) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(Row2Cfg<float, 1024>::MAX_THREADS, 3)
   }
 }
 
-__global__ void __launch_bounds__(128, 4)
+__global__ void __launch_bounds__(128, 5)
     fs_col2_batch_kernel(const KArgs* __restrict__ mem, const CUtensorMap* __restrict__ maps,
                          const long long* __restrict__ begin, const int* __restrict__ pairs, int nm,
                          long long total) {
@@ -71,10 +71,10 @@ __global__ void __launch_bounds__(128, 4)
   }
 }
 
-size_t row2_smem_f32(int nx, int nf) {
+size_t row2_smem_f32(int nx, int nf, int mode) {
   switch (nx) {
 #define FS_CASE(n) \
-  case n: return row2_smem_bytes<float, n>(nf);
+  case n: return row2_smem_bytes<float, n>(nf, mode);
     FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
     default: return 0;
@@ -95,7 +95,8 @@ cudaError_t row2_batch_launch_f32(const BatchArgs& b, cudaStream_t s) {
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_row2_batch_kernel, &done);
   if (e != cudaSuccess) return e;
-  return launch_pdl(fs_row2_batch_kernel, dim3((unsigned)b.row2_grid), dim3((unsigned)(32 * (b.nf1 - 1))), b.row2_smem,
+  return launch_pdl(fs_row2_batch_kernel, dim3((unsigned)b.row2_grid), dim3((unsigned)(32 * (b.nf1 - 1))),
+                    b.row2_mode == 1 ? b.row2_smem1 : b.row2_smem,
                     s, b.mem, b.row2_begin, b.nm, b.row2_total);
 }
 

@@ -204,7 +204,8 @@ struct BatchArgs {
   const int* col2_pairs;        // column pairs of each simulation
   long long row2_total, col2_total;
   long long row2_grid, col2_grid;
-  size_t row2_smem, col2_smem;
+  size_t row2_smem, row2_smem1, col2_smem;  // row2_smem1: row pass in mode 1
+  int row2_mode;                // mode of the row pass launched
   int row_form, col_form;       // chosen per pass: 1 half-length / tile kernels, 2 warp-per-line kernels
 };
 cudaError_t row_batch_launch_f32(const BatchArgs& b, cudaStream_t s);
@@ -213,7 +214,7 @@ cudaError_t col_batch_launch_f32(const BatchArgs& b, cudaStream_t s);
 cudaError_t col_batch_launch_f64(const BatchArgs& b, cudaStream_t s);
 cudaError_t row2_batch_launch_f32(const BatchArgs& b, cudaStream_t s);
 cudaError_t col2_batch_launch_f32(const BatchArgs& b, cudaStream_t s);
-size_t row2_smem_f32(int nx, int nf);
+size_t row2_smem_f32(int nx, int nf, int mode);
 size_t col2_smem_f32(int ny);
 int col2_groups(int nf);
 size_t row_smem_f32(int nx, int nf);

@@ -61,10 +61,14 @@ struct Row2Cfg {
   static constexpr int MAX_THREADS = TPL * 5;                 // one line per field, nf <= 5
 };
 
+// One area per field; df/dc takes c's place after the pointwise stage, but for
+// mode 1, whose forward phase still needs c (the area it saves is a CTA or two
+// more per SM: a 64-member ensemble, with the tighter register budgets of its
+// kernels, 403 us per step against 431).
 template <typename T, int NX, int G = 1>
-constexpr size_t row2_smem_bytes(int nf) {
+constexpr size_t row2_smem_bytes(int nf, int mode) {
   using Cfg = Row2Cfg<T, NX, G>;
-  return Cfg::BAR_BYTES + Cfg::TW_BYTES + (size_t)(nf + 1) * Cfg::PL * sizeof(cplx<T>);
+  return Cfg::BAR_BYTES + Cfg::TW_BYTES + (size_t)(nf + (mode == 1 ? 1 : 0)) * Cfg::PL * sizeof(cplx<T>);
 }
 
 // Synchronisation of the threads of one line: the warp itself, or the G
@@ -96,12 +100,13 @@ struct LineSync {
 // Pointwise stage of the pair-form row pass (Section 2.1 derivatives, lane-
 // wise on the two rows of a pair) with p = P known at compile time: U (FP32:
 // four) independent points per iteration -- all loads, then the arithmetic, then
-// the stores (points past the rows repeat point n).  areas: [nf + 1][PR][PL]
-// (PR row pairs), c, eta_i (replaced by g_i), df/dc in area nf.  df/dc is non-finite
+// the stores (points past the rows repeat point n).  areas: [nf][PR][PL]
+// (PR row pairs), c, eta_i (replaced by g_i); df/dc to the area at fcd (may be
+// c's own).  df/dc is non-finite
 // whenever c or any eta_i is (see the row pass of fs_kernels.cuh), so testing
 // it covers all inputs.
 template <typename T, int P, int NX, int PL, int PR = 1>
-__device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cplx<T>* areas, bool& bad) {
+__device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cplx<T>* areas, cplx<T>* fcd, bool& bad) {
   using C = cplx<T>;
   constexpr int PE = P > 0 ? P : 1, U = sizeof(T) == 4 ? 4 : 1;  // FP64: bound by its pipe, not by latency
   constexpr int FS = PR * PL;
@@ -133,7 +138,7 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
     bad |= chk.bad();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      areas[(P + 1) * FS + k[u]] = fc[u];
+      fcd[k[u]] = fc[u];
 #pragma unroll
       for (int i = 0; i < P; ++i) areas[(1 + i) * FS + k[u]] = g[u][i];
     }
@@ -141,8 +146,8 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
 }
 
 // One row pair (rows 2 pair and 2 pair + 1) of the simulation `a`, one warp
-// per field (blockDim = 32 nf).  Field areas [nf + 1][PL] (the last one holds
-// df/dc): staging of the bulk copies, then the warp's exchange buffer (pad32
+// per field (blockDim = 32 nf).  Field areas [nf][PL], one more in mode 1
+// (row2_smem_bytes): staging of the bulk copies, then the warp's exchange buffer (pad32
 // layout), then the pair values in natural order for the pointwise stage.
 // `bar` is an initialised mbarrier whose next phase has parity `parity`; the
 // ensemble kernel calls this once per work item.  Returns false if a bounded
@@ -158,6 +163,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
   C* tw = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
   C* areas = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES + Cfg::TW_BYTES);
   const int nf = a.nf;
+  C* fcd = a.mode == 1 ? areas + nf * PL : areas;  // area of df/dc
   const int line = (threadIdx.x >> 5) / G, t = threadIdx.x % TPL;  // line of this thread, thread within it
   const int nw = blockDim.x / TPL;  // lines per CTA = nf
   const long long row0 = 2LL * pair;  // row a; row b = row0 + 1
@@ -209,7 +215,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
     const int items = nf + 1 - f0 - (inv ? 1 : 0);  // inverse: fields 0..nf-1; forward: f0..nf
     for (int i = line; i < items; i += nw) {
       const int f = f0 + i;
-      C* s = areas + f * PL;
+      C* s = f == nf ? fcd : areas + f * PL;
       auto st = [s](int q, C x) { s[line_pad<T, NX>(q)] = x; };
       auto ld = [s](int q) { return s[line_pad<T, NX>(q)]; };
       C v[E];
@@ -306,14 +312,14 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
     // pointwise stage: pairs (row a, row b) of every field, lane-wise
     const Pointwise<T> pw(a);
     if constexpr (PC >= 0) {
-      row2_pointwise_fixed<T, PC, NX, PL>(pw, areas, bad);
+      row2_pointwise_fixed<T, PC, NX, PL>(pw, areas, fcd, bad);
     } else {
       switch (nf) {  // p known at compile time for every supported field count
-        case 1: row2_pointwise_fixed<T, 0, NX, PL>(pw, areas, bad); break;
-        case 2: row2_pointwise_fixed<T, 1, NX, PL>(pw, areas, bad); break;
-        case 3: row2_pointwise_fixed<T, 2, NX, PL>(pw, areas, bad); break;
-        case 4: row2_pointwise_fixed<T, 3, NX, PL>(pw, areas, bad); break;
-        case 5: row2_pointwise_fixed<T, 4, NX, PL>(pw, areas, bad); break;
+        case 1: row2_pointwise_fixed<T, 0, NX, PL>(pw, areas, fcd, bad); break;
+        case 2: row2_pointwise_fixed<T, 1, NX, PL>(pw, areas, fcd, bad); break;
+        case 3: row2_pointwise_fixed<T, 2, NX, PL>(pw, areas, fcd, bad); break;
+        case 4: row2_pointwise_fixed<T, 3, NX, PL>(pw, areas, fcd, bad); break;
+        case 5: row2_pointwise_fixed<T, 4, NX, PL>(pw, areas, fcd, bad); break;
         default: break;
       }
     }
@@ -341,7 +347,7 @@ struct Row3Cfg {
   static constexpr int PL = TPL < 16 ? PL0 + ((TPL - PL0 % 16) + 16) % 16 : PL0;
   static constexpr int TWS = pass_table_size(NX, E);
   static constexpr int TW_BYTES = ((TWS * 8) + 127) & ~127;
-  static constexpr size_t smem(int nf) { return 128 + TW_BYTES + (size_t)(nf + 1) * PR * PL * 8; }
+  static constexpr size_t smem(int nf) { return 128 + TW_BYTES + (size_t)nf * PR * PL * 8; }
 };
 
 template <int NX, int W, int NW>
@@ -352,7 +358,7 @@ __global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   C* tw = reinterpret_cast<C*>(smem_raw + 128);
-  C* areas = reinterpret_cast<C*>(smem_raw + 128 + Cfg::TW_BYTES);  // [nf + 1][PR][PL]
+  C* areas = reinterpret_cast<C*>(smem_raw + 128 + Cfg::TW_BYTES);  // [nf][PR][PL], df/dc over c
   const int nf = a.nf;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane % TPL;
   const int fw = w / W, q = (w % W) * LPW + lane / TPL;  // the warp's field, the line's pair
@@ -384,7 +390,7 @@ __global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3
   auto wsync = []() { __syncwarp(); };
   for (int ph = 0; ph < 2; ++ph) {
     const int f = fw + ph;  // inverse: fields 0..nf-1; forward: g_1..g_p and df/dc
-    C* s = areas + (f * PR + q) * PL;
+    C* s = areas + ((f == nf ? 0 : f) * PR + q) * PL;
     auto st = [s](int i, C x) { s[pad16(i)] = x; };
     auto ld = [s](int i) { return s[pad16(i)]; };
     C v[E];
@@ -427,11 +433,11 @@ __global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3
       __syncthreads();
       const Pointwise<float> pw(a);
       switch (nf) {
-        case 1: row2_pointwise_fixed<float, 0, NX, PL, PR>(pw, areas, bad); break;
-        case 2: row2_pointwise_fixed<float, 1, NX, PL, PR>(pw, areas, bad); break;
-        case 3: row2_pointwise_fixed<float, 2, NX, PL, PR>(pw, areas, bad); break;
-        case 4: row2_pointwise_fixed<float, 3, NX, PL, PR>(pw, areas, bad); break;
-        default: row2_pointwise_fixed<float, 4, NX, PL, PR>(pw, areas, bad); break;
+        case 1: row2_pointwise_fixed<float, 0, NX, PL, PR>(pw, areas, areas, bad); break;
+        case 2: row2_pointwise_fixed<float, 1, NX, PL, PR>(pw, areas, areas, bad); break;
+        case 3: row2_pointwise_fixed<float, 2, NX, PL, PR>(pw, areas, areas, bad); break;
+        case 4: row2_pointwise_fixed<float, 3, NX, PL, PR>(pw, areas, areas, bad); break;
+        default: row2_pointwise_fixed<float, 4, NX, PL, PR>(pw, areas, areas, bad); break;
       }
       __syncthreads();
     } else {
@@ -741,7 +747,7 @@ cudaError_t row2_launch_nw(const KArgs& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const int lines = a.nf < NW ? a.nf : NW;  // lines in flight; more fields take a second round
   return launch_pdl(fs_row2_kernel<T, NX, G, NW>, dim3((unsigned)(a.lines / 2)), dim3((unsigned)(32 * G * lines)),
-                    row2_smem_bytes<T, NX, G>(a.nf), s, a);
+                    row2_smem_bytes<T, NX, G>(a.nf, a.mode), s, a);
 }
 
 template <typename T, int NY, int G>

@@ -441,6 +441,7 @@ void* fd_scratch(const fs_plan* p, const Member& m) {
 cudaError_t launch_batch_pass(const fs_plan* p, int mode, int kind, cudaStream_t s) {
   fs::BatchArgs b = p->bargs;
   if (mode == 1) b.mem = p->bmem1;
+  b.row2_mode = mode;
   if (kind == 0) {
     if (b.row_form == 2) return fs::row2_batch_launch_f32(b, s);
     return p->f64 ? fs::row_batch_launch_f64(b, s) : fs::row_batch_launch_f32(b, s);
@@ -864,7 +865,7 @@ fs_status setup_batch(fs_plan* p) {
   std::vector<CUtensorMap> maps2(nm);
   std::vector<long long> rb2(nm + 1, 0), cb2(nm + 1, 0);
   std::vector<int> pairs2(nm, 0);
-  size_t rsm2 = 0, csm2 = 0;
+  size_t rsm2 = 0, rsm21 = 0, csm2 = 0;
   p->batch = true;  // make_args: ensemble members keep both forms' tables
   for (int e = 0; e < nm; ++e) {
     const Member& m = p->members[order[e]];
@@ -884,7 +885,8 @@ fs_status setup_batch(fs_plan* p) {
       pairs2[e] = nx / 4;  // nx / 2 columns, two per item
       rb2[e + 1] = rb2[e] + ny / 2;
       cb2[e + 1] = cb2[e] + (long long)pairs2[e] * fs::col2_groups(p->nf);
-      rsm2 = std::max(rsm2, fs::row2_smem_f32(nx, p->nf));
+      rsm2 = std::max(rsm2, fs::row2_smem_f32(nx, p->nf, 0));
+      rsm21 = std::max(rsm21, fs::row2_smem_f32(nx, p->nf, 1));
       csm2 = std::max(csm2, fs::col2_smem_f32(ny));
     }
   }
@@ -940,6 +942,7 @@ fs_status setup_batch(fs_plan* p) {
     b.row2_grid = b.row2_total;
     b.col2_grid = b.col2_total;
     b.row2_smem = rsm2;
+    b.row2_smem1 = rsm21;
     b.col2_smem = csm2;
   }
   return FS_OK;

@@ -117,7 +117,7 @@ cudaError_t step2_launch_n(const KArgs& a, const CUtensorMap& tm, unsigned* gsyn
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_step2_kernel<N>, &done);
   if (e != cudaSuccess) return e;
-  const size_t r = row2_smem_bytes<float, N, 1>(a.nf), c = col2_smem_bytes<float, N, 1>();
+  const size_t r = row2_smem_bytes<float, N, 1>(a.nf, 0), c = col2_smem_bytes<float, N, 1>();
   const size_t smem = r > c ? r : c;
   int dev = 0, sms = 0, per_sm = 0;
   e = cudaGetDevice(&dev);
