@@ -23,34 +23,42 @@ namespace fs {
 //   H_k,k = rho2 (cb - ca)(cb + ca - 2c) h''(eta_k)
 //           + w [2 - 12 eta_k + 12 eta_k^2 + 4 alpha sum_{j != k} eta_j^2],
 //   H_k,l = 8 w alpha eta_k eta_l (k != l),  h''(e) = 60 e (1 - e)(1 - 2e).
-template <typename T>
-__device__ __forceinline__ void hessian_apply(const Pointwise<T>& pw, T c, const T* eta, int p, const T* mu,
-                                              T* out) {
-  T S2 = T(0);
-  for (int i = 0; i < p; ++i) S2 += eta[i] * eta[i];
-  out[0] = pw.two_rho2 * mu[0];
-  const T alpha = pw.four_alpha * T(0.25);
-  for (int k = 0; k < p; ++k) {
-    const T e = eta[k];
-    const T hck = -pw.two_rho2 * pw.dcab * pw.dh(e);
-    out[0] += hck * mu[1 + k];
-    const T d2h = T(60) * e * (T(1) - e) * (T(1) - T(2) * e);
-    T hkk = pw.rho2dcab * (pw.cab - T(2) * c) * d2h +
-            pw.w * (T(2) - T(12) * e + T(12) * e * e + T(4) * alpha * (S2 - e * e));
-    T acc = hck * mu[0] + hkk * mu[1 + k];
-    for (int l = 0; l < p; ++l)
-      if (l != k) acc += T(8) * pw.w * alpha * e * eta[l] * mu[1 + l];
-    out[1 + k] = acc;
+// out = H mu on the two grid points of a pair (lane-wise), P = p known at
+// compile time.
+template <int P, typename T>
+__device__ __forceinline__ void hessian_apply(const Pointwise<T>& pw, const cplx<T> (&u)[P + 1],
+                                              const cplx<T> (&mu)[P + 1], cplx<T> (&out)[P + 1]) {
+  using C = cplx<T>;
+  auto k = [](T v) { return vsplat<C>(v); };
+  const T wa8 = T(2) * pw.w * pw.four_alpha;  // 8 w alpha
+  C S2 = k(T(0)), em = k(T(0));               // sum eta_j^2, sum eta_j mu_j
+#pragma unroll
+  for (int i = 1; i <= P; ++i) {
+    S2 = vfma(u[i], u[i], S2);
+    em = vfma(u[i], mu[i], em);
+  }
+  const C chem = vfma(u[0], k(T(-120) * pw.rho2dcab), k(T(60) * pw.rho2dcab * pw.cab));  // 60 rho2 dcab (cab - 2c)
+  out[0] = vmul(mu[0], k(pw.two_rho2));
+#pragma unroll
+  for (int i = 1; i <= P; ++i) {
+    const C e = u[i], ne = mk<C>(-e.x, -e.y);
+    const C q = vfma(e, ne, e);                                             // e (1 - e)
+    const C hck = vmul(k(T(-30) * pw.two_rho2 * pw.dcab), vmul(q, q));      // H_c,i
+    const C dw = vfma(q, k(T(-12)), k(T(2)));                               // 2 - 12 e + 12 e^2
+    const C well = vfma(vfma(e, ne, S2), k(pw.four_alpha), dw);             // + 4 alpha (S2 - e^2)
+    const C hkk = vfma(vmul(chem, q), vfma(e, k(T(-2)), k(T(1))), vmul(well, k(pw.w)));
+    out[0] = vfma(hck, mu[i], out[0]);
+    const C cross = vmul(vmul(e, k(wa8)), vfma(ne, mu[i], em));             // sum over j != i
+    out[i] = vfma(hck, mu[0], vfma(hkk, mu[i], cross));
   }
 }
 
 // ---------------------------------------------------------------------------
-// Adjoint row forward: CTA of nf + 1 warps and R rows (as the step's row
-// pass).  Inputs real: lam' (a.real), u (a.aux).  Outputs 2 x^ of lam'_phi,
+// Adjoint row forward: CTA of 3 nf warps, one per transform, and R rows.  Inputs real: lam' (a.real), u (a.aux).  Outputs 2 x^ of lam'_phi,
 // u_phi, f_phi(u) into adjoint slots [0, nf), [nf, 2nf), [2nf, 3nf).
 // ---------------------------------------------------------------------------
-template <typename T, int NX>
-__global__ void __launch_bounds__(192) fs_adj_row_fwd_kernel(KArgs a) {
+template <typename T, int NX, int P>
+__global__ void __launch_bounds__(96 * (P + 1)) fs_adj_row_fwd_kernel(KArgs a) {
   using C = cplx<T>;
   using Cfg = RowCfg<T, NX>;
   constexpr int L = Cfg::L, E = Cfg::E, TPL = Cfg::TPL, R = Cfg::R, PL = Cfg::PL;
@@ -58,7 +66,7 @@ __global__ void __launch_bounds__(192) fs_adj_row_fwd_kernel(KArgs a) {
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   C* twr = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
   C* slots = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES + Cfg::TW_BYTES);
-  const int nf = a.nf, nw = blockDim.x >> 5;
+  constexpr int nf = P + 1;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane / TPL, t = lane % TPL;
   const int Reff = a.lines < R ? (int)a.lines : R;
@@ -73,6 +81,8 @@ __global__ void __launch_bounds__(192) fs_adj_row_fwd_kernel(KArgs a) {
     mbar_init(bar, 1);
     fence_mbar_init();
   }
+  griddep_wait();  // everything read or written below may belong to the previous grid
+  griddep_launch_dependents();
   __syncthreads();
   if (threadIdx.x == 0) {
     const uint32_t bytes = (uint32_t)(L * sizeof(C));
@@ -92,28 +102,31 @@ __global__ void __launch_bounds__(192) fs_adj_row_fwd_kernel(KArgs a) {
   // f(u) into slots [2nf, 3nf)
   {
     const Pointwise<T> pw(a);
-    const int p = nf - 1;
+    const T A = T(-60) * pw.rho2dcab, B = T(30) * pw.rho2dcab * pw.cab, W = T(2) * pw.w, F = pw.w * pw.four_alpha;
     for (int idx = threadIdx.x; idx < Reff * L; idx += blockDim.x) {
       const int r = idx / L, i0 = idx % L;
       const C c = slot(nf, r)[i0];
-      C h = mk<C>(T(0), T(0)), S2 = mk<C>(T(0), T(0));
-      for (int i = 0; i < p; ++i) {
-        const C e = slot(nf + 1 + i, r)[i0];
-        h.x += pw.hpoly(e.x);
-        h.y += pw.hpoly(e.y);
-        S2.x += e.x * e.x;
-        S2.y += e.y * e.y;
+      C e[nf], h = vsplat<C>(T(0)), S2 = vsplat<C>(T(0));
+#pragma unroll
+      for (int i = 1; i < nf; ++i) {
+        e[i] = slot(nf + i, r)[i0];
+        h = pw.add_h2(e[i], h);
+        S2 = vfma(e[i], e[i], S2);
       }
-      slot(2 * nf, r)[i0] = mk<C>(pw.fc(c.x, h.x), pw.fc(c.y, h.y));
-      for (int i = 0; i < p; ++i) {
-        const C e = slot(nf + 1 + i, r)[i0];
-        slot(2 * nf + 1 + i, r)[i0] = mk<C>(pw.feta(c.x, e.x, S2.x), pw.feta(c.y, e.y, S2.y));
+      slot(2 * nf, r)[i0] = pw.fc2(c, h);
+      const C chem = vfma(c, vsplat<C>(A), vsplat<C>(B));  // 30 rho2 dcab (cab - 2c)
+#pragma unroll
+      for (int i = 1; i < nf; ++i) {
+        const C ne = mk<C>(-e[i].x, -e[i].y), q = vfma(e[i], ne, e[i]);
+        const C in = vfma(chem, q, vfma(e[i], vsplat<C>(T(-2) * W), vsplat<C>(W)));
+        slot(2 * nf + i, r)[i0] = vfma(q, in, vmul(vmul(e[i], vsplat<C>(F)), vfma(e[i], ne, S2)));
       }
     }
   }
   __syncthreads();
   C* spec = reinterpret_cast<C*>(a.spec);
-  for (int o = w; o < 3 * nf; o += nw) {
+  {
+    const int o = w;
     C* s = slot(o, g);
     auto st = [s](int i, C v) { s[Cfg::P16 ? pad16(i) : pad32(i)] = v; };
     auto ld = [s](int i) { return s[Cfg::P16 ? pad16(i) : pad32(i)]; };
@@ -150,41 +163,96 @@ __global__ void __launch_bounds__(192) fs_adj_row_fwd_kernel(KArgs a) {
 // lam'_phi, u_phi, f_phi; forward y; sensitivities into acc[0..3]; writes
 // D1 lam'^ (slot phi) and D2 lam'^ (slot nf + phi), inverse y, scaled 1/(2N).
 // ---------------------------------------------------------------------------
+// A field kind has two parameters: the rate (M or L) and its gradient
+// coefficient; their sums accumulate per thread in FP64, or in FP32 as exact
+// products added into an unevaluated pair (two-sum): GB300 issues one FP64
+// instruction where it issues 32 to 64 FP32 ones, and the FP64 sums had been
+// most of the FP32 kernel's time.
+template <typename T>
+struct AdjSum;
+template <>
+struct AdjSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct AdjSum<float> {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b), e = fmaf(a, b, -p);  // a b = p + e
+    const float t = __fadd_rn(hi, p), v = __fadd_rn(t, -hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fadd_rn(hi, -__fadd_rn(t, -v)), __fadd_rn(p, -v)), e));
+    hi = t;
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
 template <typename T>
 struct AdjCoef {
   T Mdt, Ldt, kc, ke, dt;
-  // multipliers and their parameter derivatives at K2 for field kind f (0: c)
-  __device__ __forceinline__ void eval(int f, T k2, T& d1, T& d2, T* dd1, T* dd2) const {
-    if (f == 0) {
-      const T den = T(1) + Mdt * kc * k2 * k2, i2 = T(1) / (den * den);
-      d1 = T(1) / den;
-      d2 = -Mdt * k2 / den;
-      dd1[0] = -dt * kc * k2 * k2 * i2;          // d/dM
-      dd1[1] = T(0);                             // d/dL
-      dd1[2] = -Mdt * k2 * k2 * i2;              // d/dkappa_c
-      dd1[3] = T(0);                             // d/dkappa_eta
-      dd2[0] = -dt * k2 * i2;
-      dd2[1] = T(0);
-      dd2[2] = Mdt * Mdt * k2 * k2 * k2 * i2;
-      dd2[3] = T(0);
-    } else {
-      const T den = T(1) + Ldt * ke * k2, i2 = T(1) / (den * den);
-      d1 = T(1) / den;
-      d2 = -Ldt / den;
-      dd1[0] = T(0);
-      dd1[1] = -dt * ke * k2 * i2;
-      dd1[2] = T(0);
-      dd1[3] = -Ldt * k2 * i2;
-      dd2[0] = T(0);
-      dd2[1] = -dt * i2;
-      dd2[2] = T(0);
-      dd2[3] = Ldt * Ldt * k2 * i2;
+  __device__ explicit AdjCoef(const KArgs& a) {
+    const Coef<T>& co = coef<T>(a);
+    Mdt = co.Mdt;
+    Ldt = co.Ldt;
+    kc = co.kc;
+    ke = co.ke;
+    dt = co.dt;
+  }
+  __device__ __forceinline__ static T recip(T y) {  // y >= 1
+    const T r = KUpdate<T>::quot(T(1), y);
+    if constexpr (sizeof(T) == 4) return fmaf(r, fmaf(-y, r, 1.f), r);  // one Newton step after the 2 ulp quotient
+    else return r;
+  }
+  // One mode at K2 of field kind f (0: c): va = D1 lam', vb = D2 lam' (times
+  // scale), and Re conj(lam') (dD1 u + dD2 f) of its two parameters into r, g.
+  template <typename C>
+  __device__ __forceinline__ void mode(int f, T k2, T scale, C l, C u, C fu, C& va, C& vb, AdjSum<T>& r,
+                                       AdjSum<T>& g) const {
+    const T kk = f == 0 ? k2 * k2 : k2, rate = f == 0 ? Mdt : Ldt, kap = f == 0 ? kc : ke, m2 = f == 0 ? k2 : T(1);
+    const T d1 = recip(T(1) + rate * kap * kk), i2 = d1 * d1;
+    const T d2 = -rate * m2 * d1;
+    va = cscale(l, d1 * scale);
+    vb = cscale(l, d2 * scale);
+    const T r1 = -dt * kap * kk * i2, r2 = -dt * m2 * i2;                  // d/d rate of D1, D2
+    const T g1 = -rate * kk * i2, g2 = rate * rate * kk * m2 * i2;          // d/d kappa
+    const C tr = vfma(u, vsplat<C>(r1), vmul(fu, vsplat<C>(r2))), tg = vfma(u, vsplat<C>(g1), vmul(fu, vsplat<C>(g2)));
+    r.add(l.x, tr.x);
+    r.add(l.y, tr.y);
+    g.add(l.x, tg.x);
+    g.add(l.y, tg.y);
+  }
+  // The sums of a warp, each thread's times its weight w, into acc (c: M and
+  // kappa_c; eta: L and kappa_eta).
+  __device__ __forceinline__ static void reduce(int f, const AdjSum<T>& r, const AdjSum<T>& g, double w, double* acc) {
+    double v[2] = {w * r.value(), w * g.value()};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+      if ((threadIdx.x & 31) == 0 && v[q] != 0.0) atomicAdd(&acc[2 * q + (f == 0 ? 0 : 1)], v[q]);
     }
   }
 };
 
+// Columns per CTA of the adjoint column pass: about 64 threads (tiles of 16
+// bytes or more per row), so that the pass reaches every SM on small grids:
+// three transforms forward and two back per tile and field, 512^2, p = 2,
+// FP32: 105 us with 96 CTAs of 256 threads and the sums in FP64, 20 us now.
 template <typename T, int NY>
-__global__ void __launch_bounds__(ColCfg<T, NY>::THREADS) fs_adj_col_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
+struct AdjColCfg {
+  using CC = ColCfg<T, NY>;
+  static constexpr int T0 = col_tk(NY, CC::F64, 64);
+  static constexpr int TK = (!CC::F64 && T0 < 2) ? 2 : T0;
+  // a whole number of warps (the shuffles of the sums)
+  static constexpr int THREADS = TK * CC::TPL;
+  static constexpr size_t smem(int tk) { return CC::HEAD + (size_t)3 * CC::TROWS * tk * sizeof(cplx<T>); }
+};
+
+// TKC: columns per CTA known at compile time (0: a short x axis has fewer).
+template <typename T, int NY, int TKC>
+__global__ void __launch_bounds__(AdjColCfg<T, NY>::THREADS < 32 ? 32 : AdjColCfg<T, NY>::THREADS)
+    fs_adj_col_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   using C = cplx<T>;
   using Cfg = ColCfg<T, NY>;
   constexpr int E = Cfg::E, TPL = Cfg::TPL, BH = Cfg::BH, TROWS = Cfg::TROWS, LOGE = Cfg::LOGE;
@@ -193,24 +261,30 @@ __global__ void __launch_bounds__(ColCfg<T, NY>::THREADS) fs_adj_col_kernel(KArg
   C* twc = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
   T* k2yt = reinterpret_cast<T*>(smem_raw + Cfg::BAR_BYTES + Cfg::TW_BYTES);
   C* tiles = reinterpret_cast<C*>(smem_raw + Cfg::HEAD);  // [3][TROWS][tk]
-  const int tk = blockDim.x / TPL;
-  const int j = threadIdx.x % tk, t = threadIdx.x / tk;
   const int Lh = a.nx / 2, nf = a.nf;
+  const int tk = TKC ? TKC : (AdjColCfg<T, NY>::TK < Lh ? AdjColCfg<T, NY>::TK : Lh);
+  const int j = threadIdx.x % tk, t0 = threadIdx.x / tk, t = t0 & (TPL - 1);
+  // a CTA is rounded up to whole warps: the threads beyond the tile repeat
+  // its values without storing them
+  const bool live = t0 < TPL;
   const int kx0 = blockIdx.x * tk, kx = kx0 + j, phi = blockIdx.y;
   const int fk = phi == 0 ? 0 : 1;
+  const int cx = kx0 * (int)(sizeof(C) / 8);
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
   }
   __syncthreads();
   if (threadIdx.x == 0) {
+    griddep_wait();  // the tiles are the row pass's output
     mbar_arrive_expect_tx(bar, (uint32_t)(3 * NY * tk * sizeof(C)));
-    const int cx = kx0 * (int)(sizeof(C) / 8);
     for (int i = 0; i < 3; ++i)
       for (int y0 = 0; y0 < NY; y0 += BH) tma_load_3d(tiles + (i * TROWS + y0) * tk, &tmap, cx, y0, i * nf + phi, bar);
   }
   copy_to_smem(twc, reinterpret_cast<const C*>(a.tw_col), Cfg::TWS);
   for (int i = threadIdx.x; i < NY; i += blockDim.x) k2yt[i] = reinterpret_cast<const T*>(a.k2y)[i];
+  griddep_wait();
+  griddep_launch_dependents();
   __syncthreads();
   if (!mbar_wait_bounded(bar, 0, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
@@ -219,9 +293,10 @@ __global__ void __launch_bounds__(ColCfg<T, NY>::THREADS) fs_adj_col_kernel(KArg
   }
   auto sync = []() { __syncthreads(); };
   // forward y of the three tiles, results back in natural layout
+#pragma unroll 1
   for (int i = 0; i < 3; ++i) {
     C* tl = tiles + i * TROWS * tk + j;
-    auto st = [tl, tk](int q, C x) { tl[(q + (q >> LOGE)) * tk] = x; };
+    auto st = [tl, tk, live](int q, C x) { if (live) tl[(q + (q >> LOGE)) * tk] = x; };
     auto ld = [tl, tk](int q) { return tl[(q + (q >> LOGE)) * tk]; };
     C v[E];
 #pragma unroll
@@ -229,22 +304,17 @@ __global__ void __launch_bounds__(ColCfg<T, NY>::THREADS) fs_adj_col_kernel(KArg
     line_fft<NY, E, -1>(v, t, twc, st, ld, sync);
     sync();
 #pragma unroll
-    for (int m = 0; m < E; ++m) tl[(t + TPL * m) * tk] = v[m];
+    for (int m = 0; m < E; ++m)
+      if (live) tl[(t + TPL * m) * tk] = v[m];
   }
   sync();
-  const Coef<T>& co = coef<T>(a);
-  AdjCoef<T> ac;
-  ac.Mdt = co.Mdt;
-  ac.Ldt = co.Ldt;
-  ac.kc = co.kc;
-  ac.ke = co.ke;
-  ac.dt = co.dt;
+  const AdjCoef<T> ac(a);
   const T* k2xt = reinterpret_cast<const T*>(a.k2x);
-  const T kx2 = k2xt[kx], kxn2 = k2xt[Lh], scale = co.scale;
+  const T kx2 = k2xt[kx], kxn2 = k2xt[Lh], scale = coef<T>(a).scale;
   const C* TL = tiles + 0 * TROWS * tk;  // Lam'
   const C* TU = tiles + 1 * TROWS * tk;  // U
   const C* TF = tiles + 2 * TROWS * tk;  // Fu
-  double g4[4] = {0.0, 0.0, 0.0, 0.0};
+  AdjSum<T> sr, sg;
   C va[E], vb[E];
   const bool col0 = (kx0 == 0 && j == 0);
 #pragma unroll
@@ -252,7 +322,6 @@ __global__ void __launch_bounds__(ColCfg<T, NY>::THREADS) fs_adj_col_kernel(KArg
     const int ky = t + TPL * m;
     const T ky2 = k2yt[ky];
     const C l = TL[ky * tk + j], u = TU[ky * tk + j], f = TF[ky * tk + j];
-    T d1, d2, dd1[4], dd2[4];
     if (col0) {
       // split the packed column into its kx = 0 (P) and kx = nx/2 (Q) parts
       const int kq = (NY - ky) & (NY - 1);
@@ -260,60 +329,50 @@ __global__ void __launch_bounds__(ColCfg<T, NY>::THREADS) fs_adj_col_kernel(KArg
       const C lP = cscale(cadd(l, lq), T(0.5)), lQ = cscale(mul_i<-1>(csub(l, lq)), T(0.5));
       const C uP = cscale(cadd(u, uq), T(0.5)), uQ = cscale(mul_i<-1>(csub(u, uq)), T(0.5));
       const C fP = cscale(cadd(f, fq), T(0.5)), fQ = cscale(mul_i<-1>(csub(f, fq)), T(0.5));
-      ac.eval(fk, kx2 + ky2, d1, d2, dd1, dd2);
-      C aP = cscale(lP, d1 * scale), bP = cscale(lP, d2 * scale);
-      for (int q = 0; q < 4; ++q)
-        g4[q] += (double)lP.x * (dd1[q] * uP.x + dd2[q] * fP.x) + (double)lP.y * (dd1[q] * uP.y + dd2[q] * fP.y);
-      ac.eval(fk, kxn2 + ky2, d1, d2, dd1, dd2);
-      C aQ = cscale(lQ, d1 * scale), bQ = cscale(lQ, d2 * scale);
-      for (int q = 0; q < 4; ++q)
-        g4[q] += (double)lQ.x * (dd1[q] * uQ.x + dd2[q] * fQ.x) + (double)lQ.y * (dd1[q] * uQ.y + dd2[q] * fQ.y);
+      C aP, bP, aQ, bQ;
+      ac.mode(fk, kx2 + ky2, scale, lP, uP, fP, aP, bP, sr, sg);
+      ac.mode(fk, kxn2 + ky2, scale, lQ, uQ, fQ, aQ, bQ, sr, sg);
       va[m] = cadd(aP, mul_i<1>(aQ));
       vb[m] = cadd(bP, mul_i<1>(bQ));
     } else {
-      ac.eval(fk, kx2 + ky2, d1, d2, dd1, dd2);
-      va[m] = cscale(l, d1 * scale);
-      vb[m] = cscale(l, d2 * scale);
-      for (int q = 0; q < 4; ++q)
-        g4[q] += 2.0 * ((double)l.x * (dd1[q] * u.x + dd2[q] * f.x) + (double)l.y * (dd1[q] * u.y + dd2[q] * f.y));
+      ac.mode(fk, kx2 + ky2, scale, l, u, f, va[m], vb[m], sr, sg);
     }
   }
-  for (int q = 0; q < 4; ++q) {
-    double v = g4[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(&a.acc[q], v);
-  }
+  // the conjugate half of the columns kx > 0 is not stored: weight 2
+  AdjCoef<T>::reduce(fk, sr, sg, live ? (col0 ? 1.0 : 2.0) : 0.0, a.acc);
   sync();
-  // inverse y of D1 lam'^ (exchange in tile 0) and D2 lam'^ (tile 1)
-  C* base = reinterpret_cast<C*>(a.spec) + kx;
-  {
-    C* tl = tiles + 0 * TROWS * tk + j;
-    auto st = [tl, tk](int q, C x) { tl[(q + (q >> LOGE)) * tk] = x; };
+  // inverse y of D1 lam'^ (exchange in tile 0, to slot phi) and D2 lam'^
+  // (tile 1, to slot nf + phi), out through the tiles
+  auto inverse = [&](C(&v)[E], C* tile) {
+    C* tl = tile + j;
+    auto st = [tl, tk, live](int q, C x) { if (live) tl[(q + (q >> LOGE)) * tk] = x; };
     auto ld = [tl, tk](int q) { return tl[(q + (q >> LOGE)) * tk]; };
-    line_fft<NY, E, 1>(va, t, twc, st, ld, sync);
-    C* S = base + (long long)phi * a.slot_stride;
+    line_fft<NY, E, 1>(v, t, twc, st, ld, sync);
+    sync();
 #pragma unroll
-    for (int m = 0; m < E; ++m) S[(long long)(t + TPL * m) * Lh] = va[m];
-  }
-  {
-    C* tl = tiles + 1 * TROWS * tk + j;
-    auto st = [tl, tk](int q, C x) { tl[(q + (q >> LOGE)) * tk] = x; };
-    auto ld = [tl, tk](int q) { return tl[(q + (q >> LOGE)) * tk]; };
-    line_fft<NY, E, 1>(vb, t, twc, st, ld, sync);
-    C* S = base + (long long)(nf + phi) * a.slot_stride;
-#pragma unroll
-    for (int m = 0; m < E; ++m) S[(long long)(t + TPL * m) * Lh] = vb[m];
+    for (int m = 0; m < E; ++m)
+      if (live) tl[(t + TPL * m) * tk] = v[m];
+  };
+  inverse(va, tiles);
+  inverse(vb, tiles + TROWS * tk);
+  fence_proxy_async_smem();
+  sync();
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i)
+      for (int y0 = 0; y0 < NY; y0 += BH) tma_store_3d(&tmap, cx, y0, i * nf + phi, tiles + (i * TROWS + y0) * tk);
+    bulk_commit();
+    bulk_wait_read();
   }
 }
 
 // ---------------------------------------------------------------------------
 // Adjoint row inverse: inverse x transforms of G1 lam' (slots [0, nf)) and
 // G2 lam' (slots [nf, 2nf)); lambda_phi = G1 lam'_phi + sum H_phi,psi G2 lam'_psi
-// with H at u (a.aux, real); result to a.real (lambda_out).
+// with H at u (a.aux, real); result to a.real (lambda_out).  2 nf warps, one
+// per transform.
 // ---------------------------------------------------------------------------
-template <typename T, int NX>
-__global__ void __launch_bounds__(192) fs_adj_row_inv_kernel(KArgs a) {
+template <typename T, int NX, int P>
+__global__ void __launch_bounds__(64 * (P + 1)) fs_adj_row_inv_kernel(KArgs a) {
   using C = cplx<T>;
   using Cfg = RowCfg<T, NX>;
   constexpr int L = Cfg::L, E = Cfg::E, TPL = Cfg::TPL, R = Cfg::R, PL = Cfg::PL;
@@ -321,7 +380,7 @@ __global__ void __launch_bounds__(192) fs_adj_row_inv_kernel(KArgs a) {
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   C* twr = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
   C* slots = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES + Cfg::TW_BYTES);
-  const int nf = a.nf, nw = blockDim.x >> 5;
+  constexpr int nf = P + 1;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane / TPL, t = lane % TPL;
   const int Reff = a.lines < R ? (int)a.lines : R;
@@ -335,6 +394,8 @@ __global__ void __launch_bounds__(192) fs_adj_row_inv_kernel(KArgs a) {
     mbar_init(bar, 1);
     fence_mbar_init();
   }
+  griddep_wait();  // everything read or written below may belong to the previous grid
+  griddep_launch_dependents();
   __syncthreads();
   if (threadIdx.x == 0) {
     const uint32_t bytes = (uint32_t)(L * sizeof(C));
@@ -352,7 +413,8 @@ __global__ void __launch_bounds__(192) fs_adj_row_inv_kernel(KArgs a) {
     mbar_wait_bounded(bar, 0, kWaitPolls);
     return;
   }
-  for (int o = w; o < 2 * nf; o += nw) {
+  {
+    const int o = w;
     C* s = slot(o, g);
     auto st = [s](int i, C v) { s[Cfg::P16 ? pad16(i) : pad32(i)] = v; };
     auto ld = [s](int i) { return s[Cfg::P16 ? pad16(i) : pad32(i)]; };
@@ -376,30 +438,18 @@ __global__ void __launch_bounds__(192) fs_adj_row_inv_kernel(KArgs a) {
   }
   __syncthreads();
   const Pointwise<T> pw(a);
-  const int p = nf - 1;
   C* out = reinterpret_cast<C*>(a.real);
   for (int idx = threadIdx.x; idx < Reff * L; idx += blockDim.x) {
     const int r = idx / L, i0 = idx % L;
+    C u[nf], mu[nf], res[nf];
 #pragma unroll
-    for (int h2 = 0; h2 < 2; ++h2) {
-      T eta[4], mu[5], res[5];
-      const C uc = slot(2 * nf, r)[i0];
-      const T c = h2 ? uc.y : uc.x;
-      for (int i = 0; i < p; ++i) {
-        const C e = slot(2 * nf + 1 + i, r)[i0];
-        eta[i] = h2 ? e.y : e.x;
-      }
-      for (int f = 0; f < nf; ++f) {
-        const C m2 = slot(nf + f, r)[i0];
-        mu[f] = h2 ? m2.y : m2.x;
-      }
-      hessian_apply(pw, c, eta, p, mu, res);
-      for (int f = 0; f < nf; ++f) {
-        C* sv = slot(f, r) + i0;
-        if (h2) sv->y += res[f]; else sv->x += res[f];
-      }
+    for (int f = 0; f < nf; ++f) {
+      u[f] = slot(2 * nf + f, r)[i0];
+      mu[f] = slot(nf + f, r)[i0];
     }
-    for (int f = 0; f < nf; ++f) out[f * half_stride + (row0 + r) * L + i0] = slot(f, r)[i0];
+    hessian_apply<P, T>(pw, u, mu, res);
+#pragma unroll
+    for (int f = 0; f < nf; ++f) out[f * half_stride + (row0 + r) * L + i0] = cadd(slot(f, r)[i0], res[f]);
   }
 }
 

@@ -72,14 +72,8 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 2)
     for (int m = 0; m < E; ++m) tl[(t + TPL * m) * tk] = v[m];
   }
   sync();
-  const Coef<T>& co = coef<T>(a);
-  AdjCoef<T> ac;
-  ac.Mdt = co.Mdt;
-  ac.Ldt = co.Ldt;
-  ac.kc = co.kc;
-  ac.ke = co.ke;
-  ac.dt = co.dt;
-  const T scale = co.scale;
+  const AdjCoef<T> ac(a);
+  const T scale = coef<T>(a).scale;
   const T* __restrict__ k2xt = reinterpret_cast<const T*>(a.k2x);
   const T* __restrict__ k2yt = reinterpret_cast<const T*>(a.k2y);
   // K2 of this line without the z part, as in the step's z kernel: in the
@@ -94,7 +88,7 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 2)
   const C* TL = tiles;              // Lam'
   const C* TU = tiles + TROWS * tk;  // U
   const C* TF = tiles + 2 * TROWS * tk;  // Fu
-  double g4[4] = {0.0, 0.0, 0.0, 0.0};
+  AdjSum<T> sr, sg;
   C va[E], vb[E];
   // Parseval over the stored modes: a line that is not a pair row stands for
   // itself and its conjugate partner (weight 2); a pair row's two real-packed
@@ -104,37 +98,22 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 2)
     const int kz = t + TPL * m;
     const T kz2 = k2zt[kz];
     const C l = TL[kz * tk + j], u = TU[kz * tk + j], f = TF[kz * tk + j];
-    T d1, d2, dd1[4], dd2[4];
     if (pair) {
       const int kq = (NZ - kz) & (NZ - 1);
       const C lq = cconj(TL[kq * tk + j]), uq = cconj(TU[kq * tk + j]), fq = cconj(TF[kq * tk + j]);
       const C lP = cscale(cadd(l, lq), T(0.5)), lQ = cscale(mul_i<-1>(csub(l, lq)), T(0.5));
       const C uP = cscale(cadd(u, uq), T(0.5)), uQ = cscale(mul_i<-1>(csub(u, uq)), T(0.5));
       const C fP = cscale(cadd(f, fq), T(0.5)), fQ = cscale(mul_i<-1>(csub(f, fq)), T(0.5));
-      ac.eval(fk, kxa + kya + kz2, d1, d2, dd1, dd2);
-      const C aP = cscale(lP, d1 * scale), bP = cscale(lP, d2 * scale);
-      for (int q = 0; q < 4; ++q)
-        g4[q] += (double)lP.x * (dd1[q] * uP.x + dd2[q] * fP.x) + (double)lP.y * (dd1[q] * uP.y + dd2[q] * fP.y);
-      ac.eval(fk, kxa + kyb + kz2, d1, d2, dd1, dd2);
-      const C aQ = cscale(lQ, d1 * scale), bQ = cscale(lQ, d2 * scale);
-      for (int q = 0; q < 4; ++q)
-        g4[q] += (double)lQ.x * (dd1[q] * uQ.x + dd2[q] * fQ.x) + (double)lQ.y * (dd1[q] * uQ.y + dd2[q] * fQ.y);
+      C aP, bP, aQ, bQ;
+      ac.mode(fk, kxa + kya + kz2, scale, lP, uP, fP, aP, bP, sr, sg);
+      ac.mode(fk, kxa + kyb + kz2, scale, lQ, uQ, fQ, aQ, bQ, sr, sg);
       va[m] = cadd(aP, mul_i<1>(aQ));
       vb[m] = cadd(bP, mul_i<1>(bQ));
     } else {
-      ac.eval(fk, kxy2 + kz2, d1, d2, dd1, dd2);
-      va[m] = cscale(l, d1 * scale);
-      vb[m] = cscale(l, d2 * scale);
-      for (int q = 0; q < 4; ++q)
-        g4[q] += 2.0 * ((double)l.x * (dd1[q] * u.x + dd2[q] * f.x) + (double)l.y * (dd1[q] * u.y + dd2[q] * f.y));
+      ac.mode(fk, kxy2 + kz2, scale, l, u, f, va[m], vb[m], sr, sg);
     }
   }
-  for (int q = 0; q < 4; ++q) {
-    double v = g4[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(&a.acc[q], v);
-  }
+  AdjCoef<T>::reduce(fk, sr, sg, pair ? 1.0 : 2.0, a.acc);
   sync();  // every thread has read the three tiles: they become exchange buffers
   C* base = reinterpret_cast<C*>(a.spec) + (long long)ky * Lh + kx;
   // inverse z of D1 lam'^ (exchange in tile 0) into slot phi and of D2 lam'^

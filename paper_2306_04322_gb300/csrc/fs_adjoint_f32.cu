@@ -2,6 +2,7 @@
 #include "fs_adjoint_impl.cuh"
 
 namespace fs {
+int adj_tile_width_f32(int nx, int ny) { return adj_tile_width_t<float>(nx, ny); }
 cudaError_t adjoint_launch_f32(const KArgs& a, const CUtensorMap& tm, void* lam_out, cudaStream_t s) {
   return adjoint_launch_t<float>(a, tm, lam_out, s);
 }

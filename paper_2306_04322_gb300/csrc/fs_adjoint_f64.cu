@@ -2,6 +2,7 @@
 #include "fs_adjoint_impl.cuh"
 
 namespace fs {
+int adj_tile_width_f64(int nx, int ny) { return adj_tile_width_t<double>(nx, ny); }
 cudaError_t adjoint_launch_f64(const KArgs& a, const CUtensorMap& tm, void* lam_out, cudaStream_t s) {
   return adjoint_launch_t<double>(a, tm, lam_out, s);
 }

@@ -13,40 +13,70 @@ size_t adj_row_smem(int nf) {
   return RC::BAR_BYTES + RC::TW_BYTES + (size_t)3 * nf * RC::R * RC::PL * sizeof(cplx<T>);
 }
 
-template <typename T, int NX>
-cudaError_t adj_row_n(const KArgs& a, bool inverse, cudaStream_t s) {
+template <typename T, int NX, int P>
+cudaError_t adj_row_p(const KArgs& a, bool inverse, cudaStream_t s) {
   using RC = RowCfg<T, NX>;
   const long long reff = a.lines < RC::R ? a.lines : RC::R;
   const size_t smem = adj_row_smem<T, NX>(a.nf);
-  const unsigned threads = 32 * (a.nf + 1);
   static unsigned d1 = 0, d2 = 0;
   cudaError_t e;
+  const dim3 grid((unsigned)(a.lines / reff));
   if (!inverse) {
-    e = allow_big_smem(fs_adj_row_fwd_kernel<T, NX>, &d1);
+    e = allow_big_smem(fs_adj_row_fwd_kernel<T, NX, P>, &d1);
     if (e != cudaSuccess) return e;
-    fs_adj_row_fwd_kernel<T, NX><<<(unsigned)(a.lines / reff), threads, smem, s>>>(a);
-  } else {
-    e = allow_big_smem(fs_adj_row_inv_kernel<T, NX>, &d2);
-    if (e != cudaSuccess) return e;
-    fs_adj_row_inv_kernel<T, NX><<<(unsigned)(a.lines / reff), threads, smem, s>>>(a);
+    return launch_pdl(fs_adj_row_fwd_kernel<T, NX, P>, grid, dim3(96 * (P + 1)), smem, s, a);
   }
-  return cudaGetLastError();
+  e = allow_big_smem(fs_adj_row_inv_kernel<T, NX, P>, &d2);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(fs_adj_row_inv_kernel<T, NX, P>, grid, dim3(64 * (P + 1)), smem, s, a);
+}
+
+template <typename T, int NX>
+cudaError_t adj_row_n(const KArgs& a, bool inverse, cudaStream_t s) {
+  switch (a.nf) {
+    case 1: return adj_row_p<T, NX, 0>(a, inverse, s);
+    case 2: return adj_row_p<T, NX, 1>(a, inverse, s);
+    case 3: return adj_row_p<T, NX, 2>(a, inverse, s);
+    case 4: return adj_row_p<T, NX, 3>(a, inverse, s);
+    case 5: return adj_row_p<T, NX, 4>(a, inverse, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <typename T, int NY, int TKC>
+cudaError_t adj_col_tk(const KArgs& a, const CUtensorMap& tm, int tk, cudaStream_t s) {
+  static unsigned d = 0;
+  cudaError_t e = allow_big_smem(fs_adj_col_kernel<T, NY, TKC>, &d);
+  if (e != cudaSuccess) return e;
+  const unsigned threads = ((unsigned)(tk * ColCfg<T, NY>::TPL) + 31) / 32 * 32;
+  return launch_pdl(fs_adj_col_kernel<T, NY, TKC>, dim3((unsigned)(a.nx / 2 / tk), (unsigned)a.nf), dim3(threads),
+                    AdjColCfg<T, NY>::smem(tk), s, a, tm);
+}
+
+template <typename T, int NY>
+int adj_tk(int nx) {
+  return AdjColCfg<T, NY>::TK < nx / 2 ? AdjColCfg<T, NY>::TK : nx / 2;
 }
 
 template <typename T, int NY>
 cudaError_t adj_col_n(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
-  using CC = ColCfg<T, NY>;
-  const int tk = col_tk_n<T, NY>(a.nx);
-  const size_t smem = CC::HEAD + (size_t)3 * CC::TROWS * tk * sizeof(cplx<T>);
-  static unsigned d = 0;
-  cudaError_t e = allow_big_smem(fs_adj_col_kernel<T, NY>, &d);
-  if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)(a.nx / 2 / tk), (unsigned)a.nf);
-  fs_adj_col_kernel<T, NY><<<grid, (unsigned)(tk * CC::TPL), smem, s>>>(a, tm);
-  return cudaGetLastError();
+  const int tk = adj_tk<T, NY>(a.nx);
+  if (tk == AdjColCfg<T, NY>::TK) return adj_col_tk<T, NY, AdjColCfg<T, NY>::TK>(a, tm, tk, s);
+  return adj_col_tk<T, NY, 0>(a, tm, tk, s);
 }
 
 #define FS_ADJ_SIZES(X) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024)
+
+template <typename T>
+int adj_tile_width_t(int nx, int ny) {
+  switch (ny) {
+#define FS_CASE(n) \
+  case n: return adj_tk<T, n>(nx);
+    FS_ADJ_SIZES(FS_CASE)
+#undef FS_CASE
+    default: return 0;
+  }
+}
 
 template <typename T>
 cudaError_t adjoint_launch_t(const KArgs& a0, const CUtensorMap& tm, void* lam_out, cudaStream_t s) {

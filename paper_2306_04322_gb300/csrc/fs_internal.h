@@ -167,6 +167,9 @@ cudaError_t adjoint3_launch_f32(const KArgs& a, const CUtensorMap& tm_y, const C
                                 cudaStream_t s);
 cudaError_t adjoint3_launch_f64(const KArgs& a, const CUtensorMap& tm_y, const CUtensorMap& tm_z, void* lam_out,
                                 cudaStream_t s);
+// Columns per CTA of the 2D adjoint's column pass (the box of its tensor map).
+int adj_tile_width_f32(int nx, int ny);
+int adj_tile_width_f64(int nx, int ny);
 // Columns per CTA of the 2D column pass for this grid (the TMA box width).
 int col_tile_width(bool f64, int nx, int ny);
 // 3D passes (fs_k3d_f32.cu / fs_k3d_f64.cu): y transform of `planes` z planes

@@ -1354,7 +1354,7 @@ fs_status fs_step_adjoint(fs_plan_t p, const void* const* u, const void* const* 
     // 2D: [slot][y][kx] column tiles; 3D: [slot nz + z][y][kx] tiles of the
     // y passes and [slot][z][y][kx] z lines
     const int tk = three ? (p->f64 ? fs::line_tile_width_f64(nx, ny) : fs::line_tile_width_f32(nx, ny))
-                         : fs::col_tile_width(p->f64, nx, ny);
+                         : (p->f64 ? fs::adj_tile_width_f64(nx, ny) : fs::adj_tile_width_f32(nx, ny));
     const cuuint64_t dims[3] = {W, (cuuint64_t)ny, (cuuint64_t)nz * 3 * nf};
     const cuuint64_t strides[2] = {W * 8, W * 8 * ny};
     const cuuint32_t box[3] = {(cuuint32_t)(tk * units), (cuuint32_t)(ny < 256 ? ny : 256), 1};
