@@ -63,7 +63,7 @@ class FSTrajectory(torch.autograd.Function):
             states = [ctx.checkpoints[s]]
             plan.set_fields(states[0])
             for _ in range(1, every):
-                plan.step(1)
+                plan.step_async(1)  # get_fields waits; the adjoint calls below return the status
                 states.append(plan.get_fields())
             for j in reversed(range(every)):
                 out = torch.empty_like(lam)

@@ -86,7 +86,7 @@ struct fs_plan {
   int* flag = nullptr;
   unsigned* gsync = nullptr; // grid-barrier counters of the fused step (pass form 4)
   double* acc = nullptr;     // diagnostic accumulators (device)
-  int* host_flag = nullptr;  // pinned
+  int* host_flag = nullptr;  // pinned, 64 bytes: the flag, from byte 8 the adjoint's four sums
   int state = kStateNone;
   cudaGraphExec_t gexec = nullptr;
   int gsteps = 0;
@@ -188,13 +188,18 @@ fs_status validate(const fs_params* p, std::string* why) {
   return FS_OK;
 }
 
+// Frequency of bin 1 of an axis (extended precision is slow in software on
+// some hosts: one division per axis, not one per bin).
+long double axis_step(int n, double dx) {
+  return 2.0L * 3.141592653589793238462643383279502884L / ((long double)n * (long double)dx);
+}
+
 // Squared frequency norm contribution of bin k on an axis of n points and
 // spacing dx: spectral (Eq. Gamma_fft), FS-FD O(dl^2) (Eq. Gamma_fft-fdO2),
-// FS-FD O(dl^4) (Eq. Gamma_fft-fdO4); index vector [0..n/2, -(n/2-1)..-1].
-double axis_k2(int lap, int k, int n, double dx) {
-  const long double pi = 3.141592653589793238462643383279502884L;
-  int nk = k <= n / 2 ? k : k - n;
-  double xi = (double)(2.0L * pi * (long double)nk / ((long double)n * (long double)dx));
+// FS-FD O(dl^4) (Eq. Gamma_fft-fdO4); index vector [0..n/2, -(n/2-1)..-1].  step: axis_step(n, dx).
+double axis_k2(int lap, int k, int n, double dx, long double step) {
+  const int nk = k <= n / 2 ? k : k - n;
+  const double xi = (double)(step * (long double)nk);
   if (lap == FS_LAP_FD2) return -2.0 * (std::cos(dx * xi) - 1.0) / (dx * dx);
   if (lap == FS_LAP_FD4) return -(16.0 * std::cos(dx * xi) - std::cos(2.0 * dx * xi) - 15.0) / (6.0 * dx * dx);
   return xi * xi;
@@ -725,12 +730,45 @@ TableLayout table_layout(const fs_params& prm, bool f64) {
 
 size_t member_table_bytes(const fs_params& prm, bool f64) { return table_layout(prm, f64).total; }
 
+// Roots exp(-2 pi i k / n), 0 <= k < n, n a power of two up to 2048: every
+// table of a plan looks its entries up here.  Only the octant 0 <= k <= n / 8
+// is computed, in double at the rounded angle and corrected to first order
+// for the rounding (the angle as an unevaluated sum of two doubles); the rest
+// follows by symmetry.  (A cosl and a sinl for every entry of every table took
+// two thirds of fs_plan_create where long double is software.)
+struct Roots {
+  int n;
+  std::vector<double> re, im;
+  explicit Roots(int n_) : n(n_ < 8 ? 8 : n_), re(n), im(n) {
+    const long double two_pi = 2.0L * 3.141592653589793238462643383279502884L;
+    const double hi = (double)two_pi, lo = (double)(two_pi - (long double)hi);
+    std::vector<double> c(n / 8 + 1), s(n / 8 + 1);
+    for (int k = 0; k <= n / 8; ++k) {
+      const double f = (double)k / n;  // exact
+      const double a = hi * f, e = std::fma(hi, f, -a) + lo * f;
+      c[k] = std::fma(-e, std::sin(a), std::cos(a));
+      s[k] = std::fma(e, std::cos(a), std::sin(a));
+    }
+    for (int k = 0; k < n; ++k) {
+      const int q = k / (n / 4), r = k % (n / 4);  // quadrant, angle within it
+      const double cr = r <= n / 8 ? c[r] : s[n / 4 - r], sr = r <= n / 8 ? s[r] : c[n / 4 - r];
+      re[k] = q == 0 ? cr : q == 1 ? -sr : q == 2 ? -cr : sr;
+      im[k] = -(q == 0 ? sr : q == 1 ? cr : q == 2 ? -sr : -cr);
+    }
+  }
+  // exp(-2 pi i num / den), den a power of two dividing n
+  void add(long long num, long long den, std::vector<double>& r, std::vector<double>& i) const {
+    const int k = (int)((num % den) * (n / den));
+    r.push_back(re[k]);
+    i.push_back(im[k]);
+  }
+};
+
 // Stockham pass tables of a line FFT of length L with E values per thread:
 // for every pass after the first (sub-length NS, radix R = min(E, L/NS)),
 // entries [q][j], q < R / 2, j < NS: the roots of the pass's radix-2 stages
 // (fs::stage_root).
-void pass_table(int L, int E, std::vector<long double>& re, std::vector<long double>& im) {
-  const long double pi = 3.141592653589793238462643383279502884L;
+void pass_table(const Roots& w, int L, int E, std::vector<double>& re, std::vector<double>& im) {
   for (int ns = 1; ns < L;) {
     int r = E < L / ns ? E : L / ns;
     if (ns > 1)
@@ -738,9 +776,7 @@ void pass_table(int L, int E, std::vector<long double>& re, std::vector<long dou
         for (int j = 0; j < ns; ++j) {
           long long num, den;
           fs::stage_root(q, j, ns, &num, &den);
-          long double ang = 2.0L * pi * (long double)(num % den) / (long double)den;
-          re.push_back(cosl(ang));
-          im.push_back(-sinl(ang));
+          w.add(num, den, re, im);
         }
     ns *= r;
   }
@@ -752,8 +788,7 @@ void put_real(std::vector<char>& buf, size_t off, const std::vector<double>& v) 
   for (size_t i = 0; i < v.size(); ++i) d[i] = (T)v[i];
 }
 template <typename T>
-void put_cplx(std::vector<char>& buf, size_t off, const std::vector<long double>& re,
-              const std::vector<long double>& im) {
+void put_cplx(std::vector<char>& buf, size_t off, const std::vector<double>& re, const std::vector<double>& im) {
   T* d = reinterpret_cast<T*>(buf.data() + off);
   for (size_t i = 0; i < re.size(); ++i) {
     d[2 * i] = (T)re[i];
@@ -767,26 +802,26 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   std::vector<char> buf(bytes, 0);
   int nx = prm.n[0], ny = prm.n[1], nz = prm.ndim > 2 ? prm.n[2] : 1;
   std::vector<double> kx(nx / 2 + 1), ky(ny), kz(nz, 0.0);
-  for (int k = 0; k <= nx / 2; ++k) kx[k] = axis_k2(prm.lap, k, nx, prm.dx[0]);
-  for (int k = 0; k < ny; ++k) ky[k] = axis_k2(prm.lap, k, ny, prm.dx[1]);
-  for (int k = 0; k < nz && prm.ndim > 2; ++k) kz[k] = axis_k2(prm.lap, k, nz, prm.dx[2]);
-  std::vector<long double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i, m3r, m3i;
+  auto fill = [&prm](std::vector<double>& k2, int count, int d) {
+    const long double step = axis_step(prm.n[d], prm.dx[d]);
+    for (int k = 0; k < count; ++k) k2[k] = axis_k2(prm.lap, k, prm.n[d], prm.dx[d], step);
+  };
+  fill(kx, nx / 2 + 1, 0);
+  fill(ky, ny, 1);
+  if (prm.ndim > 2) fill(kz, nz, 2);
+  const Roots w(std::max(nx, std::max(ny, nz)));
+  std::vector<double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i, m3r, m3i;
   const int er = row2_e(prm, f64), ec = col2_e(prm, f64);
-  if (er) pass_table(nx, er, r2r, r2i);
-  if (ec) pass_table(ny, ec, c2r, c2i);
-  if (row2w_form(prm, f64)) pass_table(nx, nx / 64, r3r, r3i);
-  if (col2w_form(prm, f64)) pass_table(ny, ny / 64, c3r, c3i);
-  if (row3_form(prm, f64)) pass_table(nx, 16, m3r, m3i);
-  pass_table(t.Lrow, t.Erow, rr, ii);
-  if (wide_rows(prm, f64)) pass_table(t.Lrow, 32, wr, wi);
-  pass_table(t.Lcol, t.Ecol, cr, ci);
-  if (nz > 1) pass_table(t.Lz, t.Ez, zr, zi);
-  const long double pi = 3.141592653589793238462643383279502884L;
-  for (int k = 0; k < nx / 2; ++k) {
-    long double ang = 2.0L * pi * (long double)k / (long double)nx;
-    hr.push_back(cosl(ang));
-    hi.push_back(-sinl(ang));
-  }
+  if (er) pass_table(w, nx, er, r2r, r2i);
+  if (ec) pass_table(w, ny, ec, c2r, c2i);
+  if (row2w_form(prm, f64)) pass_table(w, nx, nx / 64, r3r, r3i);
+  if (col2w_form(prm, f64)) pass_table(w, ny, ny / 64, c3r, c3i);
+  if (row3_form(prm, f64)) pass_table(w, nx, 16, m3r, m3i);
+  pass_table(w, t.Lrow, t.Erow, rr, ii);
+  if (wide_rows(prm, f64)) pass_table(w, t.Lrow, 32, wr, wi);
+  pass_table(w, t.Lcol, t.Ecol, cr, ci);
+  if (nz > 1) pass_table(w, t.Lz, t.Ez, zr, zi);
+  for (int k = 0; k < nx / 2; ++k) w.add(k, nx, hr, hi);
   if (f64) {
     put_real<double>(buf, t.k2x, kx);
     put_real<double>(buf, t.k2y, ky);
@@ -1079,7 +1114,7 @@ fs_status create_common(const fs_params* each, int count, void* stream, fs_alloc
     delete p;
     return fail(nullptr, FS_ERR_OOM, "device workspace allocation failed");
   }
-  cudaError_t e = cudaMallocHost(&p->host_flag, sizeof(int));
+  cudaError_t e = cudaMallocHost(&p->host_flag, 64);
   if (e != cudaSuccess) {
     plan_free_all(p);
     delete p;
@@ -1368,13 +1403,10 @@ fs_status fs_step_adjoint(fs_plan_t p, const void* const* u, const void* const* 
     }
     if (!ok) return fail(p, FS_ERR_CUDA, "adjoint tensor map");
   }
-  cudaError_t e = cudaSuccess;
-  for (int f = 0; f < nf && e == cudaSuccess; ++f) {
+  for (int f = 0; f < nf; ++f)
     if (!u[f] || !lam_in[f] || !lam_out[f]) return fail(p, FS_ERR_INVALID_ARG, "field pointer is NULL");
-    e = cudaMemcpyAsync((char*)m.au + f * m.npts * rs, u[f], m.npts * rs, cudaMemcpyDefault, p->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync((char*)m.alam + f * m.npts * rs, lam_in[f], m.npts * rs, cudaMemcpyDefault, p->stream);
-  }
+  cudaError_t e = copy_fields((char*)m.au, u, nf, m.npts * rs, true, p->stream);
+  if (e == cudaSuccess) e = copy_fields((char*)m.alam, lam_in, nf, m.npts * rs, true, p->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->acc, 0, sizeof(double) * 4, p->stream);
   fs::KArgs a = make_args(p, m, 0);
   a.spec = m.aspec;
@@ -1389,19 +1421,20 @@ fs_status fs_step_adjoint(fs_plan_t p, const void* const* u, const void* const* 
   else if (e == cudaSuccess)
     e = p->f64 ? fs::adjoint_launch_f64(a, m.tmap_adj, m.aout, p->stream)
                : fs::adjoint_launch_f32(a, m.tmap_adj, m.aout, p->stream);
-  for (int f = 0; f < nf && e == cudaSuccess; ++f)
-    e = cudaMemcpyAsync(lam_out[f], (char*)m.aout + f * m.npts * rs, m.npts * rs, cudaMemcpyDefault, p->stream);
+  if (e == cudaSuccess) e = copy_fields((char*)m.aout, lam_out, nf, m.npts * rs, false, p->stream);
   if (e != cudaSuccess) return cuda_fail(p, e, "fs_step_adjoint");
   p->last_launches = three ? 5 : 3;
   if (grad) {
-    double h[4];
-    e = cudaMemcpyAsync(h, p->acc, sizeof(h), cudaMemcpyDeviceToHost, p->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
+    // the sums and the flag in one wait (read_flag's)
+    const double* h = reinterpret_cast<const double*>(p->host_flag) + 1;
+    e = cudaMemcpyAsync(const_cast<double*>(h), p->acc, 4 * sizeof(double), cudaMemcpyDeviceToHost, p->stream);
     if (e != cudaSuccess) return cuda_fail(p, e, "fs_step_adjoint sensitivities");
+    const fs_status st = read_flag(p);
+    if (st != FS_OK && st != FS_ERR_NONFINITE && st != FS_ERR_TIMEOUT) return st;
     // Parseval 1/N, and both spectra carry the factor 2 of the packed x transform
     const double norm = 1.0 / (4.0 * (double)m.npts);
     for (int q = 0; q < 4; ++q) grad[q] += h[q] * norm;
-    return read_flag(p);
+    return st;
   }
   return FS_OK;
 }
@@ -1595,8 +1628,9 @@ cudaError_t slab_adopt_columns(fs_plan* p, int kx_base, const fs_params& g) {
   m.nx_full = nx;
   m.npts_full = (long long)g.n[0] * g.n[1];
   std::vector<double> k2(cols + 1);
-  for (int j = 0; j < cols; ++j) k2[j] = axis_k2(g.lap, kx_base + j, nx, g.dx[0]);
-  k2[cols] = axis_k2(g.lap, nx / 2, nx, g.dx[0]);
+  const long double step = axis_step(nx, g.dx[0]);
+  for (int j = 0; j < cols; ++j) k2[j] = axis_k2(g.lap, kx_base + j, nx, g.dx[0], step);
+  k2[cols] = axis_k2(g.lap, nx / 2, nx, g.dx[0], step);
   if (p->f64) return cudaMemcpy(m.k2x, k2.data(), sizeof(double) * k2.size(), cudaMemcpyHostToDevice);
   std::vector<float> f(k2.begin(), k2.end());
   return cudaMemcpy(m.k2x, f.data(), sizeof(float) * f.size(), cudaMemcpyHostToDevice);
