@@ -1,7 +1,6 @@
 // Batched ensemble: many independent 2D simulations of uneven grid sizes and
-// parameters advanced by one launch per pass.  The launch is persistent: a
-// grid of G CTAs (G picked by the plan's autotuner) walks a flat work list
-// of (simulation, row block) or (simulation, column tile, field group) items;
+// parameters advanced by one launch per pass, one CTA per item of a flat work
+// list of (simulation, row block) or (simulation, column tile, field group);
 // each item dispatches to the row / column body instantiated for that
 // simulation's size.  Items of one simulation are contiguous; simulations
 // are ordered largest first.
@@ -25,8 +24,7 @@ __device__ __forceinline__ int find_member(const long long* __restrict__ begin, 
 
 template <typename T>
 __global__ void __launch_bounds__(128, RowCfg<T, 1024>::MIN_BLOCKS)
-    fs_row_batch_kernel(const KArgs* __restrict__ mem, const long long* __restrict__ begin, int nm,
-                        long long total) {
+    fs_row_batch_kernel(const KArgs* __restrict__ mem, const long long* __restrict__ begin, int nm) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   if (threadIdx.x == 0) {
@@ -34,30 +32,23 @@ __global__ void __launch_bounds__(128, RowCfg<T, 1024>::MIN_BLOCKS)
     fence_mbar_init();
   }
   __syncthreads();
-  uint32_t parity = 0;
-  for (long long item = blockIdx.x; item < total; item += gridDim.x) {
-    const int m = find_member(begin, nm, item);
-    const KArgs& a = mem[m];
-    const long long rb = item - begin[m];
-    bool ok = false;
-    switch (a.nx) {
+  const long long item = blockIdx.x;
+  const int m = find_member(begin, nm, item);
+  const KArgs& a = mem[m];
+  const long long rb = item - begin[m];
+  switch (a.nx) {
 #define FS_CASE(n) \
-  case n: ok = row_body<T, n>(a, rb, smem_raw, bar, parity); break;
-      FS_BATCH_SIZES(FS_CASE)
+  case n: row_body<T, n>(a, rb, smem_raw, bar, 0); break;
+    FS_BATCH_SIZES(FS_CASE)
 #undef FS_CASE
-      default: break;
-    }
-    if (!ok) return;
-    parity ^= 1u;
-    __syncthreads();
+    default: break;
   }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256, 2)
     fs_col_batch_kernel(const KArgs* __restrict__ mem, const CUtensorMap* __restrict__ maps,
-                        const long long* __restrict__ begin, const int* __restrict__ tiles, int nm,
-                        long long total) {
+                        const long long* __restrict__ begin, const int* __restrict__ tiles, int nm) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   if (threadIdx.x == 0) {
@@ -65,24 +56,18 @@ __global__ void __launch_bounds__(256, 2)
     fence_mbar_init();
   }
   __syncthreads();
-  uint32_t parity = 0;
-  for (long long item = blockIdx.x; item < total; item += gridDim.x) {
-    const int m = find_member(begin, nm, item);
-    const KArgs& a = mem[m];
-    const int nt = tiles[m];
-    const int rem = (int)(item - begin[m]);
-    const int g = rem / nt, bx = rem % nt;
-    bool ok = false;
-    switch (a.ny) {
+  const long long item = blockIdx.x;
+  const int m = find_member(begin, nm, item);
+  const KArgs& a = mem[m];
+  const int nt = tiles[m];
+  const int rem = (int)(item - begin[m]);
+  const int g = rem / nt, bx = rem % nt;
+  switch (a.ny) {
 #define FS_CASE(n) \
-  case n: ok = col_body<T, n>(a, &maps[m], bx, g, smem_raw, bar, parity); break;
-      FS_BATCH_SIZES(FS_CASE)
+  case n: col_body<T, n>(a, &maps[m], bx, g, smem_raw, bar, 0); break;
+    FS_BATCH_SIZES(FS_CASE)
 #undef FS_CASE
-      default: break;
-    }
-    if (!ok) return;
-    parity ^= 1u;
-    __syncthreads();
+    default: break;
   }
 }
 
@@ -138,9 +123,8 @@ cudaError_t row_batch_launch_t(const BatchArgs& b, cudaStream_t s) {
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_row_batch_kernel<T>, &done);
   if (e != cudaSuccess) return e;
-  fs_row_batch_kernel<T><<<(unsigned)b.row_grid, 128, b.row_smem, s>>>(
-      b.mem, b.row_begin, b.nm, b.row_total);
-  return cudaGetLastError();
+  return launch_pdl(fs_row_batch_kernel<T>, dim3((unsigned)b.row_total), dim3(128), b.row_smem, s, b.mem, b.row_begin,
+                    b.nm);
 }
 
 template <typename T>
@@ -148,9 +132,8 @@ cudaError_t col_batch_launch_t(const BatchArgs& b, cudaStream_t s) {
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_col_batch_kernel<T>, &done);
   if (e != cudaSuccess) return e;
-  fs_col_batch_kernel<T><<<(unsigned)b.col_grid, 256, b.col_smem, s>>>(b.mem_col, b.maps, b.col_begin,
-                                                                         b.col_tiles, b.nm, b.col_total);
-  return cudaGetLastError();
+  return launch_pdl(fs_col_batch_kernel<T>, dim3((unsigned)b.col_total), dim3(256), b.col_smem, s, b.mem_col, b.maps,
+                    b.col_begin, b.col_tiles, b.nm);
 }
 
 }  // namespace fs

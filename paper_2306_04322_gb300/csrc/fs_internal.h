@@ -196,7 +196,6 @@ struct BatchArgs {
   int nm;                       // simulations
   int nf1;                      // nf + 1 (warps of a row CTA)
   long long row_total, col_total;
-  long long row_grid, col_grid; // persistent grid sizes
   size_t row_smem, col_smem;
   // warp-per-line forms (FP32 members with both axes in [64, 1024]; NULL / 0:
   // not available): row-pair and (column pair, field group) work lists,
@@ -206,7 +205,6 @@ struct BatchArgs {
   const long long* col2_begin;
   const int* col2_pairs;        // column pairs of each simulation
   long long row2_total, col2_total;
-  long long row2_grid, col2_grid;
   size_t row2_smem, row2_smem1, col2_smem;  // row2_smem1: row pass in mode 1
   int row2_mode;                // mode of the row pass launched
   int row_form, col_form;       // chosen per pass: 1 half-length / tile kernels, 2 warp-per-line kernels
@@ -235,6 +233,8 @@ cudaError_t fd_launch(bool f64, const KArgs& a, const void* in, void* out, void*
 int fd_launches_per_step(const KArgs& a);
 // FP64 sum of n values of x (float or double) added into *out.
 cudaError_t sum_launch_f32(const void* x, long long n, double* out, cudaStream_t s);
+// The same for c of every member of an FP32 ensemble, into its csum.
+cudaError_t sum_batch_launch_f32(const KArgs* mem, int nm, cudaStream_t s);
 cudaError_t sum_launch_f64(const void* x, long long n, double* out, cudaStream_t s);
 
 }  // namespace fs

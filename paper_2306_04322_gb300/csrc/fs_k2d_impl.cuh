@@ -180,18 +180,19 @@ int col_tk_t(int nx, int ny) {
   }
 }
 
-// FP64 sum reduction (grid-stride, warp shuffles, one atomic per CTA).
-// VEC: 16-byte vector loads (x 16-byte aligned, n a multiple of 16 / sizeof(T)).
+// FP64 sum of n values of x added into *out by nblk CTAs, this one blk
+// (strided, warp shuffles, one atomic per CTA).  VEC: 16-byte vector loads
+// (x 16-byte aligned, n a multiple of 16 / sizeof(T)).
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(256) fs_sum_kernel(const T* __restrict__ x, long long n, double* out) {
+__device__ __forceinline__ void sum_body(const T* __restrict__ x, long long n, double* out, long long blk,
+                                         long long nblk) {
   double s = 0.0;
   if constexpr (VEC) {
     using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
     constexpr int W = 16 / sizeof(T);
     const V* __restrict__ xv = reinterpret_cast<const V*>(x);
     const long long nv = n / W;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nv;
-         i += (long long)gridDim.x * blockDim.x) {
+    for (long long i = blk * blockDim.x + threadIdx.x; i < nv; i += nblk * blockDim.x) {
       const V v = __ldg(&xv[i]);
       if constexpr (W == 4)
         s += ((double)v.x + (double)v.y) + ((double)v.z + (double)v.w);
@@ -199,8 +200,7 @@ __global__ void __launch_bounds__(256) fs_sum_kernel(const T* __restrict__ x, lo
         s += (double)v.x + (double)v.y;
     }
   } else {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-      s += (double)x[i];
+    for (long long i = blk * blockDim.x + threadIdx.x; i < n; i += nblk * blockDim.x) s += (double)x[i];
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
@@ -212,6 +212,20 @@ __global__ void __launch_bounds__(256) fs_sum_kernel(const T* __restrict__ x, lo
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += ws[w];
     atomicAdd(out, t);
   }
+}
+
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) fs_sum_kernel(const T* __restrict__ x, long long n, double* out) {
+  sum_body<T, VEC>(x, n, out, blockIdx.x, gridDim.x);
+}
+
+// Field c of every member of an ensemble into its csum, kSumBlocks CTAs each.
+constexpr int kSumBlocks = 32;
+template <typename T>
+__global__ void __launch_bounds__(256) fs_sum_batch_kernel(const KArgs* __restrict__ mem) {
+  const KArgs& a = mem[blockIdx.x / kSumBlocks];
+  sum_body<T, true>(reinterpret_cast<const T*>(a.real), a.npts, const_cast<double*>(a.csum), blockIdx.x % kSumBlocks,
+                    kSumBlocks);
 }
 
 template <typename T>

@@ -74,6 +74,7 @@ struct fs_plan {
   bool batch = false;  // ensemble: one launch per pass for all members
   fs::BatchArgs bargs{};
   const fs::KArgs* bmem1 = nullptr;  // row arguments in mode 1 (from real fields)
+  const fs::KArgs* bmem2 = nullptr;  // row arguments in mode 2 (inverse only)
   bool tuned = false;
   int nf = 1;
   cudaStream_t stream = nullptr;
@@ -442,10 +443,11 @@ void* fd_scratch(const fs_plan* p, const Member& m) {
 }
 
 // Batched ensemble: kind 0 row pass (mode 0 from spectra, 1 from real
-// fields), kind 1 column pass, each one persistent launch for all members.
+// fields, 2 inverse only), kind 1 column pass, each one launch for all members.
 cudaError_t launch_batch_pass(const fs_plan* p, int mode, int kind, cudaStream_t s) {
   fs::BatchArgs b = p->bargs;
   if (mode == 1) b.mem = p->bmem1;
+  if (mode == 2) b.mem = p->bmem2;
   b.row2_mode = mode;
   if (kind == 0) {
     if (b.row_form == 2) return fs::row2_batch_launch_f32(b, s);
@@ -889,7 +891,7 @@ fs_status setup_batch(fs_plan* p) {
   for (int i = 0; i < nm; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(),
                    [p](int a, int b) { return p->members[a].npts > p->members[b].npts; });
-  std::vector<fs::KArgs> k0(nm), k1(nm);
+  std::vector<fs::KArgs> k0(nm), k1(nm), k2(nm);
   std::vector<CUtensorMap> maps(nm);
   std::vector<long long> rb(nm + 1, 0), cb(nm + 1, 0);
   std::vector<int> tiles(nm);
@@ -907,6 +909,7 @@ fs_status setup_batch(fs_plan* p) {
     const int nx = m.prm.n[0], ny = m.prm.n[1];
     k0[e] = make_args(p, m, 0);
     k1[e] = make_args(p, m, 1);
+    k2[e] = make_args(p, m, 2);
     maps[e] = m.tmap_col;
     const long long blocks = p->f64 ? fs::row_blocks_f64(nx, ny) : fs::row_blocks_f32(nx, ny);
     const int tk = p->f64 ? fs::col_batch_tk_f64(nx, ny) : fs::col_batch_tk_f32(nx, ny);
@@ -926,7 +929,8 @@ fs_status setup_batch(fs_plan* p) {
     }
   }
   const size_t o_maps = 0, o_k0 = align16(o_maps + sizeof(CUtensorMap) * nm);
-  const size_t o_k1 = align16(o_k0 + sizeof(fs::KArgs) * nm), o_rb = align16(o_k1 + sizeof(fs::KArgs) * nm);
+  const size_t o_k1 = align16(o_k0 + sizeof(fs::KArgs) * nm), o_k2 = align16(o_k1 + sizeof(fs::KArgs) * nm);
+  const size_t o_rb = align16(o_k2 + sizeof(fs::KArgs) * nm);
   const size_t o_cb = align16(o_rb + sizeof(long long) * (nm + 1));
   // tensor maps read by TMA from global memory must be 64-byte aligned: both
   // map arrays start on 128 bytes (the block itself is 256-byte aligned)
@@ -941,6 +945,7 @@ fs_status setup_batch(fs_plan* p) {
   std::memcpy(host.data() + o_maps, maps.data(), sizeof(CUtensorMap) * nm);
   std::memcpy(host.data() + o_k0, k0.data(), sizeof(fs::KArgs) * nm);
   std::memcpy(host.data() + o_k1, k1.data(), sizeof(fs::KArgs) * nm);
+  std::memcpy(host.data() + o_k2, k2.data(), sizeof(fs::KArgs) * nm);
   std::memcpy(host.data() + o_rb, rb.data(), sizeof(long long) * (nm + 1));
   std::memcpy(host.data() + o_cb, cb.data(), sizeof(long long) * (nm + 1));
   std::memcpy(host.data() + o_t, tiles.data(), sizeof(int) * nm);
@@ -955,6 +960,7 @@ fs_status setup_batch(fs_plan* p) {
   b.mem = reinterpret_cast<const fs::KArgs*>(dev + o_k0);
   b.mem_col = b.mem;
   p->bmem1 = reinterpret_cast<const fs::KArgs*>(dev + o_k1);
+  p->bmem2 = reinterpret_cast<const fs::KArgs*>(dev + o_k2);
   b.row_begin = reinterpret_cast<const long long*>(dev + o_rb);
   b.col_begin = reinterpret_cast<const long long*>(dev + o_cb);
   b.col_tiles = reinterpret_cast<const int*>(dev + o_t);
@@ -962,8 +968,6 @@ fs_status setup_batch(fs_plan* p) {
   b.nf1 = p->nf + 1;
   b.row_total = rb[nm];
   b.col_total = cb[nm];
-  b.row_grid = b.row_total;  // until tuned: one CTA per item
-  b.col_grid = b.col_total;
   b.row_smem = rsm;
   b.col_smem = csm;
   b.row_form = b.col_form = 1;  // until tuned
@@ -974,8 +978,6 @@ fs_status setup_batch(fs_plan* p) {
     b.col2_pairs = reinterpret_cast<const int*>(dev + o_p2);
     b.row2_total = rb2[nm];
     b.col2_total = cb2[nm];
-    b.row2_grid = b.row2_total;
-    b.col2_grid = b.col2_total;
     b.row2_smem = rsm2;
     b.row2_smem1 = rsm21;
     b.col2_smem = csm2;
@@ -983,75 +985,60 @@ fs_status setup_batch(fs_plan* p) {
   return FS_OK;
 }
 
-// Autotuner of the batched launches.  For each pass it times every form the
+// Autotuner of the batched launches.  For each pass it times the forms the
 // ensemble supports -- the half-length row / column-tile kernels (radix-16
 // line transforms, column tiles of col_tk columns) and, for FP32 members with
 // both axes in [64, 1024], the warp-per-line kernels (radix-32 / 16 / 8 ...
-// line transforms held by one warp, two-column tiles) -- at the persistent
-// grid sizes {1, 2, 3, 4, 5, 6, 8, 16} x SMs and one CTA per work item, and
-// keeps the fastest (form, grid) pair.  Runs on the state just set (row pass
-// from the real fields, column pass on its output), which it leaves
-// unchanged.
+// line transforms held by one warp, two-column tiles) -- and keeps the faster,
+// each in the steady step's own launches (row pass in mode 0), one CTA per
+// work item.  (Persistent grids of 1 to 16 CTAs per SM had been candidates,
+// timed one launch at a time: where they won that comparison the steps, whose
+// launches overlap, were slower -- 16 members of 128^2 to 1024^2, FP32, 157 us
+// per step against 122.)  Runs on the state just set, which it leaves
+// unchanged: every repetition starts again from the real fields, and bits its
+// second step sets in the status flag are dropped.
 cudaError_t autotune_batch(fs_plan* p) {
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int mult[] = {1, 2, 3, 4, 5, 6, 8, 16};
+  fs::BatchArgs& b = p->bargs;
+  const bool v2 = b.maps2 != nullptr;
+  if (!v2) {  // one form
+    b.row_form = b.col_form = 1;
+    p->tuned = true;
+    return cudaSuccess;
+  }
   cudaEvent_t e0, e1;
   cudaError_t e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   if (e != cudaSuccess) return e;
-  fs::BatchArgs& b = p->bargs;
-  const bool v2 = b.maps2 != nullptr;
-  // the column pass is timed on the output of a row pass in the current row form
-  b.row_form = 1;
+  e = cudaMemcpyAsync(p->flag + 1, p->flag, sizeof(int), cudaMemcpyDeviceToDevice, p->stream);
+  b.row_form = b.col_form = 2;
   for (int kind = 0; kind < 2 && e == cudaSuccess; ++kind) {
-    float best = 1e30f;
-    int best_form = 1;
-    long long best_g = 0;
+    int& slot = kind == 0 ? b.row_form : b.col_form;
     const int pinned = kind == 0 ? p->row_form : p->col_form;  // fs_set_pass_forms, 0: free
-    for (int form = 1; form <= (v2 ? 2 : 1) && e == cudaSuccess; ++form) {
-      if (pinned && form != pinned) continue;
-      const long long total = kind == 0 ? (form == 2 ? b.row2_total : b.row_total)
-                                        : (form == 2 ? b.col2_total : b.col_total);
-      std::vector<long long> cand;
-      for (int mm : mult)
-        if ((long long)mm * sms < total) cand.push_back((long long)mm * sms);
-      cand.push_back(total);
-      for (long long g : cand) {
-        if (kind == 0) {
-          b.row_form = form;
-          (form == 2 ? b.row2_grid : b.row_grid) = g;
-        } else {
-          b.col_form = form;
-          (form == 2 ? b.col2_grid : b.col_grid) = g;
-        }
-        float acc = 0.f;
-        for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
-          if (kind == 1) e = launch_batch_pass(p, 1, 0, p->stream);  // fresh column input
-          if (e == cudaSuccess) e = cudaEventRecord(e0, p->stream);
-          if (e == cudaSuccess) e = launch_batch_pass(p, 1, kind, p->stream);
-          if (e == cudaSuccess) e = cudaEventRecord(e1, p->stream);
-          if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-          float t = 0.f;
-          if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-          if (rep > 0) acc += t;  // first repetition warms up
-        }
-        if (acc < best) {
-          best = acc;
-          best_form = form;
-          best_g = g;
-        }
+    float best = 1e30f;
+    int best_form = pinned ? pinned : slot;
+    for (int form = 1; form <= 2 && e == cudaSuccess && !pinned; ++form) {
+      slot = form;
+      float acc = 0.f;
+      for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
+        e = launch_batch_pass(p, 1, 0, p->stream);
+        if (e == cudaSuccess) e = launch_batch_pass(p, 1, 1, p->stream);
+        if (kind == 1 && e == cudaSuccess) e = launch_batch_pass(p, 0, 0, p->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(e0, p->stream);
+        if (e == cudaSuccess) e = launch_batch_pass(p, 0, kind, p->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, p->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float t = 0.f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+        if (rep > 0) acc += t;  // first repetition warms up
+      }
+      if (acc < best) {
+        best = acc;
+        best_form = form;
       }
     }
-    if (kind == 0) {
-      b.row_form = best_form;
-      (best_form == 2 ? b.row2_grid : b.row_grid) = best_g;
-    } else {
-      b.col_form = best_form;
-      (best_form == 2 ? b.col2_grid : b.col_grid) = best_g;
-    }
+    slot = best_form;
   }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(p->flag, p->flag + 1, sizeof(int), cudaMemcpyDeviceToDevice, p->stream);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (e == cudaSuccess) p->tuned = true;
@@ -1088,6 +1075,7 @@ fs_status create_common(const fs_params* each, int count, void* stream, fs_alloc
   // Workspace first (through the allocator hook), then tables.
   p->members.resize(count);
   std::vector<size_t> table_bytes(count);
+  double* csums = (double*)plan_alloc(p, sizeof(double) * 8 * count);  // one 64-byte line per member
   for (int i = 0; i < count; ++i) {
     Member& m = p->members[i];
     m.prm = each[i];
@@ -1098,8 +1086,8 @@ fs_status create_common(const fs_params* each, int count, void* stream, fs_alloc
     m.real = plan_alloc(p, (size_t)p->nf * m.npts * rs);
     table_bytes[i] = member_table_bytes(m.prm, p->f64);
     char* tb = (char*)plan_alloc(p, table_bytes[i]);
-    m.csum = (double*)plan_alloc(p, sizeof(double) * 8);
-    if (!m.spec || !m.real || !tb || !m.csum) {
+    m.csum = csums + 8 * i;
+    if (!m.spec || !m.real || !tb || !csums) {
       plan_free_all(p);
       delete p;
       return fail(nullptr, FS_ERR_OOM, "device workspace allocation failed");
@@ -1122,9 +1110,9 @@ fs_status create_common(const fs_params* each, int count, void* stream, fs_alloc
   }
   for (int i = 0; i < count && e == cudaSuccess; ++i) {
     e = upload_tables(p->members[i], p->f64, (char*)p->members[i].k2x, table_bytes[i]);
-    if (e == cudaSuccess) e = cudaMemset(p->members[i].csum, 0, sizeof(double) * 8);
     if (e == cudaSuccess && !encode_col_map(p->members[i], p->nf + 1, p->f64)) e = cudaErrorInvalidValue;
   }
+  if (e == cudaSuccess) e = cudaMemset(csums, 0, sizeof(double) * 8 * count);
   if (e == cudaSuccess) e = cudaMemset(p->flag, 0, 256);
   if (e == cudaSuccess) e = cudaMemset(p->gsync, 0, fs::kStep2SyncBytes);
   if (e != cudaSuccess) {
@@ -1192,11 +1180,16 @@ fs_status fs_set_fields(fs_plan_t p, const void* const* fields) {
     if (ec != cudaSuccess) return cuda_fail(p, ec, "fs_set_fields copy");
     idx += p->nf;
     m.fd_cur = 0;
-    if (!p->f64 && !p->fd) {
+    if (!p->f64 && !p->fd && !p->batch) {
       cudaError_t e = cudaMemsetAsync(m.csum, 0, sizeof(double), p->stream);
       if (e == cudaSuccess) e = fs::sum_launch_f32(m.real, m.npts, m.csum, p->stream);
       if (e != cudaSuccess) return cuda_fail(p, e, "fs_set_fields mean carry");
     }
+  }
+  if (p->batch && !p->f64) {
+    cudaError_t e = cudaMemsetAsync(p->members[0].csum, 0, sizeof(double) * 8 * p->members.size(), p->stream);
+    if (e == cudaSuccess) e = fs::sum_batch_launch_f32(p->bargs.mem, p->bargs.nm, p->stream);
+    if (e != cudaSuccess) return cuda_fail(p, e, "fs_set_fields mean carry");
   }
   p->state = kStateReal;
   if (p->batch && !p->tuned) {
@@ -1236,7 +1229,7 @@ fs_status fs_step_async(fs_plan_t p, int64_t nsteps) {
       e = cudaGraphLaunch(p->gexec, p->stream);
       if (e != cudaSuccess) return cuda_fail(p, e, "graph launch");
       left -= p->gsteps;
-      launches += (int64_t)p->gsteps * 2 * (int64_t)p->members.size();
+      launches += (int64_t)p->gsteps * (p->batch ? 2 : pass_kinds(p->members[0]));
     }
   }
   for (; left > 0; --left) {
@@ -1264,11 +1257,9 @@ fs_status fs_get_fields(fs_plan_t p, void* const* out) {
   if (!out) return fail(p, FS_ERR_INVALID_ARG, "fields_out is NULL");
   if (p->state == kStateNone) return fail(p, FS_ERR_STATE, "fs_get_fields before fs_set_fields");
   if (p->state == kStateSpec && !p->fd) {
-    for (const Member& m : p->members) {
-      fs::KArgs a = make_args(p, m, 2);
-      cudaError_t e = launch_row(p, a, p->stream);
-      if (e != cudaSuccess) return cuda_fail(p, e, "inverse row pass");
-    }
+    const cudaError_t e = p->batch ? launch_batch_pass(p, 2, 0, p->stream)
+                                   : launch_row(p, make_args(p, p->members[0], 2), p->stream);
+    if (e != cudaSuccess) return cuda_fail(p, e, "inverse row pass");
     p->state = kStateBoth;  // the spectra stay valid: the next step carries on from them
   }
   const size_t rs = p->f64 ? sizeof(double) : sizeof(float);
@@ -1571,8 +1562,8 @@ fs_status fs_batch_schedule(fs_plan_t p, int64_t* row_grid, int64_t* col_grid, i
   if (!p->batch) return fail(p, FS_ERR_INVALID_ARG, "not a batched plan");
   const fs::BatchArgs& b = p->bargs;
   const bool r2 = b.row_form == 2, c2 = b.col_form == 2;
-  if (row_grid) *row_grid = r2 ? b.row2_grid : b.row_grid;
-  if (col_grid) *col_grid = c2 ? b.col2_grid : b.col_grid;
+  if (row_grid) *row_grid = r2 ? b.row2_total : b.row_total;  // one CTA per item
+  if (col_grid) *col_grid = c2 ? b.col2_total : b.col_total;
   if (row_items) *row_items = r2 ? b.row2_total : b.row_total;
   if (col_items) *col_items = c2 ? b.col2_total : b.col_total;
   if (row_form) *row_form = b.row_form;
