@@ -201,7 +201,7 @@ FS_API fs_status fs_profile_read(fs_plan_t plan, double* ms_per_pass, int64_t* l
  * form (1: half-length row pass / column tiles with radix-16 line
  * transforms; 2: warp-per-line kernels, one warp per line with radix up to
  * 32, two-column tiles -- FP32 members with both axes in [64, 1024]), the
- * persistent grid size (CTAs) and the number of work items.  Any output
+ * grid size (CTAs; one per work item) and the number of work items.  Any output
  * pointer may be NULL. */
 FS_API fs_status fs_batch_schedule(fs_plan_t plan, int64_t* row_grid, int64_t* col_grid, int64_t* row_items,
                                    int64_t* col_items, int* row_form, int* col_form);
@@ -253,14 +253,16 @@ FS_API fs_status fs_step2d_static(const fs_params* prm, void* fields, int64_t ns
  *       barriers between the passes (single 2D FS_F32 plans, square grids
  *       of 256, 512 or 1024 points, p <= 3; the first step after
  *       fs_set_fields runs the separate passes);
- *   0 = the default: form 2 for 2D lines of 256 to 1024 points, form 3 for
- *       2D columns of 2048, form 1 otherwise (3D x passes, with their many
- *       lines, keep form 1).
+ *   0 = the default: form 2 for 2D rows of 64 to 1024 points and 2D columns
+ *       of 256 to 1024 points (of 64 and 128 points while nx <= 1024), form 3
+ *       for 2D columns of 2048, form 1 otherwise; 3D x passes of 64 to 512
+ *       points run a pair-form kernel of their own.
  * A form on a plan it does not cover returns FS_ERR_UNSUPPORTED (form 4 for
  * one pass only: FS_ERR_INVALID_ARG); FP64 plans
- * always run form 1.  On a batched plan a nonzero form pins the ensemble
- * kernels' form for that pass (the autotuner then only picks the grid size,
- * at the next fs_set_fields); 0 lets the autotuner choose.  Used by the
+ * take forms 0 and 1 (0: pair-form rows and warp-per-line columns with two to
+ * eight values per thread where they exist).  On a batched plan a nonzero form pins the ensemble
+ * kernels' form for that pass (from the next fs_set_fields); 0 lets the
+ * autotuner choose.  Used by the
  * tests (both forms against the oracle) and for A/B timing. */
 FS_API fs_status fs_set_pass_forms(fs_plan_t plan, int row_form, int col_form);
 

@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(Row2Cfg<float, 1024>::MAX_THREADS, 4)
   const long long rp = item - begin[m];
   switch (a.nx) {
 #define FS_CASE(n) \
-  case n: row2_body<float, n>(a, rp, smem_raw, bar, 0); break;
+  case n: row2_body<float, n, 1, -1, true>(a, rp, smem_raw, bar, 0); break;
     FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
     default: break;
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(128, 5)
   const int group = rem / np, cp = rem % np;
   switch (a.ny) {
 #define FS_CASE(n) \
-  case n: col2_body<float, n>(a, &maps[m], cp, group, smem_raw, bar, 0); break;
+  case n: col2_body<float, n, 1, true>(a, &maps[m], cp, group, smem_raw, bar, 0); break;
     FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
     default: break;

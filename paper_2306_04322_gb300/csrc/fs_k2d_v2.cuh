@@ -154,7 +154,8 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
 // wait gave up.  PC >= 0: the caller guarantees nf = PC + 1, and the
 // pointwise stage is compiled for that p alone (the 96-thread kernel, whose
 // nf is 3: a kernel holding the code for every p measured slower there).
-template <typename T, int NX, int G = 1, int PC = -1>
+// EARLY: see griddep_launch_dependents.
+template <typename T, int NX, int G = 1, int PC = -1, bool EARLY = false>
 __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsigned char* smem_raw, uint64_t* bar,
                                           uint32_t parity) {
   using C = cplx<T>;
@@ -195,7 +196,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
   // previous pass takes, and no lane of warp 0 polls before lane 0 has issued
   griddep_wait();
   __syncwarp();
-  griddep_launch_dependents();
+  if (EARLY) griddep_launch_dependents();
   if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
     mbar_wait_bounded(bar, parity, kWaitPolls);  // let the copies land before exiting
@@ -257,6 +258,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
         for (int m = 0; m < E; ++m) v[m] = s[t + TPL * m];  // z = g_a + i g_b, natural order
       }
       line_fft<NX, E, -1>(v, t, tw, st, ld, lsync);
+      if (!EARLY && !inv) griddep_launch_dependents();
       if (inv) {
         // a + i b = conj(v)
         if (a.mode == 2) {
@@ -586,7 +588,8 @@ __device__ __noinline__ void col2_packed_update(cplx<T>* __restrict__ y, const c
 // value per lane and row.
 // Column pair (FP64: column) `cpair`, field group `group` of the simulation
 // `a` (blockDim = 64 TK G); `bar` as for row2_body.  Returns false if a bounded wait gave up.
-template <typename T, int NY, int G = 1>
+// EARLY: see griddep_launch_dependents.
+template <typename T, int NY, int G = 1, bool EARLY = false>
 __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tmap, int cpair, int group,
                                           unsigned char* smem_raw, uint64_t* bar, uint32_t parity) {
   using C = cplx<T>;
@@ -628,7 +631,7 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   // previous pass takes, and no lane of warp 0 polls before lane 0 has issued
   griddep_wait();
   __syncwarp();
-  griddep_launch_dependents();
+  if (EARLY) griddep_launch_dependents();
   if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
     mbar_wait_bounded(bar, parity, kWaitPolls);
@@ -709,6 +712,7 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   }
   // results (conj of the last transform) back to the interleaved tile layout
   // of this region, then out by TMA: c -> slot 0, eta_i -> slot i
+  if (!EARLY) griddep_launch_dependents();
   region_sync();  // both columns are done with their compact areas
 #pragma unroll
   for (int m = 0; m < E; ++m) reg[(t + TPL * m) * Cfg::TK + j] = cconj(v[m]);

@@ -285,7 +285,7 @@ __device__ __forceinline__ void row_pointwise_fixed(const Pointwise<T>& pw, cplx
 // Compute part of one row-pass work item (row block rb) once its rows have
 // landed: input slots `in` ([nf][R][PL], fields in natural layout), scratch
 // slot `scr` ([R][PL], df/dc), pass tables `twr` in shared memory.
-template <typename T, int NX, bool W = false>
+template <typename T, int NX, bool W, bool EARLY>
 __device__ __forceinline__ void row_compute(const KArgs& a, long long rb, cplx<T>* in, cplx<T>* scr,
                                             const cplx<T>* twr) {
   using C = cplx<T>;
@@ -357,6 +357,7 @@ __device__ __forceinline__ void row_compute(const KArgs& a, long long rb, cplx<T
         for (int m = 0; m < E; ++m) v[m] = s[t + TPL * m];
       }
       line_fft<L, E, -1>(v, t, twr, st, ld, wsync);
+      if (!EARLY && !inv) griddep_launch_dependents();
       if (inv) {
         if (a.mode == 2) {
           C* dst = realc + f * half_stride + row * L;
@@ -480,7 +481,7 @@ __device__ __forceinline__ void row_compute(const KArgs& a, long long rb, cplx<T
 // One row-pass work item with its own table copy and load (ensemble kernel):
 // `bar` is an initialised mbarrier whose next phase has parity `parity`.
 // Returns false if a bounded wait gave up (the caller must stop).
-template <typename T, int NX, bool W = false>
+template <typename T, int NX, bool W = false, bool EARLY = false>
 __device__ __forceinline__ bool row_body(const KArgs& a, long long rb, unsigned char* smem_raw, uint64_t* bar,
                                          uint32_t parity) {
   using C = cplx<T>;
@@ -498,13 +499,13 @@ __device__ __forceinline__ bool row_body(const KArgs& a, long long rb, unsigned 
     fence_proxy_async_smem();
     row_issue<T, NX, W>(a, rb, slots, bar);
   }
-  griddep_launch_dependents();
+  if (EARLY) griddep_launch_dependents();
   if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
     mbar_wait_bounded(bar, parity, kWaitPolls);  // let the copies land before exiting
     return false;
   }
-  row_compute<T, NX, W>(a, rb, slots, slots + a.nf * Cfg::R * Cfg::PL, twr);
+  row_compute<T, NX, W, EARLY>(a, rb, slots, slots + a.nf * Cfg::R * Cfg::PL, twr);
   return true;
 }
 
@@ -614,7 +615,7 @@ constexpr size_t col_smem_bytes(int tk) {
 // One column-pass work item: kx tile bx, field group g of the simulation
 // described by `a`, tiles loaded through the tensor map `tmap`.  TCM != 0:
 // the first radix-16 pass of each forward transform runs on tensor cores.
-template <typename T, int NY, int TCM = TC_NONE>
+template <typename T, int NY, int TCM = TC_NONE, bool EARLY = false>
 __device__ __forceinline__ bool col_body(const KArgs& a, const CUtensorMap* tmap, int bx, int g,
                                          unsigned char* smem_raw, uint64_t* bar, uint32_t parity) {
   using C = cplx<T>;
@@ -648,7 +649,7 @@ __device__ __forceinline__ bool col_body(const KArgs& a, const CUtensorMap* tmap
   copy_to_smem(twc, reinterpret_cast<const C*>(a.tw_col), Cfg::TWS);
   for (int i = threadIdx.x; i < NY; i += blockDim.x) k2yt[i] = reinterpret_cast<const T*>(a.k2y)[i];
   griddep_wait();
-  griddep_launch_dependents();
+  if (EARLY) griddep_launch_dependents();
   __syncthreads();
   if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
@@ -702,7 +703,10 @@ __device__ __forceinline__ bool col_body(const KArgs& a, const CUtensorMap* tmap
       }
       line_fft<NY, E, -1>(v, t, twc, st, ld, sync);
     }
-    if (inv) break;
+    if (inv) {
+      if (!EARLY) griddep_launch_dependents();
+      break;
+    }
     if (it + 1 < nin) {
       sync();
 #pragma unroll

@@ -266,18 +266,19 @@ fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {
   a.tw_z = m.tw_z;
   a.tw_half = m.tw_half;
   a.tw_row_w = m.tw_row_w;
-  // single plans: the warp-per-line forms by default for lines of 256 points
-  // and more (form 0) -- rows only in 2D: a 3D x pass has ny nz lines, and
-  // one row pair per CTA (table fetch and set-up per pair) loses to the
-  // several-row CTAs of the half-length kernel there -- always with form 2,
-  // never with form 1; ensemble members keep both tables (the autotuner
-  // picks the form per pass)
-  // (FP64: the pair form saves a third of the row transforms' instructions
-  // on every grid, so form 0 takes it wherever it exists)
+  // Single plans, form 0.  Rows: the pair form in 2D (a 3D x pass has ny nz
+  // lines and its own kernel) and, in FP64, on every grid (a third fewer
+  // instructions).  Columns: the warp-per-column form from 256 points, or from
+  // 64 while the columns are few: many columns of 64 or 128 points do better in
+  // the tiles of form 1, few of them leave the tiles' CTAs far apart (FP32, per
+  // step, form 1 / form 2: 64^2 p = 1 8.2 / 4.8 us, 128^2 9.3 / 5.2, 512 x 128
+  // p = 3 9.9 / 7.3, 2048 x 64 p = 3 14.0 / 16.9).  Ensemble members keep both
+  // tables (the autotuner picks the form per pass).
+  const int nx = m.prm.n[0], ny = m.prm.n[1];
   const bool r2 = p->batch || p->row_form == 2 || p->row_form == 4 ||
-                  (p->row_form == 0 && (p->f64 || (m.prm.n[0] >= 256 && m.prm.ndim == 2)));
+                  (p->row_form == 0 && (p->f64 || m.prm.ndim == 2));
   const bool c2 = p->batch || p->col_form == 2 || p->col_form == 4 ||
-                  (p->col_form == 0 && (p->f64 || m.prm.n[1] >= 256));
+                  (p->col_form == 0 && (p->f64 || ny >= 256 || (ny >= 64 && nx <= 1024)));
   a.tw_row2 = r2 ? m.tw_row2 : nullptr;
   a.tw_col2 = c2 ? m.tw_col2 : nullptr;
   a.tw_row2w = (!p->batch && p->row_form == 3) ? m.tw_row2w : nullptr;
