@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(128, 5)
   const int group = rem / np, cp = rem % np;
   switch (a.ny) {
 #define FS_CASE(n) \
-  case n: col2_body<float, n, 1, true>(a, &maps[m], cp, group, smem_raw, bar, 0); break;
+  case n: col2_body<float, n, 1, 2, 2, true>(a, &maps[m], cp, group, smem_raw, bar, 0); break;
     FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
     default: break;
@@ -70,7 +70,7 @@ size_t row2_smem_f32(int nx, int nf, int mode) {
 size_t col2_smem_f32(int ny) {
   switch (ny) {
 #define FS_CASE(n) \
-  case n: return col2_smem_bytes<float, n>();
+  case n: return Col2Cfg<float, n, 1, 2, 2>::SMEM;
     FS_V2_SIZES(FS_CASE)
 #undef FS_CASE
     default: return 0;

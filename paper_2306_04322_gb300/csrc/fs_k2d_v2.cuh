@@ -503,35 +503,39 @@ __global__ void __launch_bounds__(32 * G * NW, row2_min_blocks<T, G, NW>())
   row2_body<T, NX, G, (sizeof(T) == 4 && G == 1 && NW == 3) ? 2 : -1>(a, blockIdx.x, smem_raw, bar, 0);
 }
 
-template <typename T, int NY, int G = 1>
+// A column CTA: NR regions (slots) of TK adjacent kx columns, one line of
+// 32 G threads per (region, column).  Wide tiles matter: TMA takes 1.5 cycles
+// of an SM for a tile row of 16 or of 32 bytes alike (measured: copies in 16-,
+// 32- and 64-byte rows run at 3.3, 6.0 and 8.2 TB/s), and 16-byte rows alone
+// made 9 us of a 1024^2 pass (p = 2, FP32).  Four FP32 columns (32-byte rows)
+// come in with the 32-byte swizzle, which puts rows four apart on different
+// banks when a warp reads its column.
+template <typename T, int NY, int G, int TK_, int NR_>
 struct Col2Cfg {
   static constexpr bool F64 = sizeof(T) == 8;
   static constexpr int CS = 2 * (int)sizeof(T);               // bytes of a complex value
   static constexpr int TPL = 32 * G;                          // threads per line
   static constexpr int E = NY / TPL;
-  static constexpr int TK = F64 ? 1 : 2;                      // kx columns per CTA (16-byte TMA rows)
-  static constexpr int NE = F64 ? 1 : 2;                      // eta_i per field group
+  static constexpr int TK = TK_, NR = NR_;
+  static constexpr int NE = F64 ? 1 : NR;                     // eta_i per field group
+  static constexpr int THREADS = TPL * TK * NR;
+  static constexpr bool SWZ = TK * CS == 32;                  // 32-byte rows: swizzled (box of encode_col_map)
   static constexpr int BH = NY < 256 ? NY : 256;              // TMA box height (rows)
-  static constexpr int PL = line_pad_len<T>(NY);           // complex per compact column area
+  static constexpr int PL = line_pad_len<T>(NY);              // complex per compact column area
   // slot region: the [NY][TK] tile as loaded, then TK compact areas, then the
-  // [NY][TK] tile again for the TMA store; a multiple of 16 complex so every
-  // region starts on 128 bytes (TMA)
-  static constexpr int SLOT = (((NY * TK > TK * PL) ? NY * TK : TK * PL) + 15) & ~15;
+  // [NY][TK] tile again for the TMA store; every region starts on 256 bytes
+  // (TMA, the swizzle's period)
+  static constexpr int SLOT = (((NY * TK > TK * PL) ? NY * TK : TK * PL) + 31) & ~31;
   static constexpr int TWS = pass_table_size(NY, E);
   static constexpr int TW_BYTES = ((TWS * CS) + 127) & ~127;
   static constexpr int K2_BYTES = ((NY * (int)sizeof(T)) + 127) & ~127;
-  static constexpr int HEAD = 128 + TW_BYTES + K2_BYTES;
+  static constexpr int HEAD = (128 + TW_BYTES + K2_BYTES + 255) & ~255;
+  static constexpr size_t SMEM = HEAD + (size_t)NR * SLOT * CS;
   // CTAs per SM the registers are budgeted for: FP32 128 per thread at 32
   // values, FP64 at least 64
-  static constexpr int MIN_BLOCKS = F64 ? (G <= 2 ? 8 / G : (G == 4 ? 3 : 1)) : (E >= 32 ? 4 / G : (G == 1 ? 4 : 3));
+  static constexpr int MIN_BLOCKS =
+      F64 ? (G <= 2 ? 8 / G : (G == 4 ? 3 : 1)) : (E >= 32 ? 512 / THREADS : (G == 1 ? 512 : 768) / THREADS);
 };
-
-// Shared memory of one CTA: the head and two slot regions.
-template <typename T, int NY, int G = 1>
-constexpr size_t col2_smem_bytes() {
-  using Cfg = Col2Cfg<T, NY, G>;
-  return Cfg::HEAD + (size_t)2 * Cfg::SLOT * Cfg::CS;
-}
 
 // The packed kx = 0 / Nyquist column of the first CTA: y holds this warp's
 // forward transform Z = A + i B (A the kx = 0 column, B the kx = nx/2 one,
@@ -572,13 +576,12 @@ __device__ __noinline__ void col2_packed_update(cplx<T>* __restrict__ y, const c
   }
 }
 
-// FP32 CTA: two adjacent kx columns (kx0 = 2 blockIdx.x, kx0 + 1) of one field
-// group (blockIdx.y): group 0 holds df/dc and c, group g >= 1 eta_{2g-1} and
-// eta_{2g}; warp (region r, column j), r = 0, 1.  FP64 CTA: one column of
+// Field groups: group 0 holds df/dc and c, group g >= 1 the NE eta_i from
+// eta_{NE (g - 1) + 1}; line (region r, column j).  FP64 CTA: one column of
 // {df/dc, c} or of one eta_i, the smallest unit there is: the pass is bound by
 // the FP64 pipe, so its time is the busiest SM's share of the transforms
-// (256^2, p = 4: 9.3 transforms per SM on average; 16 on the busiest with the
-// FP32 units, 11 with these).  Four warps per CTA and
+// (256^2, p = 4: 9.3 transforms per SM on average; 16 on the busiest with
+// pairs of columns and eta_i, 11 with these).  Four warps per CTA and
 // 1 + ceil(p / 2) groups, so every CTA carries about two transforms per warp
 // and several CTAs share an SM.  The tiles come in by TMA, every warp copies
 // its column to registers, then its region becomes two compact per-column
@@ -586,27 +589,27 @@ __device__ __noinline__ void col2_packed_update(cplx<T>* __restrict__ y, const c
 // transform the results go back to the interleaved tile layout and out by
 // TMA, so the global writes are whole 16-byte rows instead of one 8-byte
 // value per lane and row.
-// Column pair (FP64: column) `cpair`, field group `group` of the simulation
-// `a` (blockDim = 64 TK G); `bar` as for row2_body.  Returns false if a bounded wait gave up.
-// EARLY: see griddep_launch_dependents.
-template <typename T, int NY, int G = 1, bool EARLY = false>
-__device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tmap, int cpair, int group,
+// Column block `cblk` (TK columns), field group `group` of the simulation `a`
+// (blockDim = THREADS); `bar` as for row2_body.  Returns false if a bounded
+// wait gave up.  EARLY: see griddep_launch_dependents.
+template <typename T, int NY, int G, int TK, int NR, bool EARLY = false>
+__device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tmap, int cblk, int group,
                                           unsigned char* smem_raw, uint64_t* bar, uint32_t parity) {
   using C = cplx<T>;
-  using Cfg = Col2Cfg<T, NY, G>;
+  using Cfg = Col2Cfg<T, NY, G, TK, NR>;
   constexpr int E = Cfg::E, BH = Cfg::BH, PL = Cfg::PL, SLOT = Cfg::SLOT, TPL = Cfg::TPL;
   C* tw = reinterpret_cast<C*>(smem_raw + 128);
   T* k2yt = reinterpret_cast<T*>(smem_raw + 128 + Cfg::TW_BYTES);
   C* regions = reinterpret_cast<C*>(smem_raw + Cfg::HEAD);
   const int nf = a.nf, p = nf - 1;
   const int line = (threadIdx.x >> 5) / G, t = threadIdx.x % TPL;  // line (region, column), thread in it
-  constexpr int TK = Cfg::TK, NE = Cfg::NE;
+  constexpr int NE = Cfg::NE;
   const int j = line % TK, r = line / TK;
   const int nreg = group == 0 ? 2 : (p - NE * (group - 1) >= NE ? NE : 1);
   // slot of region q of this group: group 0: df/dc (nf), c (0); else eta_{NE (g - 1) + 1 + q}
   auto slot_of = [nf, group](int q) { return group == 0 ? (q == 0 ? nf : 0) : NE * (group - 1) + 1 + q; };
   const bool isF = (group == 0 && r == 0), isC = (group == 0 && r == 1);
-  const int kx0 = cpair * Cfg::TK, kx = kx0 + j;
+  const int kx0 = cblk * TK, kx = kx0 + j;
   const int H = a.nx / 2;
 
   if (r >= nreg) return true;  // the second region of a last group with one eta
@@ -615,7 +618,7 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
     // generic accesses (ended by the caller's CTA barrier) before the TMA writes
     fence_proxy_async_smem();
     const uint32_t tbytes = (uint32_t)(Cfg::TWS * sizeof(C)), kbytes = (uint32_t)(NY * sizeof(T));
-    mbar_arrive_expect_tx(bar, tbytes + kbytes + (uint32_t)(nreg * NY * Cfg::TK * sizeof(C)));
+    mbar_arrive_expect_tx(bar, tbytes + kbytes + (uint32_t)(nreg * NY * TK * sizeof(C)));
     // the constant tables first, overlapping the previous grid's tail
     bulk_g2s(tw, G == 1 || Cfg::F64 ? a.tw_col2 : a.tw_col2w, tbytes, bar);
     bulk_g2s(k2yt, a.k2y, kbytes, bar);
@@ -623,7 +626,7 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
     for (int q = 0; q < nreg; ++q)
       // innermost coordinate kx0 in 8-byte units is even: 16-byte aligned
       for (int y0 = 0; y0 < NY; y0 += BH)
-        tma_load_3d(regions + q * SLOT + y0 * Cfg::TK, tmap, kx0 * (Cfg::CS / 8), y0, slot_of(q), bar);
+        tma_load_3d(regions + q * SLOT + y0 * TK, tmap, kx0 * (Cfg::CS / 8), y0, slot_of(q), bar);
   }
   const T* __restrict__ k2xt = reinterpret_cast<const T*>(a.k2x);
   const T kx2 = k2xt[kx];
@@ -638,15 +641,17 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
     return false;
   }
 
+  // this thread's first tile element; the others are TPL rows (a multiple of
+  // the swizzle's period) apart
   C* reg = regions + r * SLOT;
+  C* mine = reg + t * TK + (Cfg::SWZ ? j ^ (((t >> 2) & 1) << 1) : j);
   C v[E];
 #pragma unroll
-  for (int m = 0; m < E; ++m) v[m] = reg[(t + TPL * m) * Cfg::TK + j];
-  // named barriers with compile-time ids: 1, 2 per region (its two column
-  // lines), 3, 4 per column (df/dc^ handed to the c line), 5.. per line (its
-  // G warps, G = 2)
+  for (int m = 0; m < E; ++m) v[m] = mine[TPL * m * TK];
+  // named barriers: 1, 2 per region (its TK column lines), from 3 per column
+  // (df/dc^ handed to the c line), from 3 + TK per line (its G warps)
   auto region_sync = [r]() { if (r == 0) bar_sync(1, 32 * TK * G); else bar_sync(2, 32 * TK * G); };
-  const LineSync<G, 5, Cfg::F64> lsync{line};
+  const LineSync<G, 3 + TK, Cfg::F64> lsync{line};
   // both columns of this region have left the tile: it becomes two compact areas
   region_sync();
   C* xa = reg + j * PL;
@@ -666,11 +671,11 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
       lsync();
 #pragma unroll
       for (int m = 0; m < E; ++m) xa[t + TPL * m] = v[m];
-      if (j == 0) bar_arrive(3, 64 * G); else bar_arrive(4, 64 * G);
+      if (j == 0) bar_arrive(3, 64 * G); else if (j == 1) bar_arrive(4, 64 * G); else if (j == 2) bar_arrive(5, 64 * G); else bar_arrive(6, 64 * G);
       return true;
     }
     if (isC) {
-      if (j == 0) bar_sync(3, 64 * G); else bar_sync(4, 64 * G);
+      if (j == 0) bar_sync(3, 64 * G); else if (j == 1) bar_sync(4, 64 * G); else if (j == 2) bar_sync(5, 64 * G); else bar_sync(6, 64 * G);
     }
     if (special) {
       lsync();
@@ -715,11 +720,11 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   if (!EARLY) griddep_launch_dependents();
   region_sync();  // both columns are done with their compact areas
 #pragma unroll
-  for (int m = 0; m < E; ++m) reg[(t + TPL * m) * Cfg::TK + j] = cconj(v[m]);
+  for (int m = 0; m < E; ++m) mine[TPL * m * TK] = cconj(v[m]);
   fence_proxy_async_smem();
   region_sync();
   if (j == 0 && t == 0) {  // one thread of the region's column-0 line
-    for (int y0 = 0; y0 < NY; y0 += BH) tma_store_3d(tmap, kx0 * (Cfg::CS / 8), y0, slot_of(r), reg + y0 * Cfg::TK);
+    for (int y0 = 0; y0 < NY; y0 += BH) tma_store_3d(tmap, kx0 * (Cfg::CS / 8), y0, slot_of(r), reg + y0 * TK);
     bulk_commit();
     // the tile is read before the region is reused or the CTA exits; its
     // writes are performed before the grid completes (waiting for them here
@@ -729,8 +734,9 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
   return true;
 }
 
-template <typename T, int NY, int G>
-__global__ void __launch_bounds__(64 * Col2Cfg<T, NY, G>::TK * G, Col2Cfg<T, NY, G>::MIN_BLOCKS)
+// Uniform CTAs: grid (column blocks, field groups).
+template <typename T, int NY, int G, int TK, int NR>
+__global__ void __launch_bounds__(Col2Cfg<T, NY, G, TK, NR>::THREADS, Col2Cfg<T, NY, G, TK, NR>::MIN_BLOCKS)
     fs_col2_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
@@ -739,7 +745,24 @@ __global__ void __launch_bounds__(64 * Col2Cfg<T, NY, G>::TK * G, Col2Cfg<T, NY,
     fence_mbar_init();
   }
   __syncthreads();
-  col2_body<T, NY, G>(a, &tmap, blockIdx.x, blockIdx.y, smem_raw, bar, 0);
+  col2_body<T, NY, G, TK, NR>(a, &tmap, blockIdx.x, blockIdx.y, smem_raw, bar, 0);
+}
+
+// Mixed CTAs of four lines each (FP32): {df/dc, c} of two columns first, then
+// each eta_i of four columns.
+template <int NY, int G>
+__global__ void __launch_bounds__(128 * G, Col2Cfg<float, NY, G, 2, 2>::MIN_BLOCKS)
+    fs_col2m_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap2, const __grid_constant__ CUtensorMap tmap4) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  const int n2 = a.nx / 4, n4 = a.nx / 8, b = (int)blockIdx.x - n2;
+  if (b < 0) col2_body<float, NY, G, 2, 2>(a, &tmap2, blockIdx.x, 0, smem_raw, bar, 0);
+  else col2_body<float, NY, G, 4, 1>(a, &tmap4, b % n4, 1 + b / n4, smem_raw, bar, 0);
 }
 
 // Launchers: cudaErrorNotSupported when this form does not cover the
@@ -754,15 +777,27 @@ cudaError_t row2_launch_nw(const KArgs& a, cudaStream_t s) {
                     row2_smem_bytes<T, NX, G>(a.nf, a.mode), s, a);
 }
 
-template <typename T, int NY, int G>
+template <typename T, int NY, int G, int TK, int NR>
 cudaError_t col2_launch_n(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
   static unsigned done = 0;
-  cudaError_t e = allow_big_smem(fs_col2_kernel<T, NY, G>, &done);
+  cudaError_t e = allow_big_smem(fs_col2_kernel<T, NY, G, TK, NR>, &done);
   if (e != cudaSuccess) return e;
-  using Cfg = Col2Cfg<T, NY, G>;
+  using Cfg = Col2Cfg<T, NY, G, TK, NR>;
   const unsigned groups = (unsigned)(1 + (a.nf - 1 + Cfg::NE - 1) / Cfg::NE);  // {df/dc, c}; NE eta_i each
-  return launch_pdl(fs_col2_kernel<T, NY, G>, dim3((unsigned)(a.nx / 2 / Cfg::TK), groups),
-                    dim3((unsigned)(64 * Cfg::TK * G)), col2_smem_bytes<T, NY, G>(), s, a, tm);
+  return launch_pdl(fs_col2_kernel<T, NY, G, TK, NR>, dim3((unsigned)(a.nx / 2 / TK), groups),
+                    dim3((unsigned)Cfg::THREADS), Cfg::SMEM, s, a, tm);
+}
+
+template <int NY, int G>
+cudaError_t col2m_launch_n(const KArgs& a, const CUtensorMap& tm2, const CUtensorMap& tm4, cudaStream_t s) {
+  static unsigned done = 0;
+  cudaError_t e = allow_big_smem(fs_col2m_kernel<NY, G>, &done);
+  if (e != cudaSuccess) return e;
+  using C2 = Col2Cfg<float, NY, G, 2, 2>;
+  using C4 = Col2Cfg<float, NY, G, 4, 1>;
+  const size_t smem = C2::SMEM > C4::SMEM ? C2::SMEM : C4::SMEM;
+  return launch_pdl(fs_col2m_kernel<NY, G>, dim3((unsigned)(a.nx / 4 + (a.nf - 1) * (a.nx / 8))), dim3(128u * G), smem,
+                    s, a, tm2, tm4);
 }
 
 }  // namespace fs

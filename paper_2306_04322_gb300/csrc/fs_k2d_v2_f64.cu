@@ -57,7 +57,7 @@ cudaError_t col2_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t 
   if (a.nz != 1 || !a.tw_col2 || a.nf < 1 || a.nf > 5 || a.nx < 4) return cudaErrorNotSupported;
   switch (a.ny) {
 #define FS_CASE(n, g) \
-  case n: return col2_launch_n<double, n, g>(a, tm, s);
+  case n: return col2_launch_n<double, n, g, 1, 2>(a, tm, s);
     FS_COL64_SIZES(FS_CASE)
 #undef FS_CASE
     default: return cudaErrorNotSupported;

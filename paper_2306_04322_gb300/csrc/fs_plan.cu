@@ -54,7 +54,8 @@ struct Member {
   long long npts_full = 0;
   CUtensorMap tmap_col;  // [slot * nz + z][y][kx] tiles of the 2D column pass / 3D y passes
   CUtensorMap tmap_z;    // [slot][z][y][kx] z lines of the 3D z step
-  CUtensorMap tmap_col2; // [slot][y][kx] two-column tiles of the warp-per-column pass
+  CUtensorMap tmap_col2; // [slot][y][kx] tiles of the warp-per-column pass: 16-byte rows
+  CUtensorMap tmap_col4; // the same with 32-byte rows, swizzled (FP32 only)
   int fd_cur = 0;        // explicit FD: 0 state in `real`, 1 state in `spec` (as real fields)
   // adjoint workspace (allocated on first use)
   void* aspec = nullptr;  // 3 nf packed half-spectrum slots
@@ -342,7 +343,7 @@ cudaError_t launch_row(const fs_plan* p, const fs::KArgs& a, cudaStream_t s) {
 }
 cudaError_t launch_col(const fs_plan* p, const Member& m, const fs::KArgs& a, cudaStream_t s) {
   if (a.tw_col2 || a.tw_col2w) {
-    cudaError_t e = p->f64 ? fs::col2_launch_f64(a, m.tmap_col2, s) : fs::col2_launch_f32(a, m.tmap_col2, s);
+    cudaError_t e = p->f64 ? fs::col2_launch_f64(a, m.tmap_col2, s) : fs::col2_launch_f32(a, m.tmap_col2, m.tmap_col4, s);
     if (e != cudaErrorNotSupported) return e;
   }
   return p->f64 ? fs::col_launch_f64(a, m.tmap_col, s) : fs::col_launch_f32(a, m.tmap_col, s);
@@ -406,15 +407,20 @@ bool encode_col_map(Member& m, int nslots, bool f64) {
     if (r != CUDA_SUCCESS) return false;
   }
   if (col2_form(m.prm, f64)) {
-    // [slot][y][kx]: tiles of the warp-per-column pass with 16-byte rows (FP32 two columns, FP64 one)
+    // [slot][y][kx]: tiles of the warp-per-column pass with 16-byte rows (FP32
+    // two columns, FP64 one) and, FP32, with 32-byte rows (four columns) in
+    // the 32-byte swizzle its kernels undo
     cuuint64_t dims[3] = {W, (cuuint64_t)ny, (cuuint64_t)nslots};
     cuuint64_t strides[2] = {W * 8, W * 8 * ny};
-    cuuint32_t box[3] = {2, (cuuint32_t)(ny < 256 ? ny : 256), 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = enc(&m.tmap_col2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, m.spec, dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return false;
+    for (int wide = 0; wide < (f64 ? 1 : 2); ++wide) {
+      cuuint32_t box[3] = {wide ? 4u : 2u, (cuuint32_t)(ny < 256 ? ny : 256), 1};
+      CUresult r = enc(wide ? &m.tmap_col4 : &m.tmap_col2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, m.spec, dims, strides,
+                       box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                       wide ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                       CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (r != CUDA_SUCCESS) return false;
+    }
   }
   if (nz > 1) {
     // [slot][z][y][kx]: z lines of one (ky, kx tile), up to 256 planes per box

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(128, 4)
   __syncthreads();
   uint32_t parity = 0;
   const long long row_items = a.lines / 2;
-  const int pairs = N / 2 / Col2Cfg<float, N>::TK;
+  const int pairs = N / 2 / 2;
   const long long col_items = (long long)pairs * (1 + a.nf / 2);
   const uint32_t limit = (a.short_wait & 2) ? 0u : kGridWaitPolls;
   for (int step = 0; step < nsteps; ++step) {
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(128, 4)
     }
     if (!grid_barrier(gsync, gridDim.x, limit, a.flag)) return;
     for (long long item = blockIdx.x; item < col_items; item += gridDim.x) {
-      const bool ok = col2_body<float, N, 1>(a, &tmap, (int)(item % pairs), (int)(item / pairs), smem_raw, bar, parity);
+      const bool ok = col2_body<float, N, 1, 2, 2>(a, &tmap, (int)(item % pairs), (int)(item / pairs), smem_raw, bar, parity);
       if (__syncthreads_or(!ok)) return;
       parity ^= 1u;
     }
@@ -117,7 +117,7 @@ cudaError_t step2_launch_n(const KArgs& a, const CUtensorMap& tm, unsigned* gsyn
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_step2_kernel<N>, &done);
   if (e != cudaSuccess) return e;
-  const size_t r = row2_smem_bytes<float, N, 1>(a.nf, 0), c = col2_smem_bytes<float, N, 1>();
+  const size_t r = row2_smem_bytes<float, N, 1>(a.nf, 0), c = Col2Cfg<float, N, 1, 2, 2>::SMEM;
   const size_t smem = r > c ? r : c;
   int dev = 0, sms = 0, per_sm = 0;
   e = cudaGetDevice(&dev);
