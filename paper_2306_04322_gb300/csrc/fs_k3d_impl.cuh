@@ -52,8 +52,17 @@ struct LineCfg {
 // [slot * nz + z][y][kx].  TKC: columns per CTA (the tensor map's box) known
 // at compile time, 0 where a short x axis makes them fewer; the results leave
 // through the tile by TMA.  Both took integer instructions out of a kernel
-// that spent 39 % of its issue slots on addresses (256^3, FP32: Y1 us against
-// Y0 per pass of three slots).
+// that spent 39 % of its issue slots on addresses (256^3, FP32: 59 us against
+// 64 per pass of three slots; DRAM-bound since, 6.8 TB/s).
+// Order: each pass starts with what the one before it wrote last and L2
+// (129 MB) still holds.  The x pass writes all slots of a plane, so the
+// forward pass takes the planes from the last one down, all slots of a plane
+// together; the z step writes slot after slot, so the inverse takes the last
+// slot first (its last plane first too, as its own end, plane 0 of slot 0, is
+// where the x pass begins).  Per step against first to last in both: 256^3
+// p = 1 / 2 / 4 195 / 294 / 487 -> 185 / 284 / 482 us, 256x256x128 92.8 / 147 /
+// 248 -> 90.8 / 140 / 238; grids that L2 holds are unchanged (128^3 p = 2
+// 41.2 us).
 // ---------------------------------------------------------------------------
 template <typename T, int NY, int DIR, int TCM, int TKC>
 __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
@@ -68,7 +77,9 @@ __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
   const int tk = TKC ? TKC : blockDim.x / TPL;
   const int j = threadIdx.x % tk, t = (threadIdx.x / tk) & (TPL - 1);
   const int kx0 = blockIdx.x * tk;
-  const int plane = blockIdx.z * a.nz + blockIdx.y + a.plane0;  // slot * nz + z
+  const int islot = DIR < 0 ? blockIdx.y : gridDim.z - 1 - blockIdx.z;
+  const int z = a.nz - 1 - (DIR < 0 ? blockIdx.z : blockIdx.y);
+  const int plane = islot * a.nz + z + a.plane0;  // slot * nz + z
   // y inverse of c with the 3D carry: c's x spectrum goes to slot nf
   const int oplane = (DIR > 0 && a.carry3 && plane < a.nz) ? plane + a.nf * a.nz : plane;
   if (threadIdx.x == 0) {
@@ -189,7 +200,8 @@ __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
 // ---------------------------------------------------------------------------
 // z step: one CTA per (kx tile, ky storage row, field group).  Tensor map:
 // [slot][z][y][kx] with a box of one y row and up to 256 z planes; TKC and the
-// store as in the y pass (256^3, p = 2, FP32: Z1 us against Z0).
+// store as in the y pass (256^3, p = 2, FP32: 88 us against 107;
+// five CTAs per SM instead of four made 8 us of it).
 // ---------------------------------------------------------------------------
 template <typename T, int NZ, int TCM, int TKC>
 __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, sizeof(T) == 4 ? 5 : 4)
@@ -464,7 +476,8 @@ cudaError_t ypass_launch_tk(const KArgs& a, const CUtensorMap& tm, int planes, i
   static unsigned done = 0;
   cudaError_t e = allow_big_smem(fs_ypass_kernel<T, NY, DIR, TCM, TKC>, &done);
   if (e != cudaSuccess) return e;
-  const dim3 grid((unsigned)(a.nx / 2 / tk), (unsigned)planes, (unsigned)nslots);
+  const unsigned tiles = (unsigned)(a.nx / 2 / tk);
+  const dim3 grid = DIR < 0 ? dim3(tiles, (unsigned)nslots, (unsigned)planes) : dim3(tiles, (unsigned)planes, (unsigned)nslots);
   // The tensor-core stage holds TMEM: those launches do not overlap others.
   // Nor do the FP64 ones: CTAs of the next pass that start early gather on
   // the SMs that finish first, and a pass bound by the FP64 pipe lasts as long
