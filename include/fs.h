@@ -254,16 +254,16 @@ FS_API fs_status fs_step2d_static(const fs_params* prm, void* fields, int64_t ns
  *       of 256, 512 or 1024 points, p <= 3; the first step after
  *       fs_set_fields runs the separate passes);
  *   0 = the default: form 2 for 2D rows of 64 to 1024 points and 2D columns
- *       of 256 to 1024 points (of 64 and 128 points while nx <= 1024), form 3
- *       for 2D columns of 2048, form 1 otherwise; 3D x passes of 64 to 512
- *       points run a pair-form kernel of their own.
+ *       of 128 to 1024 points (of 64 points while nx <= 1024), form 3 for 2D
+ *       columns of 2048, form 1 otherwise; 3D x passes of 64 to 512 points
+ *       run a pair-form kernel of their own.
  * A form on a plan it does not cover returns FS_ERR_UNSUPPORTED (form 4 for
- * one pass only: FS_ERR_INVALID_ARG); FP64 plans
- * take forms 0 and 1 (0: pair-form rows and warp-per-line columns with two to
- * eight values per thread where they exist).  On a batched plan a nonzero form pins the ensemble
- * kernels' form for that pass (from the next fs_set_fields); 0 lets the
- * autotuner choose.  Used by the
- * tests (both forms against the oracle) and for A/B timing. */
+ * one pass only: FS_ERR_INVALID_ARG); FP64 plans take forms 0 and 1 (0:
+ * pair-form rows and warp-per-line columns of 64 to 2048 points with two to
+ * eight values per thread).  On a batched plan a nonzero form pins the
+ * ensemble kernels' form for that pass (from the next fs_set_fields); 0 lets
+ * the autotuner choose.  Used by the tests (both forms against the oracle)
+ * and for A/B timing. */
 FS_API fs_status fs_set_pass_forms(fs_plan_t plan, int row_form, int col_form);
 
 /* Test hook of the failure-detection path (the paper has no counterpart).

@@ -40,8 +40,8 @@ struct Member {
   void* tw_half = nullptr;
   void* tw_row_w = nullptr;  // x-pass tables with 32 values per thread (FP32 rows of 1024)
   void* tc_b = nullptr;  // split DFT matrix of the tensor-core stage (TC precisions)
-  void* tw_row2 = nullptr;  // x-line tables of the pair-form row pass (FP32, nx in {256, 512, 1024})
-  void* tw_col2 = nullptr;  // y-line tables of the warp-per-column pass (FP32 2D, ny in [64, 1024])
+  void* tw_row2 = nullptr;  // x-line tables of the pair-form row pass (nx in [64, 1024]; FP64 to 2048)
+  void* tw_col2 = nullptr;  // y-line tables of the warp-per-column pass (2D, ny in [64, 1024]; FP64 to 2048)
   void* tw_row3 = nullptr;  // x-line tables of the 3D x pass with several row pairs per CTA (FP32, nx 64 to 512)
   void* tw_row2w = nullptr; // the same with two warps per line (lines of 128 points and more)
   void* tw_col2w = nullptr;
@@ -269,17 +269,18 @@ fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {
   a.tw_row_w = m.tw_row_w;
   // Single plans, form 0.  Rows: the pair form in 2D (a 3D x pass has ny nz
   // lines and its own kernel) and, in FP64, on every grid (a third fewer
-  // instructions).  Columns: the warp-per-column form from 256 points, or from
-  // 64 while the columns are few: many columns of 64 or 128 points do better in
-  // the tiles of form 1, few of them leave the tiles' CTAs far apart (FP32, per
-  // step, form 1 / form 2: 64^2 p = 1 8.2 / 4.8 us, 128^2 9.3 / 5.2, 512 x 128
-  // p = 3 9.9 / 7.3, 2048 x 64 p = 3 14.0 / 16.9).  Ensemble members keep both
-  // tables (the autotuner picks the form per pass).
+  // instructions).  Columns: the warp-per-column form from 128 points, or from
+  // 64 while the columns are few: many columns of 64 points do better in the
+  // tiles of form 1 (FP32, per step, form 1 / form 2: 64^2 p = 1 8.2 / 4.8 us,
+  // 512 x 64 p = 2 7.8 / 6.0, 1024 x 64 9.2 / 7.7, 2048 x 64 11.1 / 11.4 and
+  // p = 4 13.6 / 14.8; 1024 x 128 p = 2 10.9 / 8.6, 2048 x 128 p = 0 to 4 12.0 /
+  // 10.3, 14.4 / 11.6, 13.7 / 12.8, 14.0 / 14.1, 16.5 / 16.5).  Ensemble members
+  // keep both tables (the autotuner picks the form per pass).
   const int nx = m.prm.n[0], ny = m.prm.n[1];
   const bool r2 = p->batch || p->row_form == 2 || p->row_form == 4 ||
                   (p->row_form == 0 && (p->f64 || m.prm.ndim == 2));
   const bool c2 = p->batch || p->col_form == 2 || p->col_form == 4 ||
-                  (p->col_form == 0 && (p->f64 || ny >= 256 || (ny >= 64 && nx <= 1024)));
+                  (p->col_form == 0 && (p->f64 || ny >= 128 || (ny >= 64 && nx <= 1024)));
   a.tw_row2 = r2 ? m.tw_row2 : nullptr;
   a.tw_col2 = c2 ? m.tw_col2 : nullptr;
   a.tw_row2w = (!p->batch && p->row_form == 3) ? m.tw_row2w : nullptr;
@@ -370,9 +371,9 @@ EncodeTiledFn encode_tiled() {
 
 // Where the warp-per-line forms apply: FP32 (plain, and the row pass also
 // for the tensor-core precisions, whose stage is in the column transforms),
-// semi-implicit FS; rows of 256, 512 or 1024 points (2D rows and 3D x
-// lines); 2D columns of 256, 512 or 1024 points with no tensor-core stage.
-// FP64: any x line of 64 to 2048 points, 2D columns of 64 to 512 points.
+// semi-implicit FS; rows of 64 to 1024 points (2D rows and 3D x lines); 2D
+// columns of 64 to 2048 points with no tensor-core stage.  FP64: x lines and
+// 2D columns of 64 to 2048 points.
 bool row2_form(const fs_params& prm, bool f64) {
   if (f64) return prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && fs::row2_g64(prm.n[0]) != 0;
   return prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && fs::row2_supported(prm.n[0], 1 + prm.p);
