@@ -125,14 +125,14 @@ cudaError_t row_launch_f64(const KArgs& a, cudaStream_t s);
 cudaError_t col_launch_f32(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
 cudaError_t col_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
 // Warp-per-line forms (FP32; fs_k2d_v2.cuh): the row pass in pair form for
-// nx in {256, 512, 1024} (modes 0, 1, 2; needs KArgs::tw_row2) and the column
-// pass with one warp per (column, slot) for ny in {256, 512, 1024} (needs
-// KArgs::tw_col2 and tensor maps with boxes of two columns and of four
-// (swizzled)).  Return cudaErrorNotSupported for other requests.
+// nx of 64 to 1024 (modes 0, 1, 2; needs KArgs::tw_row2) and the column pass
+// with one warp per (column, slot) for ny of 64 to 1024, two for 2048 (needs
+// KArgs::tw_col2 or tw_col2w and tensor maps with boxes of two columns and of
+// four (swizzled)).  Return cudaErrorNotSupported for other requests.
 cudaError_t row2_launch_f32(const KArgs& a, cudaStream_t s);
 cudaError_t col2_launch_f32(const KArgs& a, const CUtensorMap& tm, const CUtensorMap& tm4, cudaStream_t s);
-// The same in FP64: rows of 64 to 2048 points, columns of 64 to 512; warps
-// per line (0: no such kernel).
+// The same in FP64: rows and columns of 64 to 2048 points; warps per line
+// from row2_g64 / col2_g64 (0: no such kernel).
 cudaError_t row2_launch_f64(const KArgs& a, cudaStream_t s);
 cudaError_t col2_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
 // 3D x pass with several row pairs per CTA (FP32, nx of 64 to 512, modes 0

@@ -65,20 +65,10 @@ struct Pointwise {
     Ldt = k.Ldt;
   }
   __device__ __forceinline__ T hpoly(T e) const { return e * e * e * (e * (T(6) * e - T(15)) + T(10)); }
-  __device__ __forceinline__ T dh(T e) const {
-    T q = e * (T(1) - e);
-    return T(30) * q * q;
-  }
-  __device__ __forceinline__ T fc(T c, T h) const { return two_rho2 * (c - ca - dcab * h); }
-  __device__ __forceinline__ T feta(T c, T e, T S2) const {
-    T chem = rho2dcab * (cab - T(2) * c) * dh(e);
-    T well = T(2) * e * (T(1) - e) * (T(1) - T(2) * e) + four_alpha * e * (S2 - e * e);
-    return chem + w * well;
-  }
   // The step's stage on two lanes (two grid points per pair, lane-wise
   // arithmetic) with the constants multiplied out on the host: 13
-  // instructions per eta and 3 per point, against 19 and 3 for the
-  // definitions above term by term -- and fewer roundings.  FP64 (bound by its
+  // instructions per eta and 3 per point, against 19 and 3 for df/dc and
+  // df/deta_i term by term -- and fewer roundings.  FP64 (bound by its
   // pipe; with the reciprocal of KUpdate::quot), per step: 1024^2 p = 2 539 us
   // against 581, 64^3 p = 4 230 against 250; FP32: 1024^2 27.4 against 27.8.
   template <typename V>

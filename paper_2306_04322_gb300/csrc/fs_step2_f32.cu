@@ -39,7 +39,6 @@ __device__ __forceinline__ void fence_proxy_async_global() {
 // after `limit` polls (FS_FLAG_TIMEOUT is set); the host then zeroes the
 // counters.
 constexpr int kGroups = 16;
-constexpr int kSyncWords = 32 * (kGroups + 2);
 
 __device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned nblocks, uint32_t limit, int* flag) {
   fence_proxy_async_global();
