@@ -457,7 +457,7 @@ def extras(steps: int, warmup: int, device: int, peak, peak_kind):
                                                            r["total_ms"] / k, peak,
                                                            design_bytes=(4 * nf4 + 1) * N * s)
     # config 4: the ensemble advanced through its captured graph (32 steps per
-    # graph launch, one persistent launch per pass), two graph calls timed
+    # graph launch, one launch per pass), two graph calls timed
     probs = I.batch_problems(512, seed=0)
     r = time_plan(probs, "f32", 64, 1, device, chunk=32)
     kb = r["steps"]
