@@ -335,13 +335,17 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
 // steady steps and the inverse only: modes 0 and 2).  A 3D pass has ny nz
 // rows, so what counts is instructions, not the reach of a few rows over the
 // chip: 16 values per thread and 4 to 32 threads per line (two register
-// passes, one exchange), W warps per field, so that the table fetch and the
-// set-up are shared by PR = W 32 / TPL pairs.  Against the half-length kernel
-// (one real row per line of nx / 2, with its real <-> half-length step), 256^3,
-// p = 2: 100 us per pass against 118.
-template <int NX, int W>
+// passes, one exchange), so that one warp per field carries PR = 32 / TPL pairs
+// and the table fetch and the set-up are shared by them.  Against the
+// half-length kernel (one real row per line of nx / 2, with its real <->
+// half-length step), 256^3, p = 2: 97 us per pass against 118.  Small CTAs, so
+// that an SM always has some in each of load, transform and store: with two
+// warps per field a step takes 284 us (p = 4: 481) against 281 (464), with
+// four 302 (471); 64x256x256, p = 4: 124 against 116; 512-point rows, p = 1,
+// whose CTAs then hold a single pair: 96.5 against 97.
+template <int NX>
 struct Row3Cfg {
-  static constexpr int E = 16, TPL = NX / E, LPW = 32 / TPL, PR = W * LPW, H = NX / 2;
+  static constexpr int E = 16, TPL = NX / E, PR = 32 / TPL, H = NX / 2;
   // pitch of a line's area: pad16 layout, a multiple of 16 bytes, and = TPL
   // (mod 16) where a warp holds several lines, so that a half-warp's lines
   // start on different banks
@@ -352,18 +356,19 @@ struct Row3Cfg {
   static constexpr size_t smem(int nf) { return 128 + TW_BYTES + (size_t)nf * PR * PL * 8; }
 };
 
-template <int NX, int W, int NW>
-__global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3_kernel(KArgs a) {
+// NW: the most fields (warps) the instantiation takes.
+template <int NX, int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 3 ? 10 : 6) fs_row3_kernel(KArgs a) {
   using C = float2;
-  using Cfg = Row3Cfg<NX, W>;
-  constexpr int E = Cfg::E, TPL = Cfg::TPL, LPW = Cfg::LPW, PR = Cfg::PR, PL = Cfg::PL, H = Cfg::H;
+  using Cfg = Row3Cfg<NX>;
+  constexpr int E = Cfg::E, TPL = Cfg::TPL, PR = Cfg::PR, PL = Cfg::PL, H = Cfg::H;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   C* tw = reinterpret_cast<C*>(smem_raw + 128);
   C* areas = reinterpret_cast<C*>(smem_raw + 128 + Cfg::TW_BYTES);  // [nf][PR][PL], df/dc over c
   const int nf = a.nf;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane % TPL;
-  const int fw = w / W, q = (w % W) * LPW + lane / TPL;  // the warp's field, the line's pair
+  const int q = lane / TPL;                              // the line's pair; the warp's field is w
   const long long row0 = 2LL * PR * blockIdx.x;          // first row of the CTA
   C* spec = reinterpret_cast<C*>(a.spec);
   if (threadIdx.x == 0) {
@@ -391,7 +396,7 @@ __global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3
   bool bad = false;
   auto wsync = []() { __syncwarp(); };
   for (int ph = 0; ph < 2; ++ph) {
-    const int f = fw + ph;  // inverse: fields 0..nf-1; forward: g_1..g_p and df/dc
+    const int f = w + ph;  // inverse: fields 0..nf-1; forward: g_1..g_p and df/dc
     C* s = areas + ((f == nf ? 0 : f) * PR + q) * PL;
     auto st = [s](int i, C x) { s[pad16(i)] = x; };
     auto ld = [s](int i) { return s[pad16(i)]; };
@@ -467,14 +472,14 @@ __global__ void __launch_bounds__(32 * W * NW, NW == 3 ? 10 / W : 6 / W) fs_row3
   if (bad) atomicOr(a.flag, FS_FLAG_NONFINITE);
 }
 
-template <int NX, int W, int NW>
+template <int NX, int NW>
 cudaError_t row3_launch_nw(const KArgs& a, cudaStream_t s) {
-  using Cfg = Row3Cfg<NX, W>;
+  using Cfg = Row3Cfg<NX>;
   static unsigned done = 0;
-  cudaError_t e = allow_big_smem(fs_row3_kernel<NX, W, NW>, &done);
+  cudaError_t e = allow_big_smem(fs_row3_kernel<NX, NW>, &done);
   if (e != cudaSuccess) return e;
-  return launch_pdl(fs_row3_kernel<NX, W, NW>, dim3((unsigned)(a.lines / (2 * Cfg::PR))),
-                    dim3((unsigned)(32 * W * a.nf)), Cfg::smem(a.nf), s, a);
+  return launch_pdl(fs_row3_kernel<NX, NW>, dim3((unsigned)(a.lines / (2 * Cfg::PR))), dim3((unsigned)(32 * a.nf)),
+                    Cfg::smem(a.nf), s, a);
 }
 
 // NW: the most warps per line group the instantiation takes (nf <= NW).
