@@ -256,7 +256,7 @@ FS_API fs_status fs_step2d_static(const fs_params* prm, void* fields, int64_t ns
  *   0 = the default: form 2 for 2D rows of 64 to 1024 points and 2D columns
  *       of 128 to 1024 points (of 64 points while nx <= 1024), form 3 for 2D
  *       columns of 2048, form 1 otherwise; 3D x passes of 64 to 512 points
- *       run a pair-form kernel of their own.
+ *       and 2D ones of many short rows run a pair-form kernel of their own.
  * A form on a plan it does not cover returns FS_ERR_UNSUPPORTED (form 4 for
  * one pass only: FS_ERR_INVALID_ARG); FP64 plans take forms 0 and 1 (0:
  * pair-form rows and warp-per-line columns of 64 to 2048 points with two to

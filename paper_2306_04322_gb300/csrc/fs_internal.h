@@ -81,7 +81,7 @@ struct KArgs {
   const void* tw_col2;     // pass tables of the y line FFT of the warp-per-column form (L = ny, E = ny / 32)
   const void* tw_row2w;    // the same two with two warps per line (E = nx / 64, ny / 64; NULL: not this form)
   const void* tw_col2w;
-  const void* tw_row3;     // pass tables of the 3D x pass with several row pairs per CTA (L = nx, E = 16; NULL: none)
+  const void* tw_row3;     // pass tables of the x pass with several row pairs per CTA (L = nx, E = 16; NULL: none)
   const void* tc_b;        // tensor-core DFT stage: split 16-point DFT matrix, [hi | lo][32][32] float
   const void* k2x;         // |xi_x|^2 per x bin, nx/2 + 1 entries
   const void* k2y;         // |xi_y|^2 per y bin, ny entries
@@ -135,7 +135,7 @@ cudaError_t col2_launch_f32(const KArgs& a, const CUtensorMap& tm, const CUtenso
 // from row2_g64 / col2_g64 (0: no such kernel).
 cudaError_t row2_launch_f64(const KArgs& a, cudaStream_t s);
 cudaError_t col2_launch_f64(const KArgs& a, const CUtensorMap& tm, cudaStream_t s);
-// 3D x pass with several row pairs per CTA (FP32, nx of 64 to 512, modes 0
+// x pass with several row pairs per CTA (FP32, nx of 64 to 512, modes 0
 // and 2; needs KArgs::tw_row3).
 cudaError_t row3_launch_f32(const KArgs& a, cudaStream_t s);
 bool row3_supported(int nx);

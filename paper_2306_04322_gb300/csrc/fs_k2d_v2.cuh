@@ -331,11 +331,12 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
   return true;
 }
 
-// Several row pairs per CTA (3D x passes, FP32, rows of 64 to 512 points,
-// steady steps and the inverse only: modes 0 and 2).  A 3D pass has ny nz
-// rows, so what counts is instructions, not the reach of a few rows over the
-// chip: 16 values per thread and 4 to 32 threads per line (two register
-// passes, one exchange), so that one warp per field carries PR = 32 / TPL pairs
+// Several row pairs per CTA (FP32, rows of 64 to 512 points of 3D grids and of
+// 2D grids with many rows; steady steps and the inverse only: modes 0 and 2).
+// Such a pass has rows enough for every SM, so what counts is instructions, not
+// the reach of a few rows over the chip: 16 values per thread and 4 to 32
+// threads per line (two register passes, one exchange), so that one warp per
+// field carries PR = 32 / TPL pairs
 // and the table fetch and the set-up are shared by them.  Against the
 // half-length kernel (one real row per line of nx / 2, with its real <->
 // half-length step), 256^3, p = 2: 97 us per pass against 118.  Small CTAs, so
@@ -378,7 +379,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 3 ? 10 : 6) fs_row3_kernel(KArg
     bulk_g2s(tw, a.tw_row3, (uint32_t)(Cfg::TWS * sizeof(C)), bar);
   }
   griddep_wait();  // the spectra are the previous pass's output
-  griddep_launch_dependents();
+  if (a.nz > 1) griddep_launch_dependents();  // 2D: after the last transform, as row2_body
   if (w == 0) {
     __syncwarp();
     for (int i = lane; i < nf * PR; i += 32) {
@@ -423,6 +424,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 3 ? 10 : 6) fs_row3_kernel(KArg
       for (int m = 0; m < E; ++m) v[m] = s[t + TPL * m];
     }
     line_fft<NX, E, -1>(v, t, tw, st, ld, wsync);
+    if (ph == 1 && a.nz == 1) griddep_launch_dependents();
     if (ph == 0) {
       if (a.mode == 2) {
         float* ra = reinterpret_cast<float*>(a.real) + f * a.npts + (row0 + 2 * q) * NX;

@@ -1,4 +1,4 @@
-// FP32 instantiations of the 3D x pass with several row pairs per CTA.
+// FP32 instantiations of the x pass with several row pairs per CTA.
 #include "fs_k2d_v2.cuh"
 
 namespace fs {

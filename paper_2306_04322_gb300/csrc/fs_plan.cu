@@ -42,7 +42,7 @@ struct Member {
   void* tc_b = nullptr;  // split DFT matrix of the tensor-core stage (TC precisions)
   void* tw_row2 = nullptr;  // x-line tables of the pair-form row pass (nx in [64, 1024]; FP64 to 2048)
   void* tw_col2 = nullptr;  // y-line tables of the warp-per-column pass (2D, ny in [64, 1024]; FP64 to 2048)
-  void* tw_row3 = nullptr;  // x-line tables of the 3D x pass with several row pairs per CTA (FP32, nx 64 to 512)
+  void* tw_row3 = nullptr;  // x-line tables of the x pass with several row pairs per CTA (row3_form)
   void* tw_row2w = nullptr; // the same with two warps per line (lines of 128 points and more)
   void* tw_col2w = nullptr;
   double* csum = nullptr;
@@ -286,7 +286,7 @@ fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {
   a.tw_row2w = (!p->batch && p->row_form == 3) ? m.tw_row2w : nullptr;
   // columns of 2048 points have only the two-warp form, the default there
   a.tw_col2w = (!p->batch && (p->col_form == 3 || (p->col_form == 0 && m.prm.n[1] == 2048))) ? m.tw_col2w : nullptr;
-  a.tw_row3 = p->row_form == 0 ? m.tw_row3 : nullptr;
+  a.tw_row3 = (!p->batch && p->row_form == 0) ? m.tw_row3 : nullptr;
   a.tc_b = m.tc_b;
   a.k2x = m.k2x;
   a.k2y = m.k2y;
@@ -686,9 +686,18 @@ int col2_e(const fs_params& prm, bool f64) {
 bool row2w_form(const fs_params& prm, bool f64) { return !f64 && row2_form(prm, f64) && prm.n[0] >= 128; }
 bool col2w_form(const fs_params& prm, bool f64) { return !f64 && col2_form(prm, f64) && prm.n[1] >= 128; }
 
-// FP32 3D plans: the x pass with several row pairs per CTA.
+// FP32: the x pass with several row pairs per CTA, on 3D grids and on 2D ones
+// with many short rows -- 16 values per thread make two register passes of 64
+// to 256 points where the warp-per-line form makes three or four, but fewer
+// CTAs.  2D, per step, warp-per-line / this: 64 x 2048 p = 2 17.5 / 16.7 us and
+// p = 4 20.6 / 18.6, 128 x 2048 18.2 / 17.4 and 22.0 / 20.0 (128 x 1024 10.6 /
+// 11.0 and 13.2 / 13.3); 256 x 1024 p = 3 14.2 / 12.9 and p = 2 11.3 / 12.2,
+// 256 x 2048 22.7 / 20.4 and 19.6 / 21.0; 512 x 1024 p = 3 18.8 / 18.4 and p = 2
+// 15.9 / 16.2.
 bool row3_form(const fs_params& prm, bool f64) {
-  return !f64 && prm.ndim == 3 && prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS && fs::row3_supported(prm.n[0]);
+  const int nx = prm.n[0], ny = prm.n[1];
+  if (f64 || prm.scheme != FS_SCHEME_SEMI_IMPLICIT_FS || !fs::row3_supported(nx)) return false;
+  return prm.ndim == 3 || (nx <= 128 && ny >= 2048) || (nx == 256 && ny >= 1024 && prm.p >= 3);
 }
 
 // Rows of 1024 in FP32 run the x-pass variant with 32 values per thread.
@@ -732,7 +741,7 @@ TableLayout table_layout(const fs_params& prm, bool f64) {
   o = align16(o + (row2w_form(prm, f64) ? cs * fs::pass_table_size(nx, nx / 64) : 0));
   t.tw_col2w = o;
   o = align16(o + (col2w_form(prm, f64) ? cs * fs::pass_table_size(ny, ny / 64) : 0));
-  t.tw_row3 = o;  // 3D x pass with several row pairs per CTA: E = 16
+  t.tw_row3 = o;  // x pass with several row pairs per CTA: E = 16
   o = align16(o + (row3_form(prm, f64) ? cs * fs::pass_table_size(nx, 16) : 0));
   t.total = o;
   return t;

@@ -97,7 +97,8 @@ def test_fp64_update_with_denominators_out_of_the_reciprocals_range(F, O, n, kap
     ((8, 64), 2), ((16, 64), 1), ((16, 128), 4), ((32, 256), 3), ((16, 512), 2), ((8, 1024), 1), ((16, 1024), 3),
     ((512, 1024), 1), ((1024, 1024), 0), ((1024, 1024), 1), ((1024, 1024), 3), ((2048, 1024), 4), ((16, 2048), 2),
     ((8, 2048), 1), ((2048, 128), 1), ((2048, 64), 1),
-    # several row pairs per CTA of a 3D x pass: one warp per field and two
+    # several row pairs per CTA of an x pass, 2D and 3D
+    ((64, 2048), 2), ((128, 2048), 0), ((256, 1024), 3), ((256, 1024), 4),
     ((64, 8, 8), 0), ((64, 16, 16), 3), ((64, 128, 128), 2), ((128, 8, 8), 4), ((128, 64, 64), 1), ((256, 8, 8), 2),
     ((256, 32, 64), 3), ((512, 8, 8), 1), ((512, 16, 64), 4),
     # y / z lines on fewer columns than a tile has
