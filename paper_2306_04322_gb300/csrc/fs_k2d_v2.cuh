@@ -20,9 +20,9 @@
 // from real fields, 2 inverse only (mode 3, the free-energy diagnostic, keeps
 // the half-length kernel).
 //
-// Column pass, warp per column.  A CTA holds two adjacent kx columns (16-byte
-// TMA rows) of one field group -- {df/dc, c} or a pair of eta -- one warp per
-// (slot, column).  All warps transform forward; the df/dc warps publish their
+// Column pass, warp per column.  A CTA holds one, two or four adjacent kx
+// columns (16- or 32-byte TMA rows) of one field group -- {df/dc, c} or one or
+// two eta -- one warp (FP64 and 2048 points: several) per (slot, column).  All warps transform forward; the df/dc warps publish their
 // result for the c warps of the same column, and the c and eta warps apply
 // the k-space update (Eqs. A-C_discrete_fft_c, A-C_discrete_fft_eta) and
 // transform back.
@@ -588,14 +588,12 @@ __device__ __noinline__ void col2_packed_update(cplx<T>* __restrict__ y, const c
 // {df/dc, c} or of one eta_i, the smallest unit there is: the pass is bound by
 // the FP64 pipe, so its time is the busiest SM's share of the transforms
 // (256^2, p = 4: 9.3 transforms per SM on average; 16 on the busiest with
-// pairs of columns and eta_i, 11 with these).  Four warps per CTA and
-// 1 + ceil(p / 2) groups, so every CTA carries about two transforms per warp
-// and several CTAs share an SM.  The tiles come in by TMA, every warp copies
-// its column to registers, then its region becomes two compact per-column
-// areas (exchange buffers, pad32 layout).  After the update and the inverse
-// transform the results go back to the interleaved tile layout and out by
-// TMA, so the global writes are whole 16-byte rows instead of one 8-byte
-// value per lane and row.
+// pairs of columns and eta_i, 11 with these).  The tiles come in by TMA, every
+// line copies its column to registers, then its region becomes TK compact
+// per-column areas (exchange buffers, line_pad layout).  After the update and
+// the inverse transform the results go back to the interleaved tile layout
+// and out by TMA, so the global writes are whole tile rows instead of one
+// 8-byte value per lane and row.
 // Column block `cblk` (TK columns), field group `group` of the simulation `a`
 // (blockDim = THREADS); `bar` as for row2_body.  Returns false if a bounded
 // wait gave up.  EARLY: see griddep_launch_dependents.

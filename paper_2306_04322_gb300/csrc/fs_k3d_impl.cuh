@@ -1,7 +1,7 @@
 // 3D passes of the semi-implicit Fourier-spectral step (Eq. Gamma_fft_3d,
 // Algorithm 1 for 3D domains).  A step is four passes over the packed
 // x-spectra [slot][z][y][kx] (kx < nx/2, bin 0 = DC + i Nyquist):
-//   x pass     the 2D row kernel with ny * nz rows;
+//   x pass     the 2D row kernels, or fs_row3_kernel, with ny * nz rows;
 //   y forward  fs_ypass_kernel<DIR = -1> on the slots g_i, df/dc (and c in
 //              the first step after the fields are set);
 //   z step     fs_zstep_kernel: forward z transform, k-space update with
