@@ -53,14 +53,38 @@ __device__ __forceinline__ void hessian_apply(const Pointwise<T>& pw, const cplx
   }
 }
 
+// The steps' row and column tiles with the adjoint's pass tables
+// (adj_line_fft; KArgs::tw_row and tw_col of an adjoint launch hold them).
+template <typename T, int NX>
+struct AdjRowCfg : RowCfg<T, NX> {
+  using B = RowCfg<T, NX>;
+  static constexpr int TWS = adj_table_size<T>(B::L, B::E);
+  static constexpr int TW_BYTES = ((TWS * (int)sizeof(cplx<T>)) + 127) & ~127;
+  static constexpr size_t smem(int nf) {
+    return B::BAR_BYTES + TW_BYTES + (size_t)3 * nf * B::R * B::PL * sizeof(cplx<T>);
+  }
+};
+
+// B w of the row pass's post-processing; FP32 in the arithmetic the
+// sensitivities are to keep (cmul rounds the other product of the imaginary part).
+template <typename C>
+__device__ __forceinline__ C adj_cmul(C b, C w) {
+  if constexpr (sizeof(C) == 8)
+    return mk<C>(fmaf(b.x, w.x, -__fmul_rn(b.y, w.y)), fmaf(b.x, w.y, __fmul_rn(b.y, w.x)));
+  else return cmul(b, w);
+}
+
 // ---------------------------------------------------------------------------
-// Adjoint row forward: CTA of 3 nf warps, one per transform, and R rows.  Inputs real: lam' (a.real), u (a.aux).  Outputs 2 x^ of lam'_phi,
-// u_phi, f_phi(u) into adjoint slots [0, nf), [nf, 2nf), [2nf, 3nf).
+// Adjoint row forward: CTA of 3 nf warps, one per transform, and R rows.
+// Inputs real: lam' (a.real), u (a.aux).  Outputs 2 x^ of lam'_phi, u_phi,
+// f_phi(u) into adjoint slots [0, nf), [nf, 2nf), [2nf, 3nf).  f(u) in FP32 is
+// formed term by term (Pointwise::fc, feta): the sensitivities keep its
+// rounding too.
 // ---------------------------------------------------------------------------
 template <typename T, int NX, int P>
 __global__ void __launch_bounds__(96 * (P + 1)) fs_adj_row_fwd_kernel(KArgs a) {
   using C = cplx<T>;
-  using Cfg = RowCfg<T, NX>;
+  using Cfg = AdjRowCfg<T, NX>;
   constexpr int L = Cfg::L, E = Cfg::E, TPL = Cfg::TPL, R = Cfg::R, PL = Cfg::PL;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
@@ -111,15 +135,22 @@ __global__ void __launch_bounds__(96 * (P + 1)) fs_adj_row_fwd_kernel(KArgs a) {
       for (int i = 1; i < nf; ++i) {
         e[i] = slot(nf + i, r)[i0];
         h = pw.add_h2(e[i], h);
-        S2 = vfma(e[i], e[i], S2);
+        S2 = sizeof(T) == 4 ? cadd(S2, vmul(e[i], e[i])) : vfma(e[i], e[i], S2);
       }
-      slot(2 * nf, r)[i0] = pw.fc2(c, h);
-      const C chem = vfma(c, vsplat<C>(A), vsplat<C>(B));  // 30 rho2 dcab (cab - 2c)
+      if constexpr (sizeof(T) == 4) {
+        slot(2 * nf, r)[i0] = mk<C>(pw.fc(c.x, h.x), pw.fc(c.y, h.y));
 #pragma unroll
-      for (int i = 1; i < nf; ++i) {
-        const C ne = mk<C>(-e[i].x, -e[i].y), q = vfma(e[i], ne, e[i]);
-        const C in = vfma(chem, q, vfma(e[i], vsplat<C>(T(-2) * W), vsplat<C>(W)));
-        slot(2 * nf + i, r)[i0] = vfma(q, in, vmul(vmul(e[i], vsplat<C>(F)), vfma(e[i], ne, S2)));
+        for (int i = 1; i < nf; ++i)
+          slot(2 * nf + i, r)[i0] = mk<C>(pw.feta(c.x, e[i].x, S2.x), pw.feta(c.y, e[i].y, S2.y));
+      } else {
+        slot(2 * nf, r)[i0] = pw.fc2(c, h);
+        const C chem = vfma(c, vsplat<C>(A), vsplat<C>(B));  // 30 rho2 dcab (cab - 2c)
+#pragma unroll
+        for (int i = 1; i < nf; ++i) {
+          const C ne = mk<C>(-e[i].x, -e[i].y), q = vfma(e[i], ne, e[i]);
+          const C in = vfma(chem, q, vfma(e[i], vsplat<C>(T(-2) * W), vsplat<C>(W)));
+          slot(2 * nf + i, r)[i0] = vfma(q, in, vmul(vmul(e[i], vsplat<C>(F)), vfma(e[i], ne, S2)));
+        }
       }
     }
   }
@@ -133,12 +164,12 @@ __global__ void __launch_bounds__(96 * (P + 1)) fs_adj_row_fwd_kernel(KArgs a) {
     C v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = s[t + TPL * m];
-    line_fft<L, E, -1>(v, t, twr, st, ld, wsync);
+    adj_line_fft<L, E, -1>(v, t, twr, st, ld, wsync);
     wsync();
 #pragma unroll
     for (int m = 0; m < E; ++m) s[t + TPL * m] = v[m];
     wsync();
-    C* P = spec + o * a.slot_stride + row * L;
+    C* dst = spec + o * a.slot_stride + row * L;
     if (active) {
 #pragma unroll
       for (int m = 0; m < E; ++m) {
@@ -150,9 +181,9 @@ __global__ void __launch_bounds__(96 * (P + 1)) fs_adj_row_fwd_kernel(KArgs a) {
         } else {
           const C zm = cconj(s[L - k]);
           const C A = cadd(zk, zm), B = csub(zk, zm);
-          out = cadd(A, mul_i<-1>(cmul(B, __ldg(&twh[k]))));
+          out = cadd(A, mul_i<-1>(adj_cmul(B, __ldg(&twh[k]))));
         }
-        P[k] = out;
+        dst[k] = out;
       }
     }
   }
@@ -165,27 +196,36 @@ __global__ void __launch_bounds__(96 * (P + 1)) fs_adj_row_fwd_kernel(KArgs a) {
 // ---------------------------------------------------------------------------
 // A field kind has two parameters: the rate (M or L) and its gradient
 // coefficient; their sums accumulate per thread in FP64, or in FP32 as exact
-// products added into an unevaluated pair (two-sum): GB300 issues one FP64
-// instruction where it issues 32 to 64 FP32 ones, and the FP64 sums had been
-// most of the FP32 kernel's time.
+// products added into an unevaluated pair (two-sum, about 48 bits): GB300 issues
+// one FP64 instruction where it issues 32 to 64 FP32 ones, and with FP64 sums
+// (six conversions and four products per mode) the 512^2, p = 2 column pass takes
+// 51 us against 27.  A pair is as good as FP64 only while its products neither
+// overflow nor come so close to the end of the range that their rounding errors
+// vanish (an error is at least 2^-149, so 2^-69 of the largest product at 2^-80);
+// a thread whose largest product is outside (2^-80, 2^120) -- a strongly scaled
+// cotangent -- adds its modes again in FP64.
 template <typename T>
 struct AdjSum;
 template <>
 struct AdjSum<double> {
   double s = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+  template <typename V> __device__ __forceinline__ void add(V a, V b) { s = fma((double)a, (double)b, s); }
   __device__ __forceinline__ double value() const { return s; }
+  __device__ __forceinline__ bool in_range() const { return true; }
 };
 template <>
 struct AdjSum<float> {
-  float hi = 0.f, lo = 0.f;
+  float hi = 0.f, lo = 0.f, most = 0.f;
   __device__ __forceinline__ void add(float a, float b) {
     const float p = __fmul_rn(a, b), e = fmaf(a, b, -p);  // a b = p + e
     const float t = __fadd_rn(hi, p), v = __fadd_rn(t, -hi);
     lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fadd_rn(hi, -__fadd_rn(t, -v)), __fadd_rn(p, -v)), e));
     hi = t;
+    most = fmaxf(most, fabsf(p));
   }
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  // (an underflow to zero throughout is out of range too, unless lam' is zero: FP64 adds the same zeros)
+  __device__ __forceinline__ bool in_range() const { return most > 8.2718061e-25f && most < 1.3292279e36f; }
 };
 
 template <typename T>
@@ -199,33 +239,83 @@ struct AdjCoef {
     ke = co.ke;
     dt = co.dt;
   }
-  __device__ __forceinline__ static T recip(T y) {  // y >= 1
-    const T r = KUpdate<T>::quot(T(1), y);
-    if constexpr (sizeof(T) == 4) return fmaf(r, fmaf(-y, r, 1.f), r);  // one Newton step after the 2 ulp quotient
-    else return r;
+  // 1 / y rounded, y >= 1: one Newton step from the hardware's approximation
+  // (1 ulp) is the rounded reciprocal for every FP32 mantissa (all 2^23 tried),
+  // as long as it is a normal number; the factors 1/16 keep the step in range up
+  // to the largest y.  No branches: 32 rounded divisions in a thread's modes
+  // took 9 us of 36 of the 512^2, p = 2 column pass.
+  __device__ __forceinline__ static float recip(float y) {
+    const float s = y * 0.0625f;
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s));
+    r = fmaf(r, fmaf(-s, r, 1.f), r) * 0.0625f;
+    return y <= 3.402823466e38f ? r : (y != y ? y : 0.f);
   }
   // One mode at K2 of field kind f (0: c): va = D1 lam', vb = D2 lam' (times
   // scale), and Re conj(lam') (dD1 u + dD2 f) of its two parameters into r, g.
-  template <typename C>
-  __device__ __forceinline__ void mode(int f, T k2, T scale, C l, C u, C fu, C& va, C& vb, AdjSum<T>& r,
-                                       AdjSum<T>& g) const {
-    const T kk = f == 0 ? k2 * k2 : k2, rate = f == 0 ? Mdt : Ldt, kap = f == 0 ? kc : ke, m2 = f == 0 ? k2 : T(1);
-    const T d1 = recip(T(1) + rate * kap * kk), i2 = d1 * d1;
-    const T d2 = -rate * m2 * d1;
+  template <typename C, class Sum>
+  __device__ __forceinline__ void mode(int f, T k2, T scale, C l, C u, C fu, C& va, C& vb, Sum& r, Sum& g) const {
+    T d1, d2, r1, r2, g1, g2;  // D1, D2, their d/d rate, their d/d kappa
+    if constexpr (sizeof(T) == 4) {  // rounded quotients: the sensitivities keep their digits
+      if (f == 0) {
+        const T den = T(1) + Mdt * kc * k2 * k2, i2 = recip(den * den);
+        d1 = recip(den);
+        d2 = -Mdt * k2 * d1;
+        r1 = -dt * kc * k2 * k2 * i2;
+        r2 = -dt * k2 * i2;
+        g1 = -Mdt * k2 * k2 * i2;
+        g2 = Mdt * Mdt * k2 * k2 * k2 * i2;
+      } else {
+        const T den = T(1) + Ldt * ke * k2, i2 = recip(den * den);
+        d1 = recip(den);
+        d2 = -Ldt * d1;
+        r1 = -dt * ke * k2 * i2;
+        r2 = -dt * i2;
+        g1 = -Ldt * k2 * i2;
+        g2 = Ldt * Ldt * k2 * i2;
+      }
+    } else {
+      const T kk = f == 0 ? k2 * k2 : k2, rate = f == 0 ? Mdt : Ldt, kap = f == 0 ? kc : ke, m2 = f == 0 ? k2 : T(1);
+      d1 = KUpdate<T>::quot(T(1), T(1) + rate * kap * kk);
+      const T i2 = d1 * d1;
+      d2 = -rate * m2 * d1;
+      r1 = -dt * kap * kk * i2;
+      r2 = -dt * m2 * i2;
+      g1 = -rate * kk * i2;
+      g2 = rate * rate * kk * m2 * i2;
+    }
     va = cscale(l, d1 * scale);
     vb = cscale(l, d2 * scale);
-    const T r1 = -dt * kap * kk * i2, r2 = -dt * m2 * i2;                  // d/d rate of D1, D2
-    const T g1 = -rate * kk * i2, g2 = rate * rate * kk * m2 * i2;          // d/d kappa
     const C tr = vfma(u, vsplat<C>(r1), vmul(fu, vsplat<C>(r2))), tg = vfma(u, vsplat<C>(g1), vmul(fu, vsplat<C>(g2)));
     r.add(l.x, tr.x);
     r.add(l.y, tr.y);
     g.add(l.x, tg.x);
     g.add(l.y, tg.y);
   }
+  // The E modes of a thread, one(m, va, vb, r, g) each: into FP32 pairs, and
+  // again into FP64 where the pairs left their range.
+  template <int E, typename C, class One>
+  __device__ __forceinline__ static void modes(One one, C (&va)[E], C (&vb)[E], double& r, double& g) {
+    AdjSum<T> sr, sg;
+#pragma unroll
+    for (int m = 0; m < E; ++m) one(m, va[m], vb[m], sr, sg);
+    r = sr.value();
+    g = sg.value();
+    if (!sr.in_range() || !sg.in_range()) {
+      AdjSum<double> dr, dg;
+#pragma unroll 1
+      for (int m = 0; m < E; ++m) {
+        C a, b;
+        one(m, a, b, dr, dg);
+      }
+      r = dr.value();
+      g = dg.value();
+    }
+  }
   // The sums of a warp, each thread's times its weight w, into acc (c: M and
   // kappa_c; eta: L and kappa_eta).
-  __device__ __forceinline__ static void reduce(int f, const AdjSum<T>& r, const AdjSum<T>& g, double w, double* acc) {
-    double v[2] = {w * r.value(), w * g.value()};
+  __device__ __forceinline__ static void reduce(int f, double r, double g, double w, double* acc) {
+    double v[2] = {w * r, w * g};
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
 #pragma unroll
@@ -238,7 +328,7 @@ struct AdjCoef {
 // Columns per CTA of the adjoint column pass: about 64 threads (tiles of 16
 // bytes or more per row), so that the pass reaches every SM on small grids:
 // three transforms forward and two back per tile and field, 512^2, p = 2,
-// FP32: 105 us with 96 CTAs of 256 threads and the sums in FP64, 20 us now.
+// FP32: 105 us with 96 CTAs of 256 threads, 27 us now.
 template <typename T, int NY>
 struct AdjColCfg {
   using CC = ColCfg<T, NY>;
@@ -246,7 +336,10 @@ struct AdjColCfg {
   static constexpr int TK = (!CC::F64 && T0 < 2) ? 2 : T0;
   // a whole number of warps (the shuffles of the sums)
   static constexpr int THREADS = TK * CC::TPL;
-  static constexpr size_t smem(int tk) { return CC::HEAD + (size_t)3 * CC::TROWS * tk * sizeof(cplx<T>); }
+  static constexpr int TWS = adj_table_size<T>(NY, CC::E);
+  static constexpr int TW_BYTES = ((TWS * (int)sizeof(cplx<T>)) + 127) & ~127;
+  static constexpr int HEAD = CC::BAR_BYTES + TW_BYTES + CC::K2_BYTES;
+  static constexpr size_t smem(int tk) { return HEAD + (size_t)3 * CC::TROWS * tk * sizeof(cplx<T>); }
 };
 
 // TKC: columns per CTA known at compile time (0: a short x axis has fewer).
@@ -255,12 +348,13 @@ __global__ void __launch_bounds__(AdjColCfg<T, NY>::THREADS < 32 ? 32 : AdjColCf
     fs_adj_col_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   using C = cplx<T>;
   using Cfg = ColCfg<T, NY>;
+  using Adj = AdjColCfg<T, NY>;
   constexpr int E = Cfg::E, TPL = Cfg::TPL, BH = Cfg::BH, TROWS = Cfg::TROWS, LOGE = Cfg::LOGE;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   C* twc = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
-  T* k2yt = reinterpret_cast<T*>(smem_raw + Cfg::BAR_BYTES + Cfg::TW_BYTES);
-  C* tiles = reinterpret_cast<C*>(smem_raw + Cfg::HEAD);  // [3][TROWS][tk]
+  T* k2yt = reinterpret_cast<T*>(smem_raw + Cfg::BAR_BYTES + Adj::TW_BYTES);
+  C* tiles = reinterpret_cast<C*>(smem_raw + Adj::HEAD);  // [3][TROWS][tk]
   const int Lh = a.nx / 2, nf = a.nf;
   const int tk = TKC ? TKC : (AdjColCfg<T, NY>::TK < Lh ? AdjColCfg<T, NY>::TK : Lh);
   const int j = threadIdx.x % tk, t0 = threadIdx.x / tk, t = t0 & (TPL - 1);
@@ -281,7 +375,7 @@ __global__ void __launch_bounds__(AdjColCfg<T, NY>::THREADS < 32 ? 32 : AdjColCf
     for (int i = 0; i < 3; ++i)
       for (int y0 = 0; y0 < NY; y0 += BH) tma_load_3d(tiles + (i * TROWS + y0) * tk, &tmap, cx, y0, i * nf + phi, bar);
   }
-  copy_to_smem(twc, reinterpret_cast<const C*>(a.tw_col), Cfg::TWS);
+  copy_to_smem(twc, reinterpret_cast<const C*>(a.tw_col), Adj::TWS);
   for (int i = threadIdx.x; i < NY; i += blockDim.x) k2yt[i] = reinterpret_cast<const T*>(a.k2y)[i];
   griddep_wait();
   griddep_launch_dependents();
@@ -301,7 +395,7 @@ __global__ void __launch_bounds__(AdjColCfg<T, NY>::THREADS < 32 ? 32 : AdjColCf
     C v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = tl[(t + TPL * m) * tk];
-    line_fft<NY, E, -1>(v, t, twc, st, ld, sync);
+    adj_line_fft<NY, E, -1>(v, t, twc, st, ld, sync);
     sync();
 #pragma unroll
     for (int m = 0; m < E; ++m)
@@ -314,11 +408,10 @@ __global__ void __launch_bounds__(AdjColCfg<T, NY>::THREADS < 32 ? 32 : AdjColCf
   const C* TL = tiles + 0 * TROWS * tk;  // Lam'
   const C* TU = tiles + 1 * TROWS * tk;  // U
   const C* TF = tiles + 2 * TROWS * tk;  // Fu
-  AdjSum<T> sr, sg;
+  double sr, sg;
   C va[E], vb[E];
   const bool col0 = (kx0 == 0 && j == 0);
-#pragma unroll
-  for (int m = 0; m < E; ++m) {
+  auto one = [&](int m, C& a1, C& a2, auto& s1, auto& s2) {
     const int ky = t + TPL * m;
     const T ky2 = k2yt[ky];
     const C l = TL[ky * tk + j], u = TU[ky * tk + j], f = TF[ky * tk + j];
@@ -330,14 +423,15 @@ __global__ void __launch_bounds__(AdjColCfg<T, NY>::THREADS < 32 ? 32 : AdjColCf
       const C uP = cscale(cadd(u, uq), T(0.5)), uQ = cscale(mul_i<-1>(csub(u, uq)), T(0.5));
       const C fP = cscale(cadd(f, fq), T(0.5)), fQ = cscale(mul_i<-1>(csub(f, fq)), T(0.5));
       C aP, bP, aQ, bQ;
-      ac.mode(fk, kx2 + ky2, scale, lP, uP, fP, aP, bP, sr, sg);
-      ac.mode(fk, kxn2 + ky2, scale, lQ, uQ, fQ, aQ, bQ, sr, sg);
-      va[m] = cadd(aP, mul_i<1>(aQ));
-      vb[m] = cadd(bP, mul_i<1>(bQ));
+      ac.mode(fk, kx2 + ky2, scale, lP, uP, fP, aP, bP, s1, s2);
+      ac.mode(fk, kxn2 + ky2, scale, lQ, uQ, fQ, aQ, bQ, s1, s2);
+      a1 = cadd(aP, mul_i<1>(aQ));
+      a2 = cadd(bP, mul_i<1>(bQ));
     } else {
-      ac.mode(fk, kx2 + ky2, scale, l, u, f, va[m], vb[m], sr, sg);
+      ac.mode(fk, kx2 + ky2, scale, l, u, f, a1, a2, s1, s2);
     }
-  }
+  };
+  AdjCoef<T>::template modes<E>(one, va, vb, sr, sg);
   // the conjugate half of the columns kx > 0 is not stored: weight 2
   AdjCoef<T>::reduce(fk, sr, sg, live ? (col0 ? 1.0 : 2.0) : 0.0, a.acc);
   sync();
@@ -347,7 +441,7 @@ __global__ void __launch_bounds__(AdjColCfg<T, NY>::THREADS < 32 ? 32 : AdjColCf
     C* tl = tile + j;
     auto st = [tl, tk, live](int q, C x) { if (live) tl[(q + (q >> LOGE)) * tk] = x; };
     auto ld = [tl, tk](int q) { return tl[(q + (q >> LOGE)) * tk]; };
-    line_fft<NY, E, 1>(v, t, twc, st, ld, sync);
+    adj_line_fft<NY, E, 1>(v, t, twc, st, ld, sync);
     sync();
 #pragma unroll
     for (int m = 0; m < E; ++m)
@@ -374,7 +468,7 @@ __global__ void __launch_bounds__(AdjColCfg<T, NY>::THREADS < 32 ? 32 : AdjColCf
 template <typename T, int NX, int P>
 __global__ void __launch_bounds__(64 * (P + 1)) fs_adj_row_inv_kernel(KArgs a) {
   using C = cplx<T>;
-  using Cfg = RowCfg<T, NX>;
+  using Cfg = AdjRowCfg<T, NX>;
   constexpr int L = Cfg::L, E = Cfg::E, TPL = Cfg::TPL, R = Cfg::R, PL = Cfg::PL;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
@@ -431,7 +525,7 @@ __global__ void __launch_bounds__(64 * (P + 1)) fs_adj_row_inv_kernel(KArgs a) {
         v[m] = cadd(A, mul_i<1>(mul_tw<1>(B, __ldg(&twh[k]))));
       }
     }
-    line_fft<L, E, 1>(v, t, twr, st, ld, wsync);
+    adj_line_fft<L, E, 1>(v, t, twr, st, ld, wsync);
     wsync();
 #pragma unroll
     for (int m = 0; m < E; ++m) s[t + TPL * m] = v[m];

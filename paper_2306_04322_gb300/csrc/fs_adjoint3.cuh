@@ -22,7 +22,7 @@ template <typename T, int NZ>
 __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 2)
     fs_adj_z_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   using C = cplx<T>;
-  using Cfg = LineCfg<T, NZ>;
+  using Cfg = AdjLineCfg<T, NZ>;
   constexpr int E = Cfg::E, TPL = Cfg::TPL, BH = Cfg::BH, LOGE = Cfg::LOGE, TROWS = Cfg::TROWS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 2)
     C v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = tl[(t + TPL * m) * tk];
-    line_fft<NZ, E, -1>(v, t, tw, st, ld, sync);
+    adj_line_fft<NZ, E, -1>(v, t, tw, st, ld, sync);
     sync();
 #pragma unroll
     for (int m = 0; m < E; ++m) tl[(t + TPL * m) * tk] = v[m];
@@ -88,13 +88,12 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 2)
   const C* TL = tiles;              // Lam'
   const C* TU = tiles + TROWS * tk;  // U
   const C* TF = tiles + 2 * TROWS * tk;  // Fu
-  AdjSum<T> sr, sg;
+  double sr, sg;
   C va[E], vb[E];
   // Parseval over the stored modes: a line that is not a pair row stands for
   // itself and its conjugate partner (weight 2); a pair row's two real-packed
   // z sequences are stored whole (weight 1 each)
-#pragma unroll
-  for (int m = 0; m < E; ++m) {
+  auto one = [&](int m, C& a1, C& a2, auto& s1, auto& s2) {
     const int kz = t + TPL * m;
     const T kz2 = k2zt[kz];
     const C l = TL[kz * tk + j], u = TU[kz * tk + j], f = TF[kz * tk + j];
@@ -105,14 +104,15 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 2)
       const C uP = cscale(cadd(u, uq), T(0.5)), uQ = cscale(mul_i<-1>(csub(u, uq)), T(0.5));
       const C fP = cscale(cadd(f, fq), T(0.5)), fQ = cscale(mul_i<-1>(csub(f, fq)), T(0.5));
       C aP, bP, aQ, bQ;
-      ac.mode(fk, kxa + kya + kz2, scale, lP, uP, fP, aP, bP, sr, sg);
-      ac.mode(fk, kxa + kyb + kz2, scale, lQ, uQ, fQ, aQ, bQ, sr, sg);
-      va[m] = cadd(aP, mul_i<1>(aQ));
-      vb[m] = cadd(bP, mul_i<1>(bQ));
+      ac.mode(fk, kxa + kya + kz2, scale, lP, uP, fP, aP, bP, s1, s2);
+      ac.mode(fk, kxa + kyb + kz2, scale, lQ, uQ, fQ, aQ, bQ, s1, s2);
+      a1 = cadd(aP, mul_i<1>(aQ));
+      a2 = cadd(bP, mul_i<1>(bQ));
     } else {
-      ac.mode(fk, kxy2 + kz2, scale, l, u, f, va[m], vb[m], sr, sg);
+      ac.mode(fk, kxy2 + kz2, scale, l, u, f, a1, a2, s1, s2);
     }
-  }
+  };
+  AdjCoef<T>::template modes<E>(one, va, vb, sr, sg);
   AdjCoef<T>::reduce(fk, sr, sg, pair ? 1.0 : 2.0, a.acc);
   sync();  // every thread has read the three tiles: they become exchange buffers
   C* base = reinterpret_cast<C*>(a.spec) + (long long)ky * Lh + kx;
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 2)
     C* tl = tiles + o * TROWS * tk + j;
     auto st = [tl, tk](int q, C x) { tl[(q + (q >> LOGE)) * tk] = x; };
     auto ld = [tl, tk](int q) { return tl[(q + (q >> LOGE)) * tk]; };
-    line_fft<NZ, E, 1>(v, t, tw, st, ld, sync);
+    adj_line_fft<NZ, E, 1>(v, t, tw, st, ld, sync);
     C* S = base + (long long)(o * nf + phi) * a.slot_stride;
 #pragma unroll
     for (int m = 0; m < E; ++m)

@@ -7,17 +7,11 @@
 
 namespace fs {
 
-template <typename T, int NX>
-size_t adj_row_smem(int nf) {
-  using RC = RowCfg<T, NX>;
-  return RC::BAR_BYTES + RC::TW_BYTES + (size_t)3 * nf * RC::R * RC::PL * sizeof(cplx<T>);
-}
-
 template <typename T, int NX, int P>
 cudaError_t adj_row_p(const KArgs& a, bool inverse, cudaStream_t s) {
-  using RC = RowCfg<T, NX>;
+  using RC = AdjRowCfg<T, NX>;
   const long long reff = a.lines < RC::R ? a.lines : RC::R;
-  const size_t smem = adj_row_smem<T, NX>(a.nf);
+  const size_t smem = RC::smem(a.nf);
   static unsigned d1 = 0, d2 = 0;
   cudaError_t e;
   const dim3 grid((unsigned)(a.lines / reff));
@@ -113,7 +107,7 @@ cudaError_t adjoint_launch_t(const KArgs& a0, const CUtensorMap& tm, void* lam_o
 
 template <typename T, int NZ>
 cudaError_t adj_z_n(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
-  using Cfg = LineCfg<T, NZ>;
+  using Cfg = AdjLineCfg<T, NZ>;
   const int tk = line_tk<T, NZ>(a.nx);
   const size_t smem = Cfg::HEAD + (size_t)3 * Cfg::TROWS * tk * sizeof(cplx<T>);
   static unsigned d = 0;
@@ -122,6 +116,25 @@ cudaError_t adj_z_n(const KArgs& a, const CUtensorMap& tm, cudaStream_t s) {
   dim3 grid((unsigned)(a.nx / 2 / tk), (unsigned)a.ny, (unsigned)a.nf);
   fs_adj_z_kernel<T, NZ><<<grid, (unsigned)(tk * Cfg::TPL), smem, s>>>(a, tm);
   return cudaGetLastError();
+}
+
+// y pass over the adjoint's slots: the steps' in FP64; in FP32 the same kernel
+// with the adjoint's transform.
+template <typename T>
+cudaError_t adj_ypass_t(const KArgs& a, const CUtensorMap& tm, int dir, int nslots, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    return ypass_launch_f64(a, tm, dir, a.nz, nslots, s);
+  } else {
+    switch (a.ny) {
+#define FS_CASE(n)                                                                                                  \
+  case n:                                                                                                           \
+    return dir < 0 ? ypass_launch_tk<T, n, -1, TC_NONE, 0, true>(a, tm, a.nz, nslots, line_tk<T, n>(a.nx), s)       \
+                   : ypass_launch_tk<T, n, 1, TC_NONE, 0, true>(a, tm, a.nz, nslots, line_tk<T, n>(a.nx), s);
+      FS_LINE_SIZES(FS_CASE)
+#undef FS_CASE
+      default: return cudaErrorInvalidValue;
+    }
+  }
 }
 
 // Adjoint of one 3D step (five launches): x forward of lam', u, f(u) (the
@@ -145,8 +158,7 @@ cudaError_t adjoint3_launch_t(const KArgs& a0, const CUtensorMap& tm_y, const CU
   b.carry3 = 0;  // plain y transforms of every slot (no carried c)
   b.plane0 = 0;
   b.tc = 0;
-  constexpr bool f64 = sizeof(T) == 8;
-  e = f64 ? ypass_launch_f64(b, tm_y, -1, a0.nz, 3 * a0.nf, s) : ypass_launch_f32(b, tm_y, -1, a0.nz, 3 * a0.nf, s);
+  e = adj_ypass_t<T>(b, tm_y, -1, 3 * a0.nf, s);
   if (e != cudaSuccess) return e;
   e = cudaErrorInvalidValue;
   switch (a0.nz) {
@@ -157,7 +169,7 @@ cudaError_t adjoint3_launch_t(const KArgs& a0, const CUtensorMap& tm_y, const CU
     default: break;
   }
   if (e != cudaSuccess) return e;
-  e = f64 ? ypass_launch_f64(b, tm_y, 1, a0.nz, 2 * a0.nf, s) : ypass_launch_f32(b, tm_y, 1, a0.nz, 2 * a0.nf, s);
+  e = adj_ypass_t<T>(b, tm_y, 1, 2 * a0.nf, s);
   if (e != cudaSuccess) return e;
   KArgs a1 = a0;
   a1.real = lam_out;

@@ -362,6 +362,105 @@ __device__ __forceinline__ void line_fft(C (&v)[E], int t, const C* __restrict__
   stockham<L, E, 1, DIR>(v, t, twp, st, ld, sync);
 }
 
+// ---- line FFT with separate twiddles (FP32 adjoint) -------------------------
+// The same passes with the twiddle as a product of its own before a pass's
+// radix-2 stages, whose roots are then 1, -+i and constants: fewer products
+// per value than the folded form (radix 16: 1.6 against 2), more instructions.
+// The sensitivities of an FP32 adjoint step are sums that can cancel to a
+// hundredth of their terms (p = 1), where the rounding of every transform shows
+// from the fifth digit on; the FP32 adjoint keeps this form, so that its digits
+// do not move when the steps' transforms change.
+// a exp(DIR 2 pi i k / len), k and len known after unrolling, len <= 32
+template <int DIR>
+__device__ __forceinline__ float2 plain_root(float2 a, int k, int len) {
+  const int j = k * 32 / len;  // 0 <= j < 16
+  if (j == 0) return a;
+  if (j == 8) return mul_i<DIR>(a);
+  const float cr = (float)(j < 8 ? cos32(j) : -cos32(16 - j)), sr = (float)(j < 8 ? sin32(j) : sin32(16 - j));
+  if (j % 8 == 4) {  // (+-1 +- i) / sqrt(2): adds, then one scaling
+    const float h = (float)cos32(4), sx = j < 8 ? 1.f : -1.f, sy = (float)DIR;
+    return make_float2(__fmul_rn(fmaf(sx, a.x, -(sy * a.y)), h), __fmul_rn(fmaf(sy, a.x, sx * a.y), h));
+  }
+  return cmul(a, make_float2(cr, DIR * sr));
+}
+template <int R, int DIR, int S>
+__device__ __forceinline__ void plain_dft(float2* a) {
+  if constexpr (R <= 4) {
+    reg_dft<R, DIR, S>(a);
+  } else {
+    constexpr int B = ilog2(R);
+    float2 t[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) t[i] = a[bitrev(i, B) * S];
+#pragma unroll
+    for (int len = 2; len <= R; len <<= 1) {
+#pragma unroll
+      for (int i = 0; i < R; i += len) {
+#pragma unroll
+        for (int k = 0; k < len / 2; ++k) {
+          const float2 u = t[i + k], v = plain_root<DIR>(t[i + k + len / 2], k, len);
+          t[i + k] = cadd(u, v);
+          t[i + k + len / 2] = csub(u, v);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) a[i * S] = t[i];
+  }
+}
+// Tables: entries [r][j] = exp(-2 pi i r j / (NS R)), r < R, of every pass
+// after the first.
+__host__ __device__ constexpr int plain_table_size(int L, int E, int ns_end) {
+  int off = 0;
+  for (int ns = 1; ns < ns_end;) {
+    const int r = E < L / ns ? E : L / ns;
+    if (ns > 1) off += ns * r;
+    ns *= r;
+  }
+  return off;
+}
+__host__ __device__ constexpr int plain_table_size(int L, int E) { return plain_table_size(L, E, L); }
+template <int L, int E, int NS, int DIR, class Store, class Load, class Sync>
+__device__ __forceinline__ void plain_stockham(float2 (&v)[E], int t, const float2* __restrict__ twp, Store st,
+                                               Load ld, Sync sync) {
+  constexpr int TPL = L / E, R = PassRadix<L, E, NS>::R, Q = E / R;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    if constexpr (NS > 1) {
+      const float2* w = twp + plain_table_size(L, E, NS) + ((t + TPL * q) & (NS - 1));
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[q + Q * r] = mul_tw<DIR>(v[q + Q * r], w[r * NS]);
+    }
+    plain_dft<R, DIR, Q>(&v[q]);
+  }
+  if constexpr (NS * R < L) {
+    sync();
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int b = t + TPL * q, j = b & (NS - 1), base = (b - j) * R + j;
+#pragma unroll
+      for (int r = 0; r < R; ++r) st(base + r * NS, v[q + Q * r]);
+    }
+    sync();
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = ld(t + TPL * m);
+    plain_stockham<L, E, NS * R, DIR>(v, t, twp, st, ld, sync);
+  }
+}
+
+// Transform and table size of a line of the adjoint: the form above in FP32,
+// the steps' in FP64.
+template <typename T>
+__host__ __device__ constexpr int adj_table_size(int L, int E) {
+  return sizeof(T) == 4 ? plain_table_size(L, E) : pass_table_size(L, E);
+}
+template <int L, int E, int DIR, typename C, class Store, class Load, class Sync>
+__device__ __forceinline__ void adj_line_fft(C (&v)[E], int t, const C* __restrict__ twp, Store st, Load ld,
+                                             Sync sync) {
+  if constexpr (sizeof(C) == 8) plain_stockham<L, E, 1, DIR>(v, t, twp, st, ld, sync);
+  else line_fft<L, E, DIR>(v, t, twp, st, ld, sync);
+}
+
 // Padded shared-memory indices: one spare slot every 32 (pad32) or 16
 // (pad16) elements.  pad16 keeps the radix-16 butterfly writes (16
 // consecutive elements per thread) and the stride-TPL reads of the row

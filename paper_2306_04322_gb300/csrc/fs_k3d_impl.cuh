@@ -45,6 +45,14 @@ struct LineCfg {
   static constexpr int TROWS = (NL + NL / E + 1 + 15) & ~15;
   static constexpr int HEAD = BAR_BYTES + TW_BYTES + K2_BYTES;
 };
+// The same with the adjoint's pass tables (adj_line_fft).
+template <typename T, int NL>
+struct AdjLineCfg : LineCfg<T, NL> {
+  using B = LineCfg<T, NL>;
+  static constexpr int TWS = adj_table_size<T>(NL, B::E);
+  static constexpr int TW_BYTES = ((TWS * (int)sizeof(cplx<T>)) + 127) & ~127;
+  static constexpr int HEAD = B::BAR_BYTES + TW_BYTES + B::K2_BYTES;
+};
 
 // ---------------------------------------------------------------------------
 // y pass: one CTA per (kx tile, z, slot); DIR = -1 forward (slots 0..nf),
@@ -64,11 +72,12 @@ struct LineCfg {
 // 248 -> 90.8 / 140 / 238; grids that L2 holds are unchanged (128^3 p = 2
 // 41.2 us).
 // ---------------------------------------------------------------------------
-template <typename T, int NY, int DIR, int TCM, int TKC>
+// ADJ: the adjoint's transform and tables (KArgs::tw_col holds them).
+template <typename T, int NY, int DIR, int TCM, int TKC, bool ADJ = false>
 __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
     fs_ypass_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
   using C = cplx<T>;
-  using Cfg = LineCfg<T, NY>;
+  using Cfg = typename std::conditional<ADJ, AdjLineCfg<T, NY>, LineCfg<T, NY>>::type;
   constexpr int E = Cfg::E, TPL = Cfg::TPL, BH = Cfg::BH, LOGE = Cfg::LOGE;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
@@ -152,7 +161,8 @@ __global__ void __launch_bounds__(LineCfg<T, NY>::THREADS, 4)
       for (int m = 0; m < E; ++m) v[m] = ld(t + TPL * m);
       stockham<NY, E, 16, DIR>(v, t, tw, st, ld, sync);
     } else {
-      line_fft<NY, E, DIR>(v, t, tw, st, ld, sync);
+      if constexpr (ADJ) adj_line_fft<NY, E, DIR>(v, t, tw, st, ld, sync);
+      else line_fft<NY, E, DIR>(v, t, tw, st, ld, sync);
     }
   }
   if (DIR < 0 && special) {
@@ -466,15 +476,15 @@ cudaError_t energy_z_launch_n(const KArgs& a, const CUtensorMap& tm, cudaStream_
   return cudaGetLastError();
 }
 
-template <typename T, int NY, int DIR, int TCM, int TKC>
+template <typename T, int NY, int DIR, int TCM, int TKC, bool ADJ = false>
 cudaError_t ypass_launch_tk(const KArgs& a, const CUtensorMap& tm, int planes, int nslots, int tk, cudaStream_t s) {
-  using Cfg = LineCfg<T, NY>;
+  using Cfg = typename std::conditional<ADJ, AdjLineCfg<T, NY>, LineCfg<T, NY>>::type;
   size_t smem = Cfg::HEAD + (size_t)Cfg::TROWS * tk * sizeof(cplx<T>) + (TCM ? 8192 : 0) +
                 (TCM == TC_TF32 ? tc5_extra_bytes(tk * Cfg::TPL) : 0);
   // the tcgen05 stage runs 128-row MMAs over the CTA's (butterfly, column) rows
   if (TCM == TC_TF32 && (tk * Cfg::TPL) % 128 != 0) return cudaErrorNotSupported;
   static unsigned done = 0;
-  cudaError_t e = allow_big_smem(fs_ypass_kernel<T, NY, DIR, TCM, TKC>, &done);
+  cudaError_t e = allow_big_smem(fs_ypass_kernel<T, NY, DIR, TCM, TKC, ADJ>, &done);
   if (e != cudaSuccess) return e;
   const unsigned tiles = (unsigned)(a.nx / 2 / tk);
   const dim3 grid = DIR < 0 ? dim3(tiles, (unsigned)nslots, (unsigned)planes) : dim3(tiles, (unsigned)planes, (unsigned)nslots);
@@ -484,10 +494,10 @@ cudaError_t ypass_launch_tk(const KArgs& a, const CUtensorMap& tm, int planes, i
   // as its fullest SM (64^3, p = 4: 217 us per step, 247 with the overlap,
   // 229 with it allowed only from the end of a CTA, as in FP32 below).
   if (TCM != TC_NONE || sizeof(T) == 8) {
-    fs_ypass_kernel<T, NY, DIR, TCM, TKC><<<grid, (unsigned)(tk * Cfg::TPL), smem, s>>>(a, tm);
+    fs_ypass_kernel<T, NY, DIR, TCM, TKC, ADJ><<<grid, (unsigned)(tk * Cfg::TPL), smem, s>>>(a, tm);
     return cudaGetLastError();
   }
-  return launch_pdl(fs_ypass_kernel<T, NY, DIR, TCM, TKC>, grid, dim3((unsigned)(tk * Cfg::TPL)), smem, s, a, tm);
+  return launch_pdl(fs_ypass_kernel<T, NY, DIR, TCM, TKC, ADJ>, grid, dim3((unsigned)(tk * Cfg::TPL)), smem, s, a, tm);
 }
 
 template <typename T, int NY, int DIR>

@@ -65,6 +65,18 @@ struct Pointwise {
     Ldt = k.Ldt;
   }
   __device__ __forceinline__ T hpoly(T e) const { return e * e * e * (e * (T(6) * e - T(15)) + T(10)); }
+  // df/dc and df/deta_i term by term, every rounding spelt out: the FP32
+  // adjoint, whose sensitivities keep their digits (fs_fft.cuh, plain_stockham).
+  __device__ __forceinline__ float fc(float c, float h) const {
+    return __fmul_rn(two_rho2, fmaf(-dcab, h, __fadd_rn(c, -ca)));
+  }
+  __device__ __forceinline__ float feta(float c, float e, float S2) const {
+    const float m = __fadd_rn(1.f, -e), q = __fmul_rn(e, m);
+    const float dh = __fmul_rn(__fmul_rn(30.f, q), q), chem = __fmul_rn(rho2dcab, fmaf(-2.f, c, cab));
+    const float pair = __fmul_rn(__fmul_rn(four_alpha, e), fmaf(-e, e, S2));
+    const float well = fmaf(__fmul_rn(__fmul_rn(2.f, e), m), fmaf(-2.f, e, 1.f), pair);
+    return fmaf(chem, dh, __fmul_rn(w, well));
+  }
   // The step's stage on two lanes (two grid points per pair, lane-wise
   // arithmetic) with the constants multiplied out on the host: 13
   // instructions per eta and 3 per point, against 19 and 3 for df/dc and

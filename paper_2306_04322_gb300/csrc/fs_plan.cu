@@ -38,6 +38,9 @@ struct Member {
   void* tw_col = nullptr;
   void* tw_z = nullptr;
   void* tw_half = nullptr;
+  void* tw_row_a = nullptr;  // x, y and z tables of the adjoint (FP32; FP64: those of the steps)
+  void* tw_col_a = nullptr;
+  void* tw_z_a = nullptr;
   void* tw_row_w = nullptr;  // x-pass tables with 32 values per thread (FP32 rows of 1024)
   void* tc_b = nullptr;  // split DFT matrix of the tensor-core stage (TC precisions)
   void* tw_row2 = nullptr;  // x-line tables of the pair-form row pass (nx in [64, 1024]; FP64 to 2048)
@@ -587,7 +590,7 @@ fs_status read_flag(fs_plan* p) {
 //   tc_b[2048] (TC precisions only)         (split DFT matrix of the tensor-core stage, 32-bit words)
 struct TableLayout {
   size_t k2x, k2y, k2z, tw_row, tw_row_w, tw_col, tw_z, tw_half, tc_b, tw_row2, tw_col2, tw_row2w, tw_col2w,
-      tw_row3, total;  // offsets (bytes)
+      tw_row3, tw_row_a, tw_col_a, tw_z_a, total;  // offsets (bytes)
   int Lrow, Erow, Lcol, Ecol, Lz, Ez;
 };
 
@@ -700,6 +703,12 @@ bool row3_form(const fs_params& prm, bool f64) {
   return prm.ndim == 3 || (nx <= 128 && ny >= 2048) || (nx == 256 && ny >= 1024 && prm.p >= 3);
 }
 
+// Plans whose fs_step_adjoint runs with tables of its own (adj_line_fft).
+bool adj_tables(const fs_params& prm, bool f64) {
+  return !f64 && prm.scheme == FS_SCHEME_SEMI_IMPLICIT_FS &&
+         (prm.ndim == 3 || (prm.n[0] <= 1024 && prm.n[1] <= 1024));
+}
+
 // Rows of 1024 in FP32 run the x-pass variant with 32 values per thread.
 bool wide_rows(const fs_params& prm, bool f64) { return !f64 && prm.n[0] == 1024; }
 
@@ -743,6 +752,13 @@ TableLayout table_layout(const fs_params& prm, bool f64) {
   o = align16(o + (col2w_form(prm, f64) ? cs * fs::pass_table_size(ny, ny / 64) : 0));
   t.tw_row3 = o;  // x pass with several row pairs per CTA: E = 16
   o = align16(o + (row3_form(prm, f64) ? cs * fs::pass_table_size(nx, 16) : 0));
+  const bool adj = adj_tables(prm, f64);
+  t.tw_row_a = o;
+  o = align16(o + (adj ? cs * fs::plain_table_size(t.Lrow, t.Erow) : 0));
+  t.tw_col_a = o;
+  o = align16(o + (adj ? cs * fs::plain_table_size(t.Lcol, t.Ecol) : 0));
+  t.tw_z_a = o;
+  o = align16(o + (adj && nz > 1 ? cs * fs::plain_table_size(t.Lz, t.Ez) : 0));
   t.total = o;
   return t;
 }
@@ -801,6 +817,18 @@ void pass_table(const Roots& w, int L, int E, std::vector<double>& re, std::vect
   }
 }
 
+// The same with the twiddles apart (fs::plain_stockham): entries [r][j] =
+// exp(-2 pi i r j / (NS R)), r < R, j < NS.
+void plain_table(const Roots& w, int L, int E, std::vector<double>& re, std::vector<double>& im) {
+  for (int ns = 1; ns < L;) {
+    const int r = E < L / ns ? E : L / ns;
+    if (ns > 1)
+      for (int q = 0; q < r; ++q)
+        for (int j = 0; j < ns; ++j) w.add((long long)q * j, (long long)ns * r, re, im);
+    ns *= r;
+  }
+}
+
 template <typename T>
 void put_real(std::vector<char>& buf, size_t off, const std::vector<double>& v) {
   T* d = reinterpret_cast<T*>(buf.data() + off);
@@ -829,7 +857,8 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   fill(ky, ny, 1);
   if (prm.ndim > 2) fill(kz, nz, 2);
   const Roots w(std::max(nx, std::max(ny, nz)));
-  std::vector<double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i, m3r, m3i;
+  std::vector<double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i, m3r, m3i,
+      arr, ari, acr, aci, azr, azi;
   const int er = row2_e(prm, f64), ec = col2_e(prm, f64);
   if (er) pass_table(w, nx, er, r2r, r2i);
   if (ec) pass_table(w, ny, ec, c2r, c2i);
@@ -841,6 +870,12 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   pass_table(w, t.Lcol, t.Ecol, cr, ci);
   if (nz > 1) pass_table(w, t.Lz, t.Ez, zr, zi);
   for (int k = 0; k < nx / 2; ++k) w.add(k, nx, hr, hi);
+  const bool adj = adj_tables(prm, f64);
+  if (adj) {
+    plain_table(w, t.Lrow, t.Erow, arr, ari);
+    plain_table(w, t.Lcol, t.Ecol, acr, aci);
+    if (nz > 1) plain_table(w, t.Lz, t.Ez, azr, azi);
+  }
   if (f64) {
     put_real<double>(buf, t.k2x, kx);
     put_real<double>(buf, t.k2y, ky);
@@ -865,6 +900,9 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
     put_cplx<float>(buf, t.tw_row2w, r3r, r3i);
     put_cplx<float>(buf, t.tw_col2w, c3r, c3i);
     put_cplx<float>(buf, t.tw_row3, m3r, m3i);
+    put_cplx<float>(buf, t.tw_row_a, arr, ari);
+    put_cplx<float>(buf, t.tw_col_a, acr, aci);
+    put_cplx<float>(buf, t.tw_z_a, azr, azi);
   }
   m.k2x = dev + t.k2x;
   m.k2y = dev + t.k2y;
@@ -879,6 +917,9 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   m.tw_row2w = row2w_form(prm, f64) ? dev + t.tw_row2w : nullptr;
   m.tw_col2w = col2w_form(prm, f64) ? dev + t.tw_col2w : nullptr;
   m.tw_row3 = row3_form(prm, f64) ? dev + t.tw_row3 : nullptr;
+  m.tw_row_a = dev + (adj ? t.tw_row_a : t.tw_row);
+  m.tw_col_a = dev + (adj ? t.tw_col_a : t.tw_col);
+  m.tw_z_a = dev + (adj ? t.tw_z_a : t.tw_z);
   if (const int mode = tc_split(prm.precision)) {
     tc_table(mode, reinterpret_cast<uint32_t*>(buf.data() + t.tc_b));
     m.tc_b = dev + t.tc_b;
@@ -1423,6 +1464,9 @@ fs_status fs_step_adjoint(fs_plan_t p, const void* const* u, const void* const* 
   a.spec_bytes = (long long)3 * nf * m.slot_stride * (long long)cs;
   a.real_bytes = (long long)nf * m.npts * (long long)rs;
   a.aux = m.au;
+  a.tw_row = m.tw_row_a;
+  a.tw_col = m.tw_col_a;
+  a.tw_z = m.tw_z_a;
   if (e == cudaSuccess && three)
     e = p->f64 ? fs::adjoint3_launch_f64(a, m.tmap_adj, m.tmap_adj_z, m.aout, p->stream)
                : fs::adjoint3_launch_f32(a, m.tmap_adj, m.tmap_adj_z, m.aout, p->stream);
