@@ -116,9 +116,9 @@ __global__ void __launch_bounds__(FdTile<T>::THREADS) fs_fd_kernel(KArgs a, cons
   };
   const T* m = &mu[(ty + 1) * W + lx];
   const C mv = pairp(m), c = pairp(at(0, ly, lx));
-  C d = vmul(mv, vsplat<C>(k.dc_c));
-  d = vfma(xsum(m[-1], mv, m[2]), vsplat<C>(k.dc_d[0]), d);
-  d = vfma(cadd(pairp(m - W), pairp(m + W)), vsplat<C>(k.dc_d[1]), d);
+  const C m2 = vsplat<C>(T(-2));
+  C d = vmul(vfma(mv, m2, xsum(m[-1], mv, m[2])), vsplat<C>(k.dc_d[0]));
+  d = vfma(vfma(mv, m2, cadd(pairp(m - W), pairp(m + W))), vsplat<C>(k.dc_d[1]), d);
   const C cn = cadd(c, d);
   FiniteCheck<T> chk;
   chk.add(cn);
@@ -176,8 +176,9 @@ struct Vec3 {
     memcpy(&w, v, 16);
     *reinterpret_cast<int4*>(p) = w;
   }
-  // acc + sum_d w_d (sum of the two neighbours along d) of field f, whose
-  // values at the vector are v
+  // acc + sum_d w_d (sum of the two neighbours along d, DIFF: less twice the
+  // value) of field f, whose values at the vector are v
+  template <bool DIFF>
   __device__ __forceinline__ void neighbours(const T* f, const C (&v)[NC], const T (&w)[3],
                                              C (&acc)[NC]) const {
     C a0[NC], a1[NC], b0[NC], b1[NC];
@@ -188,10 +189,13 @@ struct Vec3 {
     const T l = f[xm], r = f[xp];
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
-      const C xs = xsum(q == 0 ? l : v[q - 1].y, v[q], q == NC - 1 ? r : v[q + 1].x);
-      acc[q] = vfma(xs, vsplat<C>(w[0]), acc[q]);
-      acc[q] = vfma(cadd(a0[q], a1[q]), vsplat<C>(w[1]), acc[q]);
-      acc[q] = vfma(cadd(b0[q], b1[q]), vsplat<C>(w[2]), acc[q]);
+      C s[3] = {xsum(q == 0 ? l : v[q - 1].y, v[q], q == NC - 1 ? r : v[q + 1].x), cadd(a0[q], a1[q]),
+                cadd(b0[q], b1[q])};
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        if (DIFF) s[d] = vfma(v[q], vsplat<C>(T(-2)), s[d]);
+        acc[q] = vfma(s[d], vsplat<C>(w[d]), acc[q]);
+      }
     }
   }
 };
@@ -226,7 +230,7 @@ __global__ void __launch_bounds__(256) fs_fd3_mu_eta_kernel(KArgs a, const T* in
     m[q] = vfma(c[q], vsplat<C>(k.mu_c), vfma(h, vsplat<C>(k.fc_h), vsplat<C>(k.fc_0)));
     chem[q] = vfma(c[q], vsplat<C>(k.g_c), vsplat<C>(k.g_0));
   }
-  g.neighbours(in, c, k.mu_d, m);
+  g.template neighbours<false>(in, c, k.mu_d, m);
   V3::store(mu + g.c, m);
   FiniteCheck<T> chk;
 #pragma unroll
@@ -234,7 +238,7 @@ __global__ void __launch_bounds__(256) fs_fd3_mu_eta_kernel(KArgs a, const T* in
     C r[NC];
 #pragma unroll
     for (int q = 0; q < NC; ++q) r[q] = eta_rate(k, chem[q], e[f][q], S2[q]);
-    g.neighbours(in + f * N, e[f], k.de_d, r);
+    g.template neighbours<false>(in + f * N, e[f], k.de_d, r);
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       r[q] = cadd(e[f][q], r[q]);
@@ -261,8 +265,8 @@ __global__ void __launch_bounds__(256) fs_fd3_c_kernel(KArgs a, const T* in, T* 
   V3::load(in + g.c, c);
   V3::load(mu + g.c, m);
 #pragma unroll
-  for (int q = 0; q < NC; ++q) d[q] = vmul(m[q], vsplat<C>(k.dc_c));
-  g.neighbours(mu, m, k.dc_d, d);
+  for (int q = 0; q < NC; ++q) d[q] = vsplat<C>(T(0));
+  g.template neighbours<true>(mu, m, k.dc_d, d);
   FiniteCheck<T> chk;
 #pragma unroll
   for (int q = 0; q < NC; ++q) {
