@@ -10,12 +10,12 @@
 // plus a one-point halo in shared memory, then updates its interior.  In 3D
 // two kernels: mu and the eta_i, then c.
 //
-// Both use the weights of fill_fd (stencil and pointwise constants multiplied
-// out): about 18 operations per eta and point in 2D where the stages term by
-// term take 30, which is the time of the FP64 kernels (512 x 256, p = 4: 32.6
-// us per step against 48.8); every thread takes adjacent points along x, so
+// Both use the constants of fill_pointwise and fill_fd (multiplied out): about
+// 21 operations per eta and point in 2D where the stages term by term take 30,
+// which is the time of the FP64 kernels (512 x 256, p = 4: 35.3 us per step
+// against 48.8); every thread takes adjacent points along x, so
 // that loads, index arithmetic and the FP32 arithmetic (packed two-lane
-// instructions) serve two points or more (3D 128^3, p = 4, FP32: 24 us per
+// instructions) serve two points or more (3D 128^3, p = 4, FP32: 24.8 us per
 // step against 70; one thread per point and 64-bit neighbour indices had made
 // it 530 instructions per point).
 #include "fs_k2d_impl.cuh"
@@ -36,15 +36,14 @@ __device__ __forceinline__ C xsum(T l, C v, T r) {
   return mk<C>(l + v.y, v.x + r);
 }
 
-// eta' - eta of a pair but for the neighbour terms (S2 = sum_j eta_j^2):
-//   -dt L df/deta_i + de_c eta_i   (see Pointwise::g2)
-template <typename C, typename T>
+// -dt L df/deta_i of a pair (S2 = sum_j eta_j^2; see Pointwise::g2), NF fields.
+template <int NF, typename C, typename T>
 __device__ __forceinline__ C eta_rate(const Coef<T>& k, C chem, C e, C S2) {
   const C ne = mk<C>(-e.x, -e.y);
   const C q = vfma(e, ne, e);
   const C in = vfma(chem, q, vfma(e, vsplat<C>(T(-2) * k.g_dw), vsplat<C>(k.g_dw)));
-  const C pair = vfma(vsplat<C>(k.g_pair), vfma(e, ne, S2), vsplat<C>(k.de_c));
-  return vfma(q, in, vmul(e, pair));
+  if (NF == 2) return vmul(q, in);  // one eta: the sum over the others is empty
+  return vfma(q, in, vmul(vmul(e, vsplat<C>(k.g_pair)), vfma(e, ne, S2)));
 }
 
 // 2D tile: TX x TY points, one pair of x neighbours per thread.  FP32 64 x 8;
@@ -90,6 +89,7 @@ __global__ void __launch_bounds__(FdTile<T>::THREADS) fs_fd_kernel(KArgs a, cons
   const Pointwise<T> pw(a);
   auto at = [tile](int f, int ly, int lx) { return &tile[(f * H + ly) * W + lx]; };
   auto pairp = [](const T* p) { return *reinterpret_cast<const C*>(p); };
+  const C m2 = vsplat<C>(T(-2));
   // (i) mu on the tile plus a one-point halo
   for (int i = tid; i < HW * MH; i += Cfg::THREADS) {
     const int lx = 2 * (i % HW), my = i / HW;
@@ -98,9 +98,8 @@ __global__ void __launch_bounds__(FdTile<T>::THREADS) fs_fd_kernel(KArgs a, cons
     C h = vsplat<C>(T(0));
 #pragma unroll
     for (int f = 1; f < NF; ++f) h = pw.add_h2(pairp(at(f, my + 1, lx)), h);
-    C m = vfma(v, vsplat<C>(k.mu_c), vfma(h, vsplat<C>(k.fc_h), vsplat<C>(k.fc_0)));
-    m = vfma(xsum(c[-1], v, c[2]), vsplat<C>(k.mu_d[0]), m);
-    m = vfma(cadd(pairp(c - W), pairp(c + W)), vsplat<C>(k.mu_d[1]), m);
+    C m = vfma(vfma(v, m2, xsum(c[-1], v, c[2])), vsplat<C>(k.mu_d[0]), pw.fc2(v, h));
+    m = vfma(vfma(v, m2, cadd(pairp(c - W), pairp(c + W))), vsplat<C>(k.mu_d[1]), m);
     *reinterpret_cast<C*>(&mu[my * W + lx]) = m;
   }
   __syncthreads();
@@ -116,7 +115,6 @@ __global__ void __launch_bounds__(FdTile<T>::THREADS) fs_fd_kernel(KArgs a, cons
   };
   const T* m = &mu[(ty + 1) * W + lx];
   const C mv = pairp(m), c = pairp(at(0, ly, lx));
-  const C m2 = vsplat<C>(T(-2));
   C d = vmul(vfma(mv, m2, xsum(m[-1], mv, m[2])), vsplat<C>(k.dc_d[0]));
   d = vfma(vfma(mv, m2, cadd(pairp(m - W), pairp(m + W))), vsplat<C>(k.dc_d[1]), d);
   const C cn = cadd(c, d);
@@ -134,9 +132,9 @@ __global__ void __launch_bounds__(FdTile<T>::THREADS) fs_fd_kernel(KArgs a, cons
   for (int f = 1; f < NF; ++f) {
     const T* ep = at(f, ly, lx);
     const C e = pairp(ep);
-    C r = eta_rate(k, chem, e, S2);
-    r = vfma(xsum(ep[-1], e, ep[2]), vsplat<C>(k.de_d[0]), r);
-    r = vfma(cadd(pairp(ep - W), pairp(ep + W)), vsplat<C>(k.de_d[1]), r);
+    C r = eta_rate<NF>(k, chem, e, S2);
+    r = vfma(vfma(e, m2, xsum(ep[-1], e, ep[2])), vsplat<C>(k.de_d[0]), r);
+    r = vfma(vfma(e, m2, cadd(pairp(ep - W), pairp(ep + W))), vsplat<C>(k.de_d[1]), r);
     const C en = cadd(e, r);
     chk.add(en);
     store(f, en);
@@ -176,9 +174,8 @@ struct Vec3 {
     memcpy(&w, v, 16);
     *reinterpret_cast<int4*>(p) = w;
   }
-  // acc + sum_d w_d (sum of the two neighbours along d, DIFF: less twice the
-  // value) of field f, whose values at the vector are v
-  template <bool DIFF>
+  // acc + sum_d w_d (sum of the two neighbours along d less twice the value) of
+  // field f, whose values at the vector are v
   __device__ __forceinline__ void neighbours(const T* f, const C (&v)[NC], const T (&w)[3],
                                              C (&acc)[NC]) const {
     C a0[NC], a1[NC], b0[NC], b1[NC];
@@ -192,10 +189,7 @@ struct Vec3 {
       C s[3] = {xsum(q == 0 ? l : v[q - 1].y, v[q], q == NC - 1 ? r : v[q + 1].x), cadd(a0[q], a1[q]),
                 cadd(b0[q], b1[q])};
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        if (DIFF) s[d] = vfma(v[q], vsplat<C>(T(-2)), s[d]);
-        acc[q] = vfma(s[d], vsplat<C>(w[d]), acc[q]);
-      }
+      for (int d = 0; d < 3; ++d) acc[q] = vfma(vfma(v[q], vsplat<C>(T(-2)), s[d]), vsplat<C>(w[d]), acc[q]);
     }
   }
 };
@@ -227,18 +221,18 @@ __global__ void __launch_bounds__(256) fs_fd3_mu_eta_kernel(KArgs a, const T* in
       h = pw.add_h2(e[f][q], h);
       S2[q] = vfma(e[f][q], e[f][q], S2[q]);
     }
-    m[q] = vfma(c[q], vsplat<C>(k.mu_c), vfma(h, vsplat<C>(k.fc_h), vsplat<C>(k.fc_0)));
+    m[q] = pw.fc2(c[q], h);
     chem[q] = vfma(c[q], vsplat<C>(k.g_c), vsplat<C>(k.g_0));
   }
-  g.template neighbours<false>(in, c, k.mu_d, m);
+  g.neighbours(in, c, k.mu_d, m);
   V3::store(mu + g.c, m);
   FiniteCheck<T> chk;
 #pragma unroll
   for (int f = 1; f < NF; ++f) {
     C r[NC];
 #pragma unroll
-    for (int q = 0; q < NC; ++q) r[q] = eta_rate(k, chem[q], e[f][q], S2[q]);
-    g.template neighbours<false>(in + f * N, e[f], k.de_d, r);
+    for (int q = 0; q < NC; ++q) r[q] = eta_rate<NF>(k, chem[q], e[f][q], S2[q]);
+    g.neighbours(in + f * N, e[f], k.de_d, r);
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       r[q] = cadd(e[f][q], r[q]);
@@ -266,7 +260,7 @@ __global__ void __launch_bounds__(256) fs_fd3_c_kernel(KArgs a, const T* in, T* 
   V3::load(mu + g.c, m);
 #pragma unroll
   for (int q = 0; q < NC; ++q) d[q] = vsplat<C>(T(0));
-  g.template neighbours<true>(mu, m, k.dc_d, d);
+  g.neighbours(mu, m, k.dc_d, d);
   FiniteCheck<T> chk;
 #pragma unroll
   for (int q = 0; q < NC; ++q) {

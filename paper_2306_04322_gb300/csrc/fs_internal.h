@@ -26,25 +26,23 @@ struct Coef {
   // pointwise stage with the constants multiplied out (Pointwise::fc2, g2)
   T fc_c, fc_0, fc_h, g_c, g_0, g_dw, g_pair;
   // explicit FD scheme with the constants multiplied out (fill_fd)
-  T mu_c, mu_d[3], dc_d[3], de_c, de_d[3];
+  T mu_d[3], dc_d[3], de_d[3];
 };
 
 // Stencil weights of the explicit FD scheme, formed in FP64, with l_d the sum
 // of a point's two neighbours along axis d and i_d = 1 / dx_d^2 (0 for an
 // axis the grid does not have):
-//   mu      = mu_c c + fc_0 + fc_h h + sum_d mu_d l_d(c)       (df/dc - kappa_c lap c)
+//   mu      = df/dc + sum_d mu_d (l_d(c) - 2 c)                (df/dc - kappa_c lap c)
 //   c'   - c   = sum_d dc_d (l_d(mu) - 2 mu)                   (dt M lap mu)
-//   eta' - eta = de_c eta + sum_d de_d l_d(eta) + (pointwise)  (dt L kappa_eta lap eta, ...)
-// The c update keeps the differences: a centre weight of its own, rounded by
-// itself, leaves a residue of the weights' sum (1e-9 in FP32) times mu in every
-// step, a steady drift of the mean of c, where the differences give nothing on a
-// uniform mu.  One operation per axis more.
+//   eta' - eta = (pointwise) + sum_d de_d (l_d(eta) - 2 eta)   (dt L kappa_eta lap eta, ...)
+// The differences stay, an operation per axis, field and point.  One weight for
+// the centre, rounded by itself, saves it, but leaves a residue of the weights'
+// sum (1e-9 in FP32) times mu in c at every step -- a steady drift of its mean,
+// where the differences give nothing on a uniform mu -- and rounds at the size
+// of the values where the differences are small: error against 64 bits after 32
+// steps of 64^3, FP64 8.7e-17 with differences, 1.4e-16 without.
 template <typename T>
-inline void fill_fd(Coef<T>& k, double rho2, double kappa_c, double kappa_eta, double dtM, double dtL,
-                    const double (&i)[3]) {
-  const double sum = 2.0 * (i[0] + i[1] + i[2]);
-  k.mu_c = (T)(2.0 * rho2 + kappa_c * sum);
-  k.de_c = (T)(-dtL * kappa_eta * sum);
+inline void fill_fd(Coef<T>& k, double kappa_c, double kappa_eta, double dtM, double dtL, const double (&i)[3]) {
   for (int d = 0; d < 3; ++d) {
     k.mu_d[d] = (T)(-kappa_c * i[d]);
     k.dc_d[d] = (T)(dtM * i[d]);

@@ -257,7 +257,7 @@ void fill_coef(fs::Coef<T>& k, const fs_params& q, double scale) {
   fs::fill_pointwise(k, q.rho2, q.c_alpha, q.c_beta, q.w, q.alpha, q.L * q.dt);
   const double i2[3] = {1.0 / (q.dx[0] * q.dx[0]), 1.0 / (q.dx[1] * q.dx[1]),
                         q.ndim > 2 ? 1.0 / (q.dx[2] * q.dx[2]) : 0.0};
-  fs::fill_fd(k, q.rho2, q.kappa_c, q.kappa_eta, q.dt * q.M, q.dt * q.L, i2);
+  fs::fill_fd(k, q.kappa_c, q.kappa_eta, q.dt * q.M, q.dt * q.L, i2);
 }
 
 fs::KArgs make_args(const fs_plan* p, const Member& m, int mode) {

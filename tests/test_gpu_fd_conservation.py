@@ -1,7 +1,7 @@
-"""The explicit scheme adds a multiple of lap(mu) to c, which is nothing where
-mu is uniform: a uniform state keeps its c bit for bit, however small c is
-against mu (a residue r of the stencil weights' sum would move it by r mu in
-every step: 1e-9 in FP32 against the 6e-11 of a last place of c = 1e-3)."""
+"""The Laplacians of the explicit scheme are nothing on a uniform field: a
+uniform state keeps its c bit for bit, however small c is against mu (a residue r
+of the stencil weights' sum would move it by r mu in every step: 1e-9 in FP32
+against the 6e-11 of a last place of c = 1e-3), and its eta where f_chem is 0."""
 import numpy as np
 import pytest
 
@@ -39,6 +39,23 @@ def test_uniform_state_keeps_c(F, n, dx, p, precision, c0):
     got = plan.get_fields()
     plan.close()
     assert torch.equal(got[0], t[0]), float((got[0].double() - t[0].double()).abs().max())
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+@pytest.mark.parametrize("n,dx", [((64, 16), (1.0, 0.8)), ((16, 8, 8), (1.0, 0.8, 0.9)), ((8, 16, 8), (1.0, 1.0, 1.0))])
+def test_uniform_state_without_reaction_stays(F, n, dx, precision):
+    """f_chem = 0: only the Laplacians are left, nothing on a uniform state at
+    any dt (a stencil that rounds its centre apart moves it at a large one)."""
+    import torch
+    pr = I.Problem(n=n, dx=dx, p=3, rho2=0.0, w=0.0)
+    pr.dt = 1000.0
+    t = torch.full((4,) + pr.shape, 0.3, dtype=torch.float32 if precision == "f32" else torch.float64, device="cuda")
+    plan = F.Plan(pr, precision, scheme=F.FS_SCHEME_EXPLICIT_FD)
+    plan.set_fields(t)
+    plan.step(3)
+    got = plan.get_fields()
+    plan.close()
+    assert torch.equal(got, t), float((got.double() - t.double()).abs().max())
 
 
 @pytest.mark.parametrize("n,dx", [((64, 64), (1.0, 0.8)), ((32, 32, 32), (1.0, 0.8, 0.9))])
