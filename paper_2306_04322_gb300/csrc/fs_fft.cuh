@@ -11,7 +11,7 @@
 // last pass leaves its results in the same stride-TPL order, so a line FFT of
 // P passes costs P - 1 shared-memory round trips and no global traffic.
 //
-// Twiddles: per-pass tables built on the host in long double, laid out
+// Twiddles: per-pass tables built on the host from long double roots, laid out
 // [pass][q][j] (q = 0..R/2-1, j = 0..NS-1): the roots of the pass's radix-2
 // stages with the pass twiddle folded in (fused_dft), so that the lanes of a
 // warp, which hold consecutive j, read consecutive entries.  Kernels copy the
@@ -19,6 +19,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <cmath>
 #include <stdint.h>
 
 namespace fs {
@@ -134,6 +135,19 @@ __device__ __forceinline__ double cos32(int j) {
   }
 }
 __device__ __forceinline__ double sin32(int j) { return cos32(8 - j); }
+// tan(2 pi j / 32), j = 1..7
+__device__ __forceinline__ double tan32(int j) {
+  switch (j) {
+    case 1: return 0.19891236737965800691159762264468;
+    case 2: return 0.41421356237309504880168872420970;
+    case 3: return 0.66817863791929891999775768652308;
+    case 4: return 1.0;
+    case 5: return 1.49660576266548901760113513494234;
+    case 6: return 2.41421356237309504880168872420970;
+    case 7: return 5.02733949212584810451497507106407;
+    default: return 0.0;
+  }
+}
 
 // Multiply a by exp(DIR * 2 pi i * k / len) for compile-time-known k / len
 // (after unrolling), len <= 32.  Trivial roots avoid multiplies.
@@ -161,27 +175,24 @@ __device__ __forceinline__ C twiddle_small(C a, int k, int len) {
 }
 
 // Radix-2 butterfly with the root folded in: u' = u + w v, v' = u - w v with
-// w = (wx, DIR < 0 ? wy : -wy).  FP64: u' = (u + swap(v) (-wy, wy)) + v (wx, wx)
-// by fused multiply-adds and v' = 2 u - u' by two more, 6 instructions against
-// 8 for the product followed by two additions.  FP32: four packed instructions
-// -- the swap, the broadcasts and the sign changes are operand modifiers --
-// against four scalar and two packed ones.  (FP32 keeps the product apart: in
-// fields that are a mean plus a little, u is large and v small, and the FP64
-// form rounds twice at the size of u; it cost a packed instruction less but
-// doubled the error against 64 bits at 1024^2, 1.1e-6 against 5e-7.)
+// w = wx (1 + i r), r = wy / wx (DIR > 0: conj w).  The product is scaled by wx
+// in the additions themselves: s = v + i r v by one fused multiply-add per part,
+// then u' = u + wx s and v' = u - wx s by another each (the form of Linzer and
+// Feig): 6 instructions per butterfly against 8 for the product followed by two
+// additions, in FP32 three packed ones -- the swap, the broadcasts and the sign
+// changes are operand modifiers.  Every output is rounded once at its own size
+// and once, in s, at the size of w v (however large |r|: wx shrinks with it).
+// Transforms of white noise, forward and back, relative error in units of 2^-53
+// (FP32 2^-24) sqrt(radix-2 stages): 0.52 to 0.54 (0.55 to 0.58), where
+// v' = 2 u - u' after two fused steps to u' gave 0.60 to 0.65 in FP64 and the
+// product apart 0.67 to 0.74 in FP32, at 6 and 4 instructions.
 template <int DIR, typename C>
-__device__ __forceinline__ void fused_bfly(C& u, C& v, decltype(C::x) wx, decltype(C::x) wy0) {
+__device__ __forceinline__ void fused_bfly(C& u, C& v, decltype(C::x) wx, decltype(C::x) r0) {
   using T = decltype(C::x);
-  const T wy = DIR < 0 ? wy0 : -wy0;
-  if constexpr (sizeof(T) == 8) {
-    const C x = vfma(v, vsplat<C>(wx), vfma(mk<C>(v.y, v.x), mk<C>(-wy, wy), u));
-    v = vfma(u, vsplat<C>(T(2)), mk<C>(-x.x, -x.y));
-    u = x;
-  } else {
-    const C t = vfma(v, vsplat<C>(wx), vmul(mk<C>(v.y, v.x), mk<C>(-wy, wy)));
-    v = csub(u, t);
-    u = cadd(u, t);
-  }
+  const T r = DIR < 0 ? r0 : -r0;
+  const C s = vfma(mk<C>(v.y, v.x), mk<C>(-r, r), v);
+  v = vfma(s, vsplat<C>(-wx), u);
+  u = vfma(s, vsplat<C>(wx), u);
 }
 
 // In-register DFT of length R (R <= 32) on a[0], a[S], ..., a[(R-1) S],
@@ -225,7 +236,7 @@ __device__ __forceinline__ void reg_dft(C* a) {
             using T = decltype(C::x);
             const int j = k * 32 / len;  // angle -2 pi j / 32, 0 < j < 16
             fused_bfly<DIR>(t[i + k], t[i + k + len / 2], (T)(j < 8 ? cos32(j) : -cos32(16 - j)),
-                            (T)(j < 8 ? -sin32(j) : -sin32(16 - j)));
+                            (T)(j < 8 ? -tan32(j) : tan32(16 - j)));
             continue;
           }
           C u = t[i + k], v = t[i + k + len / 2];
@@ -246,10 +257,13 @@ __device__ __forceinline__ void reg_dft(C* a) {
 // nothing beyond the stages' own fused butterflies: 3 instructions per value
 // and stage (FP32 1.5), against 3.5 to 3.6 for a separate twiddle product at
 // radix 8 or 16.  The FP64 passes are bound by the FP64 pipe, so fewer
-// instructions are less time: 1024^2, p = 2, a step 596 us against 652 us;
-// 64^3, p = 4, 290 us against 305 us.  FP32 (folded twiddles, packed products): 1024^2, p = 2, 25.4 us against 27.4; 2048^2, p = 4, 139 us against 143.  Roots with k >= len / 4 are -+i times those of k - len / 4.  tw: the
-// R / 2 roots of this j, NS entries apart, stage 2 first (stages of length
-// len = 2, 4, 8, 16 hold 1, 1, 2, 4).
+// instructions are less time.  Per step, separate twiddles / folded: 1024^2,
+// p = 2, FP64 652 / 596 us (when the rows were still half-length ones), 64^3,
+// p = 4, 305 / 290; FP32 1024^2, p = 2, 27.4 / 25.4 with the product apart in
+// every butterfly (four packed instructions), 23.8 / 22.8 for those four against
+// the three of fused_bfly, 2048^2, p = 4, 140 / 135.  Roots with k >= len / 4 are
+// -+i times those of k - len / 4.  tw: the R / 2 entries (bfly_entry) of this j, NS
+// apart, stage 2 first (stages of length len = 2, 4, 8, 16 hold 1, 1, 2, 4).
 template <int R, int DIR, int S, int NS, typename C>
 __device__ __forceinline__ void fused_dft(C* a, const C* __restrict__ tw) {
   constexpr int B = ilog2(R);
@@ -295,6 +309,22 @@ __host__ inline void stage_root(int q, int j, int ns, long long* num, long long*
   }
   *num = j + (long long)k * ns;
   *den = (long long)ns * len;
+}
+// Table entry (wx, r = wy / wx) of the root w = re + i (im + im_lo) for
+// fused_bfly, as it will be rounded to T: r belongs to the rounded wx, so that
+// wx r is wy to half a last place.  The one root without a real part, w = -i, takes
+// 2^-30 (FP64 2^-60) for it, far below a last place of the product; its s stays in
+// range for values up to 2^97 (FP64 2^963).
+template <typename T>
+__host__ inline void bfly_entry(double re, double im, double im_lo, double* wx, double* r) {
+  if (std::fabs(re) < 1e-15) {
+    *r = std::ldexp(-1.0, sizeof(T) == 4 ? 30 : 60);
+    *wx = im / *r;
+    return;
+  }
+  const double c = (double)(T)re, q = im / c;
+  *wx = c;
+  *r = (double)(T)(q + (std::fma(-q, c, im) + im_lo) / c);
 }
 // offset (in complex entries) of the table of the pass starting at NS
 template <int L, int E, int NS>

@@ -133,7 +133,7 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
       fc[u] = pw.fc2(c[u], h);
       chk.add(fc[u]);
 #pragma unroll
-      for (int i = 0; i < P; ++i) g[u][i] = pw.g2(c[u], e[u][i], S2);
+      for (int i = 0; i < P; ++i) g[u][i] = pw.template g2<P == 1>(c[u], e[u][i], S2);
     }
     bad |= chk.bad();
 #pragma unroll

@@ -44,7 +44,7 @@ namespace fs {
 // ---------------------------------------------------------------------------
 template <typename T>
 struct Pointwise {
-  T two_rho2, ca, dcab, rho2dcab, cab, w, four_alpha, Ldt;
+  T two_rho2, ca, dcab, rho2dcab, cab, w, four_alpha;
   T fc_c, fc_0, fc_h, g_c, g_0, g_dw, g_pair;  // constants multiplied out (fill_pointwise)
   __device__ explicit Pointwise(const KArgs& a) {
     const Coef<T>& k = coef<T>(a);
@@ -62,7 +62,6 @@ struct Pointwise {
     cab = k.cab;
     w = k.w;
     four_alpha = k.four_alpha;
-    Ldt = k.Ldt;
   }
   __device__ __forceinline__ T hpoly(T e) const { return e * e * e * (e * (T(6) * e - T(15)) + T(10)); }
   // df/dc and df/deta_i term by term, every rounding spelt out: the FP32
@@ -92,13 +91,15 @@ struct Pointwise {
   __device__ __forceinline__ V fc2(V c, V h) const {  // 2 rho2 (c - c_a - (c_b - c_a) h)
     return vfma(h, vsplat<V>(fc_h), vfma(c, vsplat<V>(fc_c), vsplat<V>(fc_0)));
   }
-  // g = eta - L dt df/deta
-  template <typename V>
+  // g = eta - L dt df/deta; SOLE: the only eta, whose sum over the others is
+  // empty (S2 - eta^2 would leave the rounding of a square)
+  template <bool SOLE = false, typename V>
   __device__ __forceinline__ V g2(V c, V e, V S2) const {
     const V ne = mk<V>(-e.x, -e.y);
     const V q = vfma(e, ne, e);                                               // e (1 - e)
     const V chem = vfma(c, vsplat<V>(g_c), vsplat<V>(g_0));                   // h'(e) = 30 q^2
     const V in = vfma(chem, q, vfma(e, vsplat<V>(T(-2) * g_dw), vsplat<V>(g_dw)));
+    if (SOLE) return vfma(q, in, e);
     return vfma(q, in, vfma(vmul(e, vsplat<V>(g_pair)), vfma(e, ne, S2), e));  // S2 - e^2 >= 0 first
   }
 };
@@ -272,7 +273,7 @@ __device__ __forceinline__ void row_pointwise_fixed(const Pointwise<T>& pw, cplx
       fc[u] = pw.fc2(c[u], h);
       chk += fc[u].x + fc[u].y;  // non-finite whenever any input is (see the runtime loop)
 #pragma unroll
-      for (int i = 0; i < P; ++i) gv[u][i] = pw.g2(c[u], e[u][i], S2);
+      for (int i = 0; i < P; ++i) gv[u][i] = pw.template g2<P == 1>(c[u], e[u][i], S2);
     }
     bad |= !finite_val(chk);
 #pragma unroll
@@ -471,7 +472,7 @@ __device__ __forceinline__ void row_compute(const KArgs& a, long long rb, cplx<T
         slot(nf, r)[i0] = fc;
         for (int i = 0; i < p; ++i) {
           const C e = slot(1 + i, r)[i0];
-          slot(1 + i, r)[i0] = pw.g2(c, e, S2);
+          slot(1 + i, r)[i0] = p == 1 ? pw.template g2<true>(c, e, S2) : pw.g2(c, e, S2);
         }
       }
     }
@@ -589,10 +590,12 @@ struct KUpdate {
   }
   // x / y for the denominators above (y >= 1): FP32 through the fast
   // reciprocal (2 ulp, as the warp-per-column pass); FP64 through the
-  // approximate reciprocal and one third-order Householder step
-  // r (1 + e + e^2), e = 1 - y r (about 2 ulp; four FP64 instructions where a
-  // rounded division takes twice that, of a pass bound by the FP64 pipe).
-  // Denominators near the end of the exponent range, infinite or NaN divide.
+  // approximate reciprocal (2^-20) and one third-order Householder step
+  // r (1 + e + e^2), e = 1 - y r: four FP64 instructions where a division takes
+  // twice that, of a pass bound by the FP64 pipe.  e^3 is 2^-60, so for x a power
+  // of two (the scales, and 1) the result is the rounded quotient but for one
+  // in 2700, next to a tie, that is a last place off.  Denominators near the end
+  // of the exponent range, infinite or NaN divide.
   __device__ __forceinline__ static T quot(T x, T y) {
     if constexpr (sizeof(T) == 4) {
       return __fdividef(x, y);

@@ -765,45 +765,68 @@ TableLayout table_layout(const fs_params& prm, bool f64) {
 
 size_t member_table_bytes(const fs_params& prm, bool f64) { return table_layout(prm, f64).total; }
 
-// Roots exp(-2 pi i k / n), 0 <= k < n, n a power of two up to 2048: every
-// table of a plan looks its entries up here.  Only the octant 0 <= k <= n / 8
-// is computed, in double at the rounded angle and corrected to first order
-// for the rounding (the angle as an unevaluated sum of two doubles); the rest
-// follows by symmetry.  (A cosl and a sinl for every entry of every table took
-// two thirds of fs_plan_create where long double is software.)
+// cos and sin of 2 pi k / 2048 for the octant k <= 256, as hi + lo: the roots of
+// unity every table is made of, computed in long double (software on some hosts: 60
+// us, once per process).
+struct Octant {
+  static constexpr int kN = 2048;
+  double c[kN / 8 + 1], s[kN / 8 + 1], cl[kN / 8 + 1], sl[kN / 8 + 1];
+  Octant() {
+    const long double two_pi = 2.0L * 3.141592653589793238462643383279502884L;
+    for (int k = 0; k <= kN / 8; ++k) {
+      const long double a = two_pi * ((long double)k / kN), ca = cosl(a), sa = sinl(a);
+      c[k] = (double)ca;
+      cl[k] = (double)(ca - (long double)c[k]);
+      s[k] = (double)sa;
+      sl[k] = (double)(sa - (long double)s[k]);
+    }
+  }
+};
+
+// Roots exp(-2 pi i k / n), 0 <= k < n, n a power of two from 8 to 2048, by the
+// octant's symmetry: every table of a plan looks its entries up here.
 struct Roots {
   int n;
-  std::vector<double> re, im;
-  explicit Roots(int n_) : n(n_ < 8 ? 8 : n_), re(n), im(n) {
-    const long double two_pi = 2.0L * 3.141592653589793238462643383279502884L;
-    const double hi = (double)two_pi, lo = (double)(two_pi - (long double)hi);
-    std::vector<double> c(n / 8 + 1), s(n / 8 + 1);
-    for (int k = 0; k <= n / 8; ++k) {
-      const double f = (double)k / n;  // exact
-      const double a = hi * f, e = std::fma(hi, f, -a) + lo * f;
-      c[k] = std::fma(-e, std::sin(a), std::cos(a));
-      s[k] = std::fma(e, std::cos(a), std::sin(a));
-    }
+  std::vector<double> re, im, im_lo;
+  explicit Roots(int n_) : n(n_ < 8 ? 8 : n_), re(n), im(n), im_lo(n) {
+    static const Octant o;
+    const int step = Octant::kN / n;
     for (int k = 0; k < n; ++k) {
-      const int q = k / (n / 4), r = k % (n / 4);  // quadrant, angle within it
-      const double cr = r <= n / 8 ? c[r] : s[n / 4 - r], sr = r <= n / 8 ? s[r] : c[n / 4 - r];
+      const int q = k / (n / 4), r = k % (n / 4);  // quadrant, place within it
+      const bool low = r <= n / 8;
+      const int m = (low ? r : n / 4 - r) * step;
+      const double cr = low ? o.c[m] : o.s[m], sr = low ? o.s[m] : o.c[m];
+      const double crl = low ? o.cl[m] : o.sl[m], srl = low ? o.sl[m] : o.cl[m];
       re[k] = q == 0 ? cr : q == 1 ? -sr : q == 2 ? -cr : sr;
-      im[k] = -(q == 0 ? sr : q == 1 ? cr : q == 2 ? -sr : -cr);
+      im[k] = q == 0 ? -sr : q == 1 ? -cr : q == 2 ? sr : cr;
+      im_lo[k] = q == 0 ? -srl : q == 1 ? -crl : q == 2 ? srl : crl;
     }
   }
   // exp(-2 pi i num / den), den a power of two dividing n
   void add(long long num, long long den, std::vector<double>& r, std::vector<double>& i) const {
-    const int k = (int)((num % den) * (n / den));
+    const int k = at(num, den);
     r.push_back(re[k]);
     i.push_back(im[k]);
   }
+  // the same as a butterfly's table entry (fs::bfly_entry)
+  void add_bfly(bool f64, long long num, long long den, std::vector<double>& r, std::vector<double>& i) const {
+    const int k = at(num, den);
+    double wx, t;
+    if (f64) fs::bfly_entry<double>(re[k], im[k], im_lo[k], &wx, &t);
+    else fs::bfly_entry<float>(re[k], im[k], im_lo[k], &wx, &t);
+    r.push_back(wx);
+    i.push_back(t);
+  }
+
+ private:
+  int at(long long num, long long den) const { return (int)((num % den) * (n / den)); }
 };
 
 // Stockham pass tables of a line FFT of length L with E values per thread:
 // for every pass after the first (sub-length NS, radix R = min(E, L/NS)),
 // entries [q][j], q < R / 2, j < NS: the roots of the pass's radix-2 stages
 // (fs::stage_root).
-void pass_table(const Roots& w, int L, int E, std::vector<double>& re, std::vector<double>& im) {
+void pass_table(const Roots& w, bool f64, int L, int E, std::vector<double>& re, std::vector<double>& im) {
   for (int ns = 1; ns < L;) {
     int r = E < L / ns ? E : L / ns;
     if (ns > 1)
@@ -811,7 +834,7 @@ void pass_table(const Roots& w, int L, int E, std::vector<double>& re, std::vect
         for (int j = 0; j < ns; ++j) {
           long long num, den;
           fs::stage_root(q, j, ns, &num, &den);
-          w.add(num, den, re, im);
+          w.add_bfly(f64, num, den, re, im);
         }
     ns *= r;
   }
@@ -860,15 +883,15 @@ cudaError_t upload_tables(Member& m, bool f64, char* dev, size_t bytes) {
   std::vector<double> rr, ii, wr, wi, cr, ci, zr, zi, hr, hi, r2r, r2i, c2r, c2i, r3r, r3i, c3r, c3i, m3r, m3i,
       arr, ari, acr, aci, azr, azi;
   const int er = row2_e(prm, f64), ec = col2_e(prm, f64);
-  if (er) pass_table(w, nx, er, r2r, r2i);
-  if (ec) pass_table(w, ny, ec, c2r, c2i);
-  if (row2w_form(prm, f64)) pass_table(w, nx, nx / 64, r3r, r3i);
-  if (col2w_form(prm, f64)) pass_table(w, ny, ny / 64, c3r, c3i);
-  if (row3_form(prm, f64)) pass_table(w, nx, 16, m3r, m3i);
-  pass_table(w, t.Lrow, t.Erow, rr, ii);
-  if (wide_rows(prm, f64)) pass_table(w, t.Lrow, 32, wr, wi);
-  pass_table(w, t.Lcol, t.Ecol, cr, ci);
-  if (nz > 1) pass_table(w, t.Lz, t.Ez, zr, zi);
+  if (er) pass_table(w, f64, nx, er, r2r, r2i);
+  if (ec) pass_table(w, f64, ny, ec, c2r, c2i);
+  if (row2w_form(prm, f64)) pass_table(w, f64, nx, nx / 64, r3r, r3i);
+  if (col2w_form(prm, f64)) pass_table(w, f64, ny, ny / 64, c3r, c3i);
+  if (row3_form(prm, f64)) pass_table(w, f64, nx, 16, m3r, m3i);
+  pass_table(w, f64, t.Lrow, t.Erow, rr, ii);
+  if (wide_rows(prm, f64)) pass_table(w, f64, t.Lrow, 32, wr, wi);
+  pass_table(w, f64, t.Lcol, t.Ecol, cr, ci);
+  if (nz > 1) pass_table(w, f64, t.Lz, t.Ez, zr, zi);
   for (int k = 0; k < nx / 2; ++k) w.add(k, nx, hr, hi);
   const bool adj = adj_tables(prm, f64);
   if (adj) {

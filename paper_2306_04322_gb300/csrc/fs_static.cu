@@ -70,9 +70,11 @@ size_t put_pass_table(T* dst, int L, int E) {
         for (int j = 0; j < ns; ++j) {
           long long num, den;
           fs::stage_root(q, j, ns, &num, &den);
-          long double ang = 2.0L * pi * (long double)(num % den) / (long double)den;
-          dst[2 * n] = (T)cosl(ang);
-          dst[2 * n + 1] = (T)(-sinl(ang));
+          const long double ang = 2.0L * pi * (long double)(num % den) / (long double)den, s = -sinl(ang);
+          double wx, r;
+          fs::bfly_entry<T>((double)cosl(ang), (double)s, (double)(s - (long double)(double)s), &wx, &r);
+          dst[2 * n] = (T)wx;
+          dst[2 * n + 1] = (T)r;
           ++n;
         }
     ns *= r;
