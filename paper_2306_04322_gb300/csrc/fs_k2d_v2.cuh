@@ -538,6 +538,9 @@ struct Col2Cfg {
   static constexpr int K2_BYTES = ((NY * (int)sizeof(T)) + 127) & ~127;
   static constexpr int HEAD = (128 + TW_BYTES + K2_BYTES + 255) & ~255;
   static constexpr size_t SMEM = HEAD + (size_t)NR * SLOT * CS;
+  // The 32-byte swizzle goes by the address bits 4 and 7, undone from the row
+  // in the tile (col2_body): every region on 256 bytes of a base on 256 bytes.
+  static_assert(!SWZ || (HEAD % 256 == 0 && SLOT * CS % 256 == 0 && BH * TK * CS % 256 == 0), "swizzled regions");
   // CTAs per SM the registers are budgeted for: FP32 128 per thread at 32
   // values, FP64 at least 64
   static constexpr int MIN_BLOCKS =
@@ -743,14 +746,14 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
 template <typename T, int NY, int G, int TK, int NR>
 __global__ void __launch_bounds__(Col2Cfg<T, NY, G, TK, NR>::THREADS, Col2Cfg<T, NY, G, TK, NR>::MIN_BLOCKS)
     fs_col2_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
+  extern __shared__ __align__(256) unsigned char col_smem[];  // Col2Cfg: regions on 256 bytes
+  uint64_t* bar = reinterpret_cast<uint64_t*>(col_smem);
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
   }
   __syncthreads();
-  col2_body<T, NY, G, TK, NR>(a, &tmap, blockIdx.x, blockIdx.y, smem_raw, bar, 0);
+  col2_body<T, NY, G, TK, NR>(a, &tmap, blockIdx.x, blockIdx.y, col_smem, bar, 0);
 }
 
 // Mixed CTAs of four lines each (FP32): {df/dc, c} of two columns first, then
@@ -758,16 +761,16 @@ __global__ void __launch_bounds__(Col2Cfg<T, NY, G, TK, NR>::THREADS, Col2Cfg<T,
 template <int NY, int G>
 __global__ void __launch_bounds__(128 * G, Col2Cfg<float, NY, G, 2, 2>::MIN_BLOCKS)
     fs_col2m_kernel(KArgs a, const __grid_constant__ CUtensorMap tmap2, const __grid_constant__ CUtensorMap tmap4) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
+  extern __shared__ __align__(256) unsigned char col_smem[];  // Col2Cfg: regions on 256 bytes
+  uint64_t* bar = reinterpret_cast<uint64_t*>(col_smem);
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
   }
   __syncthreads();
   const int n2 = a.nx / 4, n4 = a.nx / 8, b = (int)blockIdx.x - n2;
-  if (b < 0) col2_body<float, NY, G, 2, 2>(a, &tmap2, blockIdx.x, 0, smem_raw, bar, 0);
-  else col2_body<float, NY, G, 4, 1>(a, &tmap4, b % n4, 1 + b / n4, smem_raw, bar, 0);
+  if (b < 0) col2_body<float, NY, G, 2, 2>(a, &tmap2, blockIdx.x, 0, col_smem, bar, 0);
+  else col2_body<float, NY, G, 4, 1>(a, &tmap4, b % n4, 1 + b / n4, col_smem, bar, 0);
 }
 
 // Launchers: cudaErrorNotSupported when this form does not cover the
