@@ -318,8 +318,7 @@ struct AdjCoef {
     double v[2] = {w * r, w * g};
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+      v[q] = warp_sum(v[q]);
       if ((threadIdx.x & 31) == 0 && v[q] != 0.0) atomicAdd(&acc[2 * q + (f == 0 ? 0 : 1)], v[q]);
     }
   }

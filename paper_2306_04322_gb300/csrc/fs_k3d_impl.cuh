@@ -458,8 +458,7 @@ __global__ void __launch_bounds__(LineCfg<T, NZ>::THREADS, 4)
       sum += 2.0 * (kxy + kz2) * ((double)v[m].x * v[m].x + (double)v[m].y * v[m].y);
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  sum = warp_sum(sum);
   if ((threadIdx.x & 31) == 0) atomicAdd(&a.acc[1 + g], sum);
 }
 

@@ -131,6 +131,16 @@ __device__ __forceinline__ bool real_ok(const KArgs& a, const void* p, long long
   return in_bounds(a, p, bytes, a.real, a.real_bytes);
 }
 
+// Sum over the threads of a warp, in its first lane.  CTAs of fewer than 32
+// threads (a power of two: the line kernels on short axes) name only the lanes
+// they have: what a shuffle reads from a lane that does not exist is undefined.
+__device__ __forceinline__ double warp_sum(double v) {
+  const int width = blockDim.x < 32 ? (int)blockDim.x : 32;
+  const unsigned lanes = width < 32 ? (1u << width) - 1u : 0xffffffffu;
+  for (int o = width / 2; o > 0; o >>= 1) v += __shfl_down_sync(lanes, v, o, width);
+  return v;
+}
+
 template <typename T>
 __device__ __forceinline__ bool finite_val(T x) {
   return isfinite(x);
@@ -838,8 +848,7 @@ __global__ void __launch_bounds__(ColCfg<T, NY>::THREADS, 2)
       sum += 2.0 * (kx2 + ky2) * ((double)v[m].x * v[m].x + (double)v[m].y * v[m].y);
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  sum = warp_sum(sum);
   if ((threadIdx.x & 31) == 0) atomicAdd(&a.acc[1 + g], sum);
 }
 
