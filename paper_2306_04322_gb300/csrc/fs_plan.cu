@@ -1233,13 +1233,41 @@ fs_status fs_batch_create(const fs_params* each, int count, void* stream, fs_pla
   return create_common(each, count, stream, nullptr, nullptr, nullptr, out);
 }
 
+// End of the allocation that CUDA knows p to lie in (device, managed, pinned or
+// registered memory), NULL where it knows none (ordinary host memory).
+const char* allocation_end(const void* p) {
+  typedef CUresult (*AttributesFn)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const AttributesFn fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return reinterpret_cast<AttributesFn>(f);
+  }();
+  if (!fn) return static_cast<const char*>(p);  // unknown: an allocation of no length, nothing merges
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* to[2] = {&start, &size};
+  if (fn(2, what, to, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS || !start) return nullptr;
+  return reinterpret_cast<const char*>((uintptr_t)start) + size;
+}
+
 // Copies nf fields of n bytes each between the plan's contiguous field block
-// `dev` and the caller's nf pointers; runs of caller pointers that are
-// themselves contiguous go in one copy.
+// `dev` and the caller's nf pointers.  Fields that follow each other in one
+// allocation go in one copy; two allocations can be neighbours too, and a copy
+// across them is not promised to work.
 cudaError_t copy_fields(char* dev, const void* const* ptrs, int nf, size_t n, bool to_dev, cudaStream_t s) {
   for (int f = 0; f < nf;) {
+    const char* at = static_cast<const char*>(ptrs[f]);
     int g = f + 1;
-    while (g < nf && (const char*)ptrs[g] == (const char*)ptrs[g - 1] + n) ++g;
+    if (g < nf && ptrs[g] == at + n) {
+      const char* end = allocation_end(at);
+      while (g < nf && ptrs[g] == at + (g - f) * n &&
+             (end ? at + (g + 1 - f) * n <= end : !allocation_end(ptrs[g])))
+        ++g;
+    }
     cudaError_t e = to_dev ? cudaMemcpyAsync(dev + f * n, ptrs[f], (g - f) * n, cudaMemcpyDefault, s)
                            : cudaMemcpyAsync(const_cast<void*>(ptrs[f]), dev + f * n, (g - f) * n,
                                              cudaMemcpyDefault, s);
