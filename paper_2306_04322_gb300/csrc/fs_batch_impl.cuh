@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(128, RowCfg<T, 1024>::MIN_BLOCKS)
   const long long rb = item - begin[m];
   switch (a.nx) {
 #define FS_CASE(n) \
-  case n: row_body<T, n, false, true>(a, rb, smem_raw, bar, 0); break;
+  case n: row_body<T, n, false, true>(a, rb, smem_raw, bar); break;
     FS_BATCH_SIZES(FS_CASE)
 #undef FS_CASE
     default: break;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256, 2)
   const int g = rem / nt, bx = rem % nt;
   switch (a.ny) {
 #define FS_CASE(n) \
-  case n: col_body<T, n, TC_NONE, true>(a, &maps[m], bx, g, smem_raw, bar, 0); break;
+  case n: col_body<T, n, TC_NONE, true>(a, &maps[m], bx, g, smem_raw, bar); break;
     FS_BATCH_SIZES(FS_CASE)
 #undef FS_CASE
     default: break;

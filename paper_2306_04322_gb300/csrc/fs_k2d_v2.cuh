@@ -149,9 +149,9 @@ __device__ __forceinline__ void row2_pointwise_fixed(const Pointwise<T>& pw, cpl
 // per field (blockDim = 32 nf).  Field areas [nf][PL], one more in mode 1
 // (row2_smem_bytes): staging of the bulk copies, then the warp's exchange buffer (pad32
 // layout), then the pair values in natural order for the pointwise stage.
-// `bar` is an initialised mbarrier whose next phase has parity `parity`; the
-// ensemble kernel calls this once per work item.  Returns false if a bounded
-// wait gave up.  PC >= 0: the caller guarantees nf = PC + 1, and the
+// `bar` is an initialised mbarrier whose next phase has parity `parity` (the
+// fused step takes several items with one).  Returns false if a bounded wait
+// gave up.  PC >= 0: the caller guarantees nf = PC + 1, and the
 // pointwise stage is compiled for that p alone (the 96-thread kernel, whose
 // nf is 3: a kernel holding the code for every p measured slower there).
 // EARLY: see griddep_launch_dependents.
@@ -172,7 +172,7 @@ __device__ __forceinline__ bool row2_body(const KArgs& a, long long pair, unsign
   const bool from_real = (a.mode == 1);
 
   if (threadIdx.x == 0) {
-    // the ensemble kernel reuses the areas: order the previous item's generic
+    // the fused step reuses the areas: order the previous item's generic
     // accesses (ended by the caller's CTA barrier) before the bulk writes
     fence_proxy_async_smem();
     // both rows of a field are contiguous: NX complex (packed) or 2 NX reals
@@ -622,7 +622,7 @@ __device__ __forceinline__ bool col2_body(const KArgs& a, const CUtensorMap* tma
 
   if (r >= nreg) return true;  // the second region of a last group with one eta
   if (threadIdx.x == 0) {
-    // the ensemble kernel reuses the regions: order the previous item's
+    // the fused step reuses the regions: order the previous item's
     // generic accesses (ended by the caller's CTA barrier) before the TMA writes
     fence_proxy_async_smem();
     const uint32_t tbytes = (uint32_t)(Cfg::TWS * sizeof(C)), kbytes = (uint32_t)(NY * sizeof(T));

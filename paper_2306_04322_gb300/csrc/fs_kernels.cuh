@@ -491,12 +491,10 @@ __device__ __forceinline__ void row_compute(const KArgs& a, long long rb, cplx<T
   if (bad) atomicOr(a.flag, FS_FLAG_NONFINITE);
 }
 
-// One row-pass work item with its own table copy and load (ensemble kernel):
-// `bar` is an initialised mbarrier whose next phase has parity `parity`.
-// Returns false if a bounded wait gave up (the caller must stop).
+// One row-pass work item with its own table copy and load; `bar` is a fresh
+// mbarrier.  Returns false if a bounded wait gave up (the caller must stop).
 template <typename T, int NX, bool W = false, bool EARLY = false>
-__device__ __forceinline__ bool row_body(const KArgs& a, long long rb, unsigned char* smem_raw, uint64_t* bar,
-                                         uint32_t parity) {
+__device__ __forceinline__ bool row_body(const KArgs& a, long long rb, unsigned char* smem_raw, uint64_t* bar) {
   using C = cplx<T>;
   using Cfg = RowCfg<T, NX, W>;
   C* twr = reinterpret_cast<C*>(smem_raw + Cfg::BAR_BYTES);
@@ -506,16 +504,11 @@ __device__ __forceinline__ bool row_body(const KArgs& a, long long rb, unsigned 
   // everything above only touched constant tables; the spectra are the
   // previous pass's output
   griddep_wait();
-  if (threadIdx.x == 0) {
-    // the ensemble kernel reuses the slots: order the previous item's
-    // generic accesses (ended by the CTA barrier above) before the copies
-    fence_proxy_async_smem();
-    row_issue<T, NX, W>(a, rb, slots, bar);
-  }
+  if (threadIdx.x == 0) row_issue<T, NX, W>(a, rb, slots, bar);
   if (EARLY) griddep_launch_dependents();
-  if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
+  if (!mbar_wait_bounded(bar, 0, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
-    mbar_wait_bounded(bar, parity, kWaitPolls);  // let the copies land before exiting
+    mbar_wait_bounded(bar, 0, kWaitPolls);  // let the copies land before exiting
     return false;
   }
   row_compute<T, NX, W, EARLY>(a, rb, slots, slots + a.nf * Cfg::R * Cfg::PL, twr);
@@ -537,7 +530,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? RowCfg<T, NX, W>::MIN_BLOCK
     fence_mbar_init();
   }
   __syncthreads();
-  row_body<T, NX, W>(a, blockIdx.x, smem_raw, bar, 0);
+  row_body<T, NX, W>(a, blockIdx.x, smem_raw, bar);
 }
 
 // ---------------------------------------------------------------------------
@@ -632,7 +625,7 @@ constexpr size_t col_smem_bytes(int tk) {
 // the first radix-16 pass of each forward transform runs on tensor cores.
 template <typename T, int NY, int TCM = TC_NONE, bool EARLY = false>
 __device__ __forceinline__ bool col_body(const KArgs& a, const CUtensorMap* tmap, int bx, int g,
-                                         unsigned char* smem_raw, uint64_t* bar, uint32_t parity) {
+                                         unsigned char* smem_raw, uint64_t* bar) {
   using C = cplx<T>;
   using Cfg = ColCfg<T, NY>;
   constexpr int E = Cfg::E, TPL = Cfg::TPL, BH = Cfg::BH;
@@ -651,9 +644,6 @@ __device__ __forceinline__ bool col_body(const KArgs& a, const CUtensorMap* tmap
 
   if (threadIdx.x == 0) {
     griddep_wait();  // the tiles are the previous pass's output
-    // the ensemble kernel reuses the tiles: order the previous item's generic
-    // accesses (ended by the caller's CTA barrier) before the TMA writes
-    fence_proxy_async_smem();
     mbar_arrive_expect_tx(bar, (uint32_t)(nin * NY * tk * sizeof(C)));
     const int cx = kx0 * (int)(sizeof(C) / 8);  // innermost coordinate in 8-byte units
     for (int i = 0; i < nin; ++i) {
@@ -666,9 +656,9 @@ __device__ __forceinline__ bool col_body(const KArgs& a, const CUtensorMap* tmap
   griddep_wait();
   if (EARLY) griddep_launch_dependents();
   __syncthreads();
-  if (!mbar_wait_bounded(bar, parity, first_wait_polls(a))) {
+  if (!mbar_wait_bounded(bar, 0, first_wait_polls(a))) {
     if (threadIdx.x == 0) atomicOr(a.flag, FS_FLAG_TIMEOUT);
-    mbar_wait_bounded(bar, parity, kWaitPolls);
+    mbar_wait_bounded(bar, 0, kWaitPolls);
     return false;
   }
 
@@ -862,7 +852,7 @@ __global__ void __launch_bounds__(ColCfg<T, NY>::THREADS, 2)
     fence_mbar_init();
   }
   __syncthreads();
-  col_body<T, NY, TCM>(a, &tmap, blockIdx.x, blockIdx.y, smem_raw, bar, 0);
+  col_body<T, NY, TCM>(a, &tmap, blockIdx.x, blockIdx.y, smem_raw, bar);
 }
 
 }  // namespace fs
