@@ -45,10 +45,11 @@ __device__ __forceinline__ void hessian_apply(const Pointwise<T>& pw, const cplx
     const C q = vfma(e, ne, e);                                             // e (1 - e)
     const C hck = vmul(k(T(-30) * pw.two_rho2 * pw.dcab), vmul(q, q));      // H_c,i
     const C dw = vfma(q, k(T(-12)), k(T(2)));                               // 2 - 12 e + 12 e^2
-    const C well = vfma(vfma(e, ne, S2), k(pw.four_alpha), dw);             // + 4 alpha (S2 - e^2)
+    // + 4 alpha (S2 - e^2), the sum over the other etas (P = 1: there is none)
+    const C well = P == 1 ? dw : vfma(vfma(e, ne, S2), k(pw.four_alpha), dw);
     const C hkk = vfma(vmul(chem, q), vfma(e, k(T(-2)), k(T(1))), vmul(well, k(pw.w)));
     out[0] = vfma(hck, mu[i], out[0]);
-    const C cross = vmul(vmul(e, k(wa8)), vfma(ne, mu[i], em));             // sum over j != i
+    const C cross = P == 1 ? k(T(0)) : vmul(vmul(e, k(wa8)), vfma(ne, mu[i], em));  // sum over j != i
     out[i] = vfma(hck, mu[0], vfma(hkk, mu[i], cross));
   }
 }
@@ -149,7 +150,8 @@ __global__ void __launch_bounds__(96 * (P + 1)) fs_adj_row_fwd_kernel(KArgs a) {
         for (int i = 1; i < nf; ++i) {
           const C ne = mk<C>(-e[i].x, -e[i].y), q = vfma(e[i], ne, e[i]);
           const C in = vfma(chem, q, vfma(e[i], vsplat<C>(T(-2) * W), vsplat<C>(W)));
-          slot(2 * nf + i, r)[i0] = vfma(q, in, vmul(vmul(e[i], vsplat<C>(F)), vfma(e[i], ne, S2)));
+          slot(2 * nf + i, r)[i0] = P == 1 ? vmul(q, in)  // no other eta
+                                           : vfma(q, in, vmul(vmul(e[i], vsplat<C>(F)), vfma(e[i], ne, S2)));
         }
       }
     }
